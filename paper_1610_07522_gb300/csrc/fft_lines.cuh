@@ -183,6 +183,9 @@ constexpr int kLinesX = 64;         // most lines per block along x (smem staged
 //   cx<T> load(long long b, int idx) const;          element idx of array b
 //   void mid(cx<T>& v, long long b, int idx, int m) const;   after forward
 //   void store(long long b, int idx, cx<T> v) const;
+// or, when the store needs further loads, struct Extra, Extra extra(b, idx)
+// and store_with(b, idx, v, extra): the y / z pass loads the extras of
+// kExtraChunk points before it stores any of them.
 // idx is the point index within one array, m the position along the line.
 template <typename T, int N, class Op>
 __device__ __forceinline__ void process_line(const Op& op, cx<T>* v, long long b, int base,
@@ -192,6 +195,10 @@ __device__ __forceinline__ void process_line(const Op& op, cx<T>* v, long long b
   for (int m = 0; m < N; ++m) op.mid(v[m], b, base + m * stride, m);
   if constexpr (Op::kInv) Fft<T, N, true>::run(v);
 }
+
+constexpr int kExtraChunk = 8;      // extras in flight per thread (registers against round trips)
+template <class Op, class = void> struct HasExtra { static constexpr bool value = false; };
+template <class Op> struct HasExtra<Op, std::void_t<typename Op::Extra>> { static constexpr bool value = true; };
 
 // Lines along y (AXIS = 1) or z (AXIS = 2): one thread per line, direct loads.
 template <typename T, int N, int AXIS, class Op>
@@ -217,8 +224,21 @@ __global__ void __launch_bounds__(kLineThreads) k_line_yz(Op op, LineGeom g) {
 #pragma unroll
   for (int m = 0; m < N; ++m) v[m] = op.load(b, base + m * stride);
   process_line<T, N>(op, v, b, base, stride);
+  if constexpr (HasExtra<Op>::value) {
 #pragma unroll
-  for (int m = 0; m < N; ++m) op.store(b, base + m * stride, v[m]);
+    for (int m0 = 0; m0 < N; m0 += kExtraChunk) {
+      typename Op::Extra x[kExtraChunk];
+#pragma unroll
+      for (int k = 0; k < kExtraChunk; ++k)
+        if (m0 + k < N) x[k] = op.extra(b, base + (m0 + k) * stride);
+#pragma unroll
+      for (int k = 0; k < kExtraChunk; ++k)
+        if (m0 + k < N) op.store_with(b, base + (m0 + k) * stride, v[m0 + k], x[k]);
+    }
+  } else {
+#pragma unroll
+    for (int m = 0; m < N; ++m) op.store(b, base + m * stride, v[m]);
+  }
 }
 
 // Lines along x: a block stages blockDim.x (<= kLinesX) contiguous lines

@@ -490,6 +490,29 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_deriv(const DerivArgs a) {
       const int sc = E - 16 - 8 * (S - 1);
       constexpr int NBUF = Sh::NBUF;
       const int b = it % NBUF, use = it / NBUF;
+      // the epilogue's own operands (psi and w, or P) of a block of 4 points are
+      // loaded one block ahead, the first before the wait: behind the stores
+      // they would be a chain of round trips (24^3, 280 states: the step with
+      // its two such passes 905 us with the loads behind the stores, 840 us
+      // ahead of them)
+      constexpr bool AHEAD = OUT != kOutPlain;
+      double2 xp[4];
+      double xf[4];
+      auto ahead = [&](int cb) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int m = ((half * HALF + cb) >> 1) + c;
+          const bool on = l < a.nlines && m < N;
+          const long long at = lb + (long long)m * stride;
+          if constexpr (OUT == kOutUpdate) {
+            xp[c] = on ? __ldg(a.psi + at) : make_double2(0.0, 0.0);
+            xf[c] = on && a.w ? (double)__ldg(a.w + (at - bG)) : 1.0;
+          } else if constexpr (OUT == kOutScaleP) {
+            xf[c] = on ? __ldg(a.P + (at - bG)) : 0.0;
+          }
+        }
+      };
+      if constexpr (AHEAD) ahead(0);
       if (!mbar_wait(acc_full(b), (uint32_t)(use & 1))) {
         if (lane == 0) flag_status(a.status, SKY_ETIMEOUT);
         break;
@@ -518,6 +541,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_deriv(const DerivArgs a) {
           const int fx = __float2int_rn(__uint_as_float(v[4][c]) * 256.0f);
           acc[c] = ((long long)fu << 32) + ((long long)fw << 16) + (long long)fx;
         }
+        double2 cp[4];
+        double cf[4];
+        if constexpr (AHEAD) {
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            cp[c] = xp[c];
+            cf[c] = xf[c];
+          }
+          if (cb + 8 < HALF) ahead(cb + 8);
+        }
         if (l < a.nlines) {
 #pragma unroll
           for (int c = 0; c < 8; c += 2) {
@@ -529,12 +562,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_deriv(const DerivArgs a) {
               res.y = scaled_double(acc[c + 1], sc + s_eb[o + 1]);
               const long long at = lb + m * stride;
               if constexpr (OUT == kOutScaleP) {
-                const double f = a.P[at - bG] * a.scale;
+                const double f = cf[c >> 1] * a.scale;
                 res = make_double2(res.x * f, res.y * f);
               } else if constexpr (OUT == kOutUpdate) {
-                const double2 ps = a.psi[at];
+                const double2 ps = cp[c >> 1];
                 if (a.w) {
-                  const double f = (double)a.w[at - bG];
+                  const double f = cf[c >> 1];
                   res = make_double2(fma(-f, res.x, ps.x), fma(-f, res.y, ps.y));
                 } else {
                   res = make_double2(ps.x - res.x, ps.y - res.y);
