@@ -601,7 +601,13 @@ __global__ void k_hermitize(HermJobs h) {
 // describes.  Device gates per problem b at gate[8 b + k]: [0] Newton-Schulz
 // running, [1] eigendecomposition needed, [2] Newton-Schulz converged (one
 // final update pending or done), [3] Newton-Schulz chosen; [4..5] the row-sum
-// bound as integer bits; [6..7] ||S - I||_F^2 as a double.
+// bound as integer bits, after the choice [4] the blocks of k_ns_step that have
+// arrived and [5] the steps taken; [6..7] ||S - I||_F^2 as a double.
+//
+// Step k reads Y, Z from the buffers of parity k and writes the other ones,
+// so nothing is copied back; since skipped steps write nothing, the result is
+// in the buffer of parity [5].  The first step has Z = I: W = Z Y is S itself
+// and the new Z is T, so it takes one product instead of three.
 constexpr int kNsMaxIter = 14;
 constexpr double kNsSwitch = 2.5;      // spectral bound for the Newton-Schulz route
 constexpr double kNsFrob = 0.9;        // ||S - I||_F bound for the same route
@@ -613,11 +619,13 @@ struct NsJobs {
   double2* Y[kMaxBatch];
   double2* Z[kMaxBatch];
   double2* W[kMaxBatch];
-  double2* Yn[kMaxBatch];
-  double2* Zn[kMaxBatch];
+  double2* Zn[kMaxBatch];        // Z of odd parity
   double2* C[kMaxBatch];
   int n[kMaxBatch];
+  double* part;                  // per problem: part_stride partial sums of k_ns_step
+  size_t part_stride;
 };
+constexpr int kNsBlocks = 64;    // blocks per problem of k_ns_step at most
 
 __global__ void k_ns_reset(int* gate) {
   int* g = gate + 8 * threadIdx.x;
@@ -627,7 +635,7 @@ __global__ void k_ns_reset(int* gate) {
 }
 
 // Row sums of |S| (bounded by |Re| + |Im|) -> max into gate[4..5];
-// sum of |S - I|^2 -> gate[6..7]; Y = S, Z = I.
+// sum of |S - I|^2 -> gate[6..7]; Y = S.
 __global__ void __launch_bounds__(256) k_ns_rows(NsJobs j, int* gate) {
   __shared__ double red[8], red2[8];
   const int b = blockIdx.y, n = j.n[b], i = blockIdx.x;
@@ -640,7 +648,6 @@ __global__ void __launch_bounds__(256) k_ns_rows(NsJobs j, int* gate) {
     const double dr = v.x - (i == k ? 1.0 : 0.0);
     fro += dr * dr + v.y * v.y;
     j.Y[b][e] = v;
-    j.Z[b][e] = make_double2(i == k ? 1.0 : 0.0, 0.0);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -671,49 +678,74 @@ __global__ void k_ns_choose(int* gate) {
   g[0] = ns;
   g[1] = !ns;
   g[2] = 0;
+  g[4] = 0;
+  g[5] = 0;
 }
 
-// T = (3I - W)/2 in place of W = Z Y; records convergence; ends the
-// iteration one step after convergence was seen.  Block b serves problem b.
-__global__ void __launch_bounds__(1024) k_ns_step(NsJobs j, int* gate, long long* stats) {
-  __shared__ double red[32];
-  __shared__ int s_skip;
-  const int b = blockIdx.x, n = j.n[b];
-  int* g = gate + 8 * b;
-  if (threadIdx.x == 0) {
-    if (g[0] && g[2]) g[0] = 0;   // the final update has been applied
-    s_skip = !g[0];
-  }
-  __syncthreads();
-  if (s_skip) return;
-  if (threadIdx.x == 0) atomicAdd(reinterpret_cast<unsigned long long*>(stats + 5), 1ull);
-  double2* W = j.W[b];
-  double acc = 0.0;
-  for (long long e = threadIdx.x; e < (long long)n * n; e += blockDim.x) {
-    const int i = (int)(e / n), k = (int)(e % n);
-    double2 d = W[e];
-    if (i == k) d.x -= 1.0;                 // W - I
-    acc += d.x * d.x + d.y * d.y;
-    W[e] = make_double2((i == k ? 1.0 : 0.0) - 0.5 * d.x, -0.5 * d.y);   // I - (W - I)/2
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    if (sqrt(t) < kNsConv) g[2] = 1;
-  }
-}
-
-__global__ void k_ns_copy(NsJobs j, const int* gate) {
+// T = (3I - W)/2 in place of W = Z Y (first step: W = S, T also into the new
+// Z); records convergence; ends the iteration one step after convergence was
+// seen.  gridDim.x blocks share problem blockIdx.y; the last to arrive (a
+// counter, after every block has read the gates) adds the partial sums in
+// block order and moves the gates.  The pass is a few FP64 operations per
+// entry, bound by the FP64 rate of the SMs it runs on: one block per problem
+// took 243 us a step for 700 + 300 states; spread over the SMs and with the
+// first step's products saved, the case's Loewdin and diagonalisation went
+// from 27.6 to 23.5 ms.
+__global__ void __launch_bounds__(256) k_ns_step(NsJobs j, int* gate, long long* stats, int first) {
+  __shared__ double red[8];
+  __shared__ int s_last;
   const int b = blockIdx.y, n = j.n[b];
-  if (!gate[8 * b]) return;
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long long)n * n) return;
-  j.Y[b][e] = j.Yn[b][e];
-  j.Z[b][e] = j.Zn[b][e];
+  volatile int* g = gate + 8 * b;
+  const int g0 = g[0], g2 = g[2];
+  const bool run = g0 && !g2;
+  double acc = 0.0;
+  if (run) {
+    const double2* src = first ? j.Y[b] : j.W[b];
+    double2 *W = j.W[b], *Zn = j.Zn[b];
+    const unsigned nn = (unsigned)n * (unsigned)n, un = (unsigned)n;   // n < 2^16
+    for (unsigned e = blockIdx.x * 256u + threadIdx.x; e < nn; e += gridDim.x * 256u) {
+      const double one = (e / un == e % un) ? 1.0 : 0.0;
+      double2 d = src[e];
+      d.x -= one;                            // W - I
+      acc = fma(d.x, d.x, fma(d.y, d.y, acc));
+      const double2 t = make_double2(fma(-0.5, d.x, one), -0.5 * d.y);   // I - (W - I)/2
+      W[e] = t;
+      if (first) Zn[e] = t;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  }
+  __syncthreads();
+  double* part = j.part + (size_t)b * j.part_stride;
+  if (threadIdx.x == 0) {
+    if (run) {
+      double t = 0.0;
+      for (int w = 0; w < 8; ++w) t += red[w];
+      part[blockIdx.x] = t;
+    }
+    __threadfence();
+    s_last = atomicAdd(gate + 8 * b + 4, 1) == (int)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last || threadIdx.x >= 32) return;
+  __threadfence();
+  double t = 0.0;
+  if (run) {
+    for (int k = threadIdx.x; k < (int)gridDim.x; k += 32) t += __ldcg(part + k);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  }
+  if (threadIdx.x == 0) {
+    if (run) {
+      atomicAdd(reinterpret_cast<unsigned long long*>(stats + 5), 1ull);
+      g[5] = g[5] + 1;
+      if (sqrt(t) < kNsConv) g[2] = 1;
+    } else if (g0) {
+      g[0] = 0;                              // the final update has been applied
+    }
+    g[4] = 0;
+  }
 }
 
 // C = (Z + Z^H)/2 when Newton-Schulz converged; otherwise request the
@@ -733,21 +765,25 @@ __global__ void k_ns_final(NsJobs j, int* gate, long long* stats) {
   }
   if (e >= (long long)n * n) return;
   const int i = (int)(e / n), k = (int)(e % n);
-  j.C[b][e] = 0.5 * (j.Z[b][e] + conjx(j.Z[b][(long long)k * n + i]));
+  const double2* Z = (g[5] & 1) ? j.Zn[b] : j.Z[b];
+  j.C[b][e] = 0.5 * (Z[e] + conjx(Z[(long long)k * n + i]));
 }
 
 sky_status lowdin_batch(Ctx* c, int np, const double2* const* S, const int* I, double2* const* C) {
   if (np < 1) return SKY_OK;
   if (np > c->eig_batch) return set_err(c, SKY_EINVAL, "Loewdin batch %d > %d", np, c->eig_batch);
   NsJobs j;
+  double2* Yn[kMaxBatch];
   int nmax = 1;
   for (int b = 0; b < np; ++b) {
     const size_t off = (size_t)b * c->small_slot;
     j.S[b] = S[b]; j.n[b] = I[b]; j.C[b] = C[b];
     j.Y[b] = c->d_small[0] + off; j.Z[b] = c->d_small[1] + off; j.W[b] = c->d_small[2] + off;
-    j.Yn[b] = c->d_small[3] + off; j.Zn[b] = c->d_small[4] + off;
+    Yn[b] = c->d_small[3] + off; j.Zn[b] = c->d_small[4] + off;
     if (I[b] > nmax) nmax = I[b];
   }
+  j.part = c->d_eigpart;
+  j.part_stride = (size_t)2 * c->eig_grid_max;
   int* gate = c->d_gate;
   const long long nn = (long long)nmax * nmax;
   cudaError_t e;
@@ -762,18 +798,26 @@ sky_status lowdin_batch(Ctx* c, int np, const double2* const* S, const int* I, d
     fb[b] = gate + 8 * b + 1;
   }
   const int* none[kMaxBatch] = {nullptr};
+  // entries per block of k_ns_step: 1024 (four per thread), at most kNsBlocks
+  // blocks and as many as there are slots for partial sums
+  int step_blocks = (int)div_up(nn, 1024);
+  if (step_blocks > kNsBlocks) step_blocks = kNsBlocks;
+  if (step_blocks > 2 * c->eig_grid_max) step_blocks = 2 * c->eig_grid_max;
   for (int it = 0; it < kNsMaxIter; ++it) {
-    ZJobs w_ = zjobs(np, false, false, (const double2* const*)j.Z, (const double2* const*)j.Y, j.W, I, run, stop);
-    sky_status st = zgemm_batch(c, w_);   // W = Z Y
+    const bool odd = it & 1;
+    const double2* const* Y0 = (const double2* const*)(odd ? Yn : j.Y);
+    const double2* const* Z0 = (const double2* const*)(odd ? j.Zn : j.Z);
+    double2* const* Y1 = odd ? j.Y : Yn;
+    double2* const* Z1 = odd ? j.Z : j.Zn;
+    sky_status st;
+    if (it > 0 && (st = zgemm_batch(c, zjobs(np, false, false, Z0, Y0, j.W, I, run, stop))) != SKY_OK)
+      return st;                                                             // W = Z Y
+    k_ns_step<<<dim3(step_blocks, np), 256, 0, c->stream>>>(j, gate, c->d_stats, it == 0);
+    note_launch();
+    st = zgemm_batch(c, zjobs(np, false, false, Y0, (const double2* const*)j.W, Y1, I, run, none));   // Y T
+    if (st == SKY_OK && it > 0)
+      st = zgemm_batch(c, zjobs(np, false, false, (const double2* const*)j.W, Z0, Z1, I, run, none));   // T Z
     if (st != SKY_OK) return st;
-    k_ns_step<<<np, 1024, 0, c->stream>>>(j, gate, c->d_stats);
-    note_launch();
-    ZJobs y_ = zjobs(np, false, false, (const double2* const*)j.Y, (const double2* const*)j.W, j.Yn, I, run, none);
-    ZJobs z_ = zjobs(np, false, false, (const double2* const*)j.W, (const double2* const*)j.Z, j.Zn, I, run, none);
-    if ((st = zgemm_batch(c, y_)) != SKY_OK) return st;                      // Y T
-    if ((st = zgemm_batch(c, z_)) != SKY_OK) return st;                      // T Z
-    k_ns_copy<<<dim3(div_up(nn, 256), np), 256, 0, c->stream>>>(j, gate);
-    note_launch();
   }
   k_ns_final<<<dim3(div_up(nn, 256), np), 256, 0, c->stream>>>(j, gate, c->d_stats);
   note_launch();
@@ -836,22 +880,39 @@ struct PhaseJobs {
   double2* Z[kMaxBatch];
   int n[kMaxBatch];
 };
-__global__ void k_fix_phase(PhaseJobs j) {
+// 32 columns per block (coalesced rows), the rows dealt to its 8 warps; the
+// winners of the warps meet in shared memory, the lowest row first on ties
+// (one thread per column walking all rows: 331 us for 700 + 300 states, chains
+// of FP64 latency on six blocks).
+__global__ void __launch_bounds__(256) k_fix_phase(PhaseJobs j) {
+  __shared__ double s_max[8][32];
+  __shared__ int s_row[8][32];
   const int b = blockIdx.y, n = j.n[b];
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int k = blockIdx.x * 32 + lane;
   double2* Z = j.Z[b];
   int imax = 0;
   double amax = -1.0;
-  for (int i = 0; i < n; ++i) {
-    const double2 v = Z[(long long)i * n + k];
-    const double a = v.x * v.x + v.y * v.y;
-    if (a > amax) { amax = a; imax = i; }
+  if (k < n)
+    for (int i = w; i < n; i += 8) {
+      const double2 v = Z[(long long)i * n + k];
+      const double a = v.x * v.x + v.y * v.y;
+      if (a > amax) { amax = a; imax = i; }
+    }
+  s_max[w][lane] = amax;
+  s_row[w][lane] = imax;
+  __syncthreads();
+  for (int q = 0; q < 8; ++q) {
+    const double a = s_max[q][lane];
+    const int i = s_row[q][lane];
+    if (a > amax || (a == amax && i < imax)) { amax = a; imax = i; }
   }
-  const double2 z = Z[(long long)imax * n + k];
+  const double2 z = k < n ? Z[(long long)imax * n + k] : make_double2(1.0, 0.0);
+  __syncthreads();                         // every warp has read z before any row changes
+  if (k >= n) return;
   const double r = sqrt(z.x * z.x + z.y * z.y);
   const double2 ph = make_double2(z.x / r, -z.y / r);   // conj(z) / |z|
-  for (int i = 0; i < n; ++i) {
+  for (int i = w; i < n; i += 8) {
     const long long e = (long long)i * n + k;
     Z[e] = cmul(Z[e], ph);
   }
@@ -876,7 +937,7 @@ sky_status subspace_literal_batch(Ctx* c, int np, const double2* const* H,
     pj.n[b] = I[b];
     if (I[b] > nmax) nmax = I[b];
   }
-  k_fix_phase<<<dim3(div_up(nmax, 128), np), 128, 0, c->stream>>>(pj);
+  k_fix_phase<<<dim3(div_up(nmax, 32), np), 256, 0, c->stream>>>(pj);
   note_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_check(c, e, "fix phase");
