@@ -2,112 +2,262 @@
 // (Eq. Skyrme, Sec. 2.2, Eq. convergence).  Fields are FP64 for every
 // spinor precision; real-field derivatives are spectral with the plain
 // wavenumbers, real part kept.
-#include "fft_lines.cuh"
+#include <cmath>
+
+#include "sky_internal.cuh"
 
 namespace sky {
 
-sky_status upload_twiddles_fields(Ctx* c) {
-  return cuda_check(c, upload_twiddles_this_unit(), "twiddle upload (fields)");
-}
+// ------------------------------------------------------------ real-field operators
+// A spectral derivative of a real field along one axis is a real circulant
+// operator on its lines, Re IFFT[i k FFT[f]]_m = sum_q D1[(m - q) mod n] f_q,
+// and so is the second derivative:
+//   D1[r] = -(1/n) sum_a k_a sin(2 pi a r / n),  D2[r] = -(1/n) sum_a k_a^2 cos(2 pi a r / n).
+// The fields are small (8 kB to 2 MB, all in L2) and FP64, and on this chip a
+// dependent FP64 operation takes ~67 cycles, so an FFT with one thread per
+// line (400 lines at 20^3) was bound by that latency: 22-27 us for each axis
+// and derivative, 9 to 12 of them per call.  Here one thread per point sums
+// its 3 n terms directly, every derivative of both species in one launch,
+// with independent accumulators; the FP64 rate (2 per clock and SM) bounds it:
+// 12 n multiply-adds per point.  20^3: the nine passes of a mean field 215 us,
+// now 15; the three of a divergence 72 us, now 7.  Tables built once per
+// context in long double.
+// d_fop[axis]: [4][n] = D1, D2, cos(2 pi r / n), sin(2 pi r / n).
+constexpr int kFieldThreads = 64;    // small blocks: an 8^3 .. 24^3 field covers more SMs
+constexpr int kFieldMaxN = 64;
 
-// out (= or +=) Re IFFT[ mult FFT[in] ] along one axis; mult = i k (mode 0)
-// or -k^2 (mode 1), divided by N.
-struct OpRealD {
-  static constexpr bool kFwd = true, kInv = true;
-  const double* in; double* out; const double* k; double inv_n; int mode; int acc; long long G;
-  __device__ __forceinline__ double2 load(long long b, int i) const {
-    return make_double2(in[b * G + i], 0.0);
-  }
-  __device__ __forceinline__ void mid(double2& v, long long, int, int m) const {
-    if (mode == 0) {
-      const double kk = k[m] * inv_n;
-      v = make_double2(-kk * v.y, kk * v.x);
-    } else {
-      const double f = -k[m] * k[m] * inv_n;
-      v = make_double2(f * v.x, f * v.y);
+sky_status build_field_tables(Ctx* c) {
+  const long double two_pi = 6.283185307179586476925286766559005768L;
+  for (int j = 0; j < 3; ++j) {
+    const int n = c->n[j];
+    double t[4 * kFieldMaxN];
+    long double cs[kFieldMaxN], sn[kFieldMaxN];
+    for (int r = 0; r < n; ++r) {
+      cs[r] = cosl(two_pi * r / (long double)n);
+      sn[r] = sinl(two_pi * r / (long double)n);
     }
-  }
-  __device__ __forceinline__ void store(long long b, int i, double2 v) const {
-    out[b * G + i] = acc ? out[b * G + i] + v.x : v.x;
-  }
-};
-
-struct OpR2CFwd {   // real in -> complex, forward
-  static constexpr bool kFwd = true, kInv = false;
-  const double* in; double2* out; long long G;
-  __device__ __forceinline__ double2 load(long long b, int i) const { return make_double2(in[b * G + i], 0.0); }
-  __device__ __forceinline__ void mid(double2&, long long, int, int) const {}
-  __device__ __forceinline__ void store(long long b, int i, double2 v) const { out[b * G + i] = v; }
-};
-template <bool INV> struct OpCPass {
-  static constexpr bool kFwd = !INV, kInv = INV;
-  double2* a; long long G;
-  __device__ __forceinline__ double2 load(long long b, int i) const { return a[b * G + i]; }
-  __device__ __forceinline__ void mid(double2&, long long, int, int) const {}
-  __device__ __forceinline__ void store(long long b, int i, double2 v) const { a[b * G + i] = v; }
-};
-struct OpCoulX {    // forward x, times 4 pi e^2 / (G |k|^2), inverse x
-  static constexpr bool kFwd = true, kInv = true;
-  double2* a; const double* Pc; double scale; long long G;
-  __device__ __forceinline__ double2 load(long long b, int i) const { return a[b * G + i]; }
-  __device__ __forceinline__ void mid(double2& v, long long, int i, int) const {
-    const double f = Pc[i] * scale;
-    v = make_double2(f * v.x, f * v.y);
-  }
-  __device__ __forceinline__ void store(long long b, int i, double2 v) const { a[b * G + i] = v; }
-};
-struct OpC2RInv {   // inverse z, real part out
-  static constexpr bool kFwd = false, kInv = true;
-  const double2* a; double* out; long long G;
-  __device__ __forceinline__ double2 load(long long b, int i) const { return a[b * G + i]; }
-  __device__ __forceinline__ void mid(double2&, long long, int, int) const {}
-  __device__ __forceinline__ void store(long long b, int i, double2 v) const { out[b * G + i] = v.x; }
-};
-
-template <class Op>
-static cudaError_t run_pass(Ctx* c, int axis, const Op& op, long long nb) {
-  const int nx = c->n[0], ny = c->n[1], nz = c->n[2];
-  return dispatch_n<true>(c->n[axis], [&](auto NC) -> cudaError_t {
-    constexpr int N = decltype(NC)::value;
-    if (axis == 0) return launch_line<double, N, 0>(op, nx, ny, nz, nb, c);
-    if (axis == 1) return launch_line<double, N, 1>(op, nx, ny, nz, nb, c);
-    return launch_line<double, N, 2>(op, nx, ny, nz, nb, c);
-  });
-}
-
-// out = sum_axis (derivative or second derivative) of nb fields.
-static cudaError_t real_op_sum(Ctx* c, const double* in, double* out, long long nb, int mode) {
-  for (int ax = 0; ax < 3; ++ax) {
-    OpRealD op{in, out, c->d_kp[ax], 1.0 / c->n[ax], mode, ax > 0, (long long)c->G};
-    cudaError_t e = run_pass(c, ax, op, nb);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
-// divJ = sum_i d_i J_i for one [3][G] vector field.
-sky_status field_divergence(Ctx* c, const double* J, double* divJ) {
-  const long long G = c->G;
-  for (int ax = 0; ax < 3; ++ax) {
-    OpRealD op{J + ax * G, divJ, c->d_kp[ax], 1.0 / c->n[ax], 0, ax > 0, G};
-    cudaError_t e = run_pass(c, ax, op, 1);
-    if (e != cudaSuccess)
-      return set_err(c, SKY_ECUDA, "divergence (axis %d, n %d, blocks %d/%d): %s", ax, c->n[ax],
-                     c->line_x, c->line_yz, cudaGetErrorString(e));
+    for (int r = 0; r < n; ++r) {
+      long double d1 = 0.0L, d2 = 0.0L;
+      for (int a = 0; a < n; ++a) {
+        const int m = a < (n + 1) / 2 ? a : a - n;
+        const long double k = two_pi * m / (long double)c->L[j];
+        d1 -= k * sn[(a * r) % n];
+        d2 -= k * k * cs[(a * r) % n];
+      }
+      t[r] = (double)(d1 / n);
+      t[n + r] = (double)(d2 / n);
+      t[2 * n + r] = (double)cs[r];
+      t[3 * n + r] = (double)sn[r];
+    }
+    const cudaError_t e = cudaMemcpy(c->d_fop[j], t, 4 * n * sizeof(double), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return cuda_check(c, e, "field tables");
   }
   return SKY_OK;
+}
+
+struct FieldGeom {
+  int n[3];
+  int G;
+  const double* op[3];
+};
+static FieldGeom field_geom(const Ctx* c) {
+  FieldGeom g;
+  for (int j = 0; j < 3; ++j) {
+    g.n[j] = c->n[j];
+    g.op[j] = c->d_fop[j];
+  }
+  g.G = c->G;
+  return g;
+}
+
+// The point's position m along axis j, the line's first point and its stride.
+__device__ __forceinline__ void field_line(const FieldGeom& g, int p, int j, int& m, int& base, int& stride) {
+  const int nx = g.n[0], ny = g.n[1];
+  const int x = p % nx, t = p / nx, y = t % ny, z = t / ny;
+  stride = j == 0 ? 1 : j == 1 ? nx : nx * ny;
+  m = j == 0 ? x : j == 1 ? y : z;
+  base = p - m * stride;
+}
+
+// rho_T, Delta rho_T and (GRAD) d_j rho_T of both isospins T (the layout of
+// d_ftmp below).  The sums run over the two species (even and odd q apart:
+// eight independent chains with GRAD, four without) and combine at the end.
+template <bool GRAD>
+__global__ void __launch_bounds__(kFieldThreads) k_field_derivs(const double* __restrict__ rho,
+                                                                FieldGeom g, double* __restrict__ f) {
+  __shared__ double tab[3][2][kFieldMaxN];
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+    for (int i = threadIdx.x; i < 2 * g.n[j]; i += kFieldThreads)
+      tab[j][i >= g.n[j]][i >= g.n[j] ? i - g.n[j] : i] = g.op[j][i];
+  __syncthreads();
+  const int p = blockIdx.x * kFieldThreads + threadIdx.x, G = g.G;
+  if (p >= G) return;
+  double ln[2] = {0.0, 0.0}, lp[2] = {0.0, 0.0};
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    int m, base, stride;
+    field_line(g, p, j, m, base, stride);
+    const int n = g.n[j];
+    double gn[2] = {0.0, 0.0}, gp[2] = {0.0, 0.0};
+    int r = m;                              // (m - q) mod n
+#pragma unroll 2
+    for (int q = 0; q < n; q += 2) {        // n is even
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const double a = rho[base + (q + h) * stride], b = rho[G + base + (q + h) * stride];
+        const double d2 = tab[j][1][r];
+        ln[h] = fma(d2, a, ln[h]);
+        lp[h] = fma(d2, b, lp[h]);
+        if constexpr (GRAD) {
+          const double d1 = tab[j][0][r];
+          gn[h] = fma(d1, a, gn[h]);
+          gp[h] = fma(d1, b, gp[h]);
+        }
+        r = r == 0 ? n - 1 : r - 1;
+      }
+    }
+    if constexpr (GRAD) {
+      const double a = gn[0] + gn[1], b = gp[0] + gp[1];
+      f[(4 + 2 * j) * (long long)G + p] = a + b;
+      f[(5 + 2 * j) * (long long)G + p] = a - b;
+    }
+  }
+  const double a = ln[0] + ln[1], b = lp[0] + lp[1];
+  const double rn = rho[p], rp = rho[G + p];
+  f[p] = rn + rp;
+  f[G + p] = rn - rp;
+  f[2LL * G + p] = a + b;
+  f[3LL * G + p] = a - b;
+}
+
+// divJ = sum_j d_j J_j for one [3][G] vector field.
+__global__ void __launch_bounds__(kFieldThreads) k_field_div(const double* __restrict__ J, FieldGeom g,
+                                                             double* __restrict__ out) {
+  __shared__ double tab[3][kFieldMaxN];
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+    for (int i = threadIdx.x; i < g.n[j]; i += kFieldThreads) tab[j][i] = g.op[j][i];
+  __syncthreads();
+  const int p = blockIdx.x * kFieldThreads + threadIdx.x, G = g.G;
+  if (p >= G) return;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    int m, base, stride;
+    field_line(g, p, j, m, base, stride);
+    const int n = g.n[j];
+    const double* src = J + (long long)j * G;
+    int r = m;
+    for (int q = 0; q < n; q += 4) {        // n is a multiple of 4
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        acc[h] = fma(tab[j][r], src[base + (q + h) * stride], acc[h]);
+        r = r == 0 ? n - 1 : r - 1;
+      }
+    }
+  }
+  out[p] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+}
+
+sky_status field_divergence(Ctx* c, const double* J, double* divJ) {
+  k_field_div<<<div_up(c->G, kFieldThreads), kFieldThreads, 0, c->stream>>>(J, field_geom(c), divJ);
+  note_launch();
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess)
+    return set_err(c, SKY_ECUDA, "divergence (%d x %d x %d): %s", c->n[0], c->n[1], c->n[2],
+                   cudaGetErrorString(e));
+  return SKY_OK;
+}
+
+// Coulomb potential by the half spectrum of the real proton density: the DFT
+// along z for k_z = 0 .. n_z / 2 only (the rest are complex conjugates), then
+// y, x, times 4 pi e^2 / (G |k|^2), and back; the inverse along z takes k_z = 0
+// and n_z / 2 once and the others twice.  Direct sums with one thread per
+// output, for the same reason as above.
+// z forward (FWD: rho -> half spectrum) and inverse (half spectrum -> V).
+template <bool FWD>
+__global__ void __launch_bounds__(kFieldThreads) k_coul_z(const double* __restrict__ rho,
+                                                          double2* __restrict__ a,
+                                                          double* __restrict__ V, FieldGeom g) {
+  __shared__ double tc[kFieldMaxN], ts[kFieldMaxN];
+  const int n = g.n[2], np = g.n[0] * g.n[1];
+  for (int i = threadIdx.x; i < n; i += kFieldThreads) {
+    tc[i] = g.op[2][2 * n + i];
+    ts[i] = g.op[2][3 * n + i];
+  }
+  __syncthreads();
+  const int p = blockIdx.x * kFieldThreads + threadIdx.x;
+  const int h = n / 2 + 1;
+  if (p >= (FWD ? h : n) * np) return;
+  const int k = p / np, xy = p - k * np;
+  double s0[2] = {0.0, 0.0}, s1[2] = {0.0, 0.0};
+  int r = 0;                                // k q mod n
+  if constexpr (FWD) {
+    for (int q = 0; q < n; q += 2) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const double v = rho[(q + u) * np + xy];
+        s0[u] = fma(v, tc[r], s0[u]);
+        s1[u] = fma(-v, ts[r], s1[u]);
+        r += k;
+        if (r >= n) r -= n;
+      }
+    }
+    a[p] = make_double2(s0[0] + s0[1], s1[0] + s1[1]);
+  } else {
+    for (int q = 0; q < h; ++q) {
+      const double2 v = a[q * np + xy];
+      const double w = q == 0 || 2 * q == n ? 1.0 : 2.0;
+      s0[q & 1] = fma(w * v.x, tc[r], s0[q & 1]);
+      s1[q & 1] = fma(-w * v.y, ts[r], s1[q & 1]);
+      r += k;
+      if (r >= n) r -= n;
+    }
+    V[p] = (s0[0] + s0[1]) + (s1[0] + s1[1]);
+  }
+}
+// DFT along x or y of the half spectrum, out of place; SCALE multiplies the
+// output by Pc scale (Pc of the full grid: its first n_z / 2 + 1 planes).
+template <bool INV, bool SCALE>
+__global__ void __launch_bounds__(kFieldThreads) k_coul_xy(const double2* __restrict__ in,
+                                                           double2* __restrict__ out, FieldGeom g,
+                                                           int axis, const double* __restrict__ Pc,
+                                                           double scale) {
+  __shared__ double tc[kFieldMaxN], ts[kFieldMaxN];
+  const int n = g.n[axis];
+  for (int i = threadIdx.x; i < n; i += kFieldThreads) {
+    tc[i] = g.op[axis][2 * n + i];
+    ts[i] = INV ? g.op[axis][3 * n + i] : -g.op[axis][3 * n + i];
+  }
+  __syncthreads();
+  const int p = blockIdx.x * kFieldThreads + threadIdx.x;
+  if (p >= (g.n[2] / 2 + 1) * g.n[0] * g.n[1]) return;
+  int k, base, stride;
+  field_line(g, p, axis, k, base, stride);
+  double rc = 0.0, rs = 0.0, ic = 0.0, is = 0.0;
+  int r = 0;
+#pragma unroll 4
+  for (int q = 0; q < n; ++q) {
+    const double2 v = in[base + q * stride];
+    rc = fma(v.x, tc[r], rc);
+    rs = fma(v.x, ts[r], rs);
+    ic = fma(v.y, tc[r], ic);
+    is = fma(v.y, ts[r], is);
+    r += k;
+    if (r >= n) r -= n;
+  }
+  double2 o = make_double2(rc - is, ic + rs);
+  if constexpr (SCALE) {
+    const double s = Pc[p] * scale;
+    o = make_double2(o.x * s, o.y * s);
+  }
+  out[p] = o;
 }
 
 // Temporaries in d_ftmp ([16][G]): 0-1 rho_T, 2-3 Delta rho_T,
 // 4-9 d_j rho_T at 4 + 2j + T, 10 V_C, 11-12 reduction partials,
 // 13-15 spin-orbit density when the caller does not want it.
-__global__ void k_isospin(const double* rho, double* rT, int G) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= G) return;
-  rT[p] = rho[p] + rho[G + p];
-  rT[G + p] = rho[p] - rho[G + p];
-}
-
 __global__ void k_coul_table(double* Pc, const double* kx, const double* ky, const double* kz,
                              int nx, int ny, int nz, double e2) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -126,30 +276,27 @@ sky_status build_coulomb_table(Ctx* c) {
 
 // Shared first part of mean fields and energy: rho_T, Delta rho_T, grad rho_T, V_C.
 static sky_status field_prep(Ctx* c, const double* rho, bool need_grad) {
-  const long long G = c->G;
+  const int G = c->G, T = kFieldThreads;
   double* f = c->d_ftmp;
-  cudaError_t e;
-  k_isospin<<<div_up(G, 256), 256, 0, c->stream>>>(rho, f, (int)G); note_launch();
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_check(c, e, "isospin");
-  if ((e = real_op_sum(c, f, f + 2 * G, 2, 1)) != cudaSuccess) return cuda_check(c, e, "laplacian");
-  if (need_grad) {
-    for (int ax = 0; ax < 3; ++ax) {
-      OpRealD op{f, f + (4 + 2 * ax) * G, c->d_kp[ax], 1.0 / c->n[ax], 0, 0, G};
-      if ((e = run_pass(c, ax, op, 2)) != cudaSuccess) return cuda_check(c, e, "gradient");
-    }
-  }
+  const FieldGeom g = field_geom(c);
+  if (need_grad)
+    k_field_derivs<true><<<div_up(G, T), T, 0, c->stream>>>(rho, g, f);
+  else
+    k_field_derivs<false><<<div_up(G, T), T, 0, c->stream>>>(rho, g, f);
+  note_launch();
   if (c->cp.coulomb) {
-    OpR2CFwd o1{rho + G, c->d_fcx, G};
-    OpCPass<false> o2{c->d_fcx, G};
-    OpCoulX o3{c->d_fcx, c->d_coul, 1.0 / (double)G, G};
-    OpCPass<true> o4{c->d_fcx, G};
-    OpC2RInv o5{c->d_fcx, f + 10 * G, G};
-    if ((e = run_pass(c, 2, o1, 1)) == cudaSuccess && (e = run_pass(c, 1, o2, 1)) == cudaSuccess &&
-        (e = run_pass(c, 0, o3, 1)) == cudaSuccess && (e = run_pass(c, 1, o4, 1)) == cudaSuccess)
-      e = run_pass(c, 2, o5, 1);
-    if (e != cudaSuccess) return cuda_check(c, e, "coulomb");
+    const int gh = (c->n[2] / 2 + 1) * c->n[0] * c->n[1];
+    double2 *a = c->d_fcx, *b = c->d_fcx + gh;
+    const unsigned nb = div_up(gh, T);
+    k_coul_z<true><<<nb, T, 0, c->stream>>>(rho + G, a, nullptr, g);
+    k_coul_xy<false, false><<<nb, T, 0, c->stream>>>(a, b, g, 1, nullptr, 0.0);
+    k_coul_xy<false, true><<<nb, T, 0, c->stream>>>(b, a, g, 0, c->d_coul, 1.0 / (double)G);
+    k_coul_xy<true, false><<<nb, T, 0, c->stream>>>(a, b, g, 0, nullptr, 0.0);
+    k_coul_xy<true, false><<<nb, T, 0, c->stream>>>(b, a, g, 1, nullptr, 0.0);
+    k_coul_z<false><<<div_up(G, T), T, 0, c->stream>>>(nullptr, a, f + 10LL * G, g);
+    note_launch(6);
   }
-  return SKY_OK;
+  return cuda_check(c, cudaGetLastError(), "field derivatives");
 }
 
 __device__ __forceinline__ void rho0_powers(double r0, double alpha, double& r0a, double& r0am1) {
@@ -244,15 +391,23 @@ __global__ void __launch_bounds__(kEnBlock) k_energy_parts(Couplings cp, const d
   }
 }
 
-__global__ void k_energy_final(const double* part, int nblk, double dV, double* out, int* status) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s[kEnParts] = {0, 0, 0, 0, 0, 0, 0};
-  for (int b = 0; b < nblk; ++b)
-    for (int k = 0; k < kEnParts; ++k) s[k] += part[b * kEnParts + k];
+// One warp per part (a single thread walking the 64 x 7 partial sums: 22 us
+// of dependent FP64 additions).
+__global__ void __launch_bounds__(32 * kEnParts) k_energy_final(const double* part, int nblk, double dV,
+                                                                double* out, int* status) {
+  __shared__ double s[kEnParts];
+  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double v = 0.0;
+  for (int b = lane; b < nblk; b += 32) v += part[b * kEnParts + k];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  if (lane == 0) s[k] = v;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
   double tot = 0.0;
-  for (int k = 0; k < 6; ++k) {
-    out[1 + k] = dV * s[k];
-    tot += dV * s[k];
+  for (int q = 0; q < 6; ++q) {
+    out[1 + q] = dV * s[q];
+    tot += dV * s[q];
   }
   out[0] = tot;
   out[7] = dV * s[6];
@@ -266,7 +421,7 @@ sky_status energy_impl(Ctx* c, const double* rho, const double* tau, const doubl
   const int nblk = 64;
   double* part = c->d_ftmp + 11 * (long long)c->G;
   k_energy_parts<<<nblk, kEnBlock, 0, c->stream>>>(c->cp, rho, tau, divJ, c->d_ftmp, c->G, part); note_launch();
-  k_energy_final<<<1, 32, 0, c->stream>>>(part, nblk, c->dV, out, c->d_status); note_launch();
+  k_energy_final<<<1, 32 * kEnParts, 0, c->stream>>>(part, nblk, c->dV, out, c->d_status); note_launch();
   return cuda_check(c, cudaGetLastError(), "energy");
 }
 

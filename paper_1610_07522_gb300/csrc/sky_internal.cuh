@@ -94,7 +94,8 @@ struct Ctx {
   int red_nblk;                     // reduction blocks per state
   double* d_dpart;                  // density partials [kDensSplits][5][G]
   double* d_ftmp;                   // field temporaries [16][G]
-  double2* d_fcx;                   // complex field scratch [G]
+  double2* d_fcx;                   // half spectra of the Coulomb transform, two buffers
+  double* d_fop[3];                 // real-field operators of each axis (fields.cu)
   float* d_hf;                      // FP32 forms: U, B, W of one species as floats [5][G]
   int fused_h;                      // FP32 forms: one fused pass per axis for h psi (tunable)
   double2* d_gpart;                 // split-K partials of sky_overlap
@@ -175,7 +176,7 @@ inline unsigned div_up(long long a, long long b) { return (unsigned)((a + b - 1)
 
 // Host-side entry points of the other translation units.
 sky_status upload_twiddles_hamiltonian(Ctx* c);
-sky_status upload_twiddles_fields(Ctx* c);
+sky_status build_field_tables(Ctx* c);
 sky_status apply_h_impl(Ctx* c, const double* U, const double* B, const double* W,
                         const void* psi, void* hpsi, int I, double* eps, double* hn2);
 sky_status td_taylor_impl(Ctx* c, const double* U, const double* B, const double* W,
