@@ -82,7 +82,7 @@ static void free_all(Ctx* c) {
   void* ptrs[] = {c->d_status, c->d_kt[0], c->d_kt[1], c->d_kt[2], c->d_ktdd[0], c->d_ktdd[1],
                   c->d_ktdd[2], c->d_ktf[0], c->d_ktf[1],
                   c->d_ktf[2], c->d_kp[0], c->d_kp[1], c->d_kp[2], c->d_damp[0], c->d_damp[1],
-                  c->d_coul, c->d_gscr, c->d_red, c->d_dpart, c->d_ftmp, c->d_fcx, c->d_hf, c->d_gpart,
+                  c->d_coul, c->d_gscr, c->d_red, c->d_dpart, c->d_ftmp, c->d_fcx, c->d_fop[0], c->d_fop[1], c->d_fop[2], c->d_hf, c->d_gpart,
                   c->d_eigA[0], c->d_eigA[1], c->d_eigV, c->d_eigw, c->d_eigpart, c->d_bar, c->d_tbar,
                   c->d_eigres, c->d_eigrot, c->d_small[0], c->d_small[1], c->d_small[2],
                   c->d_small[3], c->d_small[4], c->d_small[5], c->d_gate,
@@ -290,7 +290,8 @@ sky_status sky_init(sky_ctx** out, const int grid[3], const double dx[3], const 
   }
   ALLOC(c->d_dpart, (size_t)kDensSplits * 5 * G);
   ALLOC(c->d_ftmp, (size_t)16 * G);
-  ALLOC(c->d_fcx, G);
+  ALLOC(c->d_fcx, (size_t)2 * (grid[2] / 2 + 1) * grid[0] * grid[1]);
+  for (int j = 0; j < 3; ++j) ALLOC(c->d_fop[j], 4 * grid[j]);
   ALLOC(c->d_gpart, gpart);
   // eigensolver and small-matrix workspace: eig_batch problems of size Imax
   c->eig_batch = 2;
@@ -364,7 +365,7 @@ sky_status sky_init(sky_ctx** out, const int grid[3], const double dx[3], const 
   if (s == SKY_OK) s = deriv_tc_init(c);
   if (s == SKY_OK && c->d_dop[0] && c->d_dop[1] && c->d_dop[2]) c->line_arith = 2;
   if (s == SKY_OK) s = upload_twiddles_hamiltonian(c);
-  if (s == SKY_OK) s = upload_twiddles_fields(c);
+  if (s == SKY_OK) s = build_field_tables(c);
   if (s == SKY_OK) s = build_coulomb_table(c);
   if (s == SKY_OK) s = cuda_check(c, cudaStreamSynchronize(c->stream), "init sync");
   if (s != SKY_OK) {
