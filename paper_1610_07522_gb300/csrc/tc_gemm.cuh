@@ -86,6 +86,16 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
   return (uint64_t)((saddr >> 4) & 0x3FFFu) | (1ull << 16) | (64ull << 32) | (1ull << 46) |
          (2ull << 61);
 }
+// Descriptor of an MN-major operand with 128-byte swizzle (N contiguous in
+// memory): blocks of 64 N x 64 K elements as TMA stages them, one 128-byte row
+// per K value, 8-row groups 1024 bytes apart along K (stride byte offset) and
+// blocks 8192 bytes apart along N (leading byte offset).
+constexpr int kMnBlock = 64 * 64 * 2;
+__device__ __forceinline__ uint64_t mn128_desc(uint32_t saddr) {
+  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(kMnBlock >> 4) << 16) | (64ull << 32) |
+         (1ull << 46) | (2ull << 61);
+}
+constexpr uint32_t kIdescBMn = 1u << 16;   // B MN-major (idesc_bf16 has both operands K-major)
 // Instruction descriptor, kind::f16: D fp32, A and B bf16, both K-major, M x N.
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
@@ -144,7 +154,14 @@ struct GemmArgs {
   int* status;
 };
 
-template <int BNT>
+// ROT, the recombination: B is [K][N] (the states as they are stored, N
+// contiguous: MN-major, no transposed copy) and A's rows 2a and 2a + 1 hold the
+// real and imaginary parts of coefficient row a, so that neighbouring TMEM
+// lanes hold P = M_re phi and Q = M_im phi over the interleaved (re, im)
+// columns and the epilogue forms (P_re - Q_im, P_im + Q_re) by one shuffle per
+// value: even lanes write the first half of each 32 columns of row a, odd
+// lanes the second.
+template <int BNT, bool ROT>
 __global__ void __launch_bounds__(THREADS, 1)
     k_gemm_bf16(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
                 const __grid_constant__ CUtensorMap mA2, const __grid_constant__ CUtensorMap mB0,
@@ -228,14 +245,21 @@ __global__ void __launch_bounds__(THREADS, 1)
             const CUtensorMap* mapA = i == 0 ? &mA0 : (i == 1 ? &mA1 : &mA2);
             const CUtensorMap* mapB = i == 0 ? &mB0 : (i == 1 ? &mB1 : &mB2);
             tma_load_2d(sa + i * TILE_BYTES, mapA, kb * BK, m0, full(s));
-            tma_load_2d(sa + np * TILE_BYTES + i * TILE_B, mapB, kb * BK, n0, full(s));
+            if constexpr (ROT) {
+#pragma unroll
+              for (int n = 0; n < BNT / 64; ++n)
+                tma_load_2d(sa + np * TILE_BYTES + i * TILE_B + n * kMnBlock, mapB, n0 + n * 64,
+                            kb * BK, full(s));
+            } else {
+              tma_load_2d(sa + np * TILE_BYTES + i * TILE_B, mapB, kb * BK, n0, full(s));
+            }
           }
         }
       }
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      const uint32_t idesc = idesc_bf16(BM, BNT);
+      const uint32_t idesc = idesc_bf16(BM, BNT) | (ROT ? kIdescBMn : 0u);
       long long g = 0;
       int j = 0;   // tiles done by this CTA
       bool ok = true;
@@ -262,10 +286,12 @@ __global__ void __launch_bounds__(THREADS, 1)
           const uint32_t sa = smem_u32(base + s * stage_bytes);
           for (int p = 0; p < a.nphase; ++p) {
             const uint64_t da = sw128_desc(sa + a.pa[p] * TILE_BYTES);
-            const uint64_t db = sw128_desc(sa + np * TILE_BYTES + a.pb[p] * TILE_B);
+            const uint32_t sb = sa + np * TILE_BYTES + a.pb[p] * TILE_B;
+            const uint64_t db = ROT ? mn128_desc(sb) : sw128_desc(sb);
+            constexpr uint64_t kStepB = ROT ? 128ull : 2ull;   // 16 K rows of 128 bytes, or 32 bytes
 #pragma unroll
             for (int k = 0; k < BK / 16; ++k)   // +32 bytes along K = +2 in the encoded address
-              mma_bf16(acc, da + 2ull * k, db + 2ull * k, idesc,
+              mma_bf16(acc, da + 2ull * k, db + kStepB * k, idesc,
                        (it > 0 || p > 0 || k > 0) ? 1u : 0u);
           }
           mma_commit(empty(s));
@@ -291,7 +317,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       fence_after();
       const int row = m0 + q * 32 + lane;
-      float* drow = a.D + (long long)z * a.sstride + (long long)row * a.ldd;
+      float* drow = ROT ? a.D + (long long)(row >> 1) * a.ldd
+                        : a.D + (long long)z * a.sstride + (long long)row * a.ldd;
 #pragma unroll 1
       for (int c = 0; c < BNT; c += 32) {
         float v[32];
@@ -301,7 +328,26 @@ __global__ void __launch_bounds__(THREADS, 1)
           for (int i = 0; i < 32; ++i) v[i] = 0.0f;
         }
         const int col = n0 + c;
-        if (row < a.M) {
+        if constexpr (ROT) {
+          const bool odd = lane & 1;
+          float y[16], o[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) y[i] = __shfl_xor_sync(0xffffffffu, odd ? v[i] : v[16 + i], 1);
+#pragma unroll
+          for (int i = 0; i < 16; i += 2) {
+            const float pr = odd ? y[i] : v[i], pi = odd ? y[i + 1] : v[i + 1];
+            const float qr = odd ? v[16 + i] : y[i], qi = odd ? v[17 + i] : y[i + 1];
+            o[i] = pr - qi;
+            o[i + 1] = pi + qr;
+          }
+          const int oc = col + (odd ? 16 : 0);   // N = 4 G is a multiple of 256: whole chunks
+          if (row < a.M && oc + 16 <= a.N) {
+#pragma unroll
+            for (int i = 0; i < 16; i += 4)
+              *reinterpret_cast<float4*>(drow + oc + i) =
+                  make_float4(o[i], o[i + 1], o[i + 2], o[i + 3]);
+          }
+        } else if (row < a.M) {
           if (col + 32 <= a.N) {
 #pragma unroll
             for (int i = 0; i < 32; i += 4)
@@ -374,19 +420,22 @@ inline Phases phases_for_split(int nsplit) {
   return p;
 }
 
-// D = sum over phases of A[pa] B[pb]^T.  A[i]: [M][K], B[i]: [N][K] bf16 with
+// D = sum over phases of A[pa] B[pb]^T (ROT: see k_gemm_bf16; B[i]: [K][N], D
+// M / 2 rows, no K split, N a multiple of 32).  A[i]: [M][K], B[i]: [N][K] bf16 with
 // row strides lda, ldb >= K (elements, multiples of 8), i < nsplit.  With *splits > 1
 // the K blocks are divided over blockIdx.z and partial tiles go to
 // D + z * sstride; *splits returns the number of partial tiles written.
 // Pointers 16-byte aligned, ldd a multiple of 4.
+template <bool ROT>
 inline cudaError_t gemm_bf16(const void* const* A, long long lda, const void* const* B,
                              long long ldb, int nsplit, int M, int N, int K, int* splits,
                              float* D, long long ldd, long long sstride, int* status,
                              cudaStream_t s, int tile_n = 0) {
   if (M <= 0 || N <= 0 || K <= 0) { *splits = 0; return cudaSuccess; }
   // TMA needs 16-byte row strides; columns past K read as zeros
-  if ((lda & 7) || (ldb & 7) || (ldd & 3) || lda < K || ldb < K || nsplit < 1 || nsplit > 3)
+  if ((lda & 7) || (ldb & 7) || (ldd & 3) || lda < K || ldb < (ROT ? N : K) || nsplit < 1 || nsplit > 3)
     return cudaErrorInvalidValue;
+  if (ROT && ((N & 31) || (M & 1) || *splits > 1)) return cudaErrorInvalidValue;
   // 128 x 256 tiles when the pieces of one K block still fit twice in the ring
   // (x3: 96 KiB per stage), else 128 x 128 (x6: 96 KiB per stage); tile_n
   // 128 asks for the narrow tiles (more tiles, for products that share the GPU)
@@ -396,7 +445,9 @@ inline cudaError_t gemm_bf16(const void* const* A, long long lda, const void* co
   for (int i = 0; i < 3; ++i) {
     const int j = i < nsplit ? i : 0;
     if ((e = make_map(&ma[i], A[j], M, K, lda, BM)) != cudaSuccess) return e;
-    if ((e = make_map(&mb[i], B[j], N, K, ldb, bnt)) != cudaSuccess) return e;
+    // ROT: rows of the map are K values, boxes of 64 N x 64 K
+    if ((e = ROT ? make_map(&mb[i], B[j], K, N, ldb, BK) : make_map(&mb[i], B[j], N, K, ldb, bnt)) != cudaSuccess)
+      return e;
   }
   const Phases ph = phases_for_split(nsplit);
   const int nkb = (K + BK - 1) / BK;
@@ -422,9 +473,9 @@ inline cudaError_t gemm_bf16(const void* const* A, long long lda, const void* co
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!smem_set[dev]) {
-    e = cudaFuncSetAttribute(k_gemm_bf16<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    e = cudaFuncSetAttribute(k_gemm_bf16<128, ROT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_gemm_bf16<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+      e = cudaFuncSetAttribute(k_gemm_bf16<256, ROT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
     if (e != cudaSuccess) return e;
     smem_set[dev] = true;
   }
@@ -434,9 +485,9 @@ inline cudaError_t gemm_bf16(const void* const* A, long long lda, const void* co
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const int grid = (int)(ntiles < nsm ? ntiles : nsm);   // persistent: one CTA per SM
   if (bnt == 256)
-    k_gemm_bf16<256><<<grid, THREADS, SMEM_BYTES, s>>>(ma[0], ma[1], ma[2], mb[0], mb[1], mb[2], g);
+    k_gemm_bf16<256, ROT><<<grid, THREADS, SMEM_BYTES, s>>>(ma[0], ma[1], ma[2], mb[0], mb[1], mb[2], g);
   else
-    k_gemm_bf16<128><<<grid, THREADS, SMEM_BYTES, s>>>(ma[0], ma[1], ma[2], mb[0], mb[1], mb[2], g);
+    k_gemm_bf16<128, ROT><<<grid, THREADS, SMEM_BYTES, s>>>(ma[0], ma[1], ma[2], mb[0], mb[1], mb[2], g);
   note_launch();
   *splits = z;
   return cudaGetLastError();

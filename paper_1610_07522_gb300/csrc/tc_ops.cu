@@ -9,10 +9,8 @@
 // storage:
 //   <a|b>:  Re = sum_k a_r[k] b_r[k],  Im = sum_k a_r[k] b'_r[k],
 //           b' = (Im b, -Re b) per entry, so D = a_r [b_r; b'_r]^T holds Re | Im;
-//   psi_a = sum_b M[b][a] phi_b:  psi_r = [M_re^T | M_im^T] [phi_r; (i phi)_r],
-//           i phi = (-Im phi, Re phi), with the phi operand stored transposed
-//           (K contiguous: the two halves padded with zeros to a multiple of 32
-//           states each) so that D = psi_r directly.
+//   psi_a = sum_b M[b][a] phi_b:  P = M_re^T phi_r, Q = M_im^T phi_r over phi's
+//           own layout, psi = (P_re - Q_im, P_im + Q_re) per entry.
 #include <cuda_bf16.h>
 
 #include "tc_gemm.cuh"
@@ -54,69 +52,60 @@ __global__ void k_split_rows(const float* __restrict__ src, long long rows, long
   }
 }
 
-// Transposed operand of the recombination: dst[i][v'][beta'] (row stride ld)
-// from phi_r[beta][v'] (beta' = beta) and (i phi)_r (beta' = Ipad + beta), with
-// zeros for beta in [I, Ipad); Ipad a multiple of 32.  32 x 32 tiles through
-// shared memory (coalesced on both sides, whole 32-byte sectors written).
-__global__ void __launch_bounds__(256) k_split_rot_b(const float* __restrict__ phi, int I,
-                                                     int Ipad, long long K2V, long long ld, int n,
-                                                     __nv_bfloat16* d0, __nv_bfloat16* d1,
-                                                     __nv_bfloat16* d2) {
-  __shared__ float t[32][65];    // [beta][v' (32 complex = 64 reals)]
-  const int b0 = blockIdx.y * 32;
-  const long long v0 = (long long)blockIdx.x * 64;        // real index
-  const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;  // 64 x 4
-  for (int r = ty; r < 32; r += 4) {
-    const int b = b0 + r;
-    const long long v = v0 + tx;
-    t[r][tx] = (b < I && v < K2V) ? phi[(long long)b * K2V + v] : 0.0f;
-  }
-  __syncthreads();
-  __nv_bfloat16* d[3] = {d0, d1, d2};
-  // write: each thread one (v', beta) pair; beta fastest for coalescing
-  for (int idx = threadIdx.x; idx < 64 * 32; idx += 256) {
-    const int vl = idx >> 5, bl = idx & 31;
-    const long long v = v0 + vl;
-    const int b = b0 + bl;
-    if (v >= K2V) continue;
-    const float x = t[bl][vl];            // zero for b >= I
-    // (i phi)_r: even v' (re slot) takes -Im, odd v' (im slot) takes +Re
-    const float y = (vl & 1) ? t[bl][vl - 1] : -t[bl][vl + 1];
-    __nv_bfloat16 sx[3], sy[3];
-    split3(x, n, sx);
-    split3(y, n, sy);
-    for (int i = 0; i < n; ++i) {
-      d[i][v * ld + b] = sx[i];
-      d[i][v * ld + Ipad + b] = sy[i];
+// Operand of the recombination: the n bf16 pieces of every real of phi, in
+// phi's own layout [I][2 V] (the product reads it MN-major).  Eight reals per
+// thread: two 16-byte loads, one 16-byte store per piece.  HBM-bound: 32^3, 700
+// states, x3: 734 MB in 104 us (7.1 TB/s); the transposed [V][2 I] operand that held every
+// value twice (phi and i phi) took 482 us.
+__global__ void __launch_bounds__(256) k_split_flat(const float4* __restrict__ phi, long long n8,
+                                                    int n, uint4* d0, uint4* d1, uint4* d2) {
+  const long long e = (long long)blockIdx.x * 256 + threadIdx.x;
+  if (e >= n8) return;
+  const float4 a = phi[2 * e], b = phi[2 * e + 1];
+  const float x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+  __nv_bfloat16 s[8][3];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) split3(x[k], n, s[k]);
+  uint4* d[3] = {d0, d1, d2};
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    if (i >= n) break;
+    unsigned w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      __nv_bfloat162 v;
+      v.x = s[2 * k][i];
+      v.y = s[2 * k + 1][i];
+      w[k] = *reinterpret_cast<unsigned*>(&v);
     }
+    d[i][e] = make_uint4(w[0], w[1], w[2], w[3]);
   }
 }
 
-// Row operand of the recombination: A[alpha][beta'] = M_re[beta'][alpha]
-// (beta' < I) or M_im[beta' - I][alpha], split into bf16 pieces.
-__global__ void k_split_rot_a(const double2* __restrict__ M, int I, int Ipad, long long ld, int n,
+// Coefficient operand of the recombination: rows 2a and 2a + 1 of A hold
+// M_re[beta][a] and M_im[beta][a] over beta (row stride ld, ld - I zeros),
+// split into bf16 pieces.
+__global__ void k_split_rot_a(const double2* __restrict__ M, int I, long long ld, int n,
                               __nv_bfloat16* d0, __nv_bfloat16* d1, __nv_bfloat16* d2) {
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long long)I * 2 * Ipad) return;
-  const int a = (int)(e / (2 * Ipad)), bp = (int)(e % (2 * Ipad));
-  const int beta = bp < Ipad ? bp : bp - Ipad;
-  // row a: [Re M[beta][a] for beta < I | zeros | Im M[beta][a] | zeros]
+  if (e >= 2 * I * ld) return;
+  const int r = (int)(e / ld), beta = (int)(e % ld);
   double xd = 0.0;
   if (beta < I) {
-    const double2 m = M[(long long)beta * I + a];
-    xd = bp < Ipad ? m.x : m.y;   // the FP64 value keeps its residual in the lower pieces
+    const double2 m = M[(long long)beta * I + (r >> 1)];
+    xd = (r & 1) ? m.y : m.x;   // the FP64 value keeps its residual in the lower pieces
   }
   __nv_bfloat16 s[3];
   const __nv_bfloat16 h = __double2bfloat16(xd);
   s[0] = h;
   if (n > 1) {
-    const double r = xd - (double)__bfloat162float(h);
-    const __nv_bfloat16 mm = __double2bfloat16(r);
+    const double r1 = xd - (double)__bfloat162float(h);
+    const __nv_bfloat16 mm = __double2bfloat16(r1);
     s[1] = mm;
-    if (n > 2) s[2] = __double2bfloat16(r - (double)__bfloat162float(mm));
+    if (n > 2) s[2] = __double2bfloat16(r1 - (double)__bfloat162float(mm));
   }
   __nv_bfloat16* d[3] = {d0, d1, d2};
-  for (int i = 0; i < n; ++i) d[i][(long long)a * ld + bp] = s[i];
+  for (int i = 0; i < n; ++i) d[i][e] = s[i];
 }
 
 // X[a][b] = dV sum_z (D_z[a][b] + i D_z[a][I + b]) for a >= b, mirrored.
@@ -137,10 +126,7 @@ __global__ void k_tc_overlap_reduce(const float* __restrict__ D, int nz, long lo
   if (a != b) X[(long long)b * I + a] = conjx(s);
 }
 
-// K layout of the recombination: [re | zeros | im | zeros] in halves of
-// round32(I), so that both halves of each row start on a 64-byte boundary and
-// every 32-byte sector of the transposed operand is written whole.
-static inline long long round32(long long x) { return (x + 31) / 32 * 32; }
+static inline long long round8(long long x) { return (x + 7) / 8 * 8; }   // 16-byte rows of bf16
 
 int tc_nsplit(sky_prec p) { return p == SKY_F32_BF16X6 ? 3 : 2; }
 
@@ -155,11 +141,9 @@ int tc_min_splits(long long K) { return (int)((K + kMaxAccK - 1) / kMaxAccK); }
 void tc_scratch_sizes(int I, long long V, int num_sms, size_t* piece_a, size_t* piece_b,
                       size_t* piece_rot_a, size_t* partial) {
   const long long K = 2 * V;
-  *piece_a = (size_t)I * K;
-  const size_t ov_b = (size_t)2 * I * K;
-  const size_t rot_b = (size_t)K * 2 * round32(I);
-  *piece_b = ov_b > rot_b ? ov_b : rot_b;
-  *piece_rot_a = (size_t)I * 2 * round32(I);
+  *piece_a = (size_t)I * K;              // also the states' pieces of the recombination
+  *piece_b = (size_t)2 * I * K;
+  *piece_rot_a = (size_t)2 * I * round8(I);
   const long long ldd = (2LL * I + 3) / 4 * 4;
   const int tiles = ((I + tc::BM - 1) / tc::BM) * ((2 * I + tc::BN - 1) / tc::BN);
   int z = kMaxTcWaves * num_sms / (tiles > 0 ? tiles : 1);
@@ -195,7 +179,7 @@ sky_status tc_overlap(Ctx* c, const void* a, const void* b, int I, double2* X) {
   if ((size_t)z * sstride > c->tc_partial_elems) z = (int)(c->tc_partial_elems / sstride);
   const void* pa[3] = {A[0], A[1], A[2]};
   const void* pb[3] = {Bp[0], Bp[1], Bp[2]};
-  e = tc::gemm_bf16(pa, K, pb, K, n, I, 2 * I, (int)K, &z, c->d_tcPart, ldd, sstride,
+  e = tc::gemm_bf16<false>(pa, K, pb, K, n, I, 2 * I, (int)K, &z, c->d_tcPart, ldd, sstride,
                     c->d_status, c->stream, c->tc_tile_n);
   if (e != cudaSuccess) return cuda_check(c, e, "tc overlap gemm");
   k_tc_overlap_reduce<<<div_up((long long)I * I, 256), 256, 0, c->stream>>>(
@@ -204,28 +188,33 @@ sky_status tc_overlap(Ctx* c, const void* a, const void* b, int I, double2* X) {
   return cuda_check(c, cudaGetLastError(), "tc overlap reduce");
 }
 
+// psi_a = sum_b M[b][a] phi_b as one real product over the states' own layout:
+// [P; Q] = [M_re^T; M_im^T] phi (2 I rows, K = I, N = 2 V reals), combined in
+// the epilogue.
 sky_status tc_rotate(Ctx* c, const void* phi, const double2* M, int I, void* out) {
   const long long V = 2LL * c->G, K2V = 2 * V;
   const int n = tc_nsplit(c->prec);
-  const int Ipad = (int)round32(I);
-  const long long ldk = 2LL * Ipad;
+  const long long lda = round8(I);
   __nv_bfloat16* Ra[3] = {(__nv_bfloat16*)c->d_tcRotA[0], (__nv_bfloat16*)c->d_tcRotA[1],
                           (__nv_bfloat16*)c->d_tcRotA[2]};
-  __nv_bfloat16* Bp[3] = {(__nv_bfloat16*)c->d_tcB[0], (__nv_bfloat16*)c->d_tcB[1],
-                          (__nv_bfloat16*)c->d_tcB[2]};
-  k_split_rot_a<<<div_up((long long)I * 2 * Ipad, 256), 256, 0, c->stream>>>(M, I, Ipad, ldk, n,
-                                                                            Ra[0], Ra[1], Ra[2]);
-  dim3 g2(div_up(K2V, 64), Ipad / 32);
-  k_split_rot_b<<<g2, 256, 0, c->stream>>>((const float*)phi, I, Ipad, K2V, ldk, n, Bp[0], Bp[1],
-                                           Bp[2]);
+  __nv_bfloat16* Bp[3] = {(__nv_bfloat16*)c->d_tcA[0], (__nv_bfloat16*)c->d_tcA[1],
+                          (__nv_bfloat16*)c->d_tcA[2]};
+  k_split_rot_a<<<div_up(2 * I * lda, 256), 256, 0, c->stream>>>(M, I, lda, n, Ra[0], Ra[1], Ra[2]);
+  const long long n8 = I * K2V / 8;      // K2V = 4 G, every axis a multiple of 4
+  if (((uintptr_t)phi & 15) == 0)
+    k_split_flat<<<div_up(n8, 256), 256, 0, c->stream>>>((const float4*)phi, n8, n, (uint4*)Bp[0],
+                                                         (uint4*)Bp[1], (uint4*)Bp[2]);
+  else                                   // states at an 8-byte boundary: scalar loads
+    k_split_rows<<<div_up((long long)I * V, 256), 256, 0, c->stream>>>((const float*)phi, I, K2V, n, 0,
+                                                                       Bp[0], Bp[1], Bp[2]);
   note_launch(2);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_check(c, e, "tc rotate split");
   int z = 1;
   const void* pa[3] = {Ra[0], Ra[1], Ra[2]};
   const void* pb[3] = {Bp[0], Bp[1], Bp[2]};
-  e = tc::gemm_bf16(pa, ldk, pb, ldk, n, I, (int)K2V, 2 * Ipad, &z, (float*)out, K2V, 0,
-                    c->d_status, c->stream, c->tc_tile_n);
+  e = tc::gemm_bf16<true>(pa, lda, pb, K2V, n, 2 * I, (int)K2V, I, &z, (float*)out, K2V, 0,
+                          c->d_status, c->stream, c->tc_tile_n);
   return cuda_check(c, e, "tc rotate gemm");
 }
 
