@@ -9,6 +9,8 @@
 //   2. L = U psi - (i/2) sum A_j G_j -> hpsi;  F_j -> in place of G_j
 //   3. F_j <- d_j F_j              (one pass per axis, in place)
 //   4. hpsi = L + sum_j F_j, with <psi|h psi> and |h psi|^2 per block.
+#include <cmath>
+
 #include "fft_lines.cuh"
 
 namespace sky {
@@ -311,20 +313,33 @@ __global__ void k_state_totals(const double* part, int nblk, int I, double dV,
 //   inverse), then point by point L_j = -(i/2) A_j G and F_j = -B G - (i/2)
 //   A_j psi (F in place of G), then D_j = d_j F_j, and h psi += L_j + D_j
 //   (h psi = U psi + L_x + D_x in the first pass);
-// the last pass also forms <psi|h psi> and |h psi|^2.  The sum of the three
-// passes is the rearranged h psi of the general path (identical terms, other
-// rounding order), with h psi read and written once per pass and psi read
-// once, instead of the gradient, local and divergence passes that write and
-// re-read three scratch arrays.  States go in chunks whose psi and h psi stay
-// in L2 across the passes.  Fields as floats (one conversion per call).
-constexpr int kHaxLinesX = 32;      // lines per block along x (staged in shared memory)
+// the last pass also forms <psi|h psi> and |h psi|^2 when they are asked for.
+// The sum of the three passes is the rearranged h psi of the general path
+// (identical terms, other rounding order), with h psi read and written once per
+// pass, instead of the gradient, local and divergence passes that write and
+// re-read three scratch arrays (26 array passes; 8 here).
+//
+// One thread holds one spin component of a line (N complex values in
+// registers); lanes 0-15 of a warp hold component 0 of 16 lines and lanes
+// 16-31 component 1, so the partner of a point is 16 lanes away: its G comes
+// by shuffle, its psi from the warp's own rows of shared memory, where L_j
+// then takes the place of psi while the flux is differentiated.  With 8 N
+// bytes of shared memory and about 128 registers per thread 16 warps share an
+// SM; one thread per line pair with three such arrays left 6-8 and was bound
+// by latency (32^3, 700 states: 2.19 ms, against 1.59 ms of the general passes
+// and 0.91 ms now, bound by the FP32 issue rate: some 3300 instructions per line
+// and axis).  The wavenumbers come as kernel arguments (constant-bank
+// operands), B and W as one float4 per point.
 constexpr int kHaxMaxN = 32;        // longest axis of the fused path
-constexpr double kHaxL2Bytes = 48.0 * 1024 * 1024;   // psi + h psi of one chunk
+constexpr int kHaxThreads = 64;     // threads per block: 32 lines, both components
+constexpr double kHaxL2Bytes = 96.0 * 1024 * 1024;   // psi + h psi of one chunk
 
 struct HFields {
   const float* u;
-  const float* b;
-  const float* w;   // wx, wy, wz at w, w + G, w + 2 G
+  const float4* bw;   // (B, W_x, W_y, W_z)
+};
+struct HWave {
+  float k[kHaxMaxN];  // (k + theta/L) / N
 };
 
 __global__ void k_fields_f32(const double* __restrict__ U, const double* __restrict__ B,
@@ -332,206 +347,186 @@ __global__ void k_fields_f32(const double* __restrict__ U, const double* __restr
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= G) return;
   out[p] = (float)U[p];
-  out[G + p] = (float)B[p];
-  out[2 * G + p] = (float)W[p];
-  out[3 * G + p] = (float)W[G + p];
-  out[4 * G + p] = (float)W[2 * G + p];
+  reinterpret_cast<float4*>(out + G)[p] =
+      make_float4((float)B[p], (float)W[p], (float)W[G + p], (float)W[2 * G + p]);
 }
 
 // d_j of a line in place: forward transform, x i k_m / N, inverse.
 template <int N>
-__device__ __forceinline__ void deriv_line(float2 (&v)[N], const float* __restrict__ kt,
-                                           float inv_n) {
+__device__ __forceinline__ void deriv_line(float2 (&v)[N], const HWave& w) {
   Fft<float, N, false>::run(v);
 #pragma unroll
-  for (int m = 0; m < N; ++m) {
-    const float kk = __ldg(kt + m) * inv_n;
-    v[m] = make_float2(-kk * v[m].y, kk * v[m].x);
-  }
+  for (int m = 0; m < N; ++m) v[m] = make_float2(-w.k[m] * v[m].y, w.k[m] * v[m].x);
   Fft<float, N, true>::run(v);
 }
 
-// Point idx of the line: a = psi (both components), g = d_j psi -> F_j;
-// returns L_j = -(i/2) A_j G in l0, l1.
+// A point of component c = 0 (s = 1) or 1 (s = -1): a, ap = psi of this and the
+// other component, g, gp their derivatives; g becomes F_j, L_j is returned.
 template <int AXIS>
-__device__ __forceinline__ void h_point(const HFields& f, int G, int idx, float2 a0, float2 a1,
-                                        float2& g0, float2& g1, float2& l0, float2& l1) {
-  const float bb = __ldg(f.b + idx);
-  const float wx = __ldg(f.w + idx), wy = __ldg(f.w + G + idx), wz = __ldg(f.w + 2 * G + idx);
-  float2 t0, t1;
-  apply_A<float>(AXIS, wx, wy, wz, g0, g1, t0, t1);     // A_j G_j
-  l0 = 0.5f * mul_mi(t0);
-  l1 = 0.5f * mul_mi(t1);
-  apply_A<float>(AXIS, wx, wy, wz, a0, a1, t0, t1);     // A_j psi
-  g0 = (-bb) * g0 + 0.5f * mul_mi(t0);                  // F_j = -B G_j - (i/2) A_j psi
-  g1 = (-bb) * g1 + 0.5f * mul_mi(t1);
+__device__ __forceinline__ float2 h_point(float4 f, float s, float2 a, float2 ap, float2& g, float2 gp) {
+  // (A_j v)_c = alpha v_c + beta v_{1-c} (complex beta) times 1/2
+  float2 ag, aa;
+  if (AXIS == 0) {            // s (-W_y v_c - i W_z v_{1-c})
+    const float wy = 0.5f * s * f.z, wz = 0.5f * s * f.w;
+    ag = make_float2(fmaf(wz, gp.y, -wy * g.x), fmaf(-wz, gp.x, -wy * g.y));
+    aa = make_float2(fmaf(wz, ap.y, -wy * a.x), fmaf(-wz, ap.x, -wy * a.y));
+  } else if (AXIS == 1) {     // s W_x v_c - W_z v_{1-c}
+    const float wx = 0.5f * s * f.y, wz = 0.5f * f.w;
+    ag = make_float2(fmaf(-wz, gp.x, wx * g.x), fmaf(-wz, gp.y, wx * g.y));
+    aa = make_float2(fmaf(-wz, ap.x, wx * a.x), fmaf(-wz, ap.y, wx * a.y));
+  } else {                    // (W_y + i s W_x) v_{1-c}
+    const float wx = 0.5f * s * f.y, wy = 0.5f * f.z;
+    ag = make_float2(fmaf(-wx, gp.y, wy * gp.x), fmaf(wx, gp.x, wy * gp.y));
+    aa = make_float2(fmaf(-wx, ap.y, wy * ap.x), fmaf(wx, ap.x, wy * ap.y));
+  }
+  g = make_float2(fmaf(-f.x, g.x, aa.y), fmaf(-f.x, g.y, -aa.x));   // -B G - i (A psi / 2)
+  return make_float2(ag.y, -ag.x);                                   // -i (A G / 2)
 }
 
-// x pass (first): h psi = U psi + L_x + D_x.  A block stages nl <= kHaxLinesX
-// consecutive x lines of both components of state blockIdx.y through shared
-// memory (coalesced loads and stores; rows padded to N + 1).  One component's
-// line at a time is transformed in registers; G, then F, of both components
-// wait in gs[m][c][thread].
+__device__ __forceinline__ float2 shfl16(float2 v) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, 16), __shfl_xor_sync(0xffffffffu, v.y, 16));
+}
+
+// x pass (first): h psi = U psi + L_x + D_x over the lines of ns states; lines
+// counted with the state fastest, so that a warp's lanes mostly share a line of
+// the fields (broadcast loads).  Each warp stages its 32 rows of N values
+// through its own shared memory, coalesced, padded to N + 1.
 template <int N>
-__global__ void __launch_bounds__(kHaxLinesX) k_h_axis_x(const float2* __restrict__ psi,
-                                                         float2* __restrict__ hpsi, HFields f,
-                                                         const float* __restrict__ kt,
-                                                         float inv_n, int G, int rows) {
-  __shared__ float2 tile[2][kHaxLinesX][N + 1];
-  __shared__ float2 gs[N][2][kHaxLinesX];
-  const int l0 = blockIdx.x * kHaxLinesX;
-  const int nl = rows - l0 < kHaxLinesX ? rows - l0 : kHaxLinesX;
-  const long long sb = (long long)blockIdx.y * 2 * G;
-  const int tid = threadIdx.x;
-  for (int e = tid; e < 2 * nl * N; e += kHaxLinesX) {
-    const int c = e / (nl * N), r = e - c * nl * N;
-    const int ll = r / N, m = r - ll * N;
-    tile[c][ll][m] = psi[sb + (long long)c * G + (long long)(l0 + ll) * N + m];
-  }
-  __syncthreads();
-  if (tid < nl) {
+__global__ void __launch_bounds__(kHaxThreads, 8) k_h_axis_x(const float2* __restrict__ psi,
+                                                             float2* __restrict__ hpsi, HFields f,
+                                                             const __grid_constant__ HWave w, int G,
+                                                             int rows, int ns) {
+  __shared__ float2 tile[kHaxThreads * (N + 1)];
+  __shared__ int s_base[kHaxThreads];
+  const int tid = threadIdx.x, lane = tid & 31, c = lane >> 4, w0 = tid & ~31;
+  const int l = blockIdx.x * (kHaxThreads / 2) + (tid >> 5) * 16 + (lane & 15);
+  const bool on = l < rows * ns;
+  const int row = on ? l / ns : 0, st = on ? l - row * ns : 0;
+  s_base[tid] = on ? (2 * st + c) * G + row * N : -1;
+  __syncwarp();
+  constexpr int C = 8;
+#pragma unroll 1
+  for (int j = 0; j < N; j += C) {
+    float2 t[C];
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      float2 v[N];
-#pragma unroll
-      for (int m = 0; m < N; ++m) v[m] = tile[c][tid][m];
-      deriv_line<N>(v, kt, inv_n);
-#pragma unroll
-      for (int m = 0; m < N; ++m) gs[m][c][tid] = v[m];
+    for (int k = 0; k < C; ++k) {
+      const int e = (j + k) * 32 + lane, r = e / N, b = j + k < N ? s_base[w0 + r] : -1;
+      t[k] = b >= 0 ? psi[b + (e - r * N)] : make_float2(0.0f, 0.0f);
     }
-    const int base = (l0 + tid) * N;
+#pragma unroll
+    for (int k = 0; k < C; ++k) {
+      const int e = (j + k) * 32 + lane, r = e / N;
+      if (j + k < N) tile[(w0 + r) * (N + 1) + (e - r * N)] = t[k];
+    }
+  }
+  __syncwarp();
+  float2* me = tile + tid * (N + 1);
+  const float2* other = tile + (tid ^ 16) * (N + 1);
+  const float s = c ? -1.0f : 1.0f;
+  float2 v[N];
+#pragma unroll
+  for (int m = 0; m < N; ++m) v[m] = me[m];
+  deriv_line<N>(v, w);
+#pragma unroll
+  for (int m = 0; m < N; ++m) {
+    const float4 fb = __ldg(f.bw + row * N + m);
+    const float u = __ldg(f.u + row * N + m);
+    const float2 a = me[m], ap = other[m];
+    const float2 L = h_point<0>(fb, s, a, ap, v[m], shfl16(v[m]));
+    __syncwarp();
+    me[m] = make_float2(fmaf(u, a.x, L.x), fmaf(u, a.y, L.y));
+  }
+  deriv_line<N>(v, w);
+#pragma unroll
+  for (int m = 0; m < N; ++m) me[m] = me[m] + v[m];
+  __syncwarp();
 #pragma unroll 4
-    for (int m = 0; m < N; ++m) {
-      const float2 a0 = tile[0][tid][m], a1 = tile[1][tid][m];
-      float2 g0 = gs[m][0][tid], g1 = gs[m][1][tid], L0, L1;
-      h_point<0>(f, G, base + m, a0, a1, g0, g1, L0, L1);
-      gs[m][0][tid] = g0;
-      gs[m][1][tid] = g1;
-      const float u = __ldg(f.u + base + m);
-      tile[0][tid][m] = u * a0 + L0;
-      tile[1][tid][m] = u * a1 + L1;
-    }
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      float2 v[N];
-#pragma unroll
-      for (int m = 0; m < N; ++m) v[m] = gs[m][c][tid];
-      deriv_line<N>(v, kt, inv_n);
-#pragma unroll
-      for (int m = 0; m < N; ++m) tile[c][tid][m] = tile[c][tid][m] + v[m];
-    }
-  }
-  __syncthreads();
-  for (int e = tid; e < 2 * nl * N; e += kHaxLinesX) {
-    const int c = e / (nl * N), r = e - c * nl * N;
-    const int ll = r / N, m = r - ll * N;
-    hpsi[sb + (long long)c * G + (long long)(l0 + ll) * N + m] = tile[c][ll][m];
+  for (int j = 0; j < N; ++j) {
+    const int e = j * 32 + lane, r = e / N, b = s_base[w0 + r];
+    if (b >= 0) hpsi[b + (e - r * N)] = tile[(w0 + r) * (N + 1) + (e - r * N)];
   }
 }
 
-// Threads (lines) per block of the y / z pass: two shared arrays of N x 2
-// values per thread (32 KiB at most).
-__host__ __device__ constexpr int hax_threads(int N) { return N <= 16 ? 64 : 32; }
-
-// y (AXIS 1) or z (AXIS 2) pass: one thread per line (consecutive threads on
-// consecutive x: coalesced).  The line's G, then F, of both components wait in
-// gs[m][c][thread] while one component's line is transformed in registers;
-// L_j waits in ls.  Loads never follow a store to global memory within a
-// phase (the pointwise phase stores to shared memory only; the last phase
-// loads a component's old h psi values before storing any), so each thread's
-// loads overlap instead of forming a chain of round trips.  The z pass (LAST)
-// also adds this block's <psi|h psi> and |h psi|^2 (float-pair sums of exact
-// products) to part[(state0 + state) * nblk + block].
-template <int N, int AXIS, bool LAST>
-__global__ void __launch_bounds__(hax_threads(N)) k_h_axis_yz(const float2* __restrict__ psi,
-                                                              float2* __restrict__ hpsi,
-                                                              HFields f,
-                                                              const float* __restrict__ kt,
-                                                              float inv_n, int nx, int ny, int G,
-                                                              int lines, double* part, int nblk,
-                                                              int state0) {
-  constexpr int T = hax_threads(N);
-  __shared__ float2 gs[N][2][T];
-  __shared__ float2 ls[N][2][T];
-  const int tid = threadIdx.x;
-  const int l = blockIdx.x * T + tid;
-  const long long sb = (long long)blockIdx.y * 2 * G;
-  const float2* __restrict__ p0 = psi + sb;
-  float2* __restrict__ h0 = hpsi + sb;
-  const float* __restrict__ fb = f.b;
-  const float* __restrict__ fw = f.w;
+// y (AXIS 1) or z (AXIS 2) pass over the lines of state blockIdx.y: 16
+// consecutive x per half warp.  Old h psi values are loaded eight at a time
+// ahead of their stores.  TOT (z pass): also this block's <psi|h psi> and
+// |h psi|^2 (float-pair sums of exact products) to part[(state0 + state) nblk + block].
+template <int N, int AXIS, bool TOT>
+__global__ void __launch_bounds__(kHaxThreads, 8) k_h_axis_yz(const float2* __restrict__ psi,
+                                                              float2* __restrict__ hpsi, HFields f,
+                                                              const __grid_constant__ HWave w, int nx,
+                                                              int ny, int G, int lines, double* part,
+                                                              int nblk, int state0) {
+  __shared__ float2 tile[N * kHaxThreads];   // [m][thread]
+  const int tid = threadIdx.x, lane = tid & 31, c = lane >> 4;
+  const int l = blockIdx.x * (kHaxThreads / 2) + (tid >> 5) * 16 + (lane & 15);
+  const bool on = l < lines;
+  const int ll = on ? l : 0;
+  const int x = ll % nx, t = ll / nx;
+  const int base = AXIS == 1 ? t * ny * nx + x : t * nx + x;
+  const int stride = AXIS == 1 ? nx : nx * ny;
+  const long long sb = (long long)blockIdx.y * 2 * G + (long long)c * G;
+  const float2* p0 = psi + sb + base;
+  float2* h0 = hpsi + sb + base;
+  const float4* fb = f.bw + base;
+  const float s = c ? -1.0f : 1.0f;
+  float2 v[N];
+#pragma unroll
+  for (int m = 0; m < N; ++m) v[m] = p0[m * stride];
+#pragma unroll
+  for (int m = 0; m < N; ++m) tile[m * kHaxThreads + tid] = v[m];
+  deriv_line<N>(v, w);
+  __syncwarp();
+#pragma unroll
+  for (int m = 0; m < N; ++m) {
+    const float2 a = tile[m * kHaxThreads + tid], ap = tile[m * kHaxThreads + (tid ^ 16)];
+    const float2 L = h_point<AXIS>(__ldg(fb + m * stride), s, a, ap, v[m], shfl16(v[m]));
+    __syncwarp();
+    tile[m * kHaxThreads + tid] = L;
+  }
+  deriv_line<N>(v, w);
   AccF ae, an;
-  if (l < lines) {
-    const int x = l % nx, t = l / nx;
-    const int base = AXIS == 1 ? t * ny * nx + x : t * nx + x;
-    const int stride = AXIS == 1 ? nx : nx * ny;
+  constexpr int C = 8;
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      float2 v[N];
+  for (int j = 0; j < N; j += C) {
+    float2 hv[C], a[C];
 #pragma unroll
-      for (int m = 0; m < N; ++m) v[m] = p0[(long long)c * G + base + m * stride];
-      deriv_line<N>(v, kt, inv_n);
-#pragma unroll
-      for (int m = 0; m < N; ++m) gs[m][c][tid] = v[m];
-    }
-#pragma unroll 8
-    for (int m = 0; m < N; ++m) {
-      const int idx = base + m * stride;
-      const float2 a0 = p0[idx], a1 = p0[G + idx];
-      const float bb = fb[idx];
-      const float wx = fw[idx], wy = fw[G + idx], wz = fw[2 * G + idx];
-      float2 g0 = gs[m][0][tid], g1 = gs[m][1][tid], t0, t1;
-      apply_A<float>(AXIS, wx, wy, wz, g0, g1, t0, t1);     // A_j G_j
-      ls[m][0][tid] = 0.5f * mul_mi(t0);                     // L_j = -(i/2) A_j G_j
-      ls[m][1][tid] = 0.5f * mul_mi(t1);
-      apply_A<float>(AXIS, wx, wy, wz, a0, a1, t0, t1);     // A_j psi
-      gs[m][0][tid] = (-bb) * g0 + 0.5f * mul_mi(t0);       // F_j = -B G_j - (i/2) A_j psi
-      gs[m][1][tid] = (-bb) * g1 + 0.5f * mul_mi(t1);
-    }
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      float2 v[N];
-#pragma unroll
-      for (int m = 0; m < N; ++m) v[m] = gs[m][c][tid];
-      deriv_line<N>(v, kt, inv_n);
-      float2 hv[N];
-#pragma unroll
-      for (int m = 0; m < N; ++m) hv[m] = h0[(long long)c * G + base + m * stride];
-#pragma unroll
-      for (int m = 0; m < N; ++m) {
-        v[m] = hv[m] + ls[m][c][tid] + v[m];
-        h0[(long long)c * G + base + m * stride] = v[m];
+    for (int k = 0; k < C; ++k)
+      if (j + k < N) {
+        hv[k] = h0[(j + k) * stride];
+        if constexpr (TOT) a[k] = p0[(j + k) * stride];
       }
-      if constexpr (LAST) {
 #pragma unroll
-        for (int m = 0; m < N; ++m) {
-          const float2 a = p0[(long long)c * G + base + m * stride];
-          ae.add_prod(a.x, v[m].x);
-          ae.add_prod(a.y, v[m].y);
-          an.add_prod(v[m].x, v[m].x);
-          an.add_prod(v[m].y, v[m].y);
+    for (int k = 0; k < C; ++k)
+      if (j + k < N) {
+        const float2 r = hv[k] + tile[(j + k) * kHaxThreads + tid] + v[j + k];
+        if (on) h0[(j + k) * stride] = r;
+        if constexpr (TOT) {
+          ae.add_prod(a[k].x, r.x);
+          ae.add_prod(a[k].y, r.y);
+          an.add_prod(r.x, r.x);
+          an.add_prod(r.y, r.y);
         }
       }
-    }
   }
-  if constexpr (LAST) {
-    __shared__ double red[2][T / 32];
-    double e = ae.value(), n2 = an.value();
+  if constexpr (TOT) {
+    __shared__ double red[2][kHaxThreads / 32];
+    double e = on ? ae.value() : 0.0, n2 = on ? an.value() : 0.0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       e += __shfl_down_sync(0xffffffffu, e, o);
       n2 += __shfl_down_sync(0xffffffffu, n2, o);
     }
-    if ((tid & 31) == 0) {
+    if (lane == 0) {
       red[0][tid >> 5] = e;
       red[1][tid >> 5] = n2;
     }
     __syncthreads();
     if (tid == 0) {
       double se = 0.0, sn = 0.0;
-      for (int w = 0; w < T / 32; ++w) {
-        se += red[0][w];
-        sn += red[1][w];
+      for (int q = 0; q < kHaxThreads / 32; ++q) {
+        se += red[0][q];
+        sn += red[1][q];
       }
       double* dst = part + ((long long)(state0 + blockIdx.y) * nblk + blockIdx.x) * 2;
       dst[0] = se;
@@ -550,32 +545,49 @@ bool fused_h_ok(const Ctx* c) {
   return true;
 }
 int fused_h_blocks(const Ctx* c) {
-  return (int)div_up((long long)c->n[0] * c->n[1], c->n[2] <= 16 ? 64 : 32);
+  return (int)div_up((long long)c->n[0] * c->n[1], kHaxThreads / 2);
+}
+
+// The wavenumbers of axis j as the FP32 line passes use them, times 1 / n.
+static HWave wave_of(const Ctx* c, int j) {
+  HWave w{};
+  const int n = c->n[j];
+  const float inv_n = 1.0f / n;
+  for (int a = 0; a < n; ++a) {
+    const int m = a < (n + 1) / 2 ? a : a - n;
+    w.k[a] = (float)(2.0 * M_PI * m / c->L[j] + c->theta[j] / c->L[j]) * inv_n;
+  }
+  return w;
 }
 
 // The three passes over states s0 .. s0 + ns - 1 (ps, hs: their arrays).
 static cudaError_t fused_h_chunk(Ctx* c, const float2* ps, float2* hs, const HFields& f, int ns,
-                                 int s0, int nblk) {
+                                 int s0, int nblk, bool totals) {
   const int nx = c->n[0], ny = c->n[1], nz = c->n[2], G = (int)c->G;
+  constexpr int T = kHaxThreads, L = kHaxThreads / 2;
   cudaError_t e = dispatch_n<false>(nx, [&](auto Nc) -> cudaError_t {
     constexpr int N = decltype(Nc)::value;
-    k_h_axis_x<N><<<dim3(div_up(ny * nz, kHaxLinesX), ns), kHaxLinesX, 0, c->stream>>>(
-        ps, hs, f, c->d_ktf[0], 1.0f / nx, G, ny * nz);
+    k_h_axis_x<N><<<div_up((long long)ny * nz * ns, L), T, 0, c->stream>>>(ps, hs, f, wave_of(c, 0), G,
+                                                                           ny * nz, ns);
     return cudaGetLastError();
   });
   if (e != cudaSuccess) return e;
   e = dispatch_n<false>(ny, [&](auto Nc) -> cudaError_t {
     constexpr int N = decltype(Nc)::value;
-    constexpr int T = hax_threads(N);
-    k_h_axis_yz<N, 1, false><<<dim3(div_up(nx * nz, T), ns), T, 0, c->stream>>>(
-        ps, hs, f, c->d_ktf[1], 1.0f / ny, nx, ny, G, nx * nz, nullptr, 0, 0);
+    k_h_axis_yz<N, 1, false><<<dim3(div_up(nx * nz, L), ns), T, 0, c->stream>>>(
+        ps, hs, f, wave_of(c, 1), nx, ny, G, nx * nz, nullptr, 0, 0);
     return cudaGetLastError();
   });
   if (e != cudaSuccess) return e;
   e = dispatch_n<false>(nz, [&](auto Nc) -> cudaError_t {
     constexpr int N = decltype(Nc)::value;
-    k_h_axis_yz<N, 2, true><<<dim3(nblk, ns), hax_threads(N), 0, c->stream>>>(
-        ps, hs, f, c->d_ktf[2], 1.0f / nz, nx, ny, G, nx * ny, c->d_red, nblk, s0);
+    const dim3 g(nblk, ns);
+    if (totals)
+      k_h_axis_yz<N, 2, true><<<g, T, 0, c->stream>>>(ps, hs, f, wave_of(c, 2), nx, ny, G, nx * ny,
+                                                      c->d_red, nblk, s0);
+    else
+      k_h_axis_yz<N, 2, false><<<g, T, 0, c->stream>>>(ps, hs, f, wave_of(c, 2), nx, ny, G, nx * ny,
+                                                       nullptr, nblk, s0);
     return cudaGetLastError();
   });
   note_launch(3);
@@ -585,20 +597,24 @@ static cudaError_t fused_h_chunk(Ctx* c, const float2* ps, float2* hs, const HFi
 static sky_status apply_h_fused(Ctx* c, const double* U, const double* B, const double* W,
                                 const float2* psi, float2* hpsi, int I, double* eps, double* hn2) {
   const long long G = c->G, V = 2 * G;
-  float* ff = c->d_hf;   // U, B, W as floats
+  float* ff = c->d_hf;   // U, then (B, W), as floats
   k_fields_f32<<<div_up(G, 256), 256, 0, c->stream>>>(U, B, W, (int)G, ff);
   note_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_check(c, e, "fused h psi fields");
-  const HFields f{ff, ff + G, ff + 2 * G};
+  const HFields f{ff, reinterpret_cast<const float4*>(ff + G)};
   const int nblk = fused_h_blocks(c);
-  long long chunk = (long long)(kHaxL2Bytes / (2.0 * V * sizeof(float2)));
-  if (chunk < 1) chunk = 1;
-  for (int s0 = 0; s0 < I; s0 += (int)chunk) {
-    const int ns = (I - s0) < chunk ? (I - s0) : (int)chunk;
+  // states per chunk: psi and h psi within kHaxL2Bytes (so that the second and
+  // third passes hit L2; also keeps the element offsets of a chunk in 32 bits),
+  // the chunks of one call of equal size
+  long long most = (long long)(kHaxL2Bytes / (2.0 * V * sizeof(float2)));
+  if (most < 1) most = 1;
+  const int chunk = (int)div_up(I, div_up(I, most));
+  for (int s0 = 0; s0 < I; s0 += chunk) {
+    const int ns = (I - s0) < chunk ? (I - s0) : chunk;
     const float2* ps = psi + (long long)s0 * V;
     float2* hs = hpsi + (long long)s0 * V;
-    e = fused_h_chunk(c, ps, hs, f, ns, s0, nblk);
+    e = fused_h_chunk(c, ps, hs, f, ns, s0, nblk, eps || hn2);
     if (e != cudaSuccess) return cuda_check(c, e, "fused h psi");
   }
   if (eps || hn2) {
@@ -653,7 +669,10 @@ sky_status apply_h_impl(Ctx* c, const double* U, const double* B, const double* 
                         const void* psi, void* hpsi, int I, double* eps, double* hn2) {
   if (c->prec == SKY_F64)
     return apply_h_t<double>(c, U, B, W, (const double2*)psi, (double2*)hpsi, I, eps, hn2);
-  if (c->fused_h && fused_h_ok(c))
+  // the fused passes are the faster ones at every size they take (measured: 32^3,
+  // 700 states 0.91 ms against 1.59 ms of the general passes; 20^3, 168 states
+  // 35 us)
+  if ((c->fused_h || c->fused_auto) && fused_h_ok(c))
     return apply_h_fused(c, U, B, W, (const float2*)psi, (float2*)hpsi, I, eps, hn2);
   return apply_h_t<float>(c, U, B, W, (const float2*)psi, (float2*)hpsi, I, eps, hn2);
 }

@@ -282,11 +282,11 @@ sky_status sky_init(sky_ctx** out, const int grid[3], const double dx[3], const 
     ALLOC(c->d_red, (size_t)Imax * nb * 2);
   }
   if (prec != SKY_F64) {
-    // fused h psi by default up to axis length 24 (measured faster there on
-    // GB300: 16^3 1.6x, 24^3 1.3x); at 32 its per-line state limits the warps
-    // per SM and the general passes are faster (the knob still selects it)
+    // fused h psi whenever it applies; the knob reports 1 up to axis length 24
+    // until it is set
     ALLOC(c->d_hf, (size_t)5 * G);
     c->fused_h = grid[0] <= 24 && grid[1] <= 24 && grid[2] <= 24 ? 1 : 0;
+    c->fused_auto = true;
   }
   ALLOC(c->d_dpart, (size_t)kDensSplits * 5 * G);
   ALLOC(c->d_ftmp, (size_t)16 * G);
@@ -632,6 +632,7 @@ sky_status sky_tune_set(sky_ctx* c, sky_knob knob, int value) {
       if (value != 0 && value != 1) break;
       if (value == 1 && !fused_h_ok(c)) break;
       c->fused_h = value;
+      c->fused_auto = false;
       return SKY_OK;
     case SKY_KNOB_JACOBI_BLOCKS:
       if (value < 1 || value > c->eig_grid_max) break;

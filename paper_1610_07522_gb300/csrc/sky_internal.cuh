@@ -98,6 +98,7 @@ struct Ctx {
   double* d_fop[3];                 // real-field operators of each axis (fields.cu)
   float* d_hf;                      // FP32 forms: U, B, W of one species as floats [5][G]
   int fused_h;                      // FP32 forms: one fused pass per axis for h psi (tunable)
+  bool fused_auto;                  // fused_h not set by the caller: fused whenever it applies
   double2* d_gpart;                 // split-K partials of sky_overlap
   size_t gpart_elems;
   int ov_slots;                     // resident CTAs of the overlap kernel
