@@ -13,21 +13,32 @@
 // Every G_g is a sum of integer products, so its FP32 accumulation in TMEM is
 // exact as long as it stays below 2^24: per K value |G_g| <= (g + 3) 2^14
 // (g >= 1) or 2^16 (g = 0), so a segment of 128 values of K (4 K blocks of
-// 32) is exact for every g <= 5.  One TMEM accumulator per group; group g is
-// drained ("flushed") after each of its segments, and the segments of
-// different groups end at different K blocks (staggered by g mod 4), so the
-// MMA warp waits only for the one group being drained.  The drained exact
+// 32) is exact for every g <= 5.  One TMEM accumulator of BNT columns per
+// group, the groups side by side, and the slices of B one below the other in
+// shared memory: the products of slice s of A with consecutive slices t .. t'
+// of B are one MMA of N = (t' - t + 1) BNT columns into the groups s + t ..
+// s + t'.  The groups form two sets, L = {g < S/2} and H = the rest, and no MMA
+// crosses them: 9 MMAs of up to 240 columns per 16 values of K instead of 21
+// of 80 (each reads its 128 x 16 of A from shared memory once).  A set is
+// drained ("flushed") after each of its segments, L after K blocks 1 mod 4 and
+// H after 3 mod 4; a K block issues first the set whose segment ends, commits
+// it, then the other, and the next block starts with that other set, so a
+// drain has the products of two half blocks to hide behind.  The drained exact
 // sums are added, scaled by 2^{-8g}, into an unevaluated FP32 pair (hi, lo)
 // per output element by error-free TwoSum (about 48 significant bits).
+// What bounds it: 21 x 40 tensor cycles per 16 values of K against the L2 feed
+// (78 KiB per K block and SM).  24^3, 280 states, one overlap: 560 us with one
+// MMA per slice pair issued by one lane of a diverged warp (about 160 cycles
+// from one to the next), XXX us.
 //
 // Persistent kernel, one CTA per SM; work items are (128 x BNT output tile,
 // K range).  Warp roles:
 //   warp 0     TMA producer: 3D cp.async.bulk.tensor loads of one 32-wide K
 //              block of every slice of A (128 rows) and B (BNT rows), 64-byte
 //              swizzle, into a ring of stages;
-//   warp 1     owns TMEM (S accumulators of BNT fp32 columns) and one elected
-//              lane issues tcgen05.mma (M = 128, N = BNT, K = 16): for each K
-//              block and group g all products (s, g - s);
+//   warp 1     owns TMEM (S accumulators of BNT fp32 columns) and issues
+//              tcgen05.mma (M = 128, K = 16) as a converged warp, one elected
+//              lane executing them;
 //   warps 2-9  epilogue: two warps per TMEM lane quadrant, each half of the
 //              columns; drain a group when its segment ends, accumulate
 //              (hi, lo); write the item's result at its end.
@@ -35,6 +46,8 @@
 // word, the kernel waits (bounded) for the MMAs it issued, frees TMEM and
 // returns.
 #pragma once
+
+#include <type_traits>
 
 #include "tc_gemm.cuh"
 
@@ -47,8 +60,6 @@ using tc::idesc_bf16;
 using tc::mbar_expect_tx;
 using tc::mbar_init;
 using tc::mbar_wait;
-using tc::mma_bf16;
-using tc::mma_commit;
 using tc::smem_u32;
 
 constexpr int BM = 128;
@@ -77,11 +88,11 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
 }
 // Shared-memory matrix descriptor: K-major tile with 64-byte swizzle, rows of
 // 64 bytes, 8-row groups 512 bytes apart (stride byte offset), descriptor
-// version 1, layout type 4 (64B swizzle).
-__device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
-  return (uint64_t)((saddr >> 4) & 0x3FFFu) | (1ull << 16) | (32ull << 32) | (1ull << 46) |
-         (4ull << 61);
+// version 1, layout type 4 (64B swizzle).  Low word by address, high word fixed.
+__device__ __forceinline__ uint32_t sw64_lo(uint32_t saddr) {
+  return ((saddr >> 4) & 0x3FFFu) | (1u << 16);
 }
+constexpr uint32_t kSw64Hi = 32u | (1u << 14) | (4u << 29);
 // NC consecutive fp32 columns (NC = 8, 16 or 32) of this warp's 32 TMEM lanes.
 template <int NC>
 __device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t* r);
@@ -116,19 +127,52 @@ __device__ __forceinline__ void tmem_ld<32>(uint32_t taddr, uint32_t* r) {
         "=r"(r[31])
       : "r"(taddr));
 }
-// Columns [0, NC) of a warp's share, NC = 40 or 48, as 32 + 8 or 32 + 16.
+// Columns [0, NC) of a warp's share, NC = 40 or 48, as 32 + 8 or 32 + 16
+// (complete after tmem_wait).
 template <int NC>
 __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t* r) {
   static_assert(NC == 40 || NC == 48, "column share");
   tmem_ld<32>(taddr, r);
   tmem_ld<NC - 32>(taddr + 32, r + 32);
+}
+__device__ __forceinline__ void tmem_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// Group g's segment ends after K block j (of nkb in the item): every kSegKB
-// blocks, offset by g mod kSegKB, and at the item's last block.
-__device__ __forceinline__ bool flush_at(int j, int g, int nkb) {
-  return j == nkb - 1 || ((j + 1 + (g % kSegKB)) % kSegKB) == 0;
+// The segment of set h (0: L, 1: H) ends after K block j (of nkb in the item):
+// every kSegKB blocks, H two blocks after L, and at the item's last block.
+__device__ __forceinline__ bool flush_at(int j, int h, int nkb) {
+  return j == nkb - 1 || (j & (kSegKB - 1)) == (h ? 3 : 1);
+}
+static_assert(kSegKB == 4, "segment schedule");
+
+// One lane of a converged warp, as a flag (the same lane at every use of it).
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+  return e;
+}
+// tcgen05.mma and its commit by the elected lane only, the warp converged
+// around them; descriptors as low words with one common high word.
+__device__ __forceinline__ void mma_bf16_elect(uint32_t tmem_d, uint32_t da, uint32_t db, uint32_t dhi,
+                                               uint32_t idesc, uint32_t accumulate, uint32_t el) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n .reg .b64 a, b;\n setp.ne.b32 p, %5, 0;\n setp.ne.b32 q, %6, 0;\n"
+      " mov.b64 a, {%1, %3};\n mov.b64 b, {%2, %3};\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n}\n" ::"r"(tmem_d),
+      "r"(da), "r"(db), "r"(dhi), "r"(idesc), "r"(accumulate), "r"(el)
+      : "memory");
+}
+__device__ __forceinline__ void mma_commit_elect(uint32_t bar, uint32_t el) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
+      "r"(el)
+      : "memory");
+}
+// The bounded wait by a whole converged warp.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity));
 }
 
 struct OzArgs {
@@ -290,13 +334,15 @@ __device__ __forceinline__ void oz_gemm_body(const CUtensorMap* pA, const CUtens
   constexpr int HALF = BNT / 2;
   unsigned long long* bars = (unsigned long long*)(base + STAGES * STAGE);
   uint32_t* tmem_slot = (uint32_t*)(bars + 2 * kMaxStages + 2 * kMaxS + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int HS = S / 2;                 // groups per set
+  static_assert(S % 2 == 0 && HS * BNT <= 256 && HS <= 3, "sets of groups");
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int nitems = GROUP ? grp->tile0[grp->np] : a.ntiles * a.nsplit;
   const uint32_t bar0 = smem_u32(bars);
   auto full = [&](int s) { return bar0 + 8u * s; };
   auto empty = [&](int s) { return bar0 + 8u * (kMaxStages + s); };
-  auto acc_full = [&](int g) { return bar0 + 8u * (2 * kMaxStages + g); };
-  auto acc_empty = [&](int g) { return bar0 + 8u * (2 * kMaxStages + kMaxS + g); };
+  auto acc_full = [&](int h) { return bar0 + 8u * (2 * kMaxStages + h); };
+  auto acc_empty = [&](int h) { return bar0 + 8u * (2 * kMaxStages + kMaxS + h); };
   const uint32_t drain = bar0 + 8u * (2 * kMaxStages + 2 * kMaxS);
 
   if (threadIdx.x == 0) {
@@ -304,9 +350,9 @@ __device__ __forceinline__ void oz_gemm_body(const CUtensorMap* pA, const CUtens
       mbar_init(full(s), 1);
       mbar_init(empty(s), 1);
     }
-    for (int g = 0; g < S; ++g) {
-      mbar_init(acc_full(g), 1);
-      mbar_init(acc_empty(g), kEpiWarps);   // one arrival per epilogue warp
+    for (int h = 0; h < 2; ++h) {
+      mbar_init(acc_full(h), 1);
+      mbar_init(acc_empty(h), kEpiWarps);   // one arrival per epilogue warp
     }
     mbar_init(drain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -352,70 +398,78 @@ __device__ __forceinline__ void oz_gemm_body(const CUtensorMap* pA, const CUtens
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = idesc_bf16(BM, BNT);
-      uint32_t nfl[S];
+    // the whole warp runs the loop, converged; the elected lane issues
+    const uint32_t el = elect_one();
+    uint32_t nfl[2] = {0u, 0u};
+    long long gpos = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < nitems && ok; t += gridDim.x) {
+      OzItem it;
+      if (!item_at<GROUP>(a, grp, BNT, t, it)) continue;
+      const int nkb = it.nkb;
+      for (int j = 0; j < nkb && ok; ++j, ++gpos) {
+        const int s = (int)(gpos % STAGES);
+        const long long u = gpos / STAGES;
+        if (!mbar_wait_warp(full(s), (uint32_t)(u & 1))) {
+          if (lane == 0) flag_status(a.status, SKY_ETIMEOUT);
+          ok = false;
+          break;
+        }
+        fence_after();
+        const uint32_t la = sw64_lo(smem_u32(base + s * STAGE));
+        const uint32_t lb = sw64_lo(smem_u32(base + s * STAGE + S * TILE_A));
 #pragma unroll
-      for (int g = 0; g < S; ++g) nfl[g] = 0;
-      long long gpos = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < nitems && ok; t += gridDim.x) {
-        OzItem it;
-        if (!item_at<GROUP>(a, grp, BNT, t, it)) continue;
-        const int nkb = it.nkb;
-        for (int j = 0; j < nkb && ok; ++j, ++gpos) {
-          const int s = (int)(gpos % STAGES);
-          const long long u = gpos / STAGES;
-          if (!mbar_wait(full(s), (uint32_t)(u & 1))) {
-            flag_status(a.status, SKY_ETIMEOUT);
-            ok = false;
-            break;
-          }
-          fence_after();
-          const uint32_t sa = smem_u32(base + s * STAGE);
-#pragma unroll
-          for (int g = 0; g < S; ++g) {
-            const bool seg_start = (j == 0) || flush_at(j - 1, g, nkb);
-            if (seg_start && nfl[g] > 0) {
-              // the epilogue must have drained this group's previous segment
-              if (!mbar_wait(acc_empty(g), (nfl[g] - 1) & 1)) {
-                flag_status(a.status, SKY_ETIMEOUT);
-                ok = false;
-                break;
-              }
-              fence_after();
+        for (int o = 0; o < 2; ++o) {
+          const int h = (j & 2) ? 1 - o : o;     // the set whose segment may end here first
+          const bool start = j == 0 || flush_at(j - 1, h, nkb);
+          if (start && nfl[h] > 0) {
+            // the epilogue must have drained this set's previous segment
+            if (!mbar_wait_warp(acc_empty(h), (nfl[h] - 1) & 1)) {
+              if (lane == 0) flag_status(a.status, SKY_ETIMEOUT);
+              ok = false;
+              break;
             }
-            const uint32_t acc = tmem + (uint32_t)(g * BNT);
+            fence_after();
+          }
+          auto issue = [&](auto hc) {
+            constexpr int H = decltype(hc)::value;
 #pragma unroll
-            for (int p = 0; p <= g; ++p) {
-              const uint64_t da = sw64_desc(sa + p * TILE_A);
-              const uint64_t db = sw64_desc(sa + S * TILE_A + (g - p) * TILE_B);
+            for (int p = 0; p < (H ? S : HS); ++p) {
+              constexpr int top = H ? S : HS;
+              const int g0 = H && p < HS ? HS : p;         // first group
+              const int q0 = g0 - p;                        // first slice of B
+              const uint32_t idesc = idesc_bf16(BM, (top - g0) * BNT);
 #pragma unroll
               for (int k = 0; k < BK / 16; ++k)   // +32 bytes along K = +2 in the encoded address
-                mma_bf16(acc, da + 2ull * k, db + 2ull * k, idesc,
-                         (seg_start && p == 0 && k == 0) ? 0u : 1u);
+                mma_bf16_elect(tmem + (uint32_t)(g0 * BNT), la + (uint32_t)(p * (TILE_A >> 4) + 2 * k),
+                               lb + (uint32_t)(q0 * (TILE_B >> 4) + 2 * k), kSw64Hi, idesc,
+                               (start && p == 0 && k == 0) ? 0u : 1u, el);
             }
+          };
+          if (h) issue(std::integral_constant<int, 1>{});
+          else issue(std::integral_constant<int, 0>{});
+          if (flush_at(j, h, nkb)) {
+            mma_commit_elect(acc_full(h), el);   // arrives when this set's MMAs have completed
+            ++nfl[h];
           }
-          if (!ok) break;
-          mma_commit(empty(s));
-#pragma unroll
-          for (int g = 0; g < S; ++g)
-            if (flush_at(j, g, nkb)) {
-              mma_commit(acc_full(g));   // arrives when this group's MMAs have completed
-              ++nfl[g];
-            }
         }
+        if (!ok) break;
+        mma_commit_elect(empty(s), el);
       }
-      // every MMA issued by this thread completes before TMEM is freed
-      mma_commit(drain);
-      if (!mbar_wait(drain, 0)) flag_status(a.status, SKY_ETIMEOUT);
     }
+    // every MMA issued by this warp completes before TMEM is freed
+    mma_commit_elect(drain, el);
+    if (!mbar_wait_warp(drain, 0) && lane == 0) flag_status(a.status, SKY_ETIMEOUT);
   } else {
     // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31, columns half * HALF ..
     const int q = warp & 3, half = (warp - 2) >> 2;
-    uint32_t efl[S];
-#pragma unroll
-    for (int g = 0; g < S; ++g) efl[g] = 0;
+    uint32_t efl[2] = {0u, 0u};
+    auto hand_back = [&](int h) {            // this warp's lanes of the set are read
+      fence_before();
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty(h)) : "memory");
+    };
     bool ok = true;
     for (int t = blockIdx.x; t < nitems && ok; t += gridDim.x) {
       OzItem it;
@@ -426,26 +480,44 @@ __device__ __forceinline__ void oz_gemm_body(const CUtensorMap* pA, const CUtens
       for (int c = 0; c < HALF; ++c) hi[c] = lo[c] = 0.0f;
       for (int j = 0; j < nkb && ok; ++j) {
 #pragma unroll
-        for (int g = 0; g < S; ++g) {
-          if (!flush_at(j, g, nkb)) continue;
-          if (!mbar_wait(acc_full(g), efl[g] & 1)) {
+        for (int h = 0; h < 2; ++h) {
+          if (!flush_at(j, h, nkb)) continue;
+          if (!mbar_wait_warp(acc_full(h), efl[h] & 1)) {
             if (lane == 0) flag_status(a.status, SKY_ETIMEOUT);
             ok = false;
             break;
           }
           fence_after();
-          uint32_t v[HALF];
-          tmem_ld_cols<HALF>(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(g * BNT + half * HALF),
-                             v);
-          // this warp's lanes of the accumulator are read: hand it back
-          fence_before();
-          __syncwarp();
-          if (lane == 0)
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty(g)) : "memory");
-          ++efl[g];
-          const float sc = __int_as_float((127 - 8 * g) << 23);   // 2^{-8g}, exact
+          const uint32_t col = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * HS * BNT + half * HALF);
+          auto add = [&](const uint32_t* v, int g) {
+            const float sc = __int_as_float((127 - 8 * g) << 23);   // 2^{-8g}, exact
 #pragma unroll
-          for (int c = 0; c < HALF; ++c) two_sum_acc(hi[c], lo[c], __uint_as_float(v[c]) * sc);
+            for (int c = 0; c < HALF; ++c) two_sum_acc(hi[c], lo[c], __uint_as_float(v[c]) * sc);
+          };
+          // hand the set back as early as the registers allow: two of three
+          // groups at once, the third after the first has been added; with two
+          // wider groups, one at a time
+          uint32_t v0[HALF];
+          tmem_ld_cols<HALF>(col, v0);
+          if constexpr (HS == 3) {
+            uint32_t v1[HALF];
+            tmem_ld_cols<HALF>(col + BNT, v1);
+            tmem_wait();
+            add(v0, h * HS);
+            tmem_ld_cols<HALF>(col + 2 * BNT, v0);
+            tmem_wait();
+            hand_back(h);
+            add(v1, h * HS + 1);
+            add(v0, h * HS + 2);
+          } else {
+            tmem_wait();
+            add(v0, h * HS);
+            tmem_ld_cols<HALF>(col + BNT, v0);
+            tmem_wait();
+            hand_back(h);
+            add(v0, h * HS + 1);
+          }
+          ++efl[h];
         }
       }
       if (!ok) break;
