@@ -308,7 +308,7 @@ sky_status sky_set_prec(sky_ctx* ctx, sky_prec prec);
  *   SKY_KNOB_OVERLAP_WAVES  FMA overlap: K splits filling 1 or 2 waves of blocks
  *   SKY_KNOB_TC_WAVES       split-BF16 overlap: K splits filling 1, 2 or 4 waves of SMs,
  *                           or 0: the fewest splits the FP32 accumulation bound allows
- *                           (2048 values of K each; for contexts that share the GPU with
+ *                           (at most 2048 values of K each; for contexts that share the GPU with
  *                           other boxes' work)
  *   SKY_KNOB_TC_TILE_N      split-BF16 overlap and recombination GEMM tiles: 128 x 256
  *                           (256), 128 x 128 (128) or 0 (default: 256 for x3 when N allows)

@@ -131,11 +131,20 @@ static inline long long round8(long long x) { return (x + 7) / 8 * 8; }   // 16-
 int tc_nsplit(sky_prec p) { return p == SKY_F32_BF16X6 ? 3 : 2; }
 
 // FP32 accumulation in TMEM loses accuracy over long K (its rounding error
-// grows like sqrt(K) 2^-24 of the partial sums): every split-K partial of the
-// overlap covers at most kMaxAccK values of K, and the partials are summed in
-// FP64 by the reduce.
+// grows with the length of the sum): every split-K partial of the overlap
+// covers at most kMaxAccK values of K, and the partials are summed in FP64 by
+// the reduce.  Where the partials of half that length are small enough to stay
+// in L2 (kSmallPartials), they are half as long: it costs nothing there (small
+// boxes have too few tiles to fill the GPU otherwise) and halves the error (12^3,
+// 43 states: the energy 5e-5 MeV per nucleon from that of 64-value partials
+// with 2048, 2e-5 with 1024).
 constexpr long long kMaxAccK = 2048;
-int tc_min_splits(long long K) { return (int)((K + kMaxAccK - 1) / kMaxAccK); }
+constexpr long long kSmallPartials = 4LL << 20;   // fp32 values of all partials
+int tc_min_splits(long long K, int I) {
+  const long long z = (K + kMaxAccK / 2 - 1) / (kMaxAccK / 2);
+  const long long ldd = (2LL * I + 3) / 4 * 4;
+  return (int)(z * I * ldd <= kSmallPartials ? z : (K + kMaxAccK - 1) / kMaxAccK);
+}
 
 // Scratch (bf16 elements per piece / fp32 partials) for I states of V complex.
 void tc_scratch_sizes(int I, long long V, int num_sms, size_t* piece_a, size_t* piece_b,
@@ -147,10 +156,12 @@ void tc_scratch_sizes(int I, long long V, int num_sms, size_t* piece_a, size_t* 
   const long long ldd = (2LL * I + 3) / 4 * 4;
   const int tiles = ((I + tc::BM - 1) / tc::BM) * ((2 * I + tc::BN - 1) / tc::BN);
   int z = kMaxTcWaves * num_sms / (tiles > 0 ? tiles : 1);
-  const int zacc = tc_min_splits(K);
+  const int zacc = (int)((K + kMaxAccK - 1) / kMaxAccK);
   if (z < zacc) z = zacc;
   if (z < 1) z = 1;
   *partial = (size_t)z * I * ldd;
+  // fewer states may take more splits (kSmallPartials values at most)
+  if (*partial < (size_t)kSmallPartials) *partial = (size_t)kSmallPartials;
 }
 
 sky_status tc_overlap(Ctx* c, const void* a, const void* b, int I, double2* X) {
@@ -173,7 +184,7 @@ sky_status tc_overlap(Ctx* c, const void* a, const void* b, int I, double2* X) {
   // tc_waves 0: the fewest splits the accumulation bound allows (for boxes
   // that share the GPU with others), else about that many waves of SMs
   int z = c->tc_waves * c->num_sms / tiles;
-  if (z < tc_min_splits(K)) z = tc_min_splits(K);   // bounded FP32 accumulation length
+  if (z < tc_min_splits(K, I)) z = tc_min_splits(K, I);   // bounded FP32 accumulation length
   if (z < 1) z = 1;
   const long long sstride = (long long)I * ldd;
   if ((size_t)z * sstride > c->tc_partial_elems) z = (int)(c->tc_partial_elems / sstride);
