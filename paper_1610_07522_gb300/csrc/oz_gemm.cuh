@@ -26,22 +26,33 @@
 // drain has the products of two half blocks to hide behind.  The drained exact
 // sums are added, scaled by 2^{-8g}, into an unevaluated FP32 pair (hi, lo)
 // per output element by error-free TwoSum (about 48 significant bits).
-// What bounds it: 21 x 40 tensor cycles per 16 values of K against the L2 feed
-// (78 KiB per K block and SM).  24^3, 280 states, one overlap: 560 us with one
-// MMA per slice pair issued by one lane of a diverged warp (about 160 cycles
-// from one to the next), XXX us.
+// What bounds it: shared memory.  Per 16 values of K the MMAs read 9 x 4 + 21 x
+// 2.5 KiB of operands against 840 cycles on the tensor pipe, and the copies write
+// 39 KiB: about 1000 cycles at 128 bytes per clock.  24^3, 280 states, one
+// overlap: 560 us with one MMA per slice pair issued by one lane of a diverged
+// warp (about 117 cycles from one to the next), 310 us now (1360 cycles).
 //
 // Persistent kernel, one CTA per SM; work items are (128 x BNT output tile,
 // K range).  Warp roles:
-//   warp 0     TMA producer: 3D cp.async.bulk.tensor loads of one 32-wide K
-//              block of every slice of A (128 rows) and B (BNT rows), 64-byte
-//              swizzle, into a ring of stages;
+//   warp 0     producer: bulk copies of one 32-wide K block of every slice of A
+//              (128 rows) and B (BNT rows) into a ring of stages;
 //   warp 1     owns TMEM (S accumulators of BNT fp32 columns) and issues
 //              tcgen05.mma (M = 128, K = 16) as a converged warp, one elected
 //              lane executing them;
 //   warps 2-9  epilogue: two warps per TMEM lane quadrant, each half of the
 //              columns; drain a group when its segment ends, accumulate
 //              (hi, lo); write the item's result at its end.
+// Operand layout in global memory (dig_off): the shared-memory image itself,
+// blocks of BNT rows x 32 values of K x S slices, K block outermost, then the
+// row tile, then the slice, each slice BNT rows of 64 bytes with the 16-byte
+// chunks of a row in the 64-byte swizzle's order.  A tile of B is one contiguous
+// 30 kB copy and 128 rows of A are two or three runs per slice; against tensor
+// maps over row-major digits the product itself stays the same (310-315 us), the
+// split kernels write whole blocks (103 -> 86 us per operand) and the small
+// I x I products start sooner (17 -> 15 us; no maps to encode and fetch).
+// Rows beyond an operand's last are never read as far as results go: whatever
+// they hold reaches only outputs that are not stored; K beyond the operand's
+// last value holds zeros.
 // Every mbarrier wait is bounded; a timeout sets SKY_ETIMEOUT in the status
 // word, the kernel waits (bounded) for the MMAs it issued, frees TMEM and
 // returns.
@@ -78,12 +89,22 @@ constexpr int TILE_A = BM * BK * 2;       // 8 KiB per A slice tile
 constexpr int kS64 = 6, kBN64 = 80;
 constexpr int kS32 = 4, kBN32 = 96;
 
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1,
-                                            int c2, uint32_t bar) {
+// Element (row, k) of slice s of an operand of nt row tiles of BNT rows (2-byte
+// elements); eight consecutive k from a multiple of 8 are consecutive.
+template <int S, int BNT>
+__host__ __device__ __forceinline__ long long dig_off(int row, int k, int s, int nt) {
+  const int t = row / BNT, r = row - t * BNT;
+  return (((long long)(k >> 5) * nt + t) * S + s) * (BNT * BK) + r * BK +
+         ((((k >> 3) & 3) ^ ((r >> 1) & 3)) << 3) + (k & 7);
+}
+__host__ __device__ constexpr long long dig_tiles(long long rows, int bnt) { return (rows + bnt - 1) / bnt; }
+__host__ __device__ constexpr long long dig_elems(long long rows, long long K, int S, int bnt) {
+  return (K + BK - 1) / BK * dig_tiles(rows, bnt) * S * bnt * BK;
+}
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
-      "l"((unsigned long long)map), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+      "l"(src), "r"(bytes), "r"(bar)
       : "memory");
 }
 // Shared-memory matrix descriptor: K-major tile with 64-byte swizzle, rows of
@@ -176,7 +197,10 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity) {
 }
 
 struct OzArgs {
-  int M, N, K;              // rows of A, rows of B, K (bf16 elements, within the maps)
+  const unsigned short* A;  // operands in the blocked layout, nta and ntb row tiles
+  const unsigned short* B;
+  int nta, ntb;
+  int M, N, K;              // rows of A, rows of B, K
   int kb_per_split;         // K blocks per split
   int nsplit;               // K splits
   int tri;                  // overlap lower-triangle pruning: B = [b; b'] with I rows each
@@ -239,18 +263,19 @@ __host__ __device__ inline void item_of(const OzArgs& a, int bnt, int t, int& m0
 }
 
 // Grouped products: np independent n x n complex products in one launch
-// (the many small problems of a batched eigensolve).  Problem b's operand
-// rows are stacked in the two maps (A rows ra[b] .. ra[b] + n - 1, B rows
-// rb[b] .. rb[b] + 2n - 1, K = 2n digits per row, zero beyond); its items
-// are the output tiles tile0[b] .. tile0[b+1] - 1 (one K range each); its
-// partials go to P + po[b], rows of 2n.  A tile that runs past the problem's
-// rows reads the next problem's rows, whose results are not stored.
+// (the many small problems of a batched eigensolve).  Problem b's operands lie
+// in the blocked layout from a.A + ao[b] (n rows) and a.B + bo[b] (2n rows), K =
+// 2n, their row exponents from ra[b] and rb[b]; its items are the output tiles
+// tile0[b] .. tile0[b+1] - 1 (one K range each); its partials go to P + po[b],
+// rows of 2n.
 struct OzGroup {
   int np;
   int tile0[kMaxBatch + 1];
   int n[kMaxBatch];
   int ra[kMaxBatch];
   int rb[kMaxBatch];
+  long long ao[kMaxBatch];
+  long long bo[kMaxBatch];
   long long po[kMaxBatch];
   const double2* A[kMaxBatch];
   const double2* B[kMaxBatch];
@@ -263,11 +288,13 @@ __host__ __device__ inline bool group_gated(const OzGroup& G, int b) {
   return (G.run[b] && *G.run[b] == 0) || (G.stop[b] && *G.stop[b] != 0);
 }
 
-// One work item: global map rows m0 (A) and n0 (B), K blocks kb0 .. kb0 +
-// nkb - 1, output rows / columns from (mloc, nloc) within an M x N result
-// (of problem b in a grouped launch).
+// One work item: rows from m0 (A) and n0 (B), K blocks kb0 .. kb0 + nkb - 1 of
+// the operands A, B (nta, ntb row tiles), of an M x N result (of problem b in a
+// grouped launch).
 struct OzItem {
-  int m0, n0, kb0, nkb, b, mloc, nloc, M, N;
+  const unsigned short *A, *B;
+  int nta, ntb;
+  int m0, n0, kb0, nkb, b, M, N;
 };
 
 template <bool GROUP>
@@ -284,10 +311,12 @@ __device__ __forceinline__ bool item_at(const OzArgs& a, const OzGroup* G, int b
     const int mt = (n + BM - 1) / BM, tt = t - G->tile0[b];
     const int mi = tt % mt, nj = tt / mt;
     it.b = b;
-    it.mloc = mi * BM;
-    it.nloc = nj * bnt;
-    it.m0 = G->ra[b] + it.mloc;
-    it.n0 = G->rb[b] + it.nloc;
+    it.m0 = mi * BM;
+    it.n0 = nj * bnt;
+    it.A = a.A + G->ao[b];
+    it.B = a.B + G->bo[b];
+    it.nta = (n + bnt - 1) / bnt;
+    it.ntb = (2 * n + bnt - 1) / bnt;
     it.kb0 = 0;
     it.nkb = (2 * n + BK - 1) / BK;
     it.M = n;
@@ -295,8 +324,10 @@ __device__ __forceinline__ bool item_at(const OzArgs& a, const OzGroup* G, int b
   } else {
     item_of(a, bnt, t, it.m0, it.n0, it.kb0, it.nkb);
     it.b = t / a.ntiles;   // the K split
-    it.mloc = it.m0;
-    it.nloc = it.n0;
+    it.A = a.A;
+    it.B = a.B;
+    it.nta = a.nta;
+    it.ntb = a.ntb;
     it.M = a.M;
     it.N = a.N;
   }
@@ -317,8 +348,7 @@ __device__ __forceinline__ double pow2d(int k) {
 }
 
 template <int S, int BNT, bool GROUP>
-__device__ __forceinline__ void oz_gemm_body(const CUtensorMap* pA, const CUtensorMap* pB,
-                                             const OzArgs& a, const OzGroup* grp) {
+__device__ __forceinline__ void oz_gemm_body(const OzArgs& a, const OzGroup* grp) {
   if ((a.run && *a.run == 0) || (a.stop && *a.stop != 0)) return;   // uniform in the CTA
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = (unsigned char*)(((unsigned long long)smem_raw + 1023ull) & ~1023ull);
@@ -371,30 +401,40 @@ __device__ __forceinline__ void oz_gemm_body(const CUtensorMap* pA, const CUtens
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // stage layout: A slices 0..S-1, then B slices 0..S-1
-      long long g = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < nitems && ok; t += gridDim.x) {
-        OzItem it;
-        if (!item_at<GROUP>(a, grp, BNT, t, it)) continue;
-        const int m0 = it.m0, n0 = it.n0, kb0 = it.kb0, nkb = it.nkb;
-        for (int j = 0; j < nkb; ++j, ++g) {
-          const int s = (int)(g % STAGES);
-          const long long u = g / STAGES;
-          if (u > 0 && !mbar_wait(empty(s), (uint32_t)((u - 1) & 1))) {
-            flag_status(a.status, SKY_ETIMEOUT);
-            ok = false;
-            break;
-          }
-          const uint32_t sa = smem_u32(base + s * STAGE);
-          mbar_expect_tx(full(s), STAGE);
-          const int kc = (kb0 + j) * BK;
-          for (int p = 0; p < S; ++p) {
-            tma_load_3d(sa + p * TILE_A, pA, kc, m0, p, full(s));
-            tma_load_3d(sa + S * TILE_A + p * TILE_B, pB, kc, n0, p, full(s));
-          }
+    // stage layout: A slices 0..S-1, then B slices 0..S-1.  Lane 0 arms the
+    // stage's barrier and copies B; lane i copies run i % 3 (a row tile of A) of
+    // slice i / 3.
+    static_assert(3 * S <= 32 && 2 * BNT >= BM, "runs of A");
+    long long g = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < nitems && ok; t += gridDim.x) {
+      OzItem it;
+      if (!item_at<GROUP>(a, grp, BNT, t, it)) continue;
+      const int end = it.m0 + BM < it.nta * BNT ? it.m0 + BM : it.nta * BNT;   // rows that exist
+      const int p = lane / 3, ta = it.m0 / BNT + lane % 3;
+      const int lo = ta * BNT > it.m0 ? ta * BNT : it.m0;
+      const int hi = (ta + 1) * BNT < end ? (ta + 1) * BNT : end;
+      const bool mine = lane < 3 * S && hi > lo;
+      const long long ka = (long long)it.nta * S * (BNT * BK), kb = (long long)it.ntb * S * (BNT * BK);
+      const unsigned short* srcA =
+          it.A + it.kb0 * ka + ((long long)ta * S + p) * (BNT * BK) + (long long)(lo - ta * BNT) * BK;
+      const unsigned short* srcB = it.B + it.kb0 * kb + (long long)(it.n0 / BNT) * S * (BNT * BK);
+      const uint32_t dstA = (uint32_t)(p * TILE_A + (lo - it.m0) * (BK * 2));
+      for (int j = 0; j < it.nkb; ++j, ++g, srcA += ka, srcB += kb) {
+        const int s = (int)(g % STAGES);
+        const long long u = g / STAGES;
+        if (u > 0 && !mbar_wait_warp(empty(s), (uint32_t)((u - 1) & 1))) {
+          if (lane == 0) flag_status(a.status, SKY_ETIMEOUT);
+          ok = false;
+          break;
         }
+        const uint32_t sa = smem_u32(base + s * STAGE);
+        if (lane == 0) {
+          mbar_expect_tx(full(s), (uint32_t)(S * (end - it.m0) * (BK * 2) + S * TILE_B));
+          bulk_load(sa + S * TILE_A, srcB, S * TILE_B, full(s));
+        }
+        __syncwarp();
+        if (mine) bulk_load(sa + dstA, srcA, (uint32_t)((hi - lo) * (BK * 2)), full(s));
       }
     }
   } else if (warp == 1) {
@@ -521,8 +561,8 @@ __device__ __forceinline__ void oz_gemm_body(const CUtensorMap* pA, const CUtens
         }
       }
       if (!ok) break;
-      const int row = it.mloc + q * 32 + lane;
-      const int col0 = it.nloc + half * HALF;
+      const int row = it.m0 + q * 32 + lane;
+      const int col0 = it.n0 + half * HALF;
       if (row < it.M) {
         if (GROUP || a.mode == 0) {
           float2* prow = GROUP ? a.P + grp->po[it.b] + (long long)row * it.N
@@ -564,17 +604,14 @@ __device__ __forceinline__ void oz_gemm_body(const CUtensorMap* pA, const CUtens
 }
 
 template <int S, int BNT>
-__global__ void __launch_bounds__(THREADS, 1)
-    k_oz_gemm(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB,
-              OzArgs a) {
-  oz_gemm_body<S, BNT, false>(&mA, &mB, a, nullptr);
+__global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ OzArgs a) {
+  oz_gemm_body<S, BNT, false>(a, nullptr);
 }
 
 template <int S, int BNT>
 __global__ void __launch_bounds__(THREADS, 1)
-    k_oz_gemm_group(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB,
-                    OzArgs a, const __grid_constant__ OzGroup grp) {
-  oz_gemm_body<S, BNT, true>(&mA, &mB, a, &grp);
+    k_oz_gemm_group(const __grid_constant__ OzArgs a, const __grid_constant__ OzGroup grp) {
+  oz_gemm_body<S, BNT, true>(a, &grp);
 }
 
 template <int S, int BNT>
@@ -583,31 +620,6 @@ constexpr int smem_bytes() {
   constexpr int st = (kSmemMax - kSmemExtra) / stage < kMaxStages ? (kSmemMax - kSmemExtra) / stage
                                                                     : kMaxStages;
   return st * stage + kSmemExtra;
-}
-
-// 3D bf16 map: slices [S][rows][ld] (ld, slice stride in elements, multiples
-// of 8), box BK x box_rows x 1, 64-byte swizzle; rows beyond `rows` and K
-// beyond `K` read as zeros.
-inline cudaError_t make_map3(CUtensorMap* map, const void* ptr, int S, int rows, int K, long long ld,
-                             long long slice_stride, int box_rows) {
-  static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-  if (!encode) {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000,
-                                                     cudaEnableDefault, &q);
-    if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-    encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
-  }
-  const cuuint64_t gdim[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)S};
-  const cuuint64_t gstride[2] = {(cuuint64_t)ld * 2, (cuuint64_t)slice_stride * 2};
-  const cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)box_rows, 1};
-  const cuuint32_t estride[3] = {1, 1, 1};
-  CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), gdim,
-                      gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                      CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 // Number of output tiles of an M x N product (pruned to the tiles that hold
@@ -624,20 +636,15 @@ inline int count_tiles(int M, int N, int bnt, bool tri, int I) {
   return n;
 }
 
-// Launch k_oz_gemm<S, BNT>.  A: slices [S][M][K] (row stride lda, slice
-// stride sa), B: [S][N][K] (ldb, sb), all 16-byte aligned.  *splits in: the
-// K splits wanted; out: the splits used (mode 0 writes P[z] for z < *splits).
+// Launch k_oz_gemm<S, BNT> on A (M rows) and B (N rows) in the blocked layout,
+// 16-byte aligned, nta and ntb row tiles.  *splits in: the K splits wanted; out:
+// the splits used (mode 0 writes P[z] for z < *splits).
 template <int S, int BNT>
-inline cudaError_t oz_gemm(const void* A, long long lda, long long sa, int M, const void* B,
-                           long long ldb, long long sb, int N, int K, bool tri, int I, OzArgs g,
-                           int* splits, cudaStream_t s) {
+inline cudaError_t oz_gemm(const void* A, int nta, int M, const void* B, int ntb, int N, int K, bool tri,
+                           int I, OzArgs g, int* splits, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) { *splits = 0; return cudaSuccess; }
-  if ((lda & 7) || (ldb & 7) || (sa & 7) || (sb & 7) || lda < K || ldb < K)
-    return cudaErrorInvalidValue;
-  CUtensorMap ma, mb;
+  if (dig_tiles(M, BNT) > nta || dig_tiles(N, BNT) > ntb) return cudaErrorInvalidValue;
   cudaError_t e;
-  if ((e = make_map3(&ma, A, S, M, K, lda, sa, BM)) != cudaSuccess) return e;
-  if ((e = make_map3(&mb, B, S, N, K, ldb, sb, BNT)) != cudaSuccess) return e;
   static bool smem_set[64] = {false};
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -651,6 +658,9 @@ inline cudaError_t oz_gemm(const void* A, long long lda, long long sa, int M, co
   const int nkb = (K + BK - 1) / BK;
   int z = *splits < 1 ? 1 : *splits;
   if (z > nkb) z = nkb;
+  g.A = (const unsigned short*)A;
+  g.B = (const unsigned short*)B;
+  g.nta = nta; g.ntb = ntb;
   g.M = M; g.N = N; g.K = K;
   g.kb_per_split = (nkb + z - 1) / z;
   z = (nkb + g.kb_per_split - 1) / g.kb_per_split;
@@ -662,25 +672,17 @@ inline cudaError_t oz_gemm(const void* A, long long lda, long long sa, int M, co
   int nsm = 0;
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const int grid = (int)(items < nsm ? items : nsm);
-  k_oz_gemm<S, BNT><<<grid, THREADS, smem_bytes<S, BNT>(), s>>>(ma, mb, g);
+  k_oz_gemm<S, BNT><<<grid, THREADS, smem_bytes<S, BNT>(), s>>>(g);
   note_launch();
   *splits = z;
   return cudaGetLastError();
 }
 
-// Launch the grouped form over grp's problems: A holds rowsA stacked rows,
-// B rowsB, both of row stride ld (bf16 elements, a multiple of 8; each
-// problem's digits zero from K = 2n on), slice strides sa, sb.
+// Launch the grouped form over grp's problems (operands from A + ao[b], B + bo[b]).
 template <int S, int BNT>
-inline cudaError_t oz_gemm_group(const void* A, long long sa, int rowsA, const void* B,
-                                 long long sb, int rowsB, long long ld, const OzGroup& grp,
-                                 OzArgs g, cudaStream_t s) {
+inline cudaError_t oz_gemm_group(const void* A, const void* B, const OzGroup& grp, OzArgs g, cudaStream_t s) {
   if (grp.np <= 0 || grp.tile0[grp.np] == 0) return cudaSuccess;
-  if ((ld & 7) || (sa & 7) || (sb & 7) || rowsA <= 0 || rowsB <= 0) return cudaErrorInvalidValue;
-  CUtensorMap ma, mb;
   cudaError_t e;
-  if ((e = make_map3(&ma, A, S, rowsA, (int)ld, ld, sa, BM)) != cudaSuccess) return e;
-  if ((e = make_map3(&mb, B, S, rowsB, (int)ld, ld, sb, BNT)) != cudaSuccess) return e;
   static bool smem_set[64] = {false};
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -695,9 +697,11 @@ inline cudaError_t oz_gemm_group(const void* A, long long sa, int rowsA, const v
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const int items = grp.tile0[grp.np];
   const int grid = items < nsm ? items : nsm;
+  g.A = (const unsigned short*)A;
+  g.B = (const unsigned short*)B;
   g.mode = 0;
   g.run = g.stop = nullptr;
-  k_oz_gemm_group<S, BNT><<<grid, THREADS, smem_bytes<S, BNT>(), s>>>(ma, mb, g, grp);
+  k_oz_gemm_group<S, BNT><<<grid, THREADS, smem_bytes<S, BNT>(), s>>>(g, grp);
   note_launch();
   return cudaGetLastError();
 }

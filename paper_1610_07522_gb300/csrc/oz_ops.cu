@@ -69,18 +69,24 @@ __global__ void __launch_bounds__(256) k_oz_rowexp(const T* __restrict__ src, lo
   if (threadIdx.x == 0) E[blockIdx.x] = m == INT_MIN ? 0 : m;
 }
 
+// Digits of the row pair element (row, complex entry c) into every slice.
+template <int S, int BN>
+__device__ __forceinline__ void store_digits(unsigned short* dst, int nt, int row, int c,
+                                             const unsigned (&w)[S]) {
+  unsigned* d = reinterpret_cast<unsigned*>(dst + oz::dig_off<S, BN>(row, 2 * c, 0, nt));
+#pragma unroll
+  for (int s = 0; s < S; ++s) d[s * (BN * oz::BK / 2)] = w[s];
+}
+
 // Slices of rows [0, R) of a [R][V] complex array over complex columns
-// [c0, c0 + nc): dst[s][r][2 (c - c0) + {0, 1}]; with prime_off >= 0 also
-// rows prime_off + r = (Im, -Re).
-template <typename T, int S>
+// [c0, c0 + nc) in the blocked layout (nt row tiles), K = 2 (c - c0) + {0, 1};
+// with prime_off >= 0 also rows prime_off + r = (Im, -Re).
+template <typename T, int S, int BN>
 __global__ void __launch_bounds__(256) k_oz_split_rows(const T* __restrict__ src, int R, long long V,
                                                        long long c0, long long nc,
                                                        const int* __restrict__ E,
-                                                       unsigned short* dst, long long ld,
-                                                       long long ss, int prime_off,
-                                                       const int* run, const int* stop) {
+                                                       unsigned short* dst, int nt, int prime_off) {
   using RT = decltype(T().x);
-  if (gated_off(run, stop)) return;
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (long long)R * nc) return;
   const int r = (int)(e / nc);
@@ -90,21 +96,22 @@ __global__ void __launch_bounds__(256) k_oz_split_rows(const T* __restrict__ src
   unsigned short dr[S], di[S];
   digits<S>((RT)v.x, Er, dr);
   digits<S>((RT)v.y, Er, di);
-  unsigned* d32 = reinterpret_cast<unsigned*>(dst);
+  unsigned w[S];
 #pragma unroll
-  for (int s = 0; s < S; ++s) {
-    d32[(s * ss + (long long)r * ld) / 2 + c] = pack2(dr[s], di[s]);
-    if (prime_off >= 0)
-      d32[(s * ss + (long long)(prime_off + r) * ld) / 2 + c] = pack2(di[s], neg_bf16(dr[s]));
+  for (int s = 0; s < S; ++s) w[s] = pack2(dr[s], di[s]);
+  store_digits<S, BN>(dst, nt, r, (int)c, w);
+  if (prime_off >= 0) {
+#pragma unroll
+    for (int s = 0; s < S; ++s) w[s] = pack2(di[s], neg_bf16(dr[s]));
+    store_digits<S, BN>(dst, nt, prime_off + r, (int)c, w);
   }
 }
 
 // Row operand of the recombination: row a = [Re M[b][a] (b < I) | 0 | Im M[b][a] | 0],
 // halves of Ipad; Ea[a] its exponent.  One block per row a.
-template <int S>
+template <int S, int BN>
 __global__ void __launch_bounds__(256) k_oz_rot_a(const double2* __restrict__ M, int I, int Ipad,
-                                                  unsigned short* dst, long long ld, long long ss,
-                                                  int* Ea) {
+                                                  unsigned short* dst, int nt, int* Ea) {
   const int a = blockIdx.x;
   int m = INT_MIN;
   for (int b = threadIdx.x; b < I; b += blockDim.x) {
@@ -121,8 +128,8 @@ __global__ void __launch_bounds__(256) k_oz_rot_a(const double2* __restrict__ M,
     digits<S>(v.y, E, di);
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-      dst[s * ss + (long long)a * ld + b] = dr[s];
-      dst[s * ss + (long long)a * ld + Ipad + b] = di[s];
+      dst[oz::dig_off<S, BN>(a, b, s, nt)] = dr[s];
+      dst[oz::dig_off<S, BN>(a, Ipad + b, s, nt)] = di[s];
     }
   }
 }
@@ -147,19 +154,18 @@ __global__ void __launch_bounds__(256) k_oz_colexp(const T* __restrict__ phi, in
 //   row 2v:   Re phi_b[v],  -Im phi_b[v];   row 2v+1: Im phi_b[v],  Re phi_b[v];
 // zeros for b in [I, Ipad).  32 states x 32 entries per block through shared
 // memory (coalesced reads along v, writes along b).
-template <typename T, int S>
+template <typename T, int S, int BN>
 __global__ void __launch_bounds__(256) k_oz_split_rot_b(const T* __restrict__ phi, int I, int Ipad,
                                                         long long V, long long v0, long long nv,
                                                         const int* __restrict__ F,
-                                                        unsigned short* dst, long long ld,
-                                                        long long ss) {
+                                                        unsigned short* dst, int nt) {
   using R = decltype(T().x);
   __shared__ T t[32][33];
-  const int b0 = blockIdx.y * 32;
+  const int s0 = blockIdx.y * 32;
   const long long vb = (long long)blockIdx.x * 32;   // relative to v0
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
   for (int r = ty; r < 32; r += 8) {
-    const int b = b0 + r;
+    const int b = s0 + r;
     const long long v = vb + tx;
     T z;
     z.x = 0; z.y = 0;
@@ -169,36 +175,30 @@ __global__ void __launch_bounds__(256) k_oz_split_rot_b(const T* __restrict__ ph
   for (int r = ty; r < 32; r += 8) {
     const long long v = vb + r;   // entry handled by this warp; lanes run over states
     if (v >= nv) continue;
-    const int b = b0 + tx;
+    const int b = s0 + tx;
     const T x = t[tx][r];
     const int Fv = F[v0 + v];
     unsigned short dr[S], di[S];
     digits<S>((R)x.x, Fv, dr);
     digits<S>((R)x.y, Fv, di);
+    const int row = (int)(2 * v);
+    const long long a0 = oz::dig_off<S, BN>(row, b, 0, nt), a1 = oz::dig_off<S, BN>(row, Ipad + b, 0, nt);
+    const long long b0 = oz::dig_off<S, BN>(row + 1, b, 0, nt), b1 = oz::dig_off<S, BN>(row + 1, Ipad + b, 0, nt);
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-      unsigned short* row0 = dst + s * ss + (2 * v) * ld;
-      unsigned short* row1 = row0 + ld;
-      row0[b] = dr[s];
-      row0[Ipad + b] = neg_bf16(di[s]);
-      row1[b] = di[s];
-      row1[Ipad + b] = dr[s];
+      unsigned short* d = dst + s * (BN * oz::BK);
+      d[a0] = dr[s];
+      d[a1] = neg_bf16(di[s]);
+      d[b0] = di[s];
+      d[b1] = dr[s];
     }
   }
 }
 
-// Digits of the rows of an n x n complex matrix operand in one pass per row
-// (one block per row r): the operand row is row r of src, or with trans the
-// conjugate of column r (a conjugate transpose read in place).  Its exponent
-// goes to E[r]; digits to dst[s][r][2k + {0, 1}], and with prime_off >= 0
-// (Im, -Re) to row prime_off + r.
-template <int S>
-__global__ void __launch_bounds__(256) k_oz_split_mat(const double2* __restrict__ src, int n,
-                                                      int trans, int* E, unsigned short* dst,
-                                                      long long ld, long long ss, int prime_off,
-                                                      const int* run, const int* stop) {
-  if (gated_off(run, stop)) return;
-  const int r = blockIdx.x;
+// Row r of an n x n operand by one block (k_oz_split_mat, k_oz_split_group).
+template <int S, int BN>
+__device__ __forceinline__ void split_mat_row(const double2* __restrict__ src, int n, int r, int trans,
+                                              int* E, unsigned short* dst, int nt, int prime_off) {
   auto at = [&](int k) {
     return trans ? conjx(src[(long long)k * n + r]) : src[(long long)r * n + k];
   };
@@ -209,20 +209,37 @@ __global__ void __launch_bounds__(256) k_oz_split_mat(const double2* __restrict_
   }
   m = block_max<double>(m);
   const int Er = m == INT_MIN ? 0 : m;
-  if (threadIdx.x == 0) E[r] = Er;
-  unsigned* d32 = reinterpret_cast<unsigned*>(dst);
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    const double2 v = at(k);
+  if (threadIdx.x == 0) *E = Er;
+  const int kh = (n + oz::BK / 2 - 1) / (oz::BK / 2) * (oz::BK / 2);   // whole K blocks
+  for (int k = threadIdx.x; k < kh; k += blockDim.x) {
     unsigned short dr[S], di[S];
+    const double2 v = k < n ? at(k) : make_double2(0.0, 0.0);
     digits<S>(v.x, Er, dr);
     digits<S>(v.y, Er, di);
+    unsigned w[S];
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-      d32[(s * ss + (long long)r * ld) / 2 + k] = pack2(dr[s], di[s]);
-      if (prime_off >= 0)
-        d32[(s * ss + (long long)(prime_off + r) * ld) / 2 + k] = pack2(di[s], neg_bf16(dr[s]));
+    for (int s = 0; s < S; ++s) w[s] = pack2(dr[s], di[s]);
+    store_digits<S, BN>(dst, nt, r, k, w);
+    if (prime_off >= 0) {
+#pragma unroll
+      for (int s = 0; s < S; ++s) w[s] = pack2(di[s], k < n ? neg_bf16(dr[s]) : (unsigned short)0);
+      store_digits<S, BN>(dst, nt, prime_off + r, k, w);
     }
   }
+}
+
+// Digits of the rows of an n x n complex matrix operand in one pass per row
+// (one block per row r): the operand row is row r of src, or with trans the
+// conjugate of column r (a conjugate transpose read in place).  Its exponent
+// goes to E[r]; digits to row r of the blocked layout (K = 2k + {0, 1}, zeros up
+// to a whole K block), and with prime_off >= 0 (Im, -Re) to row prime_off + r.
+template <int S, int BN>
+__global__ void __launch_bounds__(256) k_oz_split_mat(const double2* __restrict__ src, int n,
+                                                      int trans, int* E, unsigned short* dst,
+                                                      int nt, int prime_off, const int* run,
+                                                      const int* stop) {
+  if (gated_off(run, stop)) return;
+  split_mat_row<S, BN>(src, n, blockIdx.x, trans, E + blockIdx.x, dst, nt, prime_off);
 }
 
 // C[m][c] = conj(sum_z (P_z[m][c] + i P_z[m][n + c])) 2^{Ea[m] + Eb[c] - 16}: the
@@ -245,52 +262,22 @@ __global__ void k_oz_zgemm_reduce(const float2* __restrict__ P, int nz, long lon
   C[e] = make_double2(sc * re, -sc * im);
 }
 
-// Grouped form of the two kernels above (blockIdx.y = problem b of the
-// group; rows stacked at G.ra / G.rb, exponents indexed by stacked row).
+// Grouped form of the two kernels above (blockIdx.y = problem b of the group,
+// operands from G.ao / G.bo, exponents indexed by stacked row G.ra / G.rb).
 // Operand B (second) adds the (Im, -Re) rows n .. 2n - 1 of its problem.
-// Every row is written up to ld (zeros from K = 2n on), so a K block that
-// runs past 2n reads zeros.
-template <int S>
-__global__ void __launch_bounds__(256) k_oz_split_group(oz::OzGroup G, int second, int trans,
-                                                        int* E, unsigned short* dst, long long ld,
-                                                        long long ss) {
+template <int S, int BN>
+__global__ void __launch_bounds__(256) k_oz_split_group(const __grid_constant__ oz::OzGroup G, int second,
+                                                        int trans, int* E, unsigned short* dst) {
   const int b = blockIdx.y, r = blockIdx.x;
   const int n = G.n[b];
   if (r >= n || oz::group_gated(G, b)) return;
-  const double2* __restrict__ src = second ? G.B[b] : G.A[b];
-  auto at = [&](int k) {
-    return trans ? conjx(src[(long long)k * n + r]) : src[(long long)r * n + k];
-  };
-  int m = INT_MIN;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    const double2 v = at(k);
-    m = max(m, max(exp_of(v.x), exp_of(v.y)));
-  }
-  m = block_max<double>(m);
-  const int Er = m == INT_MIN ? 0 : m;
-  const long long row = (second ? G.rb[b] : G.ra[b]) + r;
-  if (threadIdx.x == 0) E[row] = Er;
-  unsigned* d32 = reinterpret_cast<unsigned*>(dst);
-  const long long kh = ld / 2;   // complex entries per row, padding included
-  for (int k = threadIdx.x; k < kh; k += blockDim.x) {
-    unsigned short dr[S], di[S];
-    if (k < n) {
-      const double2 v = at(k);
-      digits<S>(v.x, Er, dr);
-      digits<S>(v.y, Er, di);
-    } else {
-#pragma unroll
-      for (int s = 0; s < S; ++s) dr[s] = di[s] = 0;
-    }
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      d32[(s * ss + row * ld) / 2 + k] = pack2(dr[s], di[s]);
-      if (second) d32[(s * ss + (row + n) * ld) / 2 + k] = pack2(di[s], neg_bf16(dr[s]));
-    }
-  }
+  if (second)
+    split_mat_row<S, BN>(G.B[b], n, r, trans, E + G.rb[b] + r, dst + G.bo[b], (2 * n + BN - 1) / BN, n);
+  else
+    split_mat_row<S, BN>(G.A[b], n, r, trans, E + G.ra[b] + r, dst + G.ao[b], (n + BN - 1) / BN, -1);
 }
 
-__global__ void k_oz_reduce_group(const float2* __restrict__ P, oz::OzGroup G,
+__global__ void k_oz_reduce_group(const float2* __restrict__ P, const __grid_constant__ oz::OzGroup G,
                                   const int* __restrict__ Ea, const int* __restrict__ Eb) {
   const int b = blockIdx.y, n = G.n[b];
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -360,8 +347,11 @@ sky_status oz_overlap_t(Ctx* c, const void* a, const void* b, int I, double2* X)
   }
   note_launch(b != a ? 2 : 1);
   if (b == a) Eb = Ea;
-  // K chunk (complex entries) so that S slices of the 2I B rows fit the buffer
-  long long nc = c->oz_b_elems / ((long long)S * 2 * I) / 2;
+  // K chunk (complex entries) so that both operands fit their buffers
+  const int nta = (int)oz::dig_tiles(I, BN), ntb = (int)oz::dig_tiles(2LL * I, BN);
+  long long nc = c->oz_b_elems / ((long long)S * ntb * BN) / 2;
+  const long long nca = c->oz_a_elems / ((long long)S * nta * BN) / 2;
+  if (b != a && nca < nc) nc = nca;
   nc = nc / 64 * 64;   // whole 128-value segments
   if (nc > V) nc = V;
   if (nc < 64 && nc < V) return set_err(c, SKY_EINVAL, "overlap: split buffer too small for I=%d", I);
@@ -369,23 +359,18 @@ sky_status oz_overlap_t(Ctx* c, const void* a, const void* b, int I, double2* X)
   bool first = true;
   for (long long c0 = 0; c0 < V; c0 += nc) {
     const long long n = (V - c0) < nc ? (V - c0) : nc;
-    const long long K = 2 * n, ld = round_up(K, 8);
+    const long long K = 2 * n;   // n a multiple of 64, or V = 2 G with G a multiple of 64: whole K blocks
     unsigned short* Bp = (unsigned short*)c->d_ozB;
     unsigned short* Ap = (unsigned short*)c->d_ozA;
-    const long long sb = (long long)2 * I * ld, sa = (long long)I * ld;
     const long long tot = (long long)I * n;
     if (f64) {
-      k_oz_split_rows<double2, S><<<div_up(tot, 256), 256, 0, st>>>(
-          (const double2*)b, I, V, c0, n, Eb, Bp, ld, sb, I, nullptr, nullptr);
+      k_oz_split_rows<double2, S, BN><<<div_up(tot, 256), 256, 0, st>>>((const double2*)b, I, V, c0, n, Eb, Bp, ntb, I);
       if (b != a)
-        k_oz_split_rows<double2, S><<<div_up(tot, 256), 256, 0, st>>>(
-            (const double2*)a, I, V, c0, n, Ea, Ap, ld, sa, -1, nullptr, nullptr);
+        k_oz_split_rows<double2, S, BN><<<div_up(tot, 256), 256, 0, st>>>((const double2*)a, I, V, c0, n, Ea, Ap, nta, -1);
     } else {
-      k_oz_split_rows<float2, S><<<div_up(tot, 256), 256, 0, st>>>(
-          (const float2*)b, I, V, c0, n, Eb, Bp, ld, sb, I, nullptr, nullptr);
+      k_oz_split_rows<float2, S, BN><<<div_up(tot, 256), 256, 0, st>>>((const float2*)b, I, V, c0, n, Eb, Bp, ntb, I);
       if (b != a)
-        k_oz_split_rows<float2, S><<<div_up(tot, 256), 256, 0, st>>>(
-            (const float2*)a, I, V, c0, n, Ea, Ap, ld, sa, -1, nullptr, nullptr);
+        k_oz_split_rows<float2, S, BN><<<div_up(tot, 256), 256, 0, st>>>((const float2*)a, I, V, c0, n, Ea, Ap, nta, -1);
     }
     note_launch(b != a ? 2 : 1);
     cudaError_t e = cudaGetLastError();
@@ -400,9 +385,8 @@ sky_status oz_overlap_t(Ctx* c, const void* a, const void* b, int I, double2* X)
     g.ldp = ldp;
     g.sp = spart;
     g.status = c->d_status;
-    const void* Aop = b != a ? (const void*)Ap : (const void*)Bp;
-    const long long lda = ld, sA = b != a ? sa : sb;
-    e = oz::oz_gemm<S, BN>(Aop, lda, sA, I, Bp, ld, sb, 2 * I, (int)K, true, I, g, &z, st);
+    // equal operands: the rows of A are the first I rows of [b; b']
+    e = oz::oz_gemm<S, BN>(b != a ? Ap : Bp, b != a ? nta : ntb, I, Bp, ntb, 2 * I, (int)K, true, I, g, &z, st);
     if (e != cudaSuccess) return cuda_check(c, e, "oz overlap gemm");
     k_oz_overlap_reduce<<<div_up((long long)I * I, 256), 256, 0, st>>>(
         c->d_ozP, z, spart, ldp, I, Ea, Eb, c->dV, X, first ? 0 : 1);
@@ -425,10 +409,10 @@ sky_status oz_rotate_t(Ctx* c, const void* phi, const double2* M, int I, void* o
   int* F = c->d_ozE + c->max_states;
   unsigned short* Ap = (unsigned short*)c->d_ozA;
   unsigned short* Bp = (unsigned short*)c->d_ozB;
-  const long long sa = (long long)I * ldk;
-  if ((long long)S * sa > (long long)c->oz_a_elems)
+  const int nta = (int)oz::dig_tiles(I, BN);
+  if (oz::dig_elems(I, ldk, S, BN) > (long long)c->oz_a_elems)
     return set_err(c, SKY_EINVAL, "rotate: split buffer too small for I=%d", I);
-  k_oz_rot_a<S><<<I, 256, 0, st>>>(M, I, Ipad, Ap, ldk, sa, Ea);
+  k_oz_rot_a<S, BN><<<I, 256, 0, st>>>(M, I, Ipad, Ap, nta, Ea);
   if (f64) k_oz_colexp<double2><<<div_up(V, 256), 256, 0, st>>>((const double2*)phi, I, V, F);
   else k_oz_colexp<float2><<<div_up(V, 256), 256, 0, st>>>((const float2*)phi, I, V, F);
   note_launch(2);
@@ -436,19 +420,18 @@ sky_status oz_rotate_t(Ctx* c, const void* phi, const double2* M, int I, void* o
   if (e != cudaSuccess) return cuda_check(c, e, "oz rotate split a");
   // complex columns per chunk so that S slices of 2 nv rows fit the buffer
   long long nv = c->oz_b_elems / ((long long)S * 2 * ldk);
-  nv = nv / 480 * 480;   // 2 nv rows: a multiple of both tile widths
+  if (oz::dig_elems(2 * V, ldk, S, BN) <= (long long)c->oz_b_elems) nv = V;
+  else nv = nv / 480 * 480;   // 2 nv rows: a multiple of both tile widths
   if (nv > V) nv = V;
   if (nv < 480 && nv < V) return set_err(c, SKY_EINVAL, "rotate: split buffer too small for I=%d", I);
   for (long long v0 = 0; v0 < V; v0 += nv) {
     const long long n = (V - v0) < nv ? (V - v0) : nv;
-    const long long sb = 2 * n * ldk;
+    const int ntb = (int)oz::dig_tiles(2 * n, BN);
     dim3 g2(div_up(n, 32), Ipad / 32);
     if (f64)
-      k_oz_split_rot_b<double2, S><<<g2, 256, 0, st>>>((const double2*)phi, I, Ipad, V, v0, n, F,
-                                                       Bp, ldk, sb);
+      k_oz_split_rot_b<double2, S, BN><<<g2, 256, 0, st>>>((const double2*)phi, I, Ipad, V, v0, n, F, Bp, ntb);
     else
-      k_oz_split_rot_b<float2, S><<<g2, 256, 0, st>>>((const float2*)phi, I, Ipad, V, v0, n, F, Bp,
-                                                      ldk, sb);
+      k_oz_split_rot_b<float2, S, BN><<<g2, 256, 0, st>>>((const float2*)phi, I, Ipad, V, v0, n, F, Bp, ntb);
     note_launch();
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_check(c, e, "oz rotate split b");
@@ -462,8 +445,7 @@ sky_status oz_rotate_t(Ctx* c, const void* phi, const double2* M, int I, void* o
     g.eb_shift = 1;
     g.status = c->d_status;
     int z = 1;
-    e = oz::oz_gemm<S, BN>(Ap, ldk, sa, I, Bp, ldk, sb, (int)(2 * n), (int)ldk, false, I, g, &z,
-                           st);
+    e = oz::oz_gemm<S, BN>(Ap, nta, I, Bp, ntb, (int)(2 * n), (int)ldk, false, I, g, &z, st);
     if (e != cudaSuccess) return cuda_check(c, e, "oz rotate gemm");
   }
   return SKY_OK;
@@ -477,11 +459,9 @@ sky_status oz_rotate_t(Ctx* c, const void* phi, const double2* M, int I, void* o
 // of X's rows with Zt's rows (6 digits; about 1e-14 of the largest element).
 // Every kernel is skipped when the device gate (run, stop) says so.
 bool oz_zgemm_fits(const Ctx* c, int n) {
-  // the digit rows are written with the padded stride ld = round_up(2n, 8)
-  const long long ld = round_up(2LL * n, 8);
   return c->d_ozB && n <= c->max_states &&
-         (long long)oz::kS64 * 2 * n * ld <= (long long)c->oz_b_elems &&
-         (long long)oz::kS64 * n * ld <= (long long)c->oz_a_elems;
+         oz::dig_elems(2LL * n, 2LL * n, oz::kS64, oz::kBN64) <= (long long)c->oz_b_elems &&
+         oz::dig_elems(n, 2LL * n, oz::kS64, oz::kBN64) <= (long long)c->oz_a_elems;
 }
 
 sky_status oz_zgemm(Ctx* c, bool ah, bool bh, const double2* A, const double2* B, double2* C,
@@ -490,15 +470,15 @@ sky_status oz_zgemm(Ctx* c, bool ah, bool bh, const double2* A, const double2* B
   cudaStream_t st = c->stream;
   int* Ea = c->d_ozE;
   int* Eb = c->d_ozE + c->max_states;
-  const long long K = 2LL * n, ld = round_up(K, 8);
+  const long long K = 2LL * n;
+  const int nta = (int)oz::dig_tiles(n, BN), ntb = (int)oz::dig_tiles(K, BN);
   unsigned short* Bp = (unsigned short*)c->d_ozB;
   unsigned short* Ap = (unsigned short*)c->d_ozA;
-  const long long sb = 2LL * n * ld, sa = (long long)n * ld;
   const long long tot = (long long)n * n;
   // X = opA(A): rows of A, or conjugated columns; Zt = conj(opB(B))^T: rows of
   // B when opB is the conjugate transpose, else conjugated columns of B
-  k_oz_split_mat<S><<<n, 256, 0, st>>>(A, n, ah ? 1 : 0, Ea, Ap, ld, sa, -1, run, stop);
-  k_oz_split_mat<S><<<n, 256, 0, st>>>(B, n, bh ? 0 : 1, Eb, Bp, ld, sb, n, run, stop);
+  k_oz_split_mat<S, BN><<<n, 256, 0, st>>>(A, n, ah ? 1 : 0, Ea, Ap, nta, -1, run, stop);
+  k_oz_split_mat<S, BN><<<n, 256, 0, st>>>(B, n, bh ? 0 : 1, Eb, Bp, ntb, n, run, stop);
   note_launch(2);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_check(c, e, "oz zgemm split");
@@ -519,7 +499,7 @@ sky_status oz_zgemm(Ctx* c, bool ah, bool bh, const double2* A, const double2* B
   g.status = c->d_status;
   g.run = run;
   g.stop = stop;
-  e = oz::oz_gemm<S, BN>(Ap, ld, sa, n, Bp, ld, sb, 2 * n, (int)K, false, n, g, &zi, st);
+  e = oz::oz_gemm<S, BN>(Ap, nta, n, Bp, ntb, 2 * n, (int)K, false, n, g, &zi, st);
   if (e != cudaSuccess) return cuda_check(c, e, "oz zgemm");
   k_oz_zgemm_reduce<<<div_up(tot, 256), 256, 0, st>>>(c->d_ozP, zi, spart, 2LL * n, n, Ea, Eb, C,
                                                       run, stop);
@@ -531,18 +511,28 @@ sky_status oz_zgemm(Ctx* c, bool ah, bool bh, const double2* A, const double2* B
 // the context's state count) in one grouped launch sequence: two digit
 // splits, one tensor-core launch over all problems' tiles, one reduction
 // (the per-problem form above, stacked; gates per problem).
-int oz_group_slices() { return oz::kS64; }
+// Operand buffer sizes (elements) of one product of m states, and of the grouped
+// products of nb problems of up to m.
+void oz_zgemm_sizes(int m, size_t* a_elems, size_t* b_elems) { oz_group_sizes(1, m, a_elems, b_elems); }
+void oz_group_sizes(int nb, int m, size_t* a_elems, size_t* b_elems) {
+  *a_elems = (size_t)nb * oz::dig_elems(m, 2LL * m, oz::kS64, oz::kBN64);
+  *b_elems = (size_t)nb * oz::dig_elems(2LL * m, 2LL * m, oz::kS64, oz::kBN64);
+}
 
 bool oz_zgemm_group_fits(const Ctx* c, int np, const int* n) {
   if (!c->d_ozgA || np > c->ozg_np) return false;
-  long long rows = 0;
-  long long p = 0;
+  long long rows = 0, p = 0;
+  size_t ae = 0, be = 0;
   for (int b = 0; b < np; ++b) {
     if (n[b] > c->max_states) return false;
+    size_t x, y;
+    oz_group_sizes(1, n[b], &x, &y);
+    ae += x;
+    be += y;
     rows += n[b];
     p += 2LL * n[b] * n[b];
   }
-  return rows <= c->ozg_rows && p <= (long long)c->ozg_p_elems;
+  return rows <= c->ozg_rows && ae <= c->ozg_a_elems && be <= c->ozg_b_elems && p <= (long long)c->ozg_p_elems;
 }
 
 sky_status oz_zgemm_group(Ctx* c, const ZJobs& j) {
@@ -553,9 +543,15 @@ sky_status oz_zgemm_group(Ctx* c, const ZJobs& j) {
   G.tile0[0] = 0;
   int ra = 0, nmax = 0;
   long long po = 0;
+  size_t ao = 0, bo = 0;
   for (int b = 0; b < j.np; ++b) {
     const int n = j.n[b];
     G.n[b] = n; G.ra[b] = ra; G.rb[b] = 2 * ra; G.po[b] = po;
+    G.ao[b] = (long long)ao; G.bo[b] = (long long)bo;
+    size_t ae, be;
+    oz_group_sizes(1, n, &ae, &be);
+    ao += ae;
+    bo += be;
     G.A[b] = j.A[b]; G.B[b] = j.B[b]; G.C[b] = j.C[b];
     G.run[b] = j.run[b]; G.stop[b] = j.stop[b];
     G.tile0[b + 1] = G.tile0[b] + (n > 0 ? ((n + oz::BM - 1) / oz::BM) * ((2 * n + BN - 1) / BN) : 0);
@@ -564,21 +560,19 @@ sky_status oz_zgemm_group(Ctx* c, const ZJobs& j) {
     nmax = n > nmax ? n : nmax;
   }
   if (nmax == 0) return SKY_OK;
-  const long long ld = c->ozg_ld;
-  const long long sa = (long long)c->ozg_rows * ld, sb = 2 * sa;
   int* Ea = c->d_ozgE;
   int* Eb = c->d_ozgE + c->ozg_rows;
   unsigned short* Ap = (unsigned short*)c->d_ozgA;
   unsigned short* Bp = (unsigned short*)c->d_ozgB;
-  k_oz_split_group<S><<<dim3(nmax, j.np), 256, 0, st>>>(G, 0, j.ah ? 1 : 0, Ea, Ap, ld, sa);
-  k_oz_split_group<S><<<dim3(nmax, j.np), 256, 0, st>>>(G, 1, j.bh ? 0 : 1, Eb, Bp, ld, sb);
+  k_oz_split_group<S, BN><<<dim3(nmax, j.np), 256, 0, st>>>(G, 0, j.ah ? 1 : 0, Ea, Ap);
+  k_oz_split_group<S, BN><<<dim3(nmax, j.np), 256, 0, st>>>(G, 1, j.bh ? 0 : 1, Eb, Bp);
   note_launch(2);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_check(c, e, "grouped zgemm split");
   oz::OzArgs g{};
   g.P = c->d_ozgP;
   g.status = c->d_status;
-  e = oz::oz_gemm_group<S, BN>(Ap, sa, ra, Bp, sb, 2 * ra, ld, G, g, st);
+  e = oz::oz_gemm_group<S, BN>(Ap, Bp, G, g, st);
   if (e != cudaSuccess) return cuda_check(c, e, "grouped zgemm");
   k_oz_reduce_group<<<dim3(div_up((long long)nmax * nmax, 256), j.np), 256, 0, st>>>(
       c->d_ozgP, G, Ea, Eb);
@@ -609,22 +603,24 @@ void oz_scratch_sizes(sky_prec prec, int Imax, long long V, int nsm, size_t* a_e
   }
   const int S = oz_slices(prec), bn = oz_bn(prec);
   const long long Ipad = round_up(Imax, 32);
-  const long long ov_b = (long long)S * 2 * Imax * round_up(2 * V, 8);
-  const long long rot_b = (long long)S * 2 * V * 2 * Ipad;
+  const long long ov_b = oz::dig_elems(2LL * Imax, 2 * V, S, bn);
+  const long long rot_b = oz::dig_elems(2 * V, 2 * Ipad, S, bn);
   long long need_b = ov_b > rot_b ? ov_b : rot_b;
   long long cap = 4096;
   if (const char* s = getenv("SKY_OZ_MB"))
     if (atol(s) > 0) cap = atol(s);
   cap = (cap << 20) / 2;
   // at least one chunk of 64 complex columns (overlap) / 480 (recombination)
-  const long long min_b = (long long)S * 2 * Imax * 128 > (long long)S * 960 * 2 * Ipad
-                              ? (long long)S * 2 * Imax * 128
-                              : (long long)S * 960 * 2 * Ipad;
+  const long long min_ov = oz::dig_elems(2LL * Imax, 128, S, bn), min_rot = oz::dig_elems(960, 2 * Ipad, S, bn);
+  const long long min_b = min_ov > min_rot ? min_ov : min_rot;
   if (need_b > cap) need_b = cap > min_b ? cap : min_b;
   *b_elems = (size_t)need_b;
-  // A: the a rows of an overlap chunk (at most half of B) or the rotation rows
-  const long long rot_a = (long long)S * Imax * 2 * Ipad;
-  *a_elems = (size_t)(need_b / 2 > rot_a ? need_b / 2 : rot_a);
+  // A: the a rows of an overlap chunk (about half of B, a whole row tile more) or
+  // the rotation rows
+  const long long rot_a = oz::dig_elems(Imax, 2 * Ipad, S, bn);
+  const long long ov_k = need_b / ((long long)S * oz::dig_tiles(2LL * Imax, bn) * bn);
+  const long long ov_a = oz::dig_elems(Imax, ov_k < 2 * V ? ov_k : 2 * V, S, bn);
+  *a_elems = (size_t)(ov_a > rot_a ? ov_a : rot_a);
   *e_elems = (size_t)(2 * Imax + V + 64);
   size_t pmax = 1;
   for (int I = 1; I <= Imax; ++I) {

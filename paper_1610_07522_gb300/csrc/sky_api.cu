@@ -139,10 +139,11 @@ static sky_status alloc_oz_scratch(Ctx* c, bool overlap_too) {
   size_t ae, be, ee, pe;
   oz_scratch_sizes(overlap_too ? c->prec : SKY_F64, overlap_too ? Imax : 0, overlap_too ? 2LL * c->G : 0,
                    c->num_sms, &ae, &be, &ee, &pe);
-  if (Imax >= kOzZgemmMin) {   // the I x I products: 2 I rows of ld = round_up(2 I, 8)
-    const size_t zb = (size_t)6 * 2 * Imax * (size_t)((2 * Imax + 7) / 8 * 8);
+  if (Imax >= kOzZgemmMin) {   // the I x I products
+    size_t za, zb;
+    oz_zgemm_sizes(Imax, &za, &zb);
     if (zb > be) be = zb;
-    if (zb / 2 > ae) ae = zb / 2;
+    if (za > ae) ae = za;
     if ((size_t)2 * Imax * Imax > pe) pe = (size_t)2 * Imax * Imax;
   }
   if (ee < (size_t)(2 * Imax + 2LL * c->G + 64)) ee = (size_t)(2 * Imax + 2LL * c->G + 64);
@@ -721,24 +722,26 @@ sky_status sky_reserve_batch(sky_ctx* c, int nb) {
     return s;
   }
   // grouped I x I products for batches of many problems: digits of every
-  // problem's rows stacked (up to nb x Imax rows, capped at about 2 GiB)
+  // problem's operands (of nb problems of Imax states, capped at about 2 GiB)
   void *ga = nullptr, *gb = nullptr;
   float2* gp = nullptr;
   int* ge = nullptr;
-  long long grows = 0, gld = 0;
-  size_t gpe = 0;
+  long long grows = 0;
+  size_t gpe = 0, gae = 0, gbe = 0;
   if (s == SKY_OK && nb > kOzGroupMin) {
-    gld = (2LL * Imax + 7) / 8 * 8;
-    const long long per_row = (long long)oz_group_slices() * 3 * gld * 2;   // A + B bytes
-    const long long cap = 2LL << 30;
+    const size_t cap = (size_t)2 << 30;
+    oz_group_sizes(1, Imax, &gae, &gbe);
+    size_t most = cap / (2 * (gae + gbe));     // problems of Imax states within the cap
+    if (most > (size_t)nb) most = (size_t)nb;
+    gae *= most;
+    gbe *= most;
     grows = (long long)nb * Imax;
-    if (grows * per_row > cap) grows = cap / per_row;
     gpe = (size_t)nb * 2 * (size_t)Imax * (size_t)Imax;
-    if (gpe * sizeof(float2) > (size_t)cap) gpe = (size_t)cap / sizeof(float2);
-    if (grows >= Imax) {
+    if (gpe * sizeof(float2) > cap) gpe = cap / sizeof(float2);
+    if (most > 0) {
       unsigned short *pa = nullptr, *pb = nullptr;
-      s = dalloc(c, &pa, (size_t)oz_group_slices() * grows * gld);
-      if (s == SKY_OK) s = dalloc(c, &pb, (size_t)oz_group_slices() * 2 * grows * gld);
+      s = dalloc(c, &pa, gae);
+      if (s == SKY_OK) s = dalloc(c, &pb, gbe);
       if (s == SKY_OK) s = dalloc(c, &gp, gpe);
       if (s == SKY_OK) s = dalloc(c, &ge, (size_t)3 * grows);
       ga = pa;
@@ -763,7 +766,8 @@ sky_status sky_reserve_batch(sky_ctx* c, int nb) {
     for (void* p : og)
       if (p) cudaFree(p);
     c->d_ozgA = ga; c->d_ozgB = gb; c->d_ozgP = gp; c->d_ozgE = ge;
-    c->ozg_rows = (int)grows; c->ozg_ld = gld; c->ozg_p_elems = gpe; c->ozg_np = nb;
+    c->ozg_rows = (int)grows; c->ozg_a_elems = gae; c->ozg_b_elems = gbe;
+    c->ozg_p_elems = gpe; c->ozg_np = nb;
   }
   c->d_trivec = tvec;
   c->tri_vec_slots = tvec ? (nb < 8 ? nb : 8) : 0;

@@ -147,16 +147,14 @@ struct Ctx {
   float2* d_ozP;                    // split-K partials (hi, lo)
   size_t oz_a_elems, oz_b_elems, oz_p_elems;
   // grouped I x I products of a batched eigensolve (oz_zgemm_group): digits of
-  // up to ozg_rows stacked rows (A; B twice as many) of row stride ozg_ld,
-  // partials, row exponents; allocated by sky_reserve_batch for batches of
-  // more than kOzGroupMin problems
+  // every problem's operands, partials, row exponents (ozg_rows stacked rows);
+  // allocated by sky_reserve_batch for batches of more than kOzGroupMin problems
   void* d_ozgA;
   void* d_ozgB;
   float2* d_ozgP;
   int* d_ozgE;
   int ozg_rows, ozg_np;
-  long long ozg_ld;
-  size_t ozg_p_elems;
+  size_t ozg_a_elems, ozg_b_elems, ozg_p_elems;
   char err[256];
 };
 
@@ -269,7 +267,8 @@ constexpr int kOzZgemmGated = 192;
 bool oz_zgemm_fits(const Ctx* c, int n);
 bool oz_zgemm_group_fits(const Ctx* c, int np, const int* n);
 sky_status oz_zgemm_group(Ctx* c, const ZJobs& j);
-int oz_group_slices();
+void oz_group_sizes(int nb, int m, size_t* a_elems, size_t* b_elems);
+void oz_zgemm_sizes(int m, size_t* a_elems, size_t* b_elems);
 bool fused_h_ok(const Ctx* c);      // the fused FP32 h psi applies to this context
 int tri_team_plan(int np, const int* n, int blocks, int* team, int* first, int* count);
 int fused_h_blocks(const Ctx* c);   // its reduction blocks per state               // digits of the grouped products
