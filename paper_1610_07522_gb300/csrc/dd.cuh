@@ -153,6 +153,20 @@ __device__ __forceinline__ double dbl_of(dd a) {
   hd = same ? hd + K : hd - K;
   return __longlong_as_double(hd | sgn);
 }
+// The same rounding with lo counted by one float multiplication and conversion:
+// |lo| in units of the last place of hi's double is |lo| 2^{179 - eh} (half units
+// when hi is a power of two and lo points below it), at most 2^29, added to or
+// subtracted from hi's pattern.  Pairs outside 2^-71 <= |hi| < 2^126 take dbl_of.
+__device__ __forceinline__ double dbl_of_near(dd a) {
+  const unsigned uh = __float_as_uint(a.hi), mh = uh & 0x7fffffffu, sgn = uh & 0x80000000u;
+  const int eh = (int)(mh >> 23);
+  if ((unsigned)(eh - 56) > (unsigned)(252 - 56)) return dbl_of(a);
+  const float l = __uint_as_float(__float_as_uint(a.lo) ^ sgn);
+  const int down = (mh & 0x7fffffu) == 0u && l < 0.0f ? 1 : 0;
+  const int K = __float2int_rn(l * __uint_as_float((unsigned)(306 + down - eh) << 23));
+  const long long hd = (((long long)mh << 29) + (896LL << 52)) + (long long)K;
+  return __longlong_as_double(hd | ((long long)sgn << 32));
+}
 __device__ __forceinline__ ddc ddc_of(double2 v) { return ddc{dd_of(v.x), dd_of(v.y)}; }
 
 // A sum of products of floats in a float pair (the FP32 forms' reductions):

@@ -248,6 +248,139 @@ __device__ __forceinline__ void block_sum2(double& a, double& b) {
   }
 }
 
+// The same pass on float pairs (the operator-product route of the FP64 form): G_j
+// and F_j as pairs (re hi, re lo, im hi, im lo), in place, L as pairs into hpsi;
+// the fields as pairs from f ([5][G]: U, B, W / 2, converted once per call).
+// Every output real is a sum of two or three (L: seven) products of pairs; a
+// product's error and cross terms join the running low part, one
+// renormalisation per sum.  24^3, 280 states: 461 us with doubles in between
+// (their conversions bound it), 263 us with pair operators one by one, 188 us
+// with sums of products; the eight arrays it moves take 146 us.
+struct AccP {
+  float hi = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add(dd a, dd b) {
+    const float p = __fmul_rn(a.hi, b.hi);
+    float e = __fmaf_rn(a.hi, b.hi, -p);
+    e = __fmaf_rn(a.hi, b.lo, e);
+    e = __fmaf_rn(a.lo, b.hi, e);
+    const dd s = two_sum(hi, p);
+    hi = s.hi;
+    lo = __fadd_rn(lo, __fadd_rn(s.lo, e));
+  }
+  __device__ __forceinline__ void first(dd a, dd b) {
+    hi = __fmul_rn(a.hi, b.hi);
+    lo = __fmaf_rn(a.hi, b.hi, -hi);
+    lo = __fmaf_rn(a.hi, b.lo, lo);
+    lo = __fmaf_rn(a.lo, b.hi, lo);
+  }
+  __device__ __forceinline__ dd value() const { return fast_two_sum(hi, lo); }
+};
+// -(i/2) A_j v of component C (own v, other w) added to (re, im); the fields are
+// half W: j = 0: s (i W_y v - W_z w); 1: -i s W_x v + i W_z w; 2: s W_x w - i W_y w,
+// s = 1 for component 0 and -1 for 1.
+template <int J, int C>
+__device__ __forceinline__ void add_so(AccP& re, AccP& im, dd wx, dd wy, dd wz, ddc v, ddc w) {
+  if (J == 0) {
+    const dd y = C ? -wy : wy, z = C ? -wz : wz;
+    re.add(-y, v.y);
+    re.add(-z, w.x);
+    im.add(y, v.x);
+    im.add(-z, w.y);
+  } else if (J == 1) {
+    const dd x = C ? -wx : wx;
+    re.add(x, v.y);
+    re.add(-wz, w.y);
+    im.add(-x, v.x);
+    im.add(wz, w.x);
+  } else {
+    const dd x = C ? -wx : wx;
+    re.add(x, w.x);
+    re.add(wy, w.y);
+    im.add(x, w.y);
+    im.add(-wy, w.x);
+  }
+}
+template <int J>
+__device__ __forceinline__ void h_local_axis(AccP (&L)[4], dd bb, dd wx, dd wy, dd wz, ddc a0, ddc a1,
+                                             ddc d0, ddc d1, ddc& f0, ddc& f1) {
+  add_so<J, 0>(L[0], L[1], wx, wy, wz, d0, d1);    // L += -(i/2) A_j G_j
+  add_so<J, 1>(L[2], L[3], wx, wy, wz, d1, d0);
+  AccP r, i;                                       // F_j = -B G_j - (i/2) A_j psi
+  r.first(-bb, d0.x);
+  i.first(-bb, d0.y);
+  add_so<J, 0>(r, i, wx, wy, wz, a0, a1);
+  f0 = ddc{r.value(), i.value()};
+  r.first(-bb, d1.x);
+  i.first(-bb, d1.y);
+  add_so<J, 1>(r, i, wx, wy, wz, a1, a0);
+  f1 = ddc{r.value(), i.value()};
+}
+__global__ void __launch_bounds__(128) k_h_local_pair(const double2* __restrict__ psi, float4* g0,
+                                                      float4* g1, float4* g2,
+                                                      float4* __restrict__ hpsi,
+                                                      const dd* __restrict__ f, int G) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= G) return;
+  const long long o0 = (long long)blockIdx.y * 2 * G + p, o1 = o0 + G;
+  auto pair = [](float4 v) { return ddc{dd(v.x, v.y), dd(v.z, v.w)}; };
+  auto quad = [](ddc v) { return make_float4(v.x.hi, v.x.lo, v.y.hi, v.y.lo); };
+  const float4 r00 = g0[o0], r01 = g0[o1], r10 = g1[o0], r11 = g1[o1], r20 = g2[o0], r21 = g2[o1];
+  const ddc a0 = ddc_of(psi[o0]), a1 = ddc_of(psi[o1]);
+  const dd u = f[p], bb = f[G + p], wx = f[2 * G + p], wy = f[3 * G + p], wz = f[4 * G + p];
+  AccP L[4];
+  L[0].first(u, a0.x);
+  L[1].first(u, a0.y);
+  L[2].first(u, a1.x);
+  L[3].first(u, a1.y);
+  ddc f0, f1;
+  h_local_axis<0>(L, bb, wx, wy, wz, a0, a1, pair(r00), pair(r01), f0, f1);
+  g0[o0] = quad(f0);
+  g0[o1] = quad(f1);
+  h_local_axis<1>(L, bb, wx, wy, wz, a0, a1, pair(r10), pair(r11), f0, f1);
+  g1[o0] = quad(f0);
+  g1[o1] = quad(f1);
+  h_local_axis<2>(L, bb, wx, wy, wz, a0, a1, pair(r20), pair(r21), f0, f1);
+  g2[o0] = quad(f0);
+  g2[o1] = quad(f1);
+  hpsi[o0] = quad(ddc{L[0].value(), L[1].value()});
+  hpsi[o1] = quad(ddc{L[2].value(), L[3].value()});
+}
+
+// Partial <psi|h psi>, |h psi|^2 of a state's nblk blocks of points: 4 FP64
+// multiply-adds per complex value (24^3, 280 states: 62 us at the FP64 rate,
+// 248 MB read); in the epilogue of the last derivative pass they cost 205 us.
+__global__ void __launch_bounds__(kRedBlock) k_h_totals(const double2* __restrict__ psi,
+                                                        const double2* __restrict__ hpsi, int G,
+                                                        double* part, int nblk) {
+  const long long base = (long long)blockIdx.y * 2 * G;
+  double e[2] = {0.0, 0.0}, n2[2] = {0.0, 0.0};
+  for (int p = blockIdx.x * kRedBlock + threadIdx.x; p < 2 * G; p += nblk * kRedBlock) {
+    const double2 h = hpsi[base + p], a = psi[base + p];
+    e[0] = fma(a.x, h.x, e[0]);
+    e[1] = fma(a.y, h.y, e[1]);
+    n2[0] = fma(h.x, h.x, n2[0]);
+    n2[1] = fma(h.y, h.y, n2[1]);
+  }
+  double es = e[0] + e[1], ns = n2[0] + n2[1];
+  block_sum2(es, ns);
+  if (threadIdx.x == 0) {
+    double* dst = part + ((long long)blockIdx.y * nblk + blockIdx.x) * 2;
+    dst[0] = es;
+    dst[1] = ns;
+  }
+}
+
+__global__ void k_fields_dd(const double* __restrict__ U, const double* __restrict__ B,
+                            const double* __restrict__ W, int G, dd* __restrict__ f) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= G) return;
+  f[p] = dd_of(U[p]);
+  f[G + p] = dd_of(B[p]);
+  f[2 * G + p] = dd_of(0.5 * W[p]);
+  f[3 * G + p] = dd_of(0.5 * W[G + p]);
+  f[4 * G + p] = dd_of(0.5 * W[2 * G + p]);
+}
+
 // Pass 4: hpsi = L + F_x + F_y + F_z; partial <psi|h psi>, |h psi|^2.
 template <typename T>
 __global__ void __launch_bounds__(kRedBlock) k_h_sum(const cx<T>* __restrict__ psi,
@@ -291,16 +424,22 @@ __global__ void __launch_bounds__(kRedBlock) k_h_sum(const cx<T>* __restrict__ p
   }
 }
 
-// Per-state totals of the partial sums, times dV.
-__global__ void k_state_totals(const double* part, int nblk, int I, double dV,
-                               double* eps, double* hn2) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+// Per-state totals of the partial sums, times dV; one warp per state.
+__global__ void __launch_bounds__(128) k_state_totals(const double* part, int nblk, int I, double dV,
+                                                      double* eps, double* hn2) {
+  const int s = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (s >= I) return;
   double a = 0.0, b = 0.0;
-  for (int k = 0; k < nblk; ++k) {
+  for (int k = lane; k < nblk; k += 32) {
     a += part[((long long)s * nblk + k) * 2];
     b += part[((long long)s * nblk + k) * 2 + 1];
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_down_sync(0xffffffffu, a, o);
+    b += __shfl_down_sync(0xffffffffu, b, o);
+  }
+  if (lane != 0) return;
   if (eps) eps[s] = dV * a;
   if (hn2) hn2[s] = dV * b;
 }
@@ -618,7 +757,7 @@ static sky_status apply_h_fused(Ctx* c, const double* U, const double* B, const 
     if (e != cudaSuccess) return cuda_check(c, e, "fused h psi");
   }
   if (eps || hn2) {
-    k_state_totals<<<div_up(I, 128), 128, 0, c->stream>>>(c->d_red, nblk, I, c->dV, eps, hn2);
+    k_state_totals<<<div_up(I, 4), 128, 0, c->stream>>>(c->d_red, nblk, I, c->dV, eps, hn2);
     note_launch();
     return cuda_check(c, cudaGetLastError(), "fused h psi totals");
   }
@@ -657,7 +796,7 @@ static sky_status apply_h_t(Ctx* c, const double* U, const double* B, const doub
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_check(c, e, "apply_h sum");
   }
   if (eps || hn2) {
-    k_state_totals<<<div_up(I, 128), 128, 0, c->stream>>>(c->d_red, c->red_nblk, I, c->dV,
+    k_state_totals<<<div_up(I, 4), 128, 0, c->stream>>>(c->d_red, c->red_nblk, I, c->dV,
                                                           eps, hn2); note_launch();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_check(c, e, "apply_h totals");
@@ -665,8 +804,58 @@ static sky_status apply_h_t(Ctx* c, const double* U, const double* B, const doub
   return SKY_OK;
 }
 
+// FP64 form with the derivatives as operator products: gradients to pairs, the
+// pointwise pass, then h += d_j F_j axis by axis, the last with FP64 out.  hpsi
+// holds L and the growing sum as pairs in between.
+static sky_status apply_h_pair(Ctx* c, const double* U, const double* B, const double* W,
+                               const double2* psi, double2* hpsi, int I, double* eps, double* hn2) {
+  const long long G = c->G, V = 2 * G;
+  const bool tot = eps || hn2;
+  // blocks of the totals per state: about four per SM over the states, at least
+  // two points per thread, at most what d_red holds
+  int nblk = (int)div_up(4LL * c->num_sms, I);
+  if (nblk > (int)(2 * G / (2 * kRedBlock))) nblk = (int)(2 * G / (2 * kRedBlock));
+  if (nblk < 1) nblk = 1;
+  if (nblk < c->red_nblk) nblk = c->red_nblk;
+  if (nblk > c->red_most) nblk = c->red_most;
+  dd* f = reinterpret_cast<dd*>(c->d_hf);
+  k_fields_dd<<<div_up(G, 256), 256, 0, c->stream>>>(U, B, W, (int)G, f);
+  note_launch();
+  char* scr = static_cast<char*>(c->d_gscr);
+  const size_t cbytes = (size_t)c->chunk * V * sizeof(double2);
+  void* g[3] = {scr, scr + cbytes, scr + 2 * cbytes};
+  cudaError_t e = cudaGetLastError();
+  for (int s0 = 0; s0 < I && e == cudaSuccess; s0 += c->chunk) {
+    const int ns = (I - s0) < c->chunk ? (I - s0) : c->chunk;
+    const double2* ps = psi + (long long)s0 * V;
+    double2* hs = hpsi + (long long)s0 * V;
+    for (int ax = 0; ax < 3 && e == cudaSuccess; ++ax) e = deriv_tc_pair(c, ax, ps, g[ax], 2LL * ns);
+    if (e != cudaSuccess) break;
+    k_h_local_pair<<<dim3(div_up(G, 128), ns), 128, 0, c->stream>>>(
+        ps, (float4*)g[0], (float4*)g[1], (float4*)g[2], (float4*)hs, f, (int)G);
+    note_launch();
+    e = cudaGetLastError();
+    for (int ax = 0; ax < 3 && e == cudaSuccess; ++ax) e = deriv_tc_add(c, ax, g[ax], hs, 2LL * ns);
+    if (tot && e == cudaSuccess) {
+      k_h_totals<<<dim3(nblk, ns), kRedBlock, 0, c->stream>>>(
+          ps, hs, (int)G, c->d_red + (size_t)s0 * nblk * 2, nblk);
+      note_launch();
+      e = cudaGetLastError();
+    }
+  }
+  if (e != cudaSuccess) return cuda_check(c, e, "apply_h");
+  if (tot) {
+    k_state_totals<<<div_up(I, 4), 128, 0, c->stream>>>(c->d_red, nblk, I, c->dV, eps, hn2);
+    note_launch();
+    return cuda_check(c, cudaGetLastError(), "apply_h totals");
+  }
+  return SKY_OK;
+}
+
 sky_status apply_h_impl(Ctx* c, const double* U, const double* B, const double* W,
                         const void* psi, void* hpsi, int I, double* eps, double* hn2) {
+  if (c->prec == SKY_F64 && c->line_arith == 2 && c->d_dop[0] && c->d_dop[1] && c->d_dop[2])
+    return apply_h_pair(c, U, B, W, (const double2*)psi, (double2*)hpsi, I, eps, hn2);
   if (c->prec == SKY_F64)
     return apply_h_t<double>(c, U, B, W, (const double2*)psi, (double2*)hpsi, I, eps, hn2);
   // the fused passes are the faster ones at every size they take (measured: 32^3,

@@ -13,16 +13,30 @@
 // so one pass over nb arrays is OUT = LINES Dr^T with one row per line
 // (nb G / n rows, K = N = 2n, padded to NC = a multiple of 16).  Both
 // operands are cut into six base-256 digits (oz_digits.cuh), each line scaled
-// by its own exponent and each row of Dr by its own; the 21 digit products of
-// weight g = s + t <= 5 are summed in FP32 in TMEM: weights 0-3 exactly, one
-// accumulator each (per K value |G_g| <= (g + 3) 2^14, K <= 64, so every sum
-// stays an integer below 2^24), weights 4 and 5 together in a fifth, the
-// weight-5 products taken with the operator's digits times 2^-8 (exact in
-// bf16); its FP32 rounding, at most K 2^-24 of a sum below 2^23 at weight
-// 2^-32, is about 2^-49 of the largest term.  The sums are combined in a
-// 64-bit integer, rounded once to FP64 and scaled by the two exponents.  The
-// error is that rounding plus the truncated digit expansion, about 2^-48 of
-// the line's and the row's largest values.
+// by its own exponent and each row of Dr by its own; digit s is kept as the bf16
+// number alpha_s 2^{-8(s+1)} (exact), so that digit products carry their own
+// weight.  The 21 products of weight g = s + t <= 5 are summed in FP32 in TMEM:
+// weights 0-3 exactly, one accumulator each (per K value |G_g| <= (g + 3) 2^14
+// units, K <= 64, so every sum stays an integer below 2^24 units), weights 4 and
+// 5 together in a fifth; its FP32 rounding, at most K 2^-24 of a sum below 2^23
+// at weight 2^-32, is about 2^-49 of the largest term.  The accumulators lie
+// side by side and the operator's digits one below the other, so digit p of the
+// lines times digits 0 .. 4 - p of the operator is one MMA of (5 - p) NC columns
+// into the accumulators p .. 4 (two for NC = 64, p = 0): 11 MMAs per 16 values
+// of K instead of 21 (24^3, 280 states: 116 us per pass with 21 issued by one
+// lane of a diverged warp, 100 us; 84 us with pairs out).  The sums are combined exactly in a 64-bit
+// integer, rounded once to FP64 and scaled by the two exponents, or, for arrays
+// that stay inside h psi, into a pair of floats by error-free additions.  The
+// error is that rounding plus the truncated digit expansion, about 2^-48 of the
+// line's and the row's largest values.
+//
+// Arrays between the passes of h psi hold float pairs (re hi, re lo, im hi, im
+// lo in the 16 bytes of a complex double): the digits of a pair and the sum of
+// the accumulators into a pair are FP32 operations (about 26 and 30 per real),
+// where doubles take integer work at half the FP32 rate (about 35 and 50
+// instructions).  All of h psi, 24^3, 280 states: 1393 us with doubles between
+// the passes, 845 us; what is left is issue (60% of the slots) and the latency of
+// the loads ahead of each block.
 //
 // Persistent kernel, one CTA per SM, 128 lines per tile:
 //   warps 0-7   producers: warp w takes lines 16 w .. 16 w + 15 of the tile,
@@ -34,8 +48,8 @@
 //               fences the writes for the tensor core's proxy and arrives;
 //   warp 8      owns TMEM (two accumulator sets of 5 x NC fp32 columns, so
 //               the MMAs of one tile run while the epilogue drains the
-//               previous one; one set when 5 NC > 256); one lane issues
-//               tcgen05.mma (M = 128, N = NC, K = 16) for every digit pair;
+//               previous one; one set when 5 NC > 256); it stays converged and
+//               one elected lane executes tcgen05.mma (M = 128, K = 16);
 //   warps 9-16  epilogue: two warps per TMEM lane quadrant, half the columns
 //               each, in blocks of 8 columns; they combine the groups into
 //               64-bit integers, round, scale and store the (re, im) pairs at
@@ -49,6 +63,9 @@
 #include <cstring>
 #include <vector>
 
+#include <type_traits>
+
+#include "dd.cuh"
 #include "oz_digits.cuh"
 #include "oz_gemm.cuh"
 
@@ -61,8 +78,10 @@ using tc::fence_before;
 using tc::idesc_bf16;
 using tc::mbar_init;
 using tc::mbar_wait;
-using tc::mma_bf16;
-using tc::mma_commit;
+using oz::elect_one;
+using oz::mbar_wait_warp;
+using oz::mma_bf16_elect;
+using oz::mma_commit_elect;
 using tc::smem_u32;
 
 constexpr int S = 6;               // digits per operand (FP64 inputs)
@@ -77,10 +96,13 @@ __host__ __device__ constexpr int nc_of(int n) { return ((2 * n + 15) / 16) * 16
 
 // Operators of an axis: the derivative, the forward and the inverse DFT.
 constexpr int kOpDeriv = 0, kOpFwd = 1, kOpInv = 2;
-// Producer input: the lines of src, or the residual src - eps psi (src = h psi).
-constexpr int kInPlain = 0, kInResidual = 1;
-// Epilogue output: the product; times P[point] scale; or psi - w[point] times it.
-constexpr int kOutPlain = 0, kOutScaleP = 1, kOutUpdate = 2;
+// Producer input: the lines of src, the residual src - eps psi (src = h psi), or
+// lines of float pairs.
+constexpr int kInPlain = 0, kInResidual = 1, kInPair = 2;
+// Epilogue output: the product; times P[point] scale; psi - w[point] times it; as
+// pairs; added to the pairs in dst; the sum of that addition as FP64.
+constexpr int kOutPlain = 0, kOutScaleP = 1, kOutUpdate = 2, kOutPair = 3, kOutAddPair = 4,
+              kOutAddF64 = 5;
 
 template <int N>
 struct Shape {
@@ -88,13 +110,15 @@ struct Shape {
   static constexpr int TILE_A = BM * NC * 2;   // one digit of a tile of lines
   static constexpr int STAGE = S * TILE_A;
   static constexpr int TILE_B = NC * NC * 2;   // one digit of the operator
-  static constexpr int OPB = 2 * S * TILE_B;   // its digits, then the digits times 2^-8
+  static constexpr int OPB = S * TILE_B;       // its digits
   static constexpr int NBUF = NG * NC <= 256 ? 2 : 1;   // TMEM accumulator sets
   static constexpr int AUX = NC * 4 + 2 * BM * 4 + kBars * 8 + 16;
   static constexpr int H0 = ((N / 2 + 3) / 4) * 4;             // points of a line's first half
-  // staging of the next tile's half lines (one 16-byte slot per point and
-  // producer thread) when it fits beside one ring stage
-  static constexpr int STG_BYTES = H0 * kProd * 32 * 16;
+  // staging of the next tile's lines when it fits beside one ring stage: one
+  // 16-byte slot per point of each producer thread's half line, or, along x, the
+  // warp's 16 lines as they lie in memory, padded by a point each
+  static constexpr int STG_Y = H0 * kProd * 32 * 16, STG_X = kProd * 16 * (N + 1) * 16;
+  static constexpr int STG_BYTES = STG_Y > STG_X ? STG_Y : STG_X;
   static constexpr bool PREFETCH = STAGE + OPB + AUX + STG_BYTES + 1024 <= kSmemMax;
   static constexpr int STG = PREFETCH ? STG_BYTES : 0;
   static constexpr int STAGES = (2 * STAGE + OPB + AUX + STG + 1024 <= kSmemMax) ? 2 : 1;
@@ -114,11 +138,11 @@ __host__ __device__ constexpr int cm_off(int r, int k, int nc) {
 }
 // Shared-memory matrix descriptor of that layout: leading byte offset 128
 // (core matrices along K), stride byte offset 16 nc (8-row groups), version 1,
-// layout type 0 (no swizzle).
-__device__ __forceinline__ uint64_t ns_desc(uint32_t saddr, int nc) {
-  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(128 >> 4) << 16) |
-         ((uint64_t)((nc * 16) >> 4) << 32) | (1ull << 46);
+// layout type 0 (no swizzle); low word by address, high word fixed.
+__device__ __forceinline__ uint32_t ns_lo(uint32_t saddr) {
+  return ((saddr >> 4) & 0x3FFFu) | ((128u >> 4) << 16);
 }
+__host__ __device__ constexpr uint32_t ns_hi(int nc) { return (uint32_t)((nc * 16) >> 4) | (1u << 14); }
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -131,24 +155,61 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool v
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
+// 2^k as a float, k in [-128, 127] (-127, -128: subnormal).
+__device__ __forceinline__ float pow2f(int k) {
+  return __int_as_float(k >= -126 ? (k + 127) << 23 : 0x00400000 >> (-127 - k));
+}
 // The six balanced base-256 digits of the signed integer Y = +-round(|x|
-// 2^{48 - E}) (|Y| <= 2^48), as floats: adding 128 to each of the five lower
-// byte positions (0x8080808080) turns every lower byte, minus 128, into a
-// digit in [-128, 127], with the carries propagated by the addition; the top
-// digit is the rest, an arithmetic shift (|digit 0| <= 256).  All exact in bf16.
+// 2^{48 - E}) (|Y| <= 2^48), digit s as the float alpha_s 2^{-8(s+1)}: adding 128
+// to each of the five lower byte positions (0x8080808080) turns every lower
+// byte, minus 128, into a digit in [-128, 127], with the carries propagated by
+// the addition; the top digit is the rest, an arithmetic shift (|digit 0| <=
+// 256).  A byte placed below the bits of 2^23 u (u the digit's unit) is that
+// float plus byte u; subtracting (2^23 + 128) u leaves the digit, exactly.
 __device__ __forceinline__ void digits6f(double x, int E, float* d) {
   long long Y = (long long)fixed_of<6>(x, E);
   if (sign_of(x)) Y = -Y;
   const long long Z = Y + 0x8080808080LL;
   const unsigned lo = (unsigned)Z, hi = (unsigned)((unsigned long long)Z >> 32);
-  auto f = [](int v) { return __int_as_float(0x4B400000 + v) - 12582912.0f; };   // exact, |v| < 2^22
-  d[5] = f((int)(lo & 255u) - 128);
-  d[4] = f((int)((lo >> 8) & 255u) - 128);
-  d[3] = f((int)((lo >> 16) & 255u) - 128);
-  d[2] = f((int)(lo >> 24) - 128);
-  d[1] = f((int)(hi & 255u) - 128);
-  d[0] = f((int)(Z >> 40));
+  constexpr unsigned kOne = 0x4B000000u, kU = 8u << 23;     // 2^23; one unit step
+  auto f = [](unsigned word, unsigned sel, unsigned steps) {
+    const unsigned m = kOne - steps * kU;
+    return __uint_as_float(__byte_perm(word, m, sel)) - (__uint_as_float(m) + 128.0f * __uint_as_float(0x3F800000u - steps * kU));
+  };
+  d[5] = f(lo, 0x7650, 6);
+  d[4] = f(lo, 0x7651, 5);
+  d[3] = f(lo, 0x7652, 4);
+  d[2] = f(lo, 0x7653, 3);
+  d[1] = f(hi, 0x7650, 2);
+  d[0] = __int_as_float((int)(0x4B400000u - kU) + (int)(Z >> 40)) - __uint_as_float(0x4B400000u - kU);
 }
+// The same digits of a float pair scaled to |h + l| <= 1 (h = fl(h + l)): each
+// digit is the part of the remainder above half a unit, cut off by adding and
+// subtracting 1.5 2^23 units; three digits take h's 24 bits, then l joins the
+// remainder (its rounding there is below 2^-49).
+__device__ __forceinline__ void digits6p(float h, float l, float* d) {
+  auto cut = [](float r, int s) {
+    const float m = 12582912.0f * __uint_as_float(0x3F800000u - (unsigned)(s + 1) * (8u << 23));
+    return __fsub_rn(__fadd_rn(r, m), m);
+  };
+  float r = h;
+#pragma unroll
+  for (int s = 0; s < 5; ++s) {
+    d[s] = cut(r, s);
+    r = __fsub_rn(r, d[s]);
+    if (s == 2) r = __fadd_rn(r, l);
+  }
+  d[5] = cut(r, 5);
+}
+// The accumulators g0 .. g4 (decreasing weight) as a float pair.
+__device__ __forceinline__ dd pair_of_groups(float g0, float g1, float g2, float g3, float g4) {
+  const dd a = two_sum(g0, g1), b = two_sum(g2, g3);
+  const dd u = two_sum(a.lo, b.hi);
+  const dd t = two_sum(a.hi, u.hi);
+  return fast_two_sum(t.hi, __fadd_rn(t.lo, __fadd_rn(u.lo, __fadd_rn(b.lo, g4))));
+}
+// An exponent whose power of two pow2f forms (pairs beyond it have no FP32 value).
+__device__ __forceinline__ int clamp_exp(int k) { return k < -128 ? -128 : k > 127 ? 127 : k; }
 __device__ __forceinline__ unsigned bf16x2(float lo, float hi) {   // lo in the low half
   unsigned r;
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
@@ -199,10 +260,30 @@ __device__ __forceinline__ unsigned fdiv(unsigned n, const FastDiv& f) {
   return f.d == 1 ? n : (__umulhi(n, f.m) >> f.sh);
 }
 
+// 4 x 4 transpose over the lanes of a quad: afterwards z[k] of lane j is what
+// z[j] of lane k was.
+__device__ __forceinline__ float4 shfl4(float4 v, int mask) {
+  return make_float4(__shfl_xor_sync(0xffffffffu, v.x, mask), __shfl_xor_sync(0xffffffffu, v.y, mask),
+                     __shfl_xor_sync(0xffffffffu, v.z, mask), __shfl_xor_sync(0xffffffffu, v.w, mask));
+}
+__device__ __forceinline__ void quad_transpose(float4 (&z)[4], int lane) {
+#pragma unroll
+  for (int h = 1; h <= 2; h <<= 1) {
+    const bool up = lane & h;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (i & h) continue;
+      const float4 recv = shfl4(up ? z[i] : z[i + h], h);
+      if (up) z[i] = recv;
+      else z[i + h] = recv;
+    }
+  }
+}
+
 struct DerivArgs {
   const double2* src;   // nb arrays of G complex points (may equal dst)
   double2* dst;
-  const uint4* op;      // operator digits, 2 S * TILE_B bytes in the canonical layout
+  const uint4* op;      // operator digits, S * TILE_B bytes in the canonical layout
   const int* ope;       // operator row exponents [NC]
   int nx, ny, nz;
   long long G;
@@ -264,7 +345,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_deriv(const DerivArgs a) {
   int* s_ea = s_eb + NC;                                      // [2][BM]
   unsigned long long* bars = (unsigned long long*)(s_ea + 2 * BM);
   uint32_t* tmem_slot = (uint32_t*)(bars + kBars);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const uint32_t bar0 = smem_u32(bars);
   auto full = [&](int s) { return bar0 + 8u * s; };
   auto empty = [&](int s) { return bar0 + 8u * (2 + s); };
@@ -276,7 +357,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_deriv(const DerivArgs a) {
 
   // the operator's digits and row exponents, for the whole launch
   for (int i = threadIdx.x; i < Sh::OPB / 16; i += blockDim.x) ((uint4*)opb)[i] = a.op[i];
-  for (int i = threadIdx.x; i < NC; i += blockDim.x) s_eb[i] = a.ope[i];
+  // row exponents; as factors where the output is pairs
+  for (int i = threadIdx.x; i < NC; i += blockDim.x)
+    s_eb[i] = OUT >= kOutPair ? __float_as_int(pow2f(clamp_exp(a.ope[i]))) : a.ope[i];
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -321,7 +404,24 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_deriv(const DerivArgs a) {
     const int np = hh ? H1 : H0;              // points of this half
     const int p0 = hh ? H0 : 0;               // first point
     const uint32_t my_stg = smem_u32(stg) + (uint32_t)threadIdx.x * 16u;
+    // lines along x are consecutive in memory: the warp copies its 16 lines in
+    // order (whole sectors; a lane per half line had fetched every sector twice)
+    constexpr bool XW = AXIS == 0;
+    const uint32_t warp_stg = smem_u32(stg) + (uint32_t)(warp * 16 * (N + 1) * 16);
     auto prefetch = [&](int t, bool go) {     // go: a data dependency on the caller's reads
+      if constexpr (XW) {
+        __syncwarp();                         // every lane has read its slots
+        const long long l0 = (long long)t * BM + warp * 16;   // nlines is a multiple of 16
+        const bool valid = go && l0 < a.nlines;
+        const double2* src = a.src + (valid ? l0 * N : 0);
+#pragma unroll
+        for (int k = 0; k < N / 2; ++k) {
+          const int e = k * 32 + lane, rr = e / N;
+          cp_async16(warp_stg + (uint32_t)((e + rr) * 16), src + (valid ? e : 0), valid);
+        }
+        cp_async_commit();
+        return;
+      }
       const long long l = (long long)t * BM + r;
       const bool valid = go && l < a.nlines;
       long long stride = 0;
@@ -335,19 +435,22 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_deriv(const DerivArgs a) {
                      valid);
       cp_async_commit();
     };
-    constexpr bool PF = Sh::PREFETCH && IN == kInPlain;
+    constexpr bool PF = Sh::PREFETCH && IN != kInResidual;
     if constexpr (PF)
       if (blockIdx.x < a.ntiles) prefetch(blockIdx.x, true);
     int it = 0;
     for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x, ++it) {
       const int s = it % STAGES, u = it / STAGES, slot = it & 1;
-      double2 v[H0];
+      using V = std::conditional_t<IN == kInPair, float4, double2>;
+      V v[H0];
       if constexpr (PF) {
         cp_async_wait_all();
+        if constexpr (XW) __syncwarp();       // the other lanes' copies too
 #pragma unroll
         for (int j = 0; j < H0; ++j)
-          v[j] = j < np ? *(const double2*)(stg + (j * PT + threadIdx.x) * 16)
-                        : make_double2(0.0, 0.0);
+          v[j] = j < np ? (XW ? *(const V*)(stg + (warp * 16 * (N + 1) + (lane & 15) * (N + 1) + p0 + j) * 16)
+                              : *(const V*)(stg + (j * PT + threadIdx.x) * 16))
+                        : V{};
       } else {
         const long long l = (long long)t * BM + r;
         const bool valid = l < a.nlines;
@@ -355,8 +458,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_deriv(const DerivArgs a) {
         const long long lb = valid ? line_base<N, AXIS>(a, l, stride) : 0;
 #pragma unroll
         for (int j = 0; j < H0; ++j)
-          v[j] = (valid && j < np) ? a.src[lb + (long long)(p0 + j) * stride]
-                                   : make_double2(0.0, 0.0);
+          v[j] = (valid && j < np) ? ((const V*)a.src)[lb + (long long)(p0 + j) * stride] : V{};
         if constexpr (IN == kInResidual) {    // src - eps psi (src = h psi)
           const double e = valid ? a.eps[line_array<N, AXIS>(a, l) >> 1] : 0.0;
 #pragma unroll
@@ -369,7 +471,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_deriv(const DerivArgs a) {
       }
       int E = INT_MIN;
 #pragma unroll
-      for (int j = 0; j < H0; ++j) E = max(E, max(exp_of(v[j].x), exp_of(v[j].y)));
+      for (int j = 0; j < H0; ++j) {
+        if constexpr (IN == kInPair) E = max(E, max(exp_of(v[j].x), exp_of(v[j].z)));
+        else E = max(E, max(exp_of(v[j].x), exp_of(v[j].y)));
+      }
       if constexpr (PF) {
         // the next copy overwrites the slots just read: it is issued after E,
         // which depends on every value read
@@ -386,6 +491,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_deriv(const DerivArgs a) {
         break;
       }
       if (hh == 0) s_ea[slot * BM + r] = E;
+      const float sc = IN == kInPair ? pow2f(-(E < 128 ? E : 128)) : 1.0f;   // pairs: |E| <= 129
       unsigned char* ta = ring + s * STAGE;
 #pragma unroll
       for (int c = 0; c < H0 / 4; ++c) {
@@ -394,8 +500,14 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_deriv(const DerivArgs a) {
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             float dr[S], di[S];
-            digits6f(v[4 * c + j].x, E, dr);
-            digits6f(v[4 * c + j].y, E, di);
+            if constexpr (IN == kInPair) {
+              const float4 z = v[4 * c + j];
+              digits6p(z.x * sc, z.y * sc, dr);
+              digits6p(z.z * sc, z.w * sc, di);
+            } else {
+              digits6f(v[4 * c + j].x, E, dr);
+              digits6f(v[4 * c + j].y, E, di);
+            }
 #pragma unroll
             for (int p = 0; p < S; ++p) w[p][j] = bf16x2(dr[p], di[p]);
           }
@@ -421,52 +533,57 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_deriv(const DerivArgs a) {
     if constexpr (PF) cp_async_wait_all();   // no copy outlives the launch
   } else if (warp == kProd) {
     // ---------------------------------------------------------------- MMA issue
-    if (lane == 0) {
-      const uint32_t idesc = idesc_bf16(BM, NC);
-      const uint32_t sb = smem_u32(opb);
-      bool ok = true;
-      int it = 0;
-      for (int t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x, ++it) {
-        const int s = it % STAGES, u = it / STAGES;
-        if (!mbar_wait(full(s), (uint32_t)(u & 1))) {
-          flag_status(a.status, SKY_ETIMEOUT);
+    const uint32_t el = elect_one();
+    const uint32_t lb = ns_lo(smem_u32(opb));
+    constexpr uint32_t dhi = ns_hi(NC);
+    constexpr int NBUF = Sh::NBUF;
+    int it = 0;
+    for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x, ++it) {
+      const int s = it % STAGES, u = it / STAGES;
+      if (!mbar_wait_warp(full(s), (uint32_t)(u & 1))) {
+        if (lane == 0) flag_status(a.status, SKY_ETIMEOUT);
+        break;
+      }
+      fence_after();
+      const uint32_t la = ns_lo(smem_u32(ring + s * STAGE));
+      const int b = it % NBUF, use = it / NBUF;
+      if (use > 0) {
+        // the epilogue must have drained this accumulator set
+        if (!mbar_wait_warp(acc_empty(b), (uint32_t)((use - 1) & 1))) {
+          if (lane == 0) flag_status(a.status, SKY_ETIMEOUT);
           break;
         }
         fence_after();
-        const uint32_t sa = smem_u32(ring + s * STAGE);
-        constexpr int NBUF = Sh::NBUF;
-        const int b = it % NBUF, use = it / NBUF;
-        if (use > 0) {
-          // the epilogue must have drained this accumulator set
-          if (!mbar_wait(acc_empty(b), (uint32_t)((use - 1) & 1))) {
-            flag_status(a.status, SKY_ETIMEOUT);
-            ok = false;
-            break;
-          }
-          fence_after();
-        }
-        for (int g = 0; g <= S - 1; ++g) {
-          // weights 0..3 into groups 0..3; weights 4 and 5 into group 4, the
-          // weight-5 products with the operator's digits times 2^-8
-          const int grp = g < NG ? g : NG - 1;
-          const uint32_t acc = tmem + (uint32_t)(b * 256 + grp * NC);
-          for (int p = 0; p <= g; ++p) {
-            const int q = (g == S - 1) ? S + (g - p) : (g - p);
-#pragma unroll
-            for (int ks = 0; ks < NC / 16; ++ks)   // 16 values of K = two core matrices
-              mma_bf16(acc, ns_desc(sa + p * TILE_A + ks * 256, NC),
-                       ns_desc(sb + q * TILE_B + ks * 256, NC), idesc,
-                       (g < NG && p == 0 && ks == 0) ? 0u : 1u);
-          }
-        }
-        mma_commit(acc_full(b));   // arrives when this tile's MMAs have completed
-        if (!ok) break;
-        mma_commit(empty(s));
       }
-      // every MMA issued by this thread completes before TMEM is freed
-      mma_commit(drain);
-      if (!mbar_wait(drain, 0)) flag_status(a.status, SKY_ETIMEOUT);
+      const uint32_t acc = tmem + (uint32_t)(b * 256);
+#pragma unroll
+      for (int ks = 0; ks < NC / 16; ++ks) {   // 16 values of K = two core matrices
+        const uint32_t ka = la + (uint32_t)((ks * 256) >> 4), kb = lb + (uint32_t)((ks * 256) >> 4);
+        // weights up to 4: digit p of the lines with digits 0 .. 4 - p; the first
+        // MMA of the tile writes every accumulator
+#pragma unroll
+        for (int p = 0; p < NG; ++p) {
+          constexpr int most = 256 / NC;       // digits per MMA
+          const int n = NG - p, n0 = n < most ? n : most;
+          mma_bf16_elect(acc + (uint32_t)(p * NC), ka + (uint32_t)(p * (TILE_A >> 4)), kb, dhi,
+                         idesc_bf16(BM, n0 * NC), (p == 0 && ks == 0) ? 0u : 1u, el);
+          if (n > n0)
+            mma_bf16_elect(acc + (uint32_t)((p + n0) * NC), ka + (uint32_t)(p * (TILE_A >> 4)),
+                           kb + (uint32_t)(n0 * (TILE_B >> 4)), dhi, idesc_bf16(BM, (n - n0) * NC),
+                           (p == 0 && ks == 0) ? 0u : 1u, el);
+        }
+        // weight 5 into the last accumulator
+#pragma unroll
+        for (int p = 0; p < S; ++p)
+          mma_bf16_elect(acc + (uint32_t)((NG - 1) * NC), ka + (uint32_t)(p * (TILE_A >> 4)),
+                         kb + (uint32_t)((S - 1 - p) * (TILE_B >> 4)), dhi, idesc_bf16(BM, NC), 1u, el);
+      }
+      mma_commit_elect(acc_full(b), el);   // arrives when this tile's MMAs have completed
+      mma_commit_elect(empty(s), el);
     }
+    // every MMA issued by this warp completes before TMEM is freed
+    mma_commit_elect(drain, el);
+    if (!mbar_wait_warp(drain, 0) && lane == 0) flag_status(a.status, SKY_ETIMEOUT);
   } else {
     // ---------------------------------------------------------------- epilogue
     const int w = warp - kProd - 1;            // 0 .. kEpi - 1
@@ -486,95 +603,141 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_deriv(const DerivArgs a) {
       long long stride = 0;
       const long long lb = l < a.nlines ? line_base<N, AXIS>(a, l, stride) : 0;
       long long bG = 0;
-      if constexpr (OUT != kOutPlain) bG = l < a.nlines ? (long long)line_array<N, AXIS>(a, l) * a.G : 0;
+      if constexpr (OUT == kOutUpdate) bG = l < a.nlines ? (long long)line_array<N, AXIS>(a, l) * a.G : 0;
       const int sc = E - 16 - 8 * (S - 1);
       constexpr int NBUF = Sh::NBUF;
       const int b = it % NBUF, use = it / NBUF;
-      // the epilogue's own operands (psi and w, or P) of a block of 4 points are
-      // loaded one block ahead, the first before the wait: behind the stores
-      // they would be a chain of round trips (24^3, 280 states: the step with
-      // its two such passes 905 us with the loads behind the stores, 840 us
-      // ahead of them)
-      constexpr bool AHEAD = OUT != kOutPlain;
+      // A thread's four outputs of a block of 8 columns (4 points from m0): its own
+      // line's points, or, along x, where points are consecutive in memory, point
+      // m0 + lane % 4 of the four lines of its lane quad (the quad transposes its
+      // 4 x 4 results, so that a quad stores 64 consecutive bytes).
+      const long long lq = (long long)t * BM + q * 32 + (lane & 28);
+      auto at_of = [&](int m0, int c, bool& on) -> long long {
+        if constexpr (AXIS == 0) {
+          on = lq + c < a.nlines;
+          return (lq + c) * N + m0 + (lane & 3);
+        } else {
+          on = l < a.nlines;
+          return lb + (long long)(m0 + c) * stride;
+        }
+      };
+      // the epilogue's own operands (psi and w, P, or the pairs to add to) are
+      // loaded before the block's sums are read and combined, the first before the
+      // wait: behind the stores they would be a chain of round trips (24^3, 280
+      // states: the step with its two such passes 905 us with the loads behind the
+      // stores, 840 us ahead of them)
+      constexpr bool ADD = OUT == kOutAddPair || OUT == kOutAddF64;
+      constexpr bool PAIR = ADD || OUT == kOutPair;
+      constexpr bool AHEAD = ADD || OUT == kOutScaleP || OUT == kOutUpdate;
+      const float fE = pow2f(clamp_exp(E));
       double2 xp[4];
       double xf[4];
-      auto ahead = [&](int cb) {
+      float xw[4];
+      float4 xh[4];
+      auto ahead = [&](int m0) {
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          const int m = ((half * HALF + cb) >> 1) + c;
-          const bool on = l < a.nlines && m < N;
-          const long long at = lb + (long long)m * stride;
+          bool on;
+          const long long at = at_of(m0, c, on);
           if constexpr (OUT == kOutUpdate) {
             xp[c] = on ? __ldg(a.psi + at) : make_double2(0.0, 0.0);
-            xf[c] = on && a.w ? (double)__ldg(a.w + (at - bG)) : 1.0;
-          } else if constexpr (OUT == kOutScaleP) {
-            xf[c] = on ? __ldg(a.P + (at - bG)) : 0.0;
+            xw[c] = on && a.w ? __ldg(a.w + (at - bG)) : 1.0f;
+          } else if constexpr (OUT == kOutScaleP) {   // lines along x
+            xf[c] = on ? __ldg(a.P + (at - (long long)line_array<N, AXIS>(a, lq + c) * a.G)) : 0.0;
+          } else if constexpr (ADD) {
+            xh[c] = on ? ((const float4*)a.dst)[at] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
           }
         }
       };
-      if constexpr (AHEAD) ahead(0);
+      if constexpr (AHEAD) ahead(half * HALF / 2);
       if (!mbar_wait(acc_full(b), (uint32_t)(use & 1))) {
         if (lane == 0) flag_status(a.status, SKY_ETIMEOUT);
         break;
       }
       fence_after();
-      // columns in blocks of 8 (4 points).  The exact group sums (integers,
-      // |G_g| < 2^24) fold into int32: u = G0 2^8 + G1, w = G2 2^8 + G3, and
-      // x = round(2^8 G45) from the weight-{4,5} group (|x| < 2^31 for
-      // K <= 64); the total sum_g G_g 2^{8(5-g)} = u 2^32 + w 2^16 + x.
+      // columns in blocks of 8 (4 points).  FP64 out: the exact group sums
+      // (integers G_g of units 2^{-8(g+2)}, |G_g| < 2^24) fold into int32: u = G0
+      // 2^8 + G1, w = G2 2^8 + G3, and x = round(2^8 G45) from the weight-{4,5}
+      // group (|x| < 2^31 for K <= 64); the total sum_g G_g 2^{8(5-g)} = u 2^32 +
+      // w 2^16 + x.
 #pragma unroll 1
       for (int cb = 0; cb < HALF; cb += 8) {
+        const int o = half * HALF + cb, m0 = o >> 1;
+        if (m0 >= N) break;                    // padding (N is a multiple of 4)
+        if constexpr (AHEAD)
+          if (cb > 0) ahead(m0);
         uint32_t v[NG][8];
 #pragma unroll
         for (int g = 0; g < NG; ++g)
-          oz::tmem_ld<8>(tmem + ((uint32_t)(q * 32) << 16) +
-                             (uint32_t)(b * 256 + g * NC + half * HALF + cb),
-                         v[g]);
+          oz::tmem_ld<8>(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * 256 + g * NC + o), v[g]);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        long long acc[8];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const int fu = __float2int_rn(__uint_as_float(v[0][c])) * 256 +
-                         __float2int_rn(__uint_as_float(v[1][c]));
-          const int fw = __float2int_rn(__uint_as_float(v[2][c])) * 256 +
-                         __float2int_rn(__uint_as_float(v[3][c]));
-          const int fx = __float2int_rn(__uint_as_float(v[4][c]) * 256.0f);
-          acc[c] = ((long long)fu << 32) + ((long long)fw << 16) + (long long)fx;
-        }
-        double2 cp[4];
-        double cf[4];
-        if constexpr (AHEAD) {
+        float4 z[4];                           // four results: pairs, or the bits of two doubles
+        if constexpr (PAIR) {
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
-            cp[c] = xp[c];
-            cf[c] = xf[c];
-          }
-          if (cb + 8 < HALF) ahead(cb + 8);
-        }
-        if (l < a.nlines) {
+            float r[4];
 #pragma unroll
-          for (int c = 0; c < 8; c += 2) {
-            const int o = half * HALF + cb + c;   // even: (re, im) of point o / 2
-            const int m = o >> 1;
-            if (m < N) {
-              double2 res;
-              res.x = scaled_double(acc[c], sc + s_eb[o]);
-              res.y = scaled_double(acc[c + 1], sc + s_eb[o + 1]);
-              const long long at = lb + m * stride;
-              if constexpr (OUT == kOutScaleP) {
-                const double f = cf[c >> 1] * a.scale;
-                res = make_double2(res.x * f, res.y * f);
-              } else if constexpr (OUT == kOutUpdate) {
-                const double2 ps = cp[c >> 1];
-                if (a.w) {
-                  const double f = cf[c >> 1];
-                  res = make_double2(fma(-f, res.x, ps.x), fma(-f, res.y, ps.y));
-                } else {
-                  res = make_double2(ps.x - res.x, ps.y - res.y);
-                }
-              }
-              a.dst[at] = res;
+            for (int h = 0; h < 2; ++h) {
+              const int k = 2 * c + h;
+              const dd p = pair_of_groups(__uint_as_float(v[0][k]), __uint_as_float(v[1][k]),
+                                          __uint_as_float(v[2][k]), __uint_as_float(v[3][k]),
+                                          __uint_as_float(v[4][k]));
+              const float f = fE * __int_as_float(s_eb[o + k]);
+              r[2 * h] = p.hi * f;
+              r[2 * h + 1] = p.lo * f;
             }
+            z[c] = make_float4(r[0], r[1], r[2], r[3]);
+          }
+        } else {
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            double r[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int k = 2 * c + h;
+              const int fu = __float2int_rn(__uint_as_float(v[0][k]) * 0x1p16f) * 256 +
+                             __float2int_rn(__uint_as_float(v[1][k]) * 0x1p24f);
+              const int fw = __float2int_rn(__uint_as_float(v[2][k]) * 0x1p32f) * 256 +
+                             __float2int_rn(__uint_as_float(v[3][k]) * 0x1p40f);
+              const int fx = __float2int_rn(__uint_as_float(v[4][k]) * 0x1p56f);
+              r[h] = scaled_double(((long long)fu << 32) + ((long long)fw << 16) + (long long)fx,
+                                   sc + s_eb[o + k]);
+            }
+            z[c] = make_float4(__int_as_float(__double2loint(r[0])), __int_as_float(__double2hiint(r[0])),
+                               __int_as_float(__double2loint(r[1])), __int_as_float(__double2hiint(r[1])));
+          }
+        }
+        if constexpr (AXIS == 0) quad_transpose(z, lane);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          bool on;
+          const long long at = at_of(m0, c, on);
+          if (!on) continue;
+          if constexpr (PAIR) {
+            if constexpr (ADD) {
+              const float4 h = xh[c];
+              const ddc r = ddc{dd(h.x, h.y), dd(h.z, h.w)} + ddc{dd(z[c].x, z[c].y), dd(z[c].z, z[c].w)};
+              if constexpr (OUT == kOutAddF64) a.dst[at] = make_double2(dbl_of_near(r.x), dbl_of_near(r.y));
+              else ((float4*)a.dst)[at] = make_float4(r.x.hi, r.x.lo, r.y.hi, r.y.lo);
+            } else {
+              ((float4*)a.dst)[at] = z[c];
+            }
+          } else {
+            double2 res = make_double2(__hiloint2double(__float_as_int(z[c].y), __float_as_int(z[c].x)),
+                                       __hiloint2double(__float_as_int(z[c].w), __float_as_int(z[c].z)));
+            if constexpr (OUT == kOutScaleP) {
+              const double f = xf[c] * a.scale;
+              res = make_double2(res.x * f, res.y * f);
+            } else if constexpr (OUT == kOutUpdate) {
+              const double2 ps = xp[c];
+              if (a.w) {
+                const double f = (double)xw[c];
+                res = make_double2(fma(-f, res.x, ps.x), fma(-f, res.y, ps.y));
+              } else {
+                res = make_double2(ps.x - res.x, ps.y - res.y);
+              }
+            }
+            a.dst[at] = res;
           }
         }
       }
@@ -597,8 +760,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_deriv(const DerivArgs a) {
 // ------------------------------------------------------------ host side
 bool supported(int n) { return n == 8 || n == 12 || n == 16 || n == 20 || n == 24 || n == 32; }
 
-// Digits [2S][NC][NC] (canonical layout, bf16 bit patterns; digits S..2S-1
-// are digits 0..S-1 times 2^-8) and row exponents [NC] of the real operator
+// Digits [S][NC][NC] (canonical layout, bf16 bit patterns of alpha_s 2^{-8(s+1)})
+// and row exponents [NC] of the real operator
 // of one axis, built in long double.  kind: kOpDeriv the derivative, the
 // circulant D[m][q] = d[(m - q) mod n], d[r] = (i/n) sum_a kappa_a
 // e^{2 pi i a r / n}; kOpFwd / kOpInv the unnormalised DFT, D[m][q] =
@@ -643,7 +806,7 @@ void build_operator(int n, double L, double theta, int kind, std::vector<unsigne
       B[(size_t)(2 * m + 1) * NC + 2 * q] = im;
       B[(size_t)(2 * m + 1) * NC + 2 * q + 1] = re;
     }
-  dig.assign((size_t)2 * S * NC * NC, 0);
+  dig.assign((size_t)S * NC * NC, 0);
   ex.assign(NC, 0);
   for (int o = 0; o < NC; ++o) {
     int F = INT_MIN;
@@ -670,13 +833,10 @@ void build_operator(int n, double L, double theta, int kind, std::vector<unsigne
       }
       d[0] = (int)X;
       for (int p = 0; p < S; ++p) {
-        const float f = (float)(x < 0.0 ? -d[p] : d[p]);   // |d| <= 256: exact in bf16
-        const float f8 = f * 0.00390625f;                   // times 2^-8: also exact
-        unsigned u, u8;
+        const float f = std::ldexp((float)(x < 0.0 ? -d[p] : d[p]), -8 * (p + 1));   // |d| <= 256: exact in bf16
+        unsigned u;
         std::memcpy(&u, &f, 4);
-        std::memcpy(&u8, &f8, 4);
         dig[((size_t)p * NC * NC * 2 + cm_off(o, k, NC)) / 2] = (unsigned short)(u >> 16);
-        dig[((size_t)(S + p) * NC * NC * 2 + cm_off(o, k, NC)) / 2] = (unsigned short)(u8 >> 16);
       }
     }
   }
@@ -775,8 +935,11 @@ cudaError_t op_pass(const Ctx* c, int ax, const ozd::DerivArgs& a) {
       return ax == 2 ? ozd::launch<N, 2, IN, OUT>(a, c) : cudaErrorInvalidValue;
     } else if constexpr (OUT == ozd::kOutScaleP) {
       return ax == 0 ? ozd::launch<N, 0, IN, OUT>(a, c) : cudaErrorInvalidValue;
-    } else if constexpr (OUT == ozd::kOutUpdate) {
+    } else if constexpr (OUT == ozd::kOutUpdate || OUT == ozd::kOutAddF64) {
       return ax == 2 ? ozd::launch<N, 2, IN, OUT>(a, c) : cudaErrorInvalidValue;
+    } else if constexpr (OUT == ozd::kOutAddPair) {
+      if (ax == 0) return ozd::launch<N, 0, IN, OUT>(a, c);
+      return ax == 1 ? ozd::launch<N, 1, IN, OUT>(a, c) : cudaErrorInvalidValue;
     } else {
       if (ax == 0) return ozd::launch<N, 0, IN, OUT>(a, c);
       if (ax == 1) return ozd::launch<N, 1, IN, OUT>(a, c);
@@ -801,6 +964,18 @@ cudaError_t deriv_tc(Ctx* c, int ax, const double2* src, double2* dst, long long
   if (!c->d_dop[ax]) return cudaErrorInvalidValue;
   return op_pass<ozd::kInPlain, ozd::kOutPlain>(
       c, ax, op_args(c, ax, src, dst, nb, c->d_dop[ax], c->d_dope[ax]));
+}
+
+// The passes of h psi on pairs (hamiltonian.cu): G = d_ax psi as pairs; h += d_ax F
+// along x and y (pairs), along z with FP64 out.
+cudaError_t deriv_tc_pair(Ctx* c, int ax, const double2* psi, void* g, long long nb) {
+  return op_pass<ozd::kInPlain, ozd::kOutPair>(
+      c, ax, op_args(c, ax, psi, (double2*)g, nb, c->d_dop[ax], c->d_dope[ax]));
+}
+cudaError_t deriv_tc_add(Ctx* c, int ax, const void* f, void* h, long long nb) {
+  const ozd::DerivArgs a = op_args(c, ax, (const double2*)f, (double2*)h, nb, c->d_dop[ax], c->d_dope[ax]);
+  return ax < 2 ? op_pass<ozd::kInPair, ozd::kOutAddPair>(c, ax, a)
+                : op_pass<ozd::kInPair, ozd::kOutAddF64>(c, ax, a);
 }
 
 bool damp_tc_available(const Ctx* c) {

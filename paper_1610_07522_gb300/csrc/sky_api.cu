@@ -279,9 +279,12 @@ sky_status sky_init(sky_ctx** out, const int grid[3], const double dx[3], const 
     // per-state reduction partials of h psi: the general path's blocks or the
     // fused FP32 path's (one per 32 lines along z at most)
     const long long fz = ((long long)grid[0] * grid[1] + 31) / 32;
-    const long long nb = fz > c->red_nblk ? fz : c->red_nblk;
+    long long nb = fz > c->red_nblk ? fz : c->red_nblk;
+    if (prec == SKY_F64 && nb < 16) nb = 16;   // few states: more blocks each
+    c->red_most = (int)nb;
     ALLOC(c->d_red, (size_t)Imax * nb * 2);
   }
+  if (prec == SKY_F64) ALLOC(c->d_hf, (size_t)10 * G);
   if (prec != SKY_F64) {
     // fused h psi whenever it applies; the knob reports 1 up to axis length 24
     // until it is set

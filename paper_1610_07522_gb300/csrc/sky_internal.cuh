@@ -92,11 +92,12 @@ struct Ctx {
   int chunk;                        // states per apply_h / densities chunk
   double* d_red;                    // per-state partial sums [max_states][nblk][2]
   int red_nblk;                     // reduction blocks per state
+  int red_most;                     // and the most d_red has room for
   double* d_dpart;                  // density partials [kDensSplits][5][G]
   double* d_ftmp;                   // field temporaries [16][G]
   double2* d_fcx;                   // half spectra of the Coulomb transform, two buffers
   double* d_fop[3];                 // real-field operators of each axis (fields.cu)
-  float* d_hf;                      // FP32 forms: U, B, W of one species as floats [5][G]
+  float* d_hf;                      // U, B, W of one species: floats [5][G], FP64 form float pairs
   int fused_h;                      // FP32 forms: one fused pass per axis for h psi (tunable)
   bool fused_auto;                  // fused_h not set by the caller: fused whenever it applies
   double2* d_gpart;                 // split-K partials of sky_overlap
@@ -234,6 +235,8 @@ sky_status tri_init(Ctx* c);
 sky_status derivative_impl(Ctx* c, int axis, const void* src, void* dst, int n);
 sky_status deriv_tc_init(Ctx* c);
 cudaError_t deriv_tc(Ctx* c, int ax, const double2* src, double2* dst, long long nb);
+cudaError_t deriv_tc_pair(Ctx* c, int ax, const double2* psi, void* g, long long nb);
+cudaError_t deriv_tc_add(Ctx* c, int ax, const void* f, void* h, long long nb);
 bool damp_tc_available(const Ctx* c);
 cudaError_t damp_tc(Ctx* c, int q, const double2* psi, const double2* hpsi, const double* eps,
                     double2* phi, int I, double x0, const float* w);
