@@ -804,6 +804,11 @@ static sky_status apply_h_t(Ctx* c, const double* U, const double* B, const doub
   return SKY_OK;
 }
 
+// The FP64 form with every derivative as an operator product (float pairs inside).
+static bool operator_route(const Ctx* c) {
+  return c->prec == SKY_F64 && c->line_arith == 2 && c->d_dop[0] && c->d_dop[1] && c->d_dop[2];
+}
+
 // FP64 form with the derivatives as operator products: gradients to pairs, the
 // pointwise pass, then h += d_j F_j axis by axis, the last with FP64 out.  hpsi
 // holds L and the growing sum as pairs in between.
@@ -854,7 +859,7 @@ static sky_status apply_h_pair(Ctx* c, const double* U, const double* B, const d
 
 sky_status apply_h_impl(Ctx* c, const double* U, const double* B, const double* W,
                         const void* psi, void* hpsi, int I, double* eps, double* hn2) {
-  if (c->prec == SKY_F64 && c->line_arith == 2 && c->d_dop[0] && c->d_dop[1] && c->d_dop[2])
+  if (operator_route(c))
     return apply_h_pair(c, U, B, W, (const double2*)psi, (double2*)hpsi, I, eps, hn2);
   if (c->prec == SKY_F64)
     return apply_h_t<double>(c, U, B, W, (const double2*)psi, (double2*)hpsi, I, eps, hn2);
@@ -1009,6 +1014,85 @@ __global__ void __launch_bounds__(128) k_dens_accum(const cx<T>* __restrict__ ps
   dst[4 * G + p] = jz;
 }
 
+// A sum of products of pairs kept to about 2^-48 of its size: the product of the
+// high parts exactly (p + e), the cross products, both running parts by TwoSum.
+struct AccD {
+  float hi = 0.0f, mid = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add(dd a, dd b) {
+    const float p = __fmul_rn(a.hi, b.hi);
+    float e = __fmaf_rn(a.hi, b.hi, -p);
+    e = __fmaf_rn(a.hi, b.lo, e);
+    e = __fmaf_rn(a.lo, b.hi, e);
+    const dd s = two_sum(hi, p);
+    hi = s.hi;
+    const dd m = two_sum(mid, s.lo);
+    mid = m.hi;
+    lo = __fadd_rn(lo, __fadd_rn(m.lo, e));
+  }
+  // sign Re(conj(a) d) and sign Im(conj(a) d)
+  template <int SG> __device__ __forceinline__ void re_cj(ddc a, ddc d) {
+    add(SG > 0 ? a.x : -a.x, d.x);
+    add(SG > 0 ? a.y : -a.y, d.y);
+  }
+  template <int SG> __device__ __forceinline__ void im_cj(ddc a, ddc d) {
+    add(SG > 0 ? a.x : -a.x, d.y);
+    add(SG > 0 ? -a.y : a.y, d.x);
+  }
+  __device__ __forceinline__ double value() const { return ((double)hi + (double)mid) + (double)lo; }
+};
+
+// The same partial sums from gradients as float pairs (the FP64 form's operator
+// route): rho in FP64 from psi itself (four operations per state and point), tau
+// and J, whose gradients carry 48 bits, as sums of pair products on the FP32 pipe
+// (36 products; some 85 FP64 operations per state and point bound the pass
+// before: densities of 24^3, 280 states 889 us, now 464).
+__global__ void __launch_bounds__(128) k_dens_accum_pair(const double2* __restrict__ psi,
+                                                         const float4* __restrict__ g0,
+                                                         const float4* __restrict__ g1,
+                                                         const float4* __restrict__ g2, int G, int ns,
+                                                         int per_split, double* part) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= G) return;
+  const int s_beg = blockIdx.y * per_split;
+  const int s_end = (s_beg + per_split) < ns ? (s_beg + per_split) : ns;
+  double r[4] = {0.0, 0.0, 0.0, 0.0};
+  AccD ta, ax, ay, az;
+  auto pair = [](float4 v) { return ddc{dd(v.x, v.y), dd(v.z, v.w)}; };
+  for (int s = s_beg; s < s_end; ++s) {
+    const long long o0 = (long long)s * 2 * G + p, o1 = o0 + G;
+    const double2 b0 = psi[o0], b1 = psi[o1];
+    const float4 f[6] = {g0[o0], g0[o1], g1[o0], g1[o1], g2[o0], g2[o1]};
+    r[0] = fma(b0.x, b0.x, r[0]);
+    r[1] = fma(b0.y, b0.y, r[1]);
+    r[2] = fma(b1.x, b1.x, r[2]);
+    r[3] = fma(b1.y, b1.y, r[3]);
+    const ddc a0 = ddc_of(b0), a1 = ddc_of(b1);
+    const ddc x0 = pair(f[0]), x1 = pair(f[1]), y0 = pair(f[2]), y1 = pair(f[3]), z0 = pair(f[4]),
+              z1 = pair(f[5]);
+    ta.re_cj<1>(x0, x0);
+    ta.re_cj<1>(x1, x1);
+    ta.re_cj<1>(y0, y0);
+    ta.re_cj<1>(y1, y1);
+    ta.re_cj<1>(z0, z0);
+    ta.re_cj<1>(z1, z1);
+    // J_x = Im M_zy - Im M_yz
+    ax.im_cj<1>(a0, y0); ax.im_cj<-1>(a1, y1);
+    ax.re_cj<-1>(a1, z0); ax.re_cj<1>(a0, z1);
+    // J_y = Im M_xz - Im M_zx
+    ay.im_cj<1>(a0, z1); ay.im_cj<1>(a1, z0);
+    ay.im_cj<-1>(a0, x0); ay.im_cj<1>(a1, x1);
+    // J_z = Im M_yx - Im M_xy
+    az.re_cj<1>(a1, x0); az.re_cj<-1>(a0, x1);
+    az.im_cj<-1>(a0, y1); az.im_cj<-1>(a1, y0);
+  }
+  double* dst = part + (long long)blockIdx.y * 5 * G;
+  dst[p] = (r[0] + r[1]) + (r[2] + r[3]);
+  dst[G + p] = ta.value();
+  dst[2 * G + p] = ax.value();
+  dst[3 * G + p] = ay.value();
+  dst[4 * G + p] = az.value();
+}
+
 // Sum the splits in order; accumulate onto the outputs after the first chunk.
 __global__ void k_dens_reduce(const double* part, int nsplit, int G, int accumulate,
                               double* rho, double* tau, double* J) {
@@ -1045,12 +1129,25 @@ static sky_status densities_t(Ctx* c, const cx<T>* psi, int I, double* rho, doub
   for (int s0 = 0; s0 < I; s0 += c->chunk) {
     const int ns = (I - s0) < c->chunk ? (I - s0) : c->chunk;
     const cx<T>* ps = psi + (long long)s0 * V;
-    cudaError_t e = gradient_passes<T>(c, ps, g, 2LL * ns);
-    if (e != cudaSuccess) return cuda_check(c, e, "densities gradient");
     const int per = (ns + kDensSplits - 1) / kDensSplits;
     const int nsplit = (ns + per - 1) / per;
     dim3 grid(div_up(G, 128), nsplit);
-    k_dens_accum<T><<<grid, 128, 0, c->stream>>>(ps, g[0], g[1], g[2], (int)G, ns, per, c->d_dpart); note_launch();
+    bool pairs = false;
+    if constexpr (std::is_same<T, double>::value) pairs = operator_route(c);
+    cudaError_t e = cudaSuccess;
+    if (pairs) {
+      for (int ax = 0; ax < 3 && e == cudaSuccess; ++ax)
+        e = deriv_tc_pair(c, ax, (const double2*)ps, g[ax], 2LL * ns);
+      if (e != cudaSuccess) return cuda_check(c, e, "densities gradient");
+      k_dens_accum_pair<<<grid, 128, 0, c->stream>>>((const double2*)ps, (const float4*)g[0],
+                                                     (const float4*)g[1], (const float4*)g[2], (int)G,
+                                                     ns, per, c->d_dpart);
+    } else {
+      e = gradient_passes<T>(c, ps, g, 2LL * ns);
+      if (e != cudaSuccess) return cuda_check(c, e, "densities gradient");
+      k_dens_accum<T><<<grid, 128, 0, c->stream>>>(ps, g[0], g[1], g[2], (int)G, ns, per, c->d_dpart);
+    }
+    note_launch();
     k_dens_reduce<<<div_up(G, 256), 256, 0, c->stream>>>(c->d_dpart, nsplit, (int)G, s0 > 0, rho,
                                                          tau, Jout); note_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_check(c, e, "densities accumulate");
