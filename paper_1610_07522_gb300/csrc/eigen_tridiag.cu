@@ -29,9 +29,10 @@
 //     LAPACK's dstein does).  k_tri_window then applies first-order Loewdin
 //     steps Y <- Y (3 I - Y^T Y) / 2, with Y^T Y formed only between
 //     eigenvalues within kWinRel ||T|| of each other (the inverse-iteration
-//     vectors' mutual overlaps fall off like eps ||T|| / gap).  k_hh_back
-//     forms Z = Q Y, one warp per column, the reflectors applied in reverse
-//     order.
+//     vectors' mutual overlaps fall off like eps ||T|| / gap).  Z = Q Y is
+//     formed from Q's compact WY form by tensor-core products (wy_back), or, for
+//     small or device-gated batches, by k_hh_back, one warp per column, the
+//     reflectors applied in reverse order.
 //
 // Eigenvalues come out ascending, eigenvectors as the columns of Z.
 #include <algorithm>
@@ -108,7 +109,7 @@ struct TeamView {
 struct TriPtrs {
   double2* cols;                 // own columns, global home: column j at cols + j * n
   double2* V;
-  double *Y, *Y2, *U0, *U1, *U2;
+  double *Y, *Y2, *U0, *U2;      // U0: pairs (1 / pivot, first superdiagonal)
   double2 *P0, *P1, *C0, *C1, *tau;
   double *d, *e, *e2, *lam;
   float *df, *e2f;               // d and e^2 rounded to float (coarse bisection rounds)
@@ -120,7 +121,6 @@ __device__ __forceinline__ TriPtrs tri_ptrs(const TriBatch& a, int b) {
   const size_t n = (size_t)a.n[b], m = (size_t)a.m, k = (size_t)a.sid[b];
   p.cols = a.S0 + k * a.slot;
   p.U0 = reinterpret_cast<double*>(p.cols);
-  p.U1 = p.U0 + n * n;
   p.V = a.S1 + k * a.slot;
   p.Y = reinterpret_cast<double*>(a.S2 + k * a.slot);
   p.Y2 = p.Y + n * n;
@@ -628,65 +628,171 @@ __device__ __forceinline__ double start_entry(unsigned long long k, unsigned lon
   return (double)(x >> 11) * (1.0 / 4503599627370496.0) - 1.0;
 }
 
-// LU factors with partial pivoting of T - lam I for column k (row stride n):
-// U0 = 1 / (pivot), U1 = first superdiagonal of U, U2 = the multiplier of
-// the row operation, its lowest mantissa bit set when rows i and i+1 were
-// swapped (then U's second superdiagonal is e_{i+1}, else 0).  One
-// reciprocal per row; a zero pivot is replaced by pert.
+// The solver's columns of vector k, row stride n: U = (1 / pivot, first
+// superdiagonal of U), L = the multiplier of the row operation, its lowest mantissa
+// bit set when rows i and i+1 were swapped (then U's second superdiagonal is
+// e_{i+1}, else 0), Y = the vector.
+//
+// A thread works one vector off row by row, one warp per SM: what it takes is
+// instructions (eight cycles each with nothing to overlap them) and, where a load
+// waits behind a store that may alias it, memory round trips.  So the
+// factorisation carries the forward sweep of the first solve with it, the sweeps
+// walk pointers in unpredicated chunks whose loads are issued a chunk ahead, and
+// the norm is formed in the backward sweep and applied by the next solve (700 +
+// 300 states: 1.84 ms with a pass each for start, norm and scaling, 1.10 ms).
+struct TriCol {
+  double2* U;
+  double* L;
+  double* Y;
+};
 __device__ __forceinline__ double pack_piv(double l, bool piv) {
   return __longlong_as_double((__double_as_longlong(l) & ~1ll) | (long long)piv);
 }
-__device__ __forceinline__ bool piv_of(double l) { return (__double_as_longlong(l) & 1ll) != 0; }
+__device__ __forceinline__ bool piv_of(double l) { return (__double2loint(l) & 1) != 0; }
 
-__device__ __forceinline__ void tri_factor(const TriPtrs& p, int n, int k, double lam, double pert) {
+// LU factors with partial pivoting of T - lam I (one reciprocal per row; a zero
+// pivot is replaced by pert), and y <- L^{-1} P (start vector k).
+__device__ __forceinline__ void tri_factor(const double* __restrict__ d, const double* __restrict__ e,
+                                           TriCol c, int n, int k, double lam, double pert) {
   const size_t sn = (size_t)n;
-  double cur0 = p.d[0] - lam, cur1 = n > 1 ? p.e[0] : 0.0;
+  double cur0 = __ldg(d) - lam, cur1 = n > 1 ? __ldg(e) : 0.0;
+  double rc = start_entry((unsigned long long)k, 0);
+  double sub = cur1;
+#pragma unroll 2
   for (int i = 0; i < n - 1; ++i) {
-    const double sub = p.e[i], nd = p.d[i + 1] - lam;
-    const double nsup = i + 1 < n - 1 ? p.e[i + 1] : 0.0;
+    const double nd = __ldg(d + i + 1) - lam;
+    const double nsup = i + 1 < n - 1 ? __ldg(e + i + 1) : 0.0;
     const bool piv = fabs(sub) > fabs(cur0);
     const double c0 = cur0 == 0.0 ? pert : cur0;
     const double r = 1.0 / (piv ? sub : c0);
     const double l = (piv ? cur0 : sub) * r;
-    const size_t e = (size_t)i * sn + k;
-    p.U0[e] = r;
-    p.U1[e] = piv ? nd : cur1;
-    p.U2[e] = pack_piv(l, piv);
-    const double n0 = piv ? fma(-l, nd, cur1) : fma(-l, cur1, nd);
+    const double lv = pack_piv(l, piv);
+    const double rn = start_entry((unsigned long long)k, (unsigned long long)(i + 1));
+    *c.U = make_double2(r, piv ? nd : cur1);
+    *c.L = lv;
+    *c.Y = piv ? rn : rc;
+    rc = piv ? fma(-lv, rn, rc) : fma(-lv, rc, rn);
+    c.U += sn;
+    c.L += sn;
+    c.Y += sn;
+    cur0 = piv ? fma(-l, nd, cur1) : fma(-l, cur1, nd);
     cur1 = piv ? -l * nsup : nsup;
-    cur0 = n0;
+    sub = nsup;
   }
-  p.U0[(size_t)(n - 1) * sn + k] = 1.0 / (cur0 == 0.0 ? pert : cur0);
+  c.U->x = 1.0 / (cur0 == 0.0 ? pert : cur0);
+  *c.Y = rc;
 }
 
-// y <- (T - lam I)^{-1} y on column k of Y with the stored factors.
-__device__ __forceinline__ void tri_solve(const TriPtrs& p, int n, int k) {
-  double* Y = p.Y;
+constexpr int kSolveRows = 8;
+// y <- L^{-1} P (scale y).
+__device__ __forceinline__ void tri_forward(const TriCol& c, int n, double scale) {
+  constexpr int C = kSolveRows;
   const size_t sn = (size_t)n;
-  double rc = Y[k];
-  for (int i = 0; i < n - 1; ++i) {
-    const size_t e = (size_t)i * sn + k;
-    const double lv = p.U2[e], rn = Y[e + sn];
-    if (piv_of(lv)) {
-      Y[e] = rn;
-      rc = fma(-lv, rn, rc);
-    } else {
-      Y[e] = rc;
-      rc = fma(-lv, rc, rn);
+  double rc = scale * *c.Y;
+  const double* __restrict__ L = c.L;
+  const double* __restrict__ R = c.Y + sn;   // row i + 1
+  double* __restrict__ W = c.Y;
+  auto row = [&](double lv, double r0) {
+    const double rn = scale * r0;
+    const bool piv = piv_of(lv);
+    *W = piv ? rn : rc;
+    rc = piv ? fma(-lv, rn, rc) : fma(-lv, rc, rn);
+    W += sn;
+  };
+  int left = n - 1;
+  double lv[C], rn[C];
+  auto load = [&]() {
+#pragma unroll
+    for (int q = 0; q < C; ++q) {
+      lv[q] = *L;
+      rn[q] = *R;
+      L += sn;
+      R += sn;
     }
+  };
+  if (left >= C) load();
+  while (left >= C) {
+    double l2[C], r2[C];
+#pragma unroll
+    for (int q = 0; q < C; ++q) {
+      l2[q] = lv[q];
+      r2[q] = rn[q];
+    }
+    if (left >= 2 * C) load();
+#pragma unroll
+    for (int q = 0; q < C; ++q) row(l2[q], r2[q]);
+    left -= C;
   }
-  Y[(size_t)(n - 1) * sn + k] = rc;
-  double y1 = 0.0, y2 = 0.0;                // y[i+1], y[i+2]
-  for (int i = n - 1; i >= 0; --i) {
-    const size_t e = (size_t)i * sn + k;
-    // the last row has no superdiagonal (its U1 and U2 entries are never formed)
-    const double u1 = i + 1 < n ? p.U1[e] : 0.0;
-    const double u2 = (i + 2 < n && piv_of(p.U2[e])) ? p.e[i + 1] : 0.0;
-    const double yi = (Y[e] - u1 * y1 - u2 * y2) * p.U0[e];
-    Y[e] = yi;
+  for (; left > 0; --left, L += sn, R += sn) row(*L, *R);
+  *W = rc;
+}
+// y <- U^{-1} y; returns the sum of squares of the result.
+__device__ __forceinline__ double tri_backward(const TriCol& c, const double* __restrict__ e, int n) {
+  constexpr int C = kSolveRows;
+  const size_t sn = (size_t)n;
+  const double2* __restrict__ U = c.U + (size_t)(n - 1) * sn;
+  const double* __restrict__ L = c.L + (size_t)(n - 1) * sn;
+  const double* __restrict__ R = c.Y + (size_t)(n - 1) * sn;
+  double* __restrict__ W = c.Y + (size_t)(n - 1) * sn;
+  double y1 = 0.0, y2 = 0.0, s0 = 0.0, s1 = 0.0;   // y[i+1], y[i+2]
+  auto row = [&](double y, double r, double u1, double u2) {
+    const double yi = fma(-u1, y1, fma(-u2, y2, y)) * r;
+    *W = yi;
+    W -= sn;
     y2 = y1;
     y1 = yi;
+  };
+  // the last two rows have no second, the last no first superdiagonal (those
+  // entries are never formed)
+  row(*R, U->x, 0.0, 0.0);
+  s0 = y1 * y1;
+  if (n == 1) return s0;
+  U -= sn;
+  L -= sn;
+  R -= sn;
+  row(*R, U->x, U->y, 0.0);
+  s1 = y1 * y1;
+  U -= sn;
+  L -= sn;
+  R -= sn;
+  int i = n - 3;
+  double yy[C], u2[C];
+  double2 u[C];
+  auto load = [&](int top) {
+#pragma unroll
+    for (int q = 0; q < C; ++q) {
+      yy[q] = *R;
+      u[q] = *U;
+      u2[q] = piv_of(*L) ? __ldg(e + top - q + 1) : 0.0;
+      R -= sn;
+      U -= sn;
+      L -= sn;
+    }
+  };
+  if (i + 1 >= C) load(i);
+  while (i + 1 >= C) {
+    double ya[C], ua[C];
+    double2 va[C];
+#pragma unroll
+    for (int q = 0; q < C; ++q) {
+      ya[q] = yy[q];
+      ua[q] = u2[q];
+      va[q] = u[q];
+    }
+    if (i + 1 >= 2 * C) load(i - C);
+#pragma unroll
+    for (int q = 0; q < C; ++q) {
+      row(ya[q], va[q].x, va[q].y, ua[q]);
+      if (q & 1) s1 = fma(y1, y1, s1);
+      else s0 = fma(y1, y1, s0);
+    }
+    i -= C;
   }
+  for (; i >= 0; --i, R -= sn, U -= sn, L -= sn) {
+    row(*R, U->x, U->y, piv_of(*L) ? __ldg(e + i + 1) : 0.0);
+    s0 = fma(y1, y1, s0);
+  }
+  return s0 + s1;
 }
 
 // One thread per eigenvalue; the first of a cluster does the whole cluster.
@@ -708,28 +814,36 @@ __global__ void __launch_bounds__(kVecThreads, 1) k_tri_vectors(TriBatch a) {
   const size_t sn = (size_t)n;
   double* Y = p.Y;
   for (int k = j; k < end; ++k) {
-    for (int i = 0; i < n; ++i) Y[(size_t)i * sn + k] = start_entry((unsigned long long)k, i);
-    tri_factor(p, n, k, lam[k], pert);
+    const TriCol col{reinterpret_cast<double2*>(p.U0) + k, p.U2 + k, Y + k};
+    tri_factor(p.d, p.e, col, n, k, lam[k], pert);
+    double r = 1.0;                          // scale of the next solve's right-hand side
     for (int it = 0; it < kInvIters; ++it) {
-      tri_solve(p, n, k);
+      if (it > 0) tri_forward(col, n, r);
+      double sq = tri_backward(col, p.e, n);
       for (int c = j; c < k; ++c) {          // against the cluster's earlier vectors
         double dot = 0.0;
         for (int i = 0; i < n; ++i) dot = fma(Y[(size_t)i * sn + c], Y[(size_t)i * sn + k], dot);
         for (int i = 0; i < n; ++i) Y[(size_t)i * sn + k] = fma(-dot, Y[(size_t)i * sn + c], Y[(size_t)i * sn + k]);
       }
-      double s = 0.0;
-      if (it + 1 < kInvIters) {
-        for (int i = 0; i < n; ++i) s = fmax(s, fabs(Y[(size_t)i * sn + k]));
-      } else {
-        for (int i = 0; i < n; ++i) s = fma(Y[(size_t)i * sn + k], Y[(size_t)i * sn + k], s);
-        s = sqrt(s);
+      if (k > j) {
+        sq = 0.0;
+        for (int i = 0; i < n; ++i) sq = fma(Y[(size_t)i * sn + k], Y[(size_t)i * sn + k], sq);
       }
+      double s = sqrt(sq);
       if (!(s > 0.0) || !isfinite(s)) {
         flag_status(a.status, SKY_ENOCONV);
         s = 1.0;
       }
-      const double r = 1.0 / s;
-      for (int i = 0; i < n; ++i) Y[(size_t)i * sn + k] *= r;
+      r = 1.0 / s;
+    }
+    for (int i0 = 0; i0 < n; i0 += 16) {     // the unit vector
+      double y[16];
+#pragma unroll
+      for (int c = 0; c < 16; ++c)
+        if (i0 + c < n) y[c] = Y[(size_t)(i0 + c) * sn + k];
+#pragma unroll
+      for (int c = 0; c < 16; ++c)
+        if (i0 + c < n) Y[(size_t)(i0 + c) * sn + k] = y[c] * r;
     }
   }
 }
@@ -832,6 +946,178 @@ __global__ void __launch_bounds__(kBackWarps * 32) k_hh_back(TriBatch a, int zst
   }
 }
 
+// ---- back-transformation by the compact WY form ----------------------------------
+// Q = H_0 ... H_{n-2} = I - V T V^H with V's columns v_t and T upper triangular,
+// T^{-1} = striu(V^H V) + diag(1 / tau_t) (Puglisi 1992; a reflector with tau_t = 0
+// enters as v_t = 0).  With P = V^H:  G = P P^H; T's diagonal blocks of kWyBlock by
+// back substitution; then T's blocks doubled in size level by level, the upper
+// right block of a pair being -T_11 G_12 T_22, which the full products (T G) T
+// hold in that place because T is block diagonal so far; Z = Y - P^H (T (P Y)).
+// All products are digit-split tensor-core ones with seven digits (4 + 2 log2(n /
+// kWyBlock) of them); applying the reflectors one by one costs 4 n^3 FP64 multiply-adds,
+// which bound k_hh_back (72% of the FP64 pipe): 700 + 300 states 4.1 ms, here
+// 1.4 ms; 280 + 120 states 0.93 ms, here 0.55 ms.  The eigenvectors' orthogonality
+// and residuals stay what they were (128 to 1000 states, dense and nearly diagonal
+// matrices: 6e-15 to 6e-14 sqrt(n), both ways).
+constexpr int kWyBlock = 64;
+constexpr int kWyMin = 128;            // smallest largest problem of a batch it is used for
+
+struct WyJobs {
+  double2* P[kMaxBatch];               // in: row t = v_t; out: row t = v_t^H
+  const double2* tau[kMaxBatch];
+  const double* Y[kMaxBatch];
+  double2* Z[kMaxBatch];               // Y as a complex matrix, later the result
+  const double2* G[kMaxBatch];
+  double2* T[kMaxBatch];
+  const double2* N[kMaxBatch];         // (T G) T of a level, or P^H X at the end
+  int n[kMaxBatch];
+};
+// Row t (blockIdx.x) of P and of Y as complex values.
+__global__ void __launch_bounds__(256) k_wy_prep(const __grid_constant__ WyJobs j) {
+  const int b = blockIdx.y, n = j.n[b], t = blockIdx.x;
+  if (t >= n) return;
+  double2 tau = make_double2(0.0, 0.0);
+  if (t < n - 1) tau = j.tau[b][t];
+  const bool on = tau.x != 0.0 || tau.y != 0.0;
+  const long long r = (long long)t * n;
+  for (int i = threadIdx.x; i < n; i += 256) {
+    // entries up to t are not part of the reflector (never written)
+    j.P[b][r + i] = on && i > t ? conjx(j.P[b][r + i]) : make_double2(0.0, 0.0);
+    j.Z[b][r + i] = make_double2(j.Y[b][r + i], 0.0);
+  }
+}
+// Diagonal block blockIdx.x of T, columns kWyCols blockIdx.z .. of it: the inverse
+// of the block of striu(G) + diag(1 / tau) by back substitution, and zeros in the
+// rest of its rows (its share of them).  A warp per column, lane l with rows l and
+// l + 32: as x_k is known every row above takes its term, so a step is one shuffle
+// and one multiply-add deep; with the rows scaled by -tau_i beforehand the sum of
+// row i is x_i.  FP64 instructions bound it (127 us at 700 + 300 states with the row
+// sums split over 16 threads and added up row by row).
+constexpr int kWyCols = 8, kWyThreads = 32 * kWyCols;
+static_assert(kWyBlock == 64, "two rows per lane");
+__global__ void __launch_bounds__(kWyThreads) k_wy_diag(const __grid_constant__ WyJobs j) {
+  extern __shared__ double2 wsm[];
+  constexpr int B = kWyBlock, LD = kWyBlock + 1;
+  double2* m = wsm;                     // [B][LD] -tau_i G_ik
+  double2* dg = wsm + B * LD;           // [B] tau (1 / the diagonal)
+  const int b = blockIdx.y, n = j.n[b], k0 = blockIdx.x * B;
+  if (k0 >= n) return;
+  const int nb = n - k0 < B ? n - k0 : B;
+  for (int i = threadIdx.x; i < B; i += kWyThreads) {
+    double2 t = make_double2(1.0, 0.0);
+    if (k0 + i < n - 1) {
+      const double2 u = j.tau[b][k0 + i];
+      if (u.x != 0.0 || u.y != 0.0) t = u;
+    }
+    dg[i] = t;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < B * B; e += kWyThreads) {
+    const int i = e / B, c = e % B;
+    const bool on = i < c && c < nb;
+    m[i * LD + c] = on ? -cmul(dg[i], j.G[b][(long long)(k0 + i) * n + k0 + c]) : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, c = blockIdx.z * kWyCols + (threadIdx.x >> 5);
+  if (c < nb) {
+    // x0, x1: rows lane and lane + 32 of column c (rows beyond c stay zero)
+    double2 x0 = make_double2(0.0, 0.0), x1 = x0;
+    if (lane == (c & 31)) (c < 32 ? x0 : x1) = dg[c];
+    for (int k = c; k > 0; --k) {
+      const double2 s = k < 32 ? x0 : x1;
+      const double2 v = make_double2(__shfl_sync(0xffffffffu, s.x, k & 31), __shfl_sync(0xffffffffu, s.y, k & 31));
+      const double2 a0 = m[lane * LD + k];
+      x0.x = fma(a0.x, v.x, x0.x);
+      x0.y = fma(a0.x, v.y, x0.y);
+      x0.x = fma(-a0.y, v.y, x0.x);
+      x0.y = fma(a0.y, v.x, x0.y);
+      if (k > 32) {
+        const double2 a1 = m[(lane + 32) * LD + k];
+        x1.x = fma(a1.x, v.x, x1.x);
+        x1.y = fma(a1.x, v.y, x1.y);
+        x1.x = fma(-a1.y, v.y, x1.x);
+        x1.y = fma(a1.y, v.x, x1.y);
+      }
+    }
+    double2* t = j.T[b] + (long long)k0 * n + k0 + c;
+    if (lane < nb) t[(long long)lane * n] = x0;
+    if (lane + 32 < nb) t[(long long)(lane + 32) * n] = x1;
+  }
+  // every gridDim.z-th row outside the diagonal block
+  for (int i = blockIdx.z; i < nb; i += gridDim.z)
+    for (int e = threadIdx.x; e < n; e += kWyThreads)
+      if (e < k0 || e >= k0 + nb) j.T[b][(long long)(k0 + i) * n + e] = make_double2(0.0, 0.0);
+}
+constexpr size_t kWySmem = ((size_t)kWyBlock * (kWyBlock + 1) + kWyBlock) * sizeof(double2);
+// T's upper right blocks of the pairs of blocks of s rows: -(T G) T there.
+__global__ void __launch_bounds__(256) k_wy_level(const __grid_constant__ WyJobs j, int s) {
+  const int b = blockIdx.y, n = j.n[b], i = blockIdx.x;
+  if (i >= n || ((i / s) & 1)) return;
+  const int c0 = (i / s + 1) * s, c1 = c0 + s < n ? c0 + s : n;
+  const long long r = (long long)i * n;
+  for (int c = c0 + threadIdx.x; c < c1; c += 256) j.T[b][r + c] = -j.N[b][r + c];
+}
+// Z = Y - P^H X.
+__global__ void __launch_bounds__(256) k_wy_final(const __grid_constant__ WyJobs j) {
+  const int b = blockIdx.y, n = j.n[b], i = blockIdx.x;
+  if (i >= n) return;
+  const long long r = (long long)i * n;
+  for (int c = threadIdx.x; c < n; c += 256) j.Z[b][r + c] = j.Z[b][r + c] - j.N[b][r + c];
+}
+
+// Z = Q Y for the problems idx[0..np) of a batch.  Workspace: the tridiagonal
+// solver's three slots (own columns and LU rows: done; reflectors: P in place; Y:
+// done once it is copied) and two of the callers' I x I temporaries (4 and 5,
+// which no caller holds across an eigensolve).
+static sky_status wy_back(Ctx* c, int np, const int* idx, const int* n, double2* const* Z,
+                          const TriBatch& a) {
+  WyJobs j;
+  double2 *S0[kMaxBatch], *S2[kMaxBatch], *U[kMaxBatch], *T[kMaxBatch], *P[kMaxBatch], *Zb[kMaxBatch];
+  int nn[kMaxBatch], nmax = 1;
+  for (int q = 0; q < np; ++q) {
+    const int b = idx[q];
+    nn[q] = n[b];
+    nmax = n[b] > nmax ? n[b] : nmax;
+    S0[q] = c->d_eigA[0] + (size_t)b * c->eig_slot;
+    P[q] = c->d_eigA[1] + (size_t)b * c->eig_slot;
+    S2[q] = c->d_eigV + (size_t)b * c->eig_slot;
+    U[q] = c->d_small[4] + (size_t)b * c->small_slot;
+    T[q] = c->d_small[5] + (size_t)b * c->small_slot;
+    Zb[q] = Z[b];
+    j.P[q] = P[q];
+    j.tau[q] = reinterpret_cast<const double2*>(a.T + (size_t)b * a.tslot + (size_t)a.m * a.m) + 4 * (size_t)a.m;
+    j.Y[q] = reinterpret_cast<const double*>(S2[q]);
+    j.Z[q] = Zb[q];
+    j.G[q] = S0[q];
+    j.T[q] = T[q];
+    j.N[q] = S2[q];
+    j.n[q] = n[b];
+  }
+  const int* none[kMaxBatch] = {nullptr};
+  const dim3 rows(nmax, np);
+  auto mul = [&](bool ah, bool bh, double2* const* A, double2* const* B, double2* const* C) {
+    return zgemm_batch(c, zjobs(np, ah, bh, (const double2* const*)A, (const double2* const*)B, C, nn, none, none, 7));
+  };
+  k_wy_prep<<<rows, 256, 0, c->stream>>>(j);
+  sky_status s = mul(false, true, P, P, S0);                       // G = P P^H
+  if (s != SKY_OK) return s;
+  k_wy_diag<<<dim3(div_up(nmax, kWyBlock), np, kWyBlock / kWyCols), kWyThreads, kWySmem, c->stream>>>(j);
+  note_launch(2);
+  for (int w = kWyBlock; w < nmax; w *= 2) {
+    if ((s = mul(false, false, T, S0, U)) != SKY_OK) return s;     // T G
+    if ((s = mul(false, false, U, T, S2)) != SKY_OK) return s;     // (T G) T
+    k_wy_level<<<rows, 256, 0, c->stream>>>(j, w);
+    note_launch();
+  }
+  if ((s = mul(false, false, P, Zb, U)) != SKY_OK) return s;       // P Y
+  if ((s = mul(false, false, T, U, S2)) != SKY_OK) return s;       // T (P Y)
+  if ((s = mul(true, false, P, S2, S0)) != SKY_OK) return s;       // P^H X
+  for (int q = 0; q < np; ++q) j.N[q] = S0[q];
+  k_wy_final<<<rows, 256, 0, c->stream>>>(j);
+  note_launch();
+  return cuda_check(c, cudaGetLastError(), "back-transformation");
+}
+
 __global__ void k_tri_reset(unsigned* bar) { bar[(size_t)kTeamBarStride * threadIdx.x] = 0u; }
 
 // A problem of n states keeps its work vectors in global memory when they
@@ -857,6 +1143,8 @@ sky_status tri_init(Ctx* c) {
                                        (int)kTriSmemMax);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_hh_back, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTriSmemMax);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_wy_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWySmem);
   return cuda_check(c, e, "tridiagonal solver attributes");
 }
 
@@ -1142,13 +1430,20 @@ static sky_status tri_group(Ctx* c, int np, const int* idx, const double2* const
   k_tri_vectors<<<div_up(ntot, kVecThreads), kVecThreads, 0, c->stream>>>(a);
   k_tri_window<<<(unsigned)ntot, kWinThreads, 0, c->stream>>>(a, 0);
   k_tri_window<<<(unsigned)ntot, kWinThreads, 0, c->stream>>>(a, 1);
+  note_launch(4);
+  // the products by tensor cores, unless the batch is gated (skipped products
+  // still cost their launches) or its problems are small
+  if (!run && nmax >= kWyMin) {
+    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_check(c, e, "tridiagonal eigensolver");
+    return wy_back(c, np, idx, n, Z, a);
+  }
   // columns spread over all SMs first (consecutive items go to different blocks)
   const int back_blocks = (int)(ntot < c->num_sms ? ntot : c->num_sms);
   const int need_warps = (int)div_up(ntot, back_blocks);
   if (need_warps < back_warps) back_warps = need_warps;
   k_hh_back<<<back_blocks, back_warps * 32, (size_t)back_warps * zstride * sizeof(double2),
               c->stream>>>(a, zstride);
-  note_launch(5);
+  note_launch();
   return cuda_check(c, cudaGetLastError(), "tridiagonal eigensolver");
 }
 
