@@ -814,9 +814,27 @@ sky_status lowdin_batch(Ctx* c, int np, const double2* const* S, const int* I, d
       return st;                                                             // W = Z Y
     k_ns_step<<<dim3(step_blocks, np), 256, 0, c->stream>>>(j, gate, c->d_stats, it == 0);
     note_launch();
-    st = zgemm_batch(c, zjobs(np, false, false, Y0, (const double2* const*)j.W, Y1, I, run, none));   // Y T
-    if (st == SKY_OK && it > 0)
-      st = zgemm_batch(c, zjobs(np, false, false, (const double2* const*)j.W, Z0, Z1, I, run, none));   // T Z
+    // Y T and T Z: independent, so one batch of 2 np products where it fits
+    const int nj = it > 0 ? 2 * np : np;
+    if (nj <= kMaxBatch) {
+      const double2 *Aj[kMaxBatch], *Bj[kMaxBatch];
+      double2* Cj[kMaxBatch];
+      const int* rj[kMaxBatch];
+      int Ij[kMaxBatch];
+      for (int b = 0; b < nj; ++b) {
+        const int k = b < np ? b : b - np;
+        Aj[b] = b < np ? Y0[k] : j.W[k];
+        Bj[b] = b < np ? j.W[k] : Z0[k];
+        Cj[b] = b < np ? Y1[k] : Z1[k];
+        rj[b] = run[k];
+        Ij[b] = I[k];
+      }
+      st = zgemm_batch(c, zjobs(nj, false, false, Aj, Bj, Cj, Ij, rj, none));
+    } else {
+      st = zgemm_batch(c, zjobs(np, false, false, Y0, (const double2* const*)j.W, Y1, I, run, none));
+      if (st == SKY_OK && it > 0)
+        st = zgemm_batch(c, zjobs(np, false, false, (const double2* const*)j.W, Z0, Z1, I, run, none));
+    }
     if (st != SKY_OK) return st;
   }
   k_ns_final<<<dim3(div_up(nn, 256), np), 256, 0, c->stream>>>(j, gate, c->d_stats);

@@ -183,9 +183,10 @@ sky_status rotate_impl(Ctx* c, const void* phi, const double2* M, int I, void* o
 // *run[b] != 0, and stop[b] is null or *stop[b] == 0 (device-side gating, so a
 // fixed launch sequence can skip work the device decided is not needed).
 ZJobs zjobs(int np, bool ah, bool bh, const double2* const* A, const double2* const* B,
-            double2* const* C, const int* n, const int* const* run, const int* const* stop) {
+            double2* const* C, const int* n, const int* const* run, const int* const* stop,
+            int slices) {
   ZJobs j;
-  j.np = np; j.ah = ah; j.bh = bh;
+  j.np = np; j.ah = ah; j.bh = bh; j.slices = slices;
   for (int b = 0; b < kMaxBatch; ++b) {
     const bool in = b < np;
     j.A[b] = in ? A[b] : nullptr;
@@ -279,17 +280,23 @@ static void launch_zgemm(Ctx* c, const ZJobs& j, int nmax) {
 }
 
 sky_status zgemm_batch(Ctx* c, const ZJobs& jin) {
-  // a batch of many problems: every product in one grouped tensor-core launch
-  // sequence (oz_zgemm_group), when its buffers hold them
-  if (jin.np > kOzGroupMin && oz_zgemm_group_fits(c, jin.np, jin.n)) return oz_zgemm_group(c, jin);
+  // several problems: every product in one grouped tensor-core launch sequence
+  // (oz_zgemm_group), when its buffers hold them.  Up to kOzGroupMin problems
+  // only when one has kOzZgemmMin states or more: four launches for all (280 +
+  // 120 states: 25 us) instead of four for each large one and an FP64 launch for
+  // the rest (21 + 75 us); batches of small problems stay with the one FP64 launch
+  int nbig = 0;
+  for (int b = 0; b < jin.np; ++b) nbig = jin.n[b] > nbig ? jin.n[b] : nbig;
+  if (jin.np > 1 && (jin.np > kOzGroupMin || nbig >= kOzZgemmMin) && oz_zgemm_group_fits(c, jin.np, jin.n, jin.slices))
+    return oz_zgemm_group(c, jin);
   // problems of kOzZgemmMin states or more: tensor-core digit-split products
   // (one launch sequence each, gated like the rest); the others in one
   // batched FP64 launch
   ZJobs j = jin;
   for (int b = 0; b < j.np; ++b) {
     const bool gated = j.run[b] || j.stop[b];
-    if (j.n[b] >= (gated ? kOzZgemmGated : kOzZgemmMin) && oz_zgemm_fits(c, j.n[b])) {
-      const sky_status s = oz_zgemm(c, j.ah, j.bh, j.A[b], j.B[b], j.C[b], j.n[b], j.run[b], j.stop[b]);
+    if (j.n[b] >= (gated ? kOzZgemmGated : kOzZgemmMin) && oz_zgemm_fits(c, j.n[b], j.slices)) {
+      const sky_status s = oz_zgemm(c, j.ah, j.bh, j.A[b], j.B[b], j.C[b], j.n[b], j.run[b], j.stop[b], j.slices);
       if (s != SKY_OK) return s;
       j.n[b] = 0;
     }

@@ -25,7 +25,10 @@
 // it, then the other, and the next block starts with that other set, so a
 // drain has the products of two half blocks to hide behind.  The drained exact
 // sums are added, scaled by 2^{-8g}, into an unevaluated FP32 pair (hi, lo)
-// per output element by error-free TwoSum (about 48 significant bits).
+// per output element (about 48 significant bits): groups 0 .. 3 by error-free
+// TwoSum, groups 4 and 5, which lie below hi's last bit, straight into lo.  With
+// seven slices a third sum takes what lo drops, and the partial results keep all
+// three (a pair's own rounding, 2^-49, is 16 times that of FP64).
 // What bounds it: shared memory.  Per 16 values of K the MMAs read 9 x 4 + 21 x
 // 2.5 KiB of operands against 840 cycles on the tensor pipe, and the copies write
 // 39 KiB: about 1000 cycles at 128 bytes per clock.  24^3, 280 states, one
@@ -75,10 +78,12 @@ using tc::smem_u32;
 
 constexpr int BM = 128;
 constexpr int BK = 32;                    // bf16 K block: one 64-byte swizzle row
-constexpr int kSegKB = 4;                 // K blocks per exact segment (128 values)
+// K blocks per exact segment: 128 values for S <= 6; with seven slices group 6
+// reaches 9 x 2^14 per value, so 96
+__host__ __device__ constexpr int seg_kb(int S) { return S <= 6 ? 4 : 3; }
 constexpr int kEpiWarps = 8;
 constexpr int THREADS = 64 + 32 * kEpiWarps;
-constexpr int kMaxS = 6;
+constexpr int kMaxS = 7;
 constexpr int kMaxStages = 4;
 constexpr int kSmemMax = 232448;          // dynamic shared memory opt-in limit per CTA
 constexpr int kSmemExtra = 1024 + 256;    // alignment slack + barriers
@@ -88,6 +93,26 @@ constexpr int TILE_A = BM * BK * 2;       // 8 KiB per A slice tile
 // columns of TMEM <= 512).
 constexpr int kS64 = 6, kBN64 = 80;
 constexpr int kS32 = 4, kBN32 = 96;
+// Seven slices hold a double's 53 bits whole; with them the products of weight 7
+// count too (the last of two sets of four groups).  For the back-transformation of
+// the eigensolver, whose reflectors' entries spread far below their largest one:
+// the orthogonality it leaves at 700 states (Frobenius norm over sqrt(n)) is 1e-12
+// with six slices, 3e-14 with seven and float-pair sums, 7.1e-15 as it is and
+// 7.1e-15 with the reflectors applied in FP64.
+constexpr int kS7 = 7, kBN7 = 64;
+__host__ __device__ constexpr int num_groups(int S) { return S == kMaxS ? S + 1 : S; }
+// Float pairs of a partial result: (hi, lo), with seven slices (hi, lo), (tail, 0).
+__host__ __device__ constexpr int part_width(int S) { return S == kMaxS ? 2 : 1; }
+template <int S>
+__device__ __forceinline__ double part_value(const float2* row, int c) {
+  if constexpr (S == kMaxS) {
+    const float4 r = reinterpret_cast<const float4*>(row)[c];
+    return (double)r.x + ((double)r.y + (double)r.z);
+  } else {
+    const float2 r = row[c];
+    return (double)r.x + (double)r.y;
+  }
+}
 
 // Element (row, k) of slice s of an operand of nt row tiles of BNT rows (2-byte
 // elements); eight consecutive k from a multiple of 8 are consecutive.
@@ -148,24 +173,25 @@ __device__ __forceinline__ void tmem_ld<32>(uint32_t taddr, uint32_t* r) {
         "=r"(r[31])
       : "r"(taddr));
 }
-// Columns [0, NC) of a warp's share, NC = 40 or 48, as 32 + 8 or 32 + 16
+// Columns [0, NC) of a warp's share, NC = 32, 40 or 48, as 32, 32 + 8 or 32 + 16
 // (complete after tmem_wait).
 template <int NC>
 __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t* r) {
-  static_assert(NC == 40 || NC == 48, "column share");
+  static_assert(NC == 32 || NC == 40 || NC == 48, "column share");
   tmem_ld<32>(taddr, r);
-  tmem_ld<NC - 32>(taddr + 32, r + 32);
+  if constexpr (NC > 32) tmem_ld<NC - 32>(taddr + 32, r + 32);
 }
 __device__ __forceinline__ void tmem_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
 // The segment of set h (0: L, 1: H) ends after K block j (of nkb in the item):
-// every kSegKB blocks, H two blocks after L, and at the item's last block.
+// every SEG blocks, L after the second and H after the last of them, and at the
+// item's last block.
+template <int SEG>
 __device__ __forceinline__ bool flush_at(int j, int h, int nkb) {
-  return j == nkb - 1 || (j & (kSegKB - 1)) == (h ? 3 : 1);
+  return j == nkb - 1 || j % SEG == (h ? SEG - 1 : 1);
 }
-static_assert(kSegKB == 4, "segment schedule");
 
 // One lane of a converged warp, as a flag (the same lane at every use of it).
 __device__ __forceinline__ uint32_t elect_one() {
@@ -207,7 +233,7 @@ struct OzArgs {
   int I;
   int ntiles;               // output tiles in use (pruned when tri)
   int mode;                 // 0: (hi, lo) partials; 1: scaled final output
-  float2* P;                // mode 0: P[z][m][n], row stride ldp, split stride sp
+  float2* P;                // mode 0: P[z][m][n], row stride ldp, split stride sp (float2s)
   long long ldp, sp;
   void* out;                // mode 1: out[m][n] (double, or float when out_f32), row stride ldo
   long long ldo;
@@ -358,16 +384,28 @@ __device__ __forceinline__ void oz_gemm_body(const OzArgs& a, const OzGroup* grp
                              ? (kSmemMax - kSmemExtra) / STAGE
                              : kMaxStages;
   static_assert(STAGES >= 2, "ring");
-  static_assert(S * BNT <= 512, "TMEM");
+  constexpr int NG = num_groups(S);
+  static_assert(NG * BNT <= 512, "TMEM");
   static_assert(TILE_B % 1024 == 0, "swizzle alignment");
   constexpr uint32_t TMEM_COLS = 512;
   constexpr int HALF = BNT / 2;
   unsigned long long* bars = (unsigned long long*)(base + STAGES * STAGE);
   uint32_t* tmem_slot = (uint32_t*)(bars + 2 * kMaxStages + 2 * kMaxS + 1);
-  constexpr int HS = S / 2;                 // groups per set
-  static_assert(S % 2 == 0 && HS * BNT <= 256 && HS <= 3, "sets of groups");
+  constexpr int HS = NG / 2;                // groups of set L; H has the rest
+  constexpr int SEG = seg_kb(S);
+  static_assert((NG - HS) * BNT <= 256 && HS >= 2 && NG - HS <= 4, "sets of groups");
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int nitems = GROUP ? grp->tile0[grp->np] : a.ntiles * a.nsplit;
+  // items of this CTA: every second round in reverse, so that the CTAs whose last
+  // item was a short one (the later problems of a group) take the next first;
+  // -1 at the end
+  auto item_index = [&](int w) {
+    const int g = (int)gridDim.x, b = (int)blockIdx.x;
+    const long long first = (long long)w * g;
+    if (first >= nitems) return -1;
+    const int t = (int)first + ((w & 1) ? g - 1 - b : b);
+    return t < nitems ? t : -1;
+  };
   const uint32_t bar0 = smem_u32(bars);
   auto full = [&](int s) { return bar0 + 8u * s; };
   auto empty = [&](int s) { return bar0 + 8u * (kMaxStages + s); };
@@ -407,7 +445,7 @@ __device__ __forceinline__ void oz_gemm_body(const OzArgs& a, const OzGroup* grp
     static_assert(3 * S <= 32 && 2 * BNT >= BM, "runs of A");
     long long g = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < nitems && ok; t += gridDim.x) {
+    for (int w = 0, t; (t = item_index(w)) >= 0 && ok; ++w) {
       OzItem it;
       if (!item_at<GROUP>(a, grp, BNT, t, it)) continue;
       const int end = it.m0 + BM < it.nta * BNT ? it.m0 + BM : it.nta * BNT;   // rows that exist
@@ -443,7 +481,7 @@ __device__ __forceinline__ void oz_gemm_body(const OzArgs& a, const OzGroup* grp
     uint32_t nfl[2] = {0u, 0u};
     long long gpos = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < nitems && ok; t += gridDim.x) {
+    for (int w = 0, t; (t = item_index(w)) >= 0 && ok; ++w) {
       OzItem it;
       if (!item_at<GROUP>(a, grp, BNT, t, it)) continue;
       const int nkb = it.nkb;
@@ -460,8 +498,8 @@ __device__ __forceinline__ void oz_gemm_body(const OzArgs& a, const OzGroup* grp
         const uint32_t lb = sw64_lo(smem_u32(base + s * STAGE + S * TILE_A));
 #pragma unroll
         for (int o = 0; o < 2; ++o) {
-          const int h = (j & 2) ? 1 - o : o;     // the set whose segment may end here first
-          const bool start = j == 0 || flush_at(j - 1, h, nkb);
+          const int h = j % SEG >= 2 ? 1 - o : o;     // the set whose segment may end here first
+          const bool start = j == 0 || flush_at<SEG>(j - 1, h, nkb);
           if (start && nfl[h] > 0) {
             // the epilogue must have drained this set's previous segment
             if (!mbar_wait_warp(acc_empty(h), (nfl[h] - 1) & 1)) {
@@ -474,8 +512,11 @@ __device__ __forceinline__ void oz_gemm_body(const OzArgs& a, const OzGroup* grp
           auto issue = [&](auto hc) {
             constexpr int H = decltype(hc)::value;
 #pragma unroll
-            for (int p = 0; p < (H ? S : HS); ++p) {
-              constexpr int top = H ? S : HS;
+            for (int i = 0; i < (H ? S : HS); ++i) {
+              // the first MMA of a segment sets every group of its set, so with a
+              // group beyond S slice 1 of A goes first
+              const int p = H && NG > S && i < 2 ? 1 - i : i;
+              const int top = !H ? HS : p + S < NG ? p + S : NG;
               const int g0 = H && p < HS ? HS : p;         // first group
               const int q0 = g0 - p;                        // first slice of B
               const uint32_t idesc = idesc_bf16(BM, (top - g0) * BNT);
@@ -483,12 +524,12 @@ __device__ __forceinline__ void oz_gemm_body(const OzArgs& a, const OzGroup* grp
               for (int k = 0; k < BK / 16; ++k)   // +32 bytes along K = +2 in the encoded address
                 mma_bf16_elect(tmem + (uint32_t)(g0 * BNT), la + (uint32_t)(p * (TILE_A >> 4) + 2 * k),
                                lb + (uint32_t)(q0 * (TILE_B >> 4) + 2 * k), kSw64Hi, idesc,
-                               (start && p == 0 && k == 0) ? 0u : 1u, el);
+                               (start && i == 0 && k == 0) ? 0u : 1u, el);
             }
           };
           if (h) issue(std::integral_constant<int, 1>{});
           else issue(std::integral_constant<int, 0>{});
-          if (flush_at(j, h, nkb)) {
+          if (flush_at<SEG>(j, h, nkb)) {
             mma_commit_elect(acc_full(h), el);   // arrives when this set's MMAs have completed
             ++nfl[h];
           }
@@ -511,17 +552,22 @@ __device__ __forceinline__ void oz_gemm_body(const OzArgs& a, const OzGroup* grp
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty(h)) : "memory");
     };
     bool ok = true;
-    for (int t = blockIdx.x; t < nitems && ok; t += gridDim.x) {
+    for (int w = 0, t; (t = item_index(w)) >= 0 && ok; ++w) {
       OzItem it;
       if (!item_at<GROUP>(a, grp, BNT, t, it)) continue;
       const int nkb = it.nkb;
       float hi[HALF], lo[HALF];
 #pragma unroll
       for (int c = 0; c < HALF; ++c) hi[c] = lo[c] = 0.0f;
+      float tail[S == kMaxS ? HALF : 1];     // seven slices: what lies below lo
+      if constexpr (S == kMaxS) {
+#pragma unroll
+        for (int c = 0; c < HALF; ++c) tail[c] = 0.0f;
+      }
       for (int j = 0; j < nkb && ok; ++j) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          if (!flush_at(j, h, nkb)) continue;
+          if (!flush_at<SEG>(j, h, nkb)) continue;
           if (!mbar_wait_warp(acc_full(h), efl[h] & 1)) {
             if (lane == 0) flag_status(a.status, SKY_ETIMEOUT);
             ok = false;
@@ -532,23 +578,61 @@ __device__ __forceinline__ void oz_gemm_body(const OzArgs& a, const OzGroup* grp
           auto add = [&](const uint32_t* v, int g) {
             const float sc = __int_as_float((127 - 8 * g) << 23);   // 2^{-8g}, exact
 #pragma unroll
-            for (int c = 0; c < HALF; ++c) two_sum_acc(hi[c], lo[c], __uint_as_float(v[c]) * sc);
+            for (int c = 0; c < HALF; ++c) {
+              const float y = __uint_as_float(v[c]);
+              if (g < 4) two_sum_acc(hi[c], lo[c], y * sc);
+              else lo[c] = fmaf(y, sc, lo[c]);
+            }
           };
-          // hand the set back as early as the registers allow: two of three
-          // groups at once, the third after the first has been added; with two
-          // wider groups, one at a time
+          if constexpr (S == kMaxS) {
+            // 16 columns at a time, so that the set's four groups are at hand: the
+            // rounding errors of groups 0 .. 2 (whole numbers below 2^4 times 2^-16)
+            // add up exactly, and lo takes them and groups 3 and 4 by TwoSum, with
+            // what it drops and groups 5 .. 7 in tail
+            static_assert(NG == 8 && HS == 4 && HALF % 16 == 0, "two sets of four groups");
+#pragma unroll
+            for (int cc = 0; cc < HALF; cc += 16) {
+              uint32_t v[4][16];
+#pragma unroll
+              for (int g = 0; g < 4; ++g) tmem_ld<16>(col + (uint32_t)(g * BNT + cc), v[g]);
+              tmem_wait();
+              if (cc + 16 == HALF) hand_back(h);
+#pragma unroll
+              for (int c = 0; c < 16; ++c) {
+                auto y = [&](int g) {
+                  return __uint_as_float(v[g][c]) * __int_as_float((127 - 8 * (g + 4 * h)) << 23);
+                };
+                if (h == 0) {
+                  float e = 0.0f;
+                  two_sum_acc(hi[cc + c], e, y(0));
+                  two_sum_acc(hi[cc + c], e, y(1));
+                  two_sum_acc(hi[cc + c], e, y(2));
+                  two_sum_acc(lo[cc + c], tail[cc + c], e);
+                  two_sum_acc(lo[cc + c], tail[cc + c], y(3));
+                } else {
+                  two_sum_acc(lo[cc + c], tail[cc + c], y(0));
+                  tail[cc + c] += y(1) + (y(2) + y(3));
+                }
+              }
+            }
+            ++efl[h];
+            continue;
+          }
+          // hand the set back as early as the registers allow: with narrow shares
+          // two groups at once, the next ones read as the first are added
           uint32_t v0[HALF];
           tmem_ld_cols<HALF>(col, v0);
-          if constexpr (HS == 3) {
+          if constexpr (HALF <= 40) {
             uint32_t v1[HALF];
+            const int g = h * HS;
             tmem_ld_cols<HALF>(col + BNT, v1);
             tmem_wait();
-            add(v0, h * HS);
+            add(v0, g);
             tmem_ld_cols<HALF>(col + 2 * BNT, v0);
             tmem_wait();
             hand_back(h);
-            add(v1, h * HS + 1);
-            add(v0, h * HS + 2);
+            add(v1, g + 1);
+            add(v0, g + 2);
           } else {
             tmem_wait();
             add(v0, h * HS);
@@ -565,12 +649,17 @@ __device__ __forceinline__ void oz_gemm_body(const OzArgs& a, const OzGroup* grp
       const int col0 = it.n0 + half * HALF;
       if (row < it.M) {
         if (GROUP || a.mode == 0) {
-          float2* prow = GROUP ? a.P + grp->po[it.b] + (long long)row * it.N
+          float2* prow = GROUP ? a.P + part_width(S) * (grp->po[it.b] + (long long)row * it.N)
                                : a.P + (long long)it.b * a.sp + (long long)row * a.ldp;
 #pragma unroll
           for (int c = 0; c < HALF; ++c)
-            if (col0 + c < it.N) prow[col0 + c] = make_float2(hi[c], lo[c]);
-        } else {
+            if (col0 + c < it.N) {
+              if constexpr (S == kMaxS)
+                reinterpret_cast<float4*>(prow)[col0 + c] = make_float4(hi[c], lo[c], tail[c], 0.0f);
+              else
+                prow[col0 + c] = make_float2(hi[c], lo[c]);
+            }
+        } else if constexpr (S < kMaxS) {      // seven slices: partials only
           const int er = a.ea[row] - 16;
           if (a.out_f32) {
             float* orow = (float*)a.out + (long long)row * a.ldo;

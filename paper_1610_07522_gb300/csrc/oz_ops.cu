@@ -244,6 +244,7 @@ __global__ void __launch_bounds__(256) k_oz_split_mat(const double2* __restrict_
 
 // C[m][c] = conj(sum_z (P_z[m][c] + i P_z[m][n + c])) 2^{Ea[m] + Eb[c] - 16}: the
 // product X Y from the full overlap of X with Zt = conj(Y)^T.
+template <int S>
 __global__ void k_oz_zgemm_reduce(const float2* __restrict__ P, int nz, long long sp, long long ldp,
                                   int n, const int* __restrict__ Ea, const int* __restrict__ Eb,
                                   double2* C, const int* run, const int* stop) {
@@ -254,9 +255,8 @@ __global__ void k_oz_zgemm_reduce(const float2* __restrict__ P, int nz, long lon
   double re = 0.0, im = 0.0;
   for (int z = 0; z < nz; ++z) {
     const float2* Pz = P + z * sp + (long long)m * ldp;
-    const float2 r = Pz[c], i = Pz[n + c];
-    re += (double)r.x + (double)r.y;
-    im += (double)i.x + (double)i.y;
+    re += oz::part_value<S>(Pz, c);
+    im += oz::part_value<S>(Pz, n + c);
   }
   const double sc = oz::pow2d(Ea[m] + Eb[c] - 16);
   C[e] = make_double2(sc * re, -sc * im);
@@ -277,15 +277,15 @@ __global__ void __launch_bounds__(256) k_oz_split_group(const __grid_constant__ 
     split_mat_row<S, BN>(G.A[b], n, r, trans, E + G.ra[b] + r, dst + G.ao[b], (n + BN - 1) / BN, -1);
 }
 
+template <int S>
 __global__ void k_oz_reduce_group(const float2* __restrict__ P, const __grid_constant__ oz::OzGroup G,
                                   const int* __restrict__ Ea, const int* __restrict__ Eb) {
   const int b = blockIdx.y, n = G.n[b];
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (long long)n * n || oz::group_gated(G, b)) return;
   const int m = (int)(e / n), c = (int)(e % n);
-  const float2* Pm = P + G.po[b] + (long long)m * 2 * n;
-  const float2 r = Pm[c], i = Pm[n + c];
-  const double re = (double)r.x + (double)r.y, im = (double)i.x + (double)i.y;
+  const float2* Pm = P + oz::part_width(S) * (G.po[b] + (long long)m * 2 * n);
+  const double re = oz::part_value<S>(Pm, c), im = oz::part_value<S>(Pm, n + c);
   const double sc = oz::pow2d(Ea[G.ra[b] + m] + Eb[G.rb[b] + c] - 16);
   G.C[b][e] = make_double2(sc * re, -sc * im);
 }
@@ -458,15 +458,17 @@ sky_status oz_rotate_t(Ctx* c, const void* phi, const double2* M, int I, void* o
 // C[m][c] = conj(sum_k conj(X[m][k]) Zt[c][k]), the full digit-split overlap
 // of X's rows with Zt's rows (6 digits; about 1e-14 of the largest element).
 // Every kernel is skipped when the device gate (run, stop) says so.
-bool oz_zgemm_fits(const Ctx* c, int n) {
+static inline int zbn(int slices) { return slices == oz::kS7 ? oz::kBN7 : oz::kBN64; }
+bool oz_zgemm_fits(const Ctx* c, int n, int slices) {
+  const int bn = zbn(slices);
   return c->d_ozB && n <= c->max_states &&
-         oz::dig_elems(2LL * n, 2LL * n, oz::kS64, oz::kBN64) <= (long long)c->oz_b_elems &&
-         oz::dig_elems(n, 2LL * n, oz::kS64, oz::kBN64) <= (long long)c->oz_a_elems;
+         oz::dig_elems(2LL * n, 2LL * n, slices, bn) <= (long long)c->oz_b_elems &&
+         oz::dig_elems(n, 2LL * n, slices, bn) <= (long long)c->oz_a_elems;
 }
 
-sky_status oz_zgemm(Ctx* c, bool ah, bool bh, const double2* A, const double2* B, double2* C,
-                    int n, const int* run, const int* stop) {
-  constexpr int S = oz::kS64, BN = oz::kBN64;
+template <int S, int BN>
+static sky_status oz_zgemm_t(Ctx* c, bool ah, bool bh, const double2* A, const double2* B, double2* C,
+                             int n, const int* run, const int* stop) {
   cudaStream_t st = c->stream;
   int* Ea = c->d_ozE;
   int* Eb = c->d_ozE + c->max_states;
@@ -487,56 +489,77 @@ sky_status oz_zgemm(Ctx* c, bool ah, bool bh, const double2* A, const double2* B
   long long z = (c->num_sms + tiles - 1) / tiles;
   if (z > nkb / 8) z = nkb / 8;
   if (z < 1) z = 1;
-  const long long spart = 2LL * n * n;
+  const long long spart = 2LL * n * n * oz::part_width(S);
   if ((size_t)z * spart > c->oz_p_elems) z = (long long)(c->oz_p_elems / spart);
   if (z < 1) return set_err(c, SKY_EINVAL, "zgemm: partial buffer too small for n=%d", n);
   int zi = (int)z;
   oz::OzArgs g{};
   g.mode = 0;
   g.P = c->d_ozP;
-  g.ldp = 2LL * n;
+  g.ldp = 2LL * n * oz::part_width(S);
   g.sp = spart;
   g.status = c->d_status;
   g.run = run;
   g.stop = stop;
   e = oz::oz_gemm<S, BN>(Ap, nta, n, Bp, ntb, 2 * n, (int)K, false, n, g, &zi, st);
   if (e != cudaSuccess) return cuda_check(c, e, "oz zgemm");
-  k_oz_zgemm_reduce<<<div_up(tot, 256), 256, 0, st>>>(c->d_ozP, zi, spart, 2LL * n, n, Ea, Eb, C,
-                                                      run, stop);
+  k_oz_zgemm_reduce<S><<<div_up(tot, 256), 256, 0, st>>>(c->d_ozP, zi, spart, g.ldp, n, Ea, Eb, C,
+                                                         run, stop);
   note_launch();
   return cuda_check(c, cudaGetLastError(), "oz zgemm reduce");
+}
+
+sky_status oz_zgemm(Ctx* c, bool ah, bool bh, const double2* A, const double2* B, double2* C,
+                    int n, const int* run, const int* stop, int slices) {
+  return slices == oz::kS7 ? oz_zgemm_t<oz::kS7, oz::kBN7>(c, ah, bh, A, B, C, n, run, stop)
+                           : oz_zgemm_t<oz::kS64, oz::kBN64>(c, ah, bh, A, B, C, n, run, stop);
 }
 
 // The products C_b = opA(A_b) opB(B_b) of every problem of a batch (n_b <=
 // the context's state count) in one grouped launch sequence: two digit
 // splits, one tensor-core launch over all problems' tiles, one reduction
 // (the per-problem form above, stacked; gates per problem).
-// Operand buffer sizes (elements) of one product of m states, and of the grouped
-// products of nb problems of up to m.
-void oz_zgemm_sizes(int m, size_t* a_elems, size_t* b_elems) { oz_group_sizes(1, m, a_elems, b_elems); }
+// Operand buffer sizes (elements) of one product of m states with the given
+// digits; of the larger of both forms; and of the grouped products of nb problems
+// of up to m.
+static void zgemm_elems(int m, int slices, size_t* a_elems, size_t* b_elems) {
+  *a_elems = (size_t)oz::dig_elems(m, 2LL * m, slices, zbn(slices));
+  *b_elems = (size_t)oz::dig_elems(2LL * m, 2LL * m, slices, zbn(slices));
+}
+void oz_zgemm_sizes(int m, size_t* a_elems, size_t* b_elems) {
+  size_t a6, b6, a7, b7;
+  zgemm_elems(m, oz::kS64, &a6, &b6);
+  zgemm_elems(m, oz::kS7, &a7, &b7);
+  *a_elems = a6 > a7 ? a6 : a7;
+  *b_elems = b6 > b7 ? b6 : b7;
+}
 void oz_group_sizes(int nb, int m, size_t* a_elems, size_t* b_elems) {
-  *a_elems = (size_t)nb * oz::dig_elems(m, 2LL * m, oz::kS64, oz::kBN64);
-  *b_elems = (size_t)nb * oz::dig_elems(2LL * m, 2LL * m, oz::kS64, oz::kBN64);
+  oz_zgemm_sizes(m, a_elems, b_elems);
+  *a_elems *= nb;
+  *b_elems *= nb;
 }
 
-bool oz_zgemm_group_fits(const Ctx* c, int np, const int* n) {
+// Partials (float2s) of a product of m states, either form.
+size_t oz_partial_elems(int m) { return (size_t)oz::part_width(oz::kS7) * 2 * m * m; }
+
+bool oz_zgemm_group_fits(const Ctx* c, int np, const int* n, int slices) {
   if (!c->d_ozgA || np > c->ozg_np) return false;
   long long rows = 0, p = 0;
   size_t ae = 0, be = 0;
   for (int b = 0; b < np; ++b) {
     if (n[b] > c->max_states) return false;
     size_t x, y;
-    oz_group_sizes(1, n[b], &x, &y);
+    zgemm_elems(n[b], slices, &x, &y);
     ae += x;
     be += y;
     rows += n[b];
-    p += 2LL * n[b] * n[b];
+    p += 2LL * n[b] * n[b] * oz::part_width(slices);
   }
   return rows <= c->ozg_rows && ae <= c->ozg_a_elems && be <= c->ozg_b_elems && p <= (long long)c->ozg_p_elems;
 }
 
-sky_status oz_zgemm_group(Ctx* c, const ZJobs& j) {
-  constexpr int S = oz::kS64, BN = oz::kBN64;
+template <int S, int BN>
+static sky_status oz_zgemm_group_t(Ctx* c, const ZJobs& j) {
   cudaStream_t st = c->stream;
   oz::OzGroup G;
   G.np = j.np;
@@ -549,7 +572,7 @@ sky_status oz_zgemm_group(Ctx* c, const ZJobs& j) {
     G.n[b] = n; G.ra[b] = ra; G.rb[b] = 2 * ra; G.po[b] = po;
     G.ao[b] = (long long)ao; G.bo[b] = (long long)bo;
     size_t ae, be;
-    oz_group_sizes(1, n, &ae, &be);
+    zgemm_elems(n, S, &ae, &be);
     ao += ae;
     bo += be;
     G.A[b] = j.A[b]; G.B[b] = j.B[b]; G.C[b] = j.C[b];
@@ -574,10 +597,15 @@ sky_status oz_zgemm_group(Ctx* c, const ZJobs& j) {
   g.status = c->d_status;
   e = oz::oz_gemm_group<S, BN>(Ap, Bp, G, g, st);
   if (e != cudaSuccess) return cuda_check(c, e, "grouped zgemm");
-  k_oz_reduce_group<<<dim3(div_up((long long)nmax * nmax, 256), j.np), 256, 0, st>>>(
+  k_oz_reduce_group<S><<<dim3(div_up((long long)nmax * nmax, 256), j.np), 256, 0, st>>>(
       c->d_ozgP, G, Ea, Eb);
   note_launch();
   return cuda_check(c, cudaGetLastError(), "grouped zgemm reduce");
+}
+
+sky_status oz_zgemm_group(Ctx* c, const ZJobs& j) {
+  return j.slices == oz::kS7 ? oz_zgemm_group_t<oz::kS7, oz::kBN7>(c, j)
+                             : oz_zgemm_group_t<oz::kS64, oz::kBN64>(c, j);
 }
 
 sky_status oz_overlap(Ctx* c, const void* a, const void* b, int I, double2* X) {

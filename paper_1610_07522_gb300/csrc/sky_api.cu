@@ -144,7 +144,7 @@ static sky_status alloc_oz_scratch(Ctx* c, bool overlap_too) {
     oz_zgemm_sizes(Imax, &za, &zb);
     if (zb > be) be = zb;
     if (za > ae) ae = za;
-    if ((size_t)2 * Imax * Imax > pe) pe = (size_t)2 * Imax * Imax;
+    if (oz_partial_elems(Imax) > pe) pe = oz_partial_elems(Imax);
   }
   if (ee < (size_t)(2 * Imax + 2LL * c->G + 64)) ee = (size_t)(2 * Imax + 2LL * c->G + 64);
   if (c->d_ozB && c->oz_a_elems >= ae && c->oz_b_elems >= be && c->oz_p_elems >= pe)
@@ -326,6 +326,23 @@ sky_status sky_init(sky_ctx** out, const int grid[3], const double dx[3], const 
   if (s == SKY_OK && is_tc(prec)) s = alloc_tc_scratch(c, tc_nsplit(prec));
   c->oz_on = is_tc(prec) ? 0 : 1;
   if (s == SKY_OK && (c->oz_on || Imax >= kOzZgemmMin)) s = alloc_oz_scratch(c, c->oz_on != 0);
+  if (s == SKY_OK && Imax >= kOzZgemmMin) {
+    // grouped I x I products of two species, two products each at once
+    size_t ga, gb;
+    const size_t np = 4, gp = np * oz_partial_elems(Imax);
+    oz_group_sizes((int)np, Imax, &ga, &gb);
+    if (2 * (ga + gb) + gp * sizeof(float2) <= kOzGroupInit) {
+      unsigned short *pa = nullptr, *pb = nullptr;
+      ALLOC(pa, ga);
+      c->d_ozgA = pa;
+      ALLOC(pb, gb);
+      c->d_ozgB = pb;
+      ALLOC(c->d_ozgP, gp);
+      ALLOC(c->d_ozgE, 3 * np * Imax);
+      c->ozg_rows = (int)np * Imax; c->ozg_a_elems = ga; c->ozg_b_elems = gb;
+      c->ozg_p_elems = gp; c->ozg_np = (int)np;
+    }
+  }
   ALLOC(c->d_stats, 8);
   ALLOC(c->d_netpart, net_partial_elems(c->G));
   if (s == SKY_OK) {
@@ -730,16 +747,18 @@ sky_status sky_reserve_batch(sky_ctx* c, int nb) {
   float2* gp = nullptr;
   int* ge = nullptr;
   long long grows = 0;
+  int gnp = 0;
   size_t gpe = 0, gae = 0, gbe = 0;
   if (s == SKY_OK && nb > kOzGroupMin) {
     const size_t cap = (size_t)2 << 30;
     oz_group_sizes(1, Imax, &gae, &gbe);
-    size_t most = cap / (2 * (gae + gbe));     // problems of Imax states within the cap
-    if (most > (size_t)nb) most = (size_t)nb;
+    gnp = 2 * nb <= kMaxBatch ? 2 * nb : kMaxBatch;   // products: two per problem where they fit
+    size_t most = cap / (2 * (gae + gbe));     // of Imax states within the cap
+    if (most > (size_t)gnp) most = (size_t)gnp;
     gae *= most;
     gbe *= most;
-    grows = (long long)nb * Imax;
-    gpe = (size_t)nb * 2 * (size_t)Imax * (size_t)Imax;
+    grows = (long long)gnp * Imax;
+    gpe = (size_t)gnp * oz_partial_elems(Imax);
     if (gpe * sizeof(float2) > cap) gpe = cap / sizeof(float2);
     if (most > 0) {
       unsigned short *pa = nullptr, *pb = nullptr;
@@ -770,7 +789,7 @@ sky_status sky_reserve_batch(sky_ctx* c, int nb) {
       if (p) cudaFree(p);
     c->d_ozgA = ga; c->d_ozgB = gb; c->d_ozgP = gp; c->d_ozgE = ge;
     c->ozg_rows = (int)grows; c->ozg_a_elems = gae; c->ozg_b_elems = gbe;
-    c->ozg_p_elems = gpe; c->ozg_np = nb;
+    c->ozg_p_elems = gpe; c->ozg_np = gnp;
   }
   c->d_trivec = tvec;
   c->tri_vec_slots = tvec ? (nb < 8 ? nb : 8) : 0;

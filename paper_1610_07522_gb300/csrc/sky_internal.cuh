@@ -212,9 +212,11 @@ struct ZJobs {
   const int* stop[kMaxBatch];
   int np;
   bool ah, bh;
+  int slices;                       // tensor-core products: 6 digits, or 7 (FP64's whole mantissa)
 };
 ZJobs zjobs(int np, bool ah, bool bh, const double2* const* A, const double2* const* B,
-            double2* const* C, const int* n, const int* const* run, const int* const* stop);
+            double2* const* C, const int* n, const int* const* run, const int* const* stop,
+            int slices = 6);
 sky_status zgemm_batch(Ctx* c, const ZJobs& j);
 sky_status zgemm_small(Ctx* c, bool ah, bool bh, const double2* A, const double2* B,
                        double2* C, int n, const int* run = nullptr, const int* stop = nullptr);
@@ -267,17 +269,19 @@ sky_status oz_rotate(Ctx* c, const void* phi, const double2* M, int I, void* out
 // tensor cores) take the tensor cores too (19.81 ms)
 constexpr int kOzZgemmMin = 96;
 constexpr int kOzZgemmGated = 192;
-bool oz_zgemm_fits(const Ctx* c, int n);
-bool oz_zgemm_group_fits(const Ctx* c, int np, const int* n);
+bool oz_zgemm_fits(const Ctx* c, int n, int slices = 6);
+bool oz_zgemm_group_fits(const Ctx* c, int np, const int* n, int slices = 6);
 sky_status oz_zgemm_group(Ctx* c, const ZJobs& j);
+size_t oz_partial_elems(int m);
 void oz_group_sizes(int nb, int m, size_t* a_elems, size_t* b_elems);
 void oz_zgemm_sizes(int m, size_t* a_elems, size_t* b_elems);
 bool fused_h_ok(const Ctx* c);      // the fused FP32 h psi applies to this context
 int tri_team_plan(int np, const int* n, int blocks, int* team, int* first, int* count);
 int fused_h_blocks(const Ctx* c);   // its reduction blocks per state               // digits of the grouped products
-constexpr int kOzGroupMin = 8;      // batches of more problems take the grouped products
+constexpr int kOzGroupMin = 8;      // batches of more problems always take the grouped products
+constexpr size_t kOzGroupInit = (size_t)512 << 20;   // bytes a context spends on them by default
 sky_status oz_zgemm(Ctx* c, bool ah, bool bh, const double2* A, const double2* B, double2* C,
-                    int n, const int* run, const int* stop);
+                    int n, const int* run, const int* stop, int slices = 6);
 sky_status tc_rotate(Ctx* c, const void* phi, const double2* M, int I, void* out);
 inline bool is_tc(sky_prec p) { return p == SKY_F32_BF16X3 || p == SKY_F32_BF16X6; }
 size_t jacobi_rot_bytes(int m);
