@@ -10,13 +10,14 @@
 //     diagonal onto beta_t e_1 with beta_t real (T is real symmetric).  One
 //     cooperative kernel: the blocks keep the columns of the (full, Hermitian)
 //     trailing matrix cyclically in shared memory.  The update by H_t is
-//     A <- A - v w^H - w v^H with p = A v, w = tau p - (|tau|^2 v^H p / 2) v.
-//     Each owner forms p_j = col_j^H v_t for its own columns, fused with that
-//     column's update by the previous reflector, and publishes p, the next
-//     column and its block's partial of v^H p; after one grid barrier every
-//     block recomputes the next column and reflector itself (the same
-//     arithmetic in every block), so each step costs one barrier.  The heads
-//     of up to four problems run side by side on separate warp groups.
+//     A <- A - u w^H - w u^H with u the reflector's unscaled vector, p = A u and
+//     w = tau p - (|tau|^2 u^H p / 2) u (tau for u).  Each owner forms p_j =
+//     col_j^H u_t for its own columns, fused with that column's update by the
+//     previous reflector, and publishes p, the next column and its block's
+//     partial of u^H p; after one grid barrier every block recomputes the next
+//     column itself (the same arithmetic in every block), so each step costs one
+//     barrier.  The heads of up to four problems run side by side on separate
+//     warp groups.
 //  2. k_tri_bisect: eigenvalues of T by multisection on the count of
 //     negative LDL^T pivots of T - x I, one warp (kBisLanes points) per
 //     eigenvalue and round: FP32 counts first, then double-float ones (the
@@ -156,13 +157,40 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// Warp sums of two values, in lane 0 (five additions for both).
+__device__ __forceinline__ void warp_sum2(double& x, double& y) {
+  const int lane = threadIdx.x & 31;
+  double v = lane < 16 ? x : y;
+  v += __shfl_xor_sync(0xffffffffu, lane < 16 ? y : x, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  x = v;
+  y = __shfl_sync(0xffffffffu, v, 16);
+}
+
 // ---- stage 1: Householder reduction ------------------------------------------
+// What a step takes is FP64 instructions (a warp's takes the SM's unit 16 cycles
+// whatever lanes are active) and the latency of what stands in a row (67 cycles
+// each, a barrier over the blocks and its loads some thousands).  So:
+//  - scalars are formed by one warp and passed on in shared memory, sums over a
+//    block's threads go through shared memory to one warp;
+//  - w is not formed (column j <- column j - u a_j - p b_j with a_j = conj(w_j) -
+//    c conj(u_j), b_j = tau conj(u_j), c = |tau|^2 u^H p / 2), u stays unscaled
+//    until k_hh_scale;
+//  - norm, beta and tau are formed while the other warps update their columns:
+//    these need only row t + 1 of u from it, whose term is added at the end;
+//  - a block's columns are split over its warps by rows.
+// 700 + 300 states: 12.0 ms before, 9.9 ms; 280 + 120: 3.3, 2.7 ms.
 // The per-step vectors of a problem are short (n - t entries): its head work
-// runs on one group of kHeadWarps warps, and the heads of up to kHeadGroups
-// problems run side by side (one set of __syncthreads for all of them).
-constexpr int kHeadWarps = 4;
-constexpr int kHeadThreads = kHeadWarps * 32;
-constexpr int kHeadGroups = kTriWarps / kHeadWarps;
+// runs on a group of 16, 8 or 4 warps for one, two or more problems left, and the
+// heads of up to kHeadGroups problems run side by side (one set of __syncthreads
+// for all of them).
+constexpr int kHeadGroups = 4;
+constexpr int kHeadLoad = 4;            // elements per thread loaded ahead of the sums
+constexpr int kTabProbs = 4;            // problems of a team whose a_j, b_j are tabulated
+constexpr int kTabCols = 31;            // own columns of them
+constexpr int kBodyItems = 64;          // column shares per pass of tri_body
+constexpr int kMaxParts = 8;            // row shares of a column at most
 
 __device__ __forceinline__ TeamView team_view(const TriBatch& a) {
   const int k = find_prob(a.tg0, a.nteam, (int)blockIdx.x);
@@ -196,271 +224,415 @@ __device__ __forceinline__ double* sp_row(const TriBatch& a, int b, int t) {
 }
 
 struct HeadShared {
-  double red[kHeadGroups][kHeadWarps + 1];
-  double2 sc[kHeadGroups][2];
+  double sg[kTriWarps][16];                 // the threads' |column|^2, pairs of lanes added
+  double2 at[kHeadGroups][2];               // a_t, b_t
+  double2 tab[kTabProbs][kTabCols][2];      // a_j, b_j of the own columns from slot smin on
+  double2 acc[kBodyItems];                  // column shares' col^H u but for row t + 1
+  double2 x1[kBodyItems];                   // row t + 1 of the columns
+  int rescaled;                             // a reflector of this step has scl != 1
+};
+// Reflector t of a problem, the same in every block; entry b + kMaxBatch (t & 1).
+struct TriStep {
+  double2 tau;                              // for the unscaled u: H = I - tau u u^H
+  double kap;                               // |tau|^2 / 2
+  double c;                                 // of the reflector before: kap u^H p
+  double scl;                               // power of two u was scaled by
+  double beta, den;                         // den = |u_{t+1}|^2
+};
+// A problem of the team (by position): its size (0: not to be run), this block's
+// own columns j0 + s G, s < ns, and the first s with j >= t + 1.
+struct TriOwn {
+  int n, j0, ns, smin;
 };
 
-// Step t of the team's problems tmem[k0 .. k0 + kHeadGroups - 1] (group q
-// serves tmem[k0 + q]), every block of the team alike: column t of the trailing matrix (updated by reflector
-// t-1 from the published copy), d_t, and reflector t.  Work vectors: vn = v_t
-// (built in place from the column), vo = v_{t-1}, w.  v_{t-1}^H p_{t-1} is the
-// sum of the owners' published per-block partials (the same order in every
-// block); beta, tau and 1/(alpha - beta) are formed once per problem by the
-// group's first thread and passed on in shared memory.  The published p and
-// column are loaded in one pass (one L2 round trip per step).
-__device__ void tri_heads(const TriBatch& a, const TeamView& tv, int k0, int t, double2* dsm,
-                          HeadShared& hs, double2* s_tau, const unsigned char* s_run) {
-  const int q = threadIdx.x / kHeadThreads, ht = threadIdx.x % kHeadThreads;
-  const int lane = threadIdx.x & 31, hwarp = ht >> 5;
-  const bool has = k0 + q < tv.p1;
-  const int b = has ? a.tmem[k0 + q] : 0;
-  const bool on = has && s_run[b] && t <= a.n[b] - 1;
-  const int n = on ? a.n[b] : 0;
+// The r-th problem (position) still at work at step t, or -1; how many there are.
+__device__ __forceinline__ int nth_active(const TriOwn* own, int np, int t, int r) {
+  for (int k = 0; k < np; ++k)
+    if (t < own[k].n && r-- == 0) return k;
+  return -1;
+}
+__device__ __forceinline__ int count_active(const TriOwn* own, int np, int t) {
+  int c = 0;
+  for (int k = 0; k < np; ++k) c += t < own[k].n;
+  return c;
+}
+// Active own columns of a problem at step t (none at its last).
+__device__ __forceinline__ int active_cols(const TriOwn& o, int t) {
+  return t < o.n - 1 ? o.ns - o.smin : 0;
+}
+// a_j, b_j of column j from p_j, u_j.
+__device__ __forceinline__ void column_factors(const TriStep& st, double2 pj, double2 uj, double2& fa,
+                                               double2& fb) {
+  const double c2 = 2.0 * st.c;
+  fa = make_double2(fma(-c2, uj.x, fma(st.tau.x, pj.x, -st.tau.y * pj.y)),
+                    fma(c2, uj.y, -fma(st.tau.x, pj.y, st.tau.y * pj.x)));
+  fb = make_double2(fma(st.tau.x, uj.x, st.tau.y * uj.y), fma(st.tau.y, uj.x, -st.tau.x * uj.y));
+}
+// x - u a - p b.
+__device__ __forceinline__ double2 column_update(double2 x, double2 u, double2 p, double2 fa,
+                                                 double2 fb) {
+  return make_double2(
+      fma(-u.x, fa.x, fma(u.y, fa.y, fma(-p.x, fb.x, fma(p.y, fb.y, x.x)))),
+      fma(-u.x, fa.y, fma(-u.y, fa.x, fma(-p.x, fb.y, fma(-p.y, fb.x, x.y)))));
+}
+
+// Heads of the problems at active positions r0 .. r0 + 16 / gw - 1, step t, every
+// block of the team alike, gw = 2^lg warps each: column t of the trailing matrix
+// (updated by reflector t-1 from the published copy) into vn, the published p
+// into w, and reflector t.  vo = u_{t-1}.  u_{t-1}^H p_{t-1} is the sum of the
+// owners' published per-block partials (the same order in every block).  The
+// published p and column are loaded in one pass (one L2 round trip per step).
+// The group's first warp ends with reflector t after the last barrier here: its
+// results, u_{t+1} among them, are there after the next one.
+__device__ void tri_heads(const TriBatch& a, const TeamView& tv, int r0, int lg, int t, double2* dsm,
+                          HeadShared& hs, TriStep* s_st, const TriOwn* own) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int q = wid >> lg, hwarp = wid & ((1 << lg) - 1), HT = 32 << lg, ht = hwarp * 32 + lane;
+  const int k = nth_active(own, tv.p1 - tv.p0, t, r0 + q);
+  const bool on = k >= 0;
+  const int b = on ? a.tmem[tv.p0 + k] : 0, n = on ? own[k].n : 0;
   double2* vb = on ? vec_base(a, b, dsm) : dsm;
   double2* vn = vb + (size_t)(t & 1) * n;
   const double2* vo = vb + (size_t)((t + 1) & 1) * n;
   double2* w = vb + 2 * (size_t)n;
-  TriPtrs p;
-  if (on) p = tri_ptrs(a, b);
   double sg = 0.0;                           // |column|^2 below the subdiagonal
   if (t == 0) {
-    if (on) {
-      const double2* A = a.A[b];
-      for (int i = ht; i < n; i += kHeadThreads) {
-        double2 x = A[i];
-        x.y = i == 0 ? 0.0 : -x.y;         // column 0 = conj(row 0)
-        vn[i] = x;
-        if (i >= 2) sg = fma(x.x, x.x, fma(x.y, x.y, sg));
-      }
+    const double2* A = on ? a.A[b] : nullptr;
+    for (int i = ht; i < n; i += HT) {
+      double2 x = A[i];
+      x.y = i == 0 ? 0.0 : -x.y;             // column 0 = conj(row 0)
+      vn[i] = x;
+      if (i >= 2) sg = fma(x.x, x.x, fma(x.y, x.y, sg));
     }
+    if (r0 == 0 && threadIdx.x == 0) hs.rescaled = 0;
   } else {
+    double2 xp[kHeadLoad], xc[kHeadLoad];
+    const double2 *Pp = nullptr, *Cp = nullptr;
     if (on) {
-      const double2* Pp = ((t - 1) & 1) ? p.P1 : p.P0;
-      const double2* Cp = ((t - 1) & 1) ? p.C1 : p.C0;
-      for (int i = t + ht; i < n; i += kHeadThreads) {
-        const double2 x = __ldcg(Pp + i);
-        w[i] = x;
-        vn[i] = __ldcg(Cp + i);            // the column after step t-2's update, for now
-        if (i == t) hs.sc[q][0] = x;       // p_{t-1}[t], for w_t in every thread
+      const TriPtrs p = tri_ptrs(a, b);
+      Pp = ((t - 1) & 1) ? p.P1 : p.P0;
+      Cp = ((t - 1) & 1) ? p.C1 : p.C0;
+#pragma unroll
+      for (int r = 0; r < kHeadLoad; ++r) {
+        const int i = t + ht + r * HT;
+        if (i < n) {
+          xp[r] = __ldcg(Pp + i);
+          xc[r] = __ldcg(Cp + i);            // the column after step t-2's update
+        }
       }
       if (hwarp == 0) {
+        // lanes 0 .. 30: own columns; lane 31: column t
         const double* ps = sp_row(a, b, t - 1);
-        double S = 0.0;
-        for (int g = lane; g < tv.G; g += 32) S += __ldcg(ps + g);
-        S = warp_sum(S);
-        if (lane == 0) {
-          const double2 tau = s_tau[b];
-          hs.red[q][kHeadWarps] = 0.5 * (tau.x * tau.x + tau.y * tau.y) * S;
+        double S0 = 0.0, S1 = 0.0;
+#pragma unroll 4
+        for (int g = lane; g < tv.G; g += 64) {
+          S0 += __ldcg(ps + g);
+          if (g + 32 < tv.G) S1 += __ldcg(ps + g + 32);
+        }
+        const int cb = active_cols(own[k], t);
+        const int j = lane == 31 ? t : lane < cb ? own[k].j0 + (own[k].smin + lane) * tv.G : -1;
+        const double2 pj = j >= 0 ? __ldcg(Pp + j) : make_double2(0.0, 0.0);
+        const double2 uj = j >= 0 ? vo[j] : make_double2(0.0, 0.0);
+        TriStep& prev = s_st[b + (size_t)((t + 1) & 1) * kMaxBatch];
+        TriStep st = prev;
+        st.c = st.kap * warp_sum(S0 + S1);
+        double2 fa, fb;
+        column_factors(st, pj, uj, fa, fb);
+        if (lane == 31) {
+          hs.at[q][0] = fa;
+          hs.at[q][1] = fb;
+          prev.c = st.c;
+        } else if (lane < cb && k < kTabProbs) {
+          hs.tab[k][lane][0] = fa;
+          hs.tab[k][lane][1] = fb;
         }
       }
     }
+    if (r0 == 0 && threadIdx.x == 0) hs.rescaled = 0;
     __syncthreads();
     if (on) {
-      // w = tau p - c v_{t-1}; w_t (v_{t-1}[t] = 1) the same bits in every thread;
-      // then column t = Cb - v_{t-1} conj(w_t) - w
-      const double c = hs.red[q][kHeadWarps];
-      const double2 tau = s_tau[b];
-      const double2 pt = hs.sc[q][0], vt = vo[t];
-      const double2 wt = make_double2(fma(tau.x, pt.x, fma(-tau.y, pt.y, -c * vt.x)),
-                                      fma(tau.x, pt.y, fma(tau.y, pt.x, -c * vt.y)));
-      for (int i = t + ht; i < n; i += kHeadThreads) {
-        const double2 x = w[i], v = vo[i], cb = vn[i];
-        const double2 u = make_double2(fma(tau.x, x.x, fma(-tau.y, x.y, -c * v.x)),
-                                       fma(tau.x, x.y, fma(tau.y, x.x, -c * v.y)));
-        w[i] = u;
-        const double2 y = make_double2(fma(-v.x, wt.x, fma(-v.y, wt.y, cb.x - u.x)),
-                                       fma(-v.y, wt.x, fma(v.x, wt.y, cb.y - u.y)));
+      const double2 fa = hs.at[q][0], fb = hs.at[q][1];
+      auto row = [&](int i, double2 pi, double2 ci) {
+        const double2 y = column_update(ci, vo[i], pi, fa, fb);
+        w[i] = pi;
         vn[i] = y;
         if (i >= t + 2) sg = fma(y.x, y.x, fma(y.y, y.y, sg));
+      };
+#pragma unroll
+      for (int r = 0; r < kHeadLoad; ++r) {
+        const int i = t + ht + r * HT;
+        if (i < n) row(i, xp[r], xc[r]);
       }
+      for (int i = t + ht + kHeadLoad * HT; i < n; i += HT) row(i, __ldcg(Pp + i), __ldcg(Cp + i));
     }
   }
-  const bool refl = on && t <= n - 2;
-  if (refl) {
-    sg = warp_sum(sg);
-    if (lane == 0) hs.red[q][hwarp] = sg;
-  }
+  if (t + hwarp * 32 < n || t == 0) sg += __shfl_xor_sync(0xffffffffu, sg, 16);
+  if (lane < 16) hs.sg[wid][lane] = sg;
   __syncthreads();
-  if (refl && ht == 0) {
-    double sig = hs.red[q][0];
-    for (int k = 1; k < kHeadWarps; ++k) sig += hs.red[q][k];
-    const double2 al = vn[t + 1];
-    double beta;
-    double2 tn, sc;
-    if (sig == 0.0 && al.y == 0.0) {
-      beta = al.x;                          // already real: H_t = I
-      tn = make_double2(0.0, 0.0);
-      sc = make_double2(1.0, 0.0);
-    } else {
-      const double nr = sqrt(al.x * al.x + al.y * al.y + sig);
-      beta = al.x >= 0.0 ? -nr : nr;
-      const double rb = 1.0 / beta;
-      tn = make_double2((beta - al.x) * rb, -al.y * rb);
-      const double dx = al.x - beta;        // |Re alpha| + nr: no cancellation
-      const double r = 1.0 / fma(dx, dx, al.y * al.y);
-      sc = make_double2(dx * r, -al.y * r);  // 1 / (alpha - beta)
-    }
-    s_tau[b] = tn;
-    hs.sc[q][0] = sc;
-    hs.sc[q][1] = make_double2(beta, vn[t].x);
-    vn[t + 1] = make_double2(1.0, 0.0);
+  if (hwarp != 0 || !on || t > n - 2) return;
+  double sig = 0.0;
+  {
+    double s2[8];                            // 16 gw values, half as many per lane
+    const int half = lane >> 4;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) s2[r] = r < (1 << lg) / 2 ? hs.sg[wid + 2 * r + half][lane & 15] : 0.0;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1)
+      if (o < (1 << lg) / 2)
+#pragma unroll
+        for (int r = 0; r + o < 8; r += 2 * o) s2[r] += s2[r + o];
+    sig = warp_sum(s2[0]);
   }
-  __syncthreads();
-  if (refl) {
-    const double2 sc = hs.sc[q][0];
-    for (int i = t + 2 + ht; i < n; i += kHeadThreads) {
-      const double2 x = vn[i];
-      vn[i] = make_double2(fma(x.x, sc.x, -x.y * sc.y), fma(x.x, sc.y, x.y * sc.x));
+  if (lane != 0) return;
+  double2 al = vn[t + 1];
+  TriStep st;
+  st.c = 0.0;
+  st.scl = 1.0;
+  st.tau = make_double2(0.0, 0.0);
+  st.kap = 0.0;
+  st.den = 1.0;
+  double2 u1 = make_double2(1.0, 0.0);
+  if (sig == 0.0 && al.y == 0.0) {
+    st.beta = al.x;                          // already real: H_t = I
+  } else {
+    double s2 = fma(al.x, al.x, fma(al.y, al.y, sig));
+    double unscl = 1.0;
+    if (!(s2 > 0x1p-60 && s2 < 0x1p+60) && s2 > 0.0 && s2 < 1.7e308) {
+      // far from 1: u times a power of two, so that tau stays in range, as does what
+      // the reciprocals below start from
+      const int ex = (int)((__double_as_longlong(s2) >> 52) & 0x7FF);
+      const int h = ex == 0 ? -537 : (ex - 1023) >> 1;
+      st.scl = __longlong_as_double((long long)(1023 - h) << 52);
+      unscl = __longlong_as_double((long long)(1023 + h) << 52);
+      s2 = (s2 * st.scl) * st.scl;
+      al.x *= st.scl;
+      al.y *= st.scl;
+      hs.rescaled = 1;
     }
+    // |column|, by one step of Heron's rule from the refined reciprocal root
+    const double rs = rsqrt_refined(s2);
+    double nr = s2 * rs;
+    nr = fma(0.5 * rs, fma(-nr, nr, s2), nr);
+    const double beta = al.x >= 0.0 ? -nr : nr;
+    st.beta = beta * unscl;
+    const double dx = al.x - beta;           // |Re alpha| + nr: no cancellation
+    st.den = fma(dx, dx, al.y * al.y);
+    const double r = rcp_refined(beta * st.den);
+    st.tau = make_double2(-dx * r, -al.y * r);
+    st.kap = 0.5 * fma(st.tau.x, st.tau.x, st.tau.y * st.tau.y);
+    u1 = make_double2(dx, al.y);             // alpha - beta
   }
-  __syncthreads();
-  if (on && tv.gb == 0) {
-    if (refl) {
-      if (ht == 0) {
-        const double2 bd = hs.sc[q][1];
-        p.d[t] = bd.y;
-        p.e[t] = bd.x;
-        p.e2[t] = bd.x * bd.x;
-        p.ddd[t] = dd_of(bd.y);
-        p.e2dd[t] = dd_of(bd.x) * dd_of(bd.x);
-        p.df[t] = __double2float_rn(bd.y);
-        p.e2f[t] = __double2float_rn(bd.x * bd.x);
-        p.tau[t] = s_tau[b];
-      }
-      double2* Vt = p.V + (size_t)t * n;
-      for (int i = t + 1 + ht; i < n; i += kHeadThreads) Vt[i] = vn[i];
-    } else if (ht == 0) {
-      p.d[t] = vn[t].x;                     // t = n - 1
-      p.ddd[t] = dd_of(vn[t].x);
-      p.df[t] = __double2float_rn(vn[t].x);
+  vn[t + 1] = u1;
+  s_st[b + (size_t)(t & 1) * kMaxBatch] = st;
+}
+
+// d_t, beta_t, the unscaled reflector t and its tau and |u_{t+1}|^2 (in e2) of the
+// team's problems, by one block, a different one each step, while the arrivals
+// are under way (k_hh_scale makes of them what is kept).
+__device__ void tri_store(const TriBatch& a, const TeamView& tv, int t, double2* dsm,
+                          const TriStep* s_st, const TriOwn* own) {
+  for (int k = 0; k < tv.p1 - tv.p0; ++k) {
+    const int b = a.tmem[tv.p0 + k], n = own[k].n;
+    if (t >= n) continue;
+    const double2* vn = vec_base(a, b, dsm) + (size_t)(t & 1) * n;
+    const TriPtrs p = tri_ptrs(a, b);
+    if (threadIdx.x == 0) p.d[t] = vn[t].x;
+    if (t > n - 2) continue;
+    if (threadIdx.x == 32) {
+      const TriStep& st = s_st[b + (size_t)(t & 1) * kMaxBatch];
+      p.e[t] = st.beta;
+      p.e2[t] = st.den;
+      p.tau[t] = st.tau;
     }
+    double2* Vt = p.V + (size_t)t * n;
+    for (int i = t + 1 + (int)threadIdx.x; i < n; i += kTriThreads) Vt[i] = vn[i];
   }
 }
 
-// Own columns of problem b active at step t (j >= t+1): first slot and count.
-__device__ __forceinline__ void active_own(const TriBatch& a, const TeamView& tv, int b, int t,
-                                           int& j0, int& smin, int& cb) {
-  const int G = tv.G;
-  int ns;
-  own_range(a, tv, b, j0, ns);
-  smin = t + 1 > j0 ? (t + 1 - j0 + G - 1) / G : 0;
-  cb = ns > smin ? ns - smin : 0;
-}
-
-// Own columns j >= t+1, one warp per column: update by reflector t-1 (rows
-// > t), p_j = col_j^H v_t, publication of p_j and of column t+1, and the
-// block's partial of Re(v_t^H p_t) per problem (over its own columns, in
-// column order), for the team's problems.
-__device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, double2* dsm,
-                         double* contrib, const unsigned char* s_run) {
-  const int G = tv.G, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  int C = 0;
-  for (int k = tv.p0; k < tv.p1; ++k) {
-    const int b = a.tmem[k];
-    if (!s_run[b] || t > a.n[b] - 2) continue;
-    int j0, smin, cb;
-    active_own(a, tv, b, t, j0, smin, cb);
-    C += cb;
+// Own columns j >= t+1: update by reflector t-1 (rows > t), p_j = col_j^H u_t,
+// publication of p_j and of column t+1, and the block's partial of Re(u_t^H p_t)
+// per problem (over its own columns, in column order), for the team's problems.
+// A column's rows go to `parts` warps in turn.  The first shares are begun while
+// the first warps of the last ng groups of heads are at reflector t (so those get
+// theirs last), and row t + 1 of u is added after the barrier.
+__device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, int ng, double2* dsm,
+                         double* contrib, HeadShared& hs, const TriStep* s_st, TriOwn* own) {
+  const int G = tv.G, np = tv.p1 - tv.p0, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int grp = wid >> lg;
+  const int rank = grp >= ng ? wid - ng
+                             : (wid & ((1 << lg) - 1)) == 0 ? kTriWarps - ng + grp : wid - grp - 1;
+  int C = 0, mmax = 0;
+  for (int k = 0; k < np; ++k) {
+    C += active_cols(own[k], t);
+    mmax = own[k].n - t > mmax ? own[k].n - t : mmax;
   }
-  for (int ci = wid; ci < C; ci += kTriWarps) {
-    // column ci -> problem b, column j, slot s
-    int b = 0, j = 0, s = 0, rest = ci;
-    for (int k = tv.p0; k < tv.p1; ++k) {
-      b = a.tmem[k];
-      if (!s_run[b] || t > a.n[b] - 2) continue;
-      int j0, smin, cb;
-      active_own(a, tv, b, t, j0, smin, cb);
-      if (rest < cb) {
-        s = smin + rest;
-        j = j0 + s * G;
-        break;
-      }
+  // at least two rows per lane and share; no more shares than warps
+  int parts = C > 0 ? (kTriWarps - 1) / C : 1;
+  const int most = (mmax + 63) >> 6;
+  parts = parts > most ? most : parts;
+  parts = parts < 1 ? 1 : parts > kMaxParts ? kMaxParts : parts;
+  const TriStep* cur = s_st + (size_t)(t & 1) * kMaxBatch;
+  const TriStep* before = s_st + (size_t)((t + 1) & 1) * kMaxBatch;
+  // column ci -> position k of its problem, its place among the active ones
+  auto find = [&](int ci, int& k, int& rest) {
+    rest = ci;
+    for (k = 0; k < np; ++k) {
+      const int cb = active_cols(own[k], t);
+      if (rest < cb) return;
       rest -= cb;
     }
-    const int n = a.n[b];
-    double2* col = own_col(a, b, dsm, j, s);
-    const double2* vb = vec_base(a, b, dsm);
-    const double2* vn = vb + (size_t)(t & 1) * n;
-    const double2* vo = vb + (size_t)((t + 1) & 1) * n;
-    const double2* w = vb + 2 * (size_t)n;
-    const TriPtrs p = tri_ptrs(a, b);
-    double2* Cb = (t & 1) ? p.C1 : p.C0;
-    const bool upd = t >= 1, pub = (j == t + 1);
-    const double2 wj = upd ? conjx(w[j]) : make_double2(0.0, 0.0);
-    const double2 vj = upd ? conjx(vo[j]) : make_double2(0.0, 0.0);
-    double ax = 0.0, ay = 0.0;
-    for (int i = t + 1 + lane; i < n; i += 32) {
-      double2 x = col[i];
-      if (upd) {                            // x -= vo_i conj(w_j) + w_i conj(vo_j)
-        const double2 v = vo[i], u = w[i];
-        x.x = fma(-v.x, wj.x, fma(v.y, wj.y, fma(-u.x, vj.x, fma(u.y, vj.y, x.x))));
-        x.y = fma(-v.x, wj.y, fma(-v.y, wj.x, fma(-u.x, vj.y, fma(-u.y, vj.x, x.y))));
-        col[i] = x;
+  };
+  for (int c0 = 0; c0 < C || c0 == 0; c0 += kBodyItems) {
+    const int cols = C - c0 < kBodyItems ? C - c0 : kBodyItems;
+    for (int it = rank; it < cols * parts; it += kTriWarps) {
+      const int part = parts == 1 ? 0 : it / cols, cj = it - part * cols;
+      int k, rest;
+      find(c0 + cj, k, rest);
+      const int b = a.tmem[tv.p0 + k], n = own[k].n, s = own[k].smin + rest, j = own[k].j0 + s * G;
+      double2* col = own_col(a, b, dsm, j, s);
+      const double2* vb = vec_base(a, b, dsm);
+      const double2* vn = vb + (size_t)(t & 1) * n;
+      const double2* vo = vb + (size_t)((t + 1) & 1) * n;
+      const double2* w = vb + 2 * (size_t)n;
+      const bool upd = t >= 1, pub = (j == t + 1);
+      double2* Cb = nullptr;
+      if (pub) {
+        const TriPtrs p = tri_ptrs(a, b);
+        Cb = (t & 1) ? p.C1 : p.C0;
       }
-      const double2 v = vn[i];
-      ax = fma(x.x, v.x, fma(x.y, v.y, ax));      // conj(x) v
-      ay = fma(x.x, v.y, fma(-x.y, v.x, ay));
-      if (pub) Cb[i] = x;
+      double2 fa = make_double2(0.0, 0.0), fb = fa;
+      if (upd) {
+        if (k < kTabProbs && rest < kTabCols) {
+          fa = hs.tab[k][rest][0];
+          fb = hs.tab[k][rest][1];
+        } else {
+          column_factors(before[b], w[j], vo[j], fa, fb);
+        }
+      }
+      double ax = 0.0, ay = 0.0, bx = 0.0, by = 0.0;
+      double2 x1 = make_double2(0.0, 0.0);
+      const int step = 32 * parts;
+      // two rows at a time, loads first
+      for (int i = t + 1 + part * 32 + lane; i < n; i += 2 * step) {
+        const int i2 = i + step;
+        const bool two = i2 < n;
+        double2 xa = col[i], xb = make_double2(0.0, 0.0), v2 = xb, va = xb;
+        if (two) {
+          xb = col[i2];
+          v2 = vn[i2];
+        }
+        if (i > t + 1) va = vn[i];
+        if (upd) {
+          xa = column_update(xa, vo[i], w[i], fa, fb);
+          if (two) xb = column_update(xb, vo[i2], w[i2], fa, fb);
+          col[i] = xa;
+          if (two) col[i2] = xb;
+        }
+        if (i == t + 1) x1 = xa;
+        if (pub) {
+          Cb[i] = xa;
+          if (two) Cb[i2] = xb;
+        }
+        ax = fma(xa.x, va.x, fma(xa.y, va.y, ax));      // conj(x) u
+        ay = fma(xa.x, va.y, fma(-xa.y, va.x, ay));
+        bx = fma(xb.x, v2.x, fma(xb.y, v2.y, bx));
+        by = fma(xb.x, v2.y, fma(-xb.y, v2.x, by));
+      }
+      ax += bx;
+      ay += by;
+      warp_sum2(ax, ay);
+      if (lane == 0) {
+        hs.acc[part * cols + cj] = make_double2(ax, ay);
+        if (part == 0) hs.x1[cj] = x1;
+      }
     }
-    ax = warp_sum(ax);
-    ay = warp_sum(ay);
-    if (lane == 0) {
-      ((t & 1) ? p.P1 : p.P0)[j] = make_double2(ax, ay);
-      const double2 vnj = vn[j];
-      contrib[ci] = fma(vnj.x, ax, vnj.y * ay);   // Re(conj(v_t[j]) p_j)
+    __syncthreads();                         // reflector t; the shares
+    if (c0 == 0 && hs.rescaled) {
+      for (int k = 0; k < np; ++k) {
+        const int b = a.tmem[tv.p0 + k], n = own[k].n;
+        if (t > n - 2 || cur[b].scl == 1.0) continue;
+        double2* v = vec_base(a, b, dsm) + (size_t)(t & 1) * n;
+        const double sc = cur[b].scl;
+        for (int i = t + 2 + (int)threadIdx.x; i < n; i += kTriThreads)
+          v[i] = make_double2(v[i].x * sc, v[i].y * sc);
+      }
+      __syncthreads();
     }
+    if (wid == 0)
+      for (int cj = lane; cj < cols; cj += 32) {
+        int k, rest;
+        find(c0 + cj, k, rest);
+        const int b = a.tmem[tv.p0 + k], n = own[k].n, j = own[k].j0 + (own[k].smin + rest) * G;
+        const double2* vn = vec_base(a, b, dsm) + (size_t)(t & 1) * n;
+        double2 z[kMaxParts];
+#pragma unroll
+        for (int q = 0; q < kMaxParts; ++q)
+          z[q] = q < parts ? hs.acc[q * cols + cj] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int o = 1; o < kMaxParts; o <<= 1)
+          if (o < parts)
+#pragma unroll
+            for (int q = 0; q + o < kMaxParts; q += 2 * o) z[q] = z[q] + z[q + o];
+        const double2 u1 = vn[t + 1], x1 = hs.x1[cj], uj = vn[j];
+        const double sc = cur[b].scl;        // (the shares are of u before its scaling)
+        const double ax = fma(x1.x, u1.x, fma(x1.y, u1.y, sc * z[0].x));
+        const double ay = fma(x1.x, u1.y, fma(-x1.y, u1.x, sc * z[0].y));
+        const TriPtrs p = tri_ptrs(a, b);
+        ((t & 1) ? p.P1 : p.P0)[j] = make_double2(ax, ay);
+        contrib[c0 + cj] = fma(uj.x, ax, uj.y * ay);   // Re(conj(u_t[j]) p_j)
+      }
+    if (c0 + kBodyItems < C) __syncthreads();
   }
-  __syncthreads();
-  // per-problem partials, one thread per problem, own columns in order
-  for (int k = tv.p0 + (int)threadIdx.x; k < tv.p1; k += blockDim.x) {
-    const int b = a.tmem[k];
-    if (!s_run[b] || t > a.n[b] - 2) continue;
+  // per-problem partials, one lane per problem, own columns in order; the next
+  // step's first own columns
+  if (wid != 0) return;
+  __syncwarp();
+  for (int k = lane; k < np; k += 32) {
+    TriOwn& o = own[k];
+    if (t > o.n - 2) continue;
     int first = 0;
-    for (int kq = tv.p0; kq < k; ++kq) {
-      const int q = a.tmem[kq];
-      if (!s_run[q] || t > a.n[q] - 2) continue;
-      int j0, smin, cb;
-      active_own(a, tv, q, t, j0, smin, cb);
-      first += cb;
-    }
-    int j0, smin, cb;
-    active_own(a, tv, b, t, j0, smin, cb);
+    for (int kq = 0; kq < k; ++kq) first += active_cols(own[kq], t);
+    const int cb = active_cols(o, t);
     double acc = 0.0;
     for (int i = 0; i < cb; ++i) acc += contrib[first + i];
-    sp_row(a, b, t)[tv.gb] = acc;
+    sp_row(a, a.tmem[tv.p0 + k], t)[tv.gb] = acc;
   }
+  __syncwarp();
+  for (int k = lane; k < np; k += 32)
+    if (own[k].smin < own[k].ns && own[k].j0 + own[k].smin * G < t + 2) ++own[k].smin;
 }
 
 __global__ void __launch_bounds__(kTriThreads, 1) k_hh_tridiag(TriBatch a) {
   extern __shared__ double2 dsm[];
   __shared__ HeadShared hs;
-  __shared__ double2 s_tau[kMaxBatch];
-  __shared__ unsigned char s_run[kMaxBatch];
+  __shared__ TriStep s_st[2 * kMaxBatch];
+  __shared__ TriOwn own[kMaxBatch];
   const int tid = threadIdx.x, nt = blockDim.x;
   double* contrib = reinterpret_cast<double*>(dsm + a.coff);
   const TeamView tv = team_view(a);
+  const int np = tv.p1 - tv.p0;
   unsigned epoch = 0;
   int nrun = 0;
-  for (int k = tv.p0; k < tv.p1; ++k) {
-    const int b = a.tmem[k];
+  for (int k = 0; k < np; ++k) {
+    const int b = a.tmem[tv.p0 + k];
     const bool r = tri_run(a, b);
     if (tid == 0) {
-      s_run[b] = r;
-      s_tau[b] = make_double2(0.0, 0.0);
+      TriOwn o;
+      own_range(a, tv, b, o.j0, o.ns);
+      o.n = r ? a.n[b] : 0;
+      o.smin = o.j0 < 1 ? 1 : 0;             // the first column >= 1
+      own[k] = o;
     }
     if (r && a.n[b] > nrun) nrun = a.n[b];
   }
   __syncthreads();
   // own columns: column j = conj(row j) of the Hermitian input
-  for (int k = tv.p0; k < tv.p1; ++k) {
-    const int b = a.tmem[k];
-    if (!s_run[b]) continue;
-    int j0, ns;
-    own_range(a, tv, b, j0, ns);
-    const int n = a.n[b];
+  for (int k = 0; k < np; ++k) {
+    const int b = a.tmem[tv.p0 + k], n = own[k].n;
+    if (n == 0) continue;
     const double2* A = a.A[b];
-    for (int s = 0; s < ns; ++s) {
-      const int j = j0 + s * tv.G;
+    for (int s = 0; s < own[k].ns; ++s) {
+      const int j = own[k].j0 + s * tv.G;
       double2* col = own_col(a, b, dsm, j, s);
       for (int i = tid; i < n; i += nt) {
         double2 x = A[(size_t)j * n + i];
@@ -471,21 +643,64 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_hh_tridiag(TriBatch a) {
   }
   __syncthreads();
   for (int t = 0; t < nrun; ++t) {
-    for (int k0 = tv.p0; k0 < tv.p1; k0 += kHeadGroups)
-      tri_heads(a, tv, k0, t, dsm, hs, s_tau, s_run);
-    tri_body(a, tv, t, dsm, contrib, s_run);
-    if (t + 1 < nrun) {
-      if (tv.G == 1) {
-        __syncthreads();
-      } else if (!blocks_barrier(tv.bar, epoch, (unsigned)tv.G, a.status, a.spins)) {
-        return;
-      }
+    const int nact = count_active(own, np, t);
+    const int lg = nact == 1 ? 4 : nact == 2 ? 3 : 2;
+    const int per = kTriWarps >> lg;
+    int last = 0;                            // problems of the last round of heads
+    for (int r0 = 0; r0 < nact; r0 += per) {
+      if (r0 > 0) __syncthreads();
+      tri_heads(a, tv, r0, lg, t, dsm, hs, s_st, own);
+      last = nact - r0 < per ? nact - r0 : per;
+    }
+    tri_body(a, tv, t, lg, last, dsm, contrib, hs, s_st, own);
+    auto store = [&] {
+      if (tv.gb == t % tv.G) tri_store(a, tv, t, dsm, s_st, own);
+    };
+    if (t + 1 == nrun) {
+      store();
+    } else if (tv.G == 1) {
+      store();
+      __syncthreads();
+    } else if (!blocks_barrier(tv.bar, epoch, (unsigned)tv.G, a.status, a.spins, store)) {
+      return;
     }
   }
   if (tv.gb == 0 && tid == 0) {
     long long k = 0;
-    for (int q = tv.p0; q < tv.p1; ++q) k += s_run[a.tmem[q]];
+    for (int q = 0; q < np; ++q) k += own[q].n > 0;
     atomicAdd(reinterpret_cast<unsigned long long*>(a.stats + 6), (unsigned long long)k);
+  }
+}
+
+// What is kept of reflector t (blockIdx.x) and of T: v = u / u_{t+1} and its tau, d
+// and e in the forms the bisection reads.
+__global__ void __launch_bounds__(128) k_hh_scale(TriBatch a) {
+  const int b = blockIdx.y, t = blockIdx.x, n = a.n[b];
+  if (t >= n || !tri_run(a, b)) return;
+  const TriPtrs p = tri_ptrs(a, b);
+  if (threadIdx.x == 0) {
+    const double d = p.d[t];
+    p.ddd[t] = dd_of(d);
+    p.df[t] = __double2float_rn(d);
+  }
+  if (t > n - 2) return;
+  double2* Vt = p.V + (size_t)t * n;
+  const double2 u1 = Vt[t + 1];
+  const double den = p.e2[t], r = 1.0 / den;
+  const double2 sc = make_double2(u1.x * r, -u1.y * r);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const double e = p.e[t];
+    const double2 tau = p.tau[t];
+    p.e2[t] = e * e;
+    p.e2dd[t] = dd_of(e) * dd_of(e);
+    p.e2f[t] = __double2float_rn(e * e);
+    p.tau[t] = make_double2(tau.x * den, tau.y * den);
+    Vt[t + 1] = make_double2(1.0, 0.0);
+  }
+  for (int i = t + 2 + (int)threadIdx.x; i < n; i += 128) {
+    const double2 x = Vt[i];
+    Vt[i] = make_double2(fma(x.x, sc.x, -x.y * sc.y), fma(x.x, sc.y, x.y * sc.x));
   }
 }
 
@@ -1426,11 +1641,12 @@ static sky_status tri_group(Ctx* c, int np, const int* idx, const double2* const
   e = cudaLaunchCooperativeKernel((const void*)k_hh_tridiag, dim3(G), dim3(kTriThreads), args,
                                   used * sizeof(double2), c->stream);
   if (e != cudaSuccess) return cuda_check(c, e, "householder tridiagonalisation");
+  k_hh_scale<<<dim3(nmax, np), 128, 0, c->stream>>>(a);
   k_tri_bisect<<<(unsigned)ntot, 32, 0, c->stream>>>(a);
   k_tri_vectors<<<div_up(ntot, kVecThreads), kVecThreads, 0, c->stream>>>(a);
   k_tri_window<<<(unsigned)ntot, kWinThreads, 0, c->stream>>>(a, 0);
   k_tri_window<<<(unsigned)ntot, kWinThreads, 0, c->stream>>>(a, 1);
-  note_launch(4);
+  note_launch(5);
   // the products by tensor cores, unless the batch is gated (skipped products
   // still cost their launches) or its problems are small
   if (!run && nmax >= kWyMin) {
