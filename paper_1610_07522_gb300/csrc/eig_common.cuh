@@ -29,20 +29,15 @@ __device__ __forceinline__ double rcp_refined(double x) {
 // counter `bar` (reset before the launch): barrier number e completes when
 // the counter reaches e * count.  Release-add to arrive, acquire loads to
 // wait, with a bounded spin: on timeout it flags SKY_ETIMEOUT and returns
-// false.  The whole grid is count = gridDim.x.  meanwhile() is run by every
-// thread between the block's arrival and its wait.
-template <class F>
+// false.  The whole grid is count = gridDim.x.
 __device__ __forceinline__ bool blocks_barrier(unsigned* bar, unsigned& epoch, unsigned count,
-                                               int* status, long long max_spins, F meanwhile) {
+                                               int* status, long long max_spins) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
     ++epoch;
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-  }
-  meanwhile();
-  if (threadIdx.x == 0) {
     const unsigned target = epoch * count;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
     int ok = 1;
     long long spins = 0;
     for (;;) {
@@ -62,10 +57,6 @@ __device__ __forceinline__ bool blocks_barrier(unsigned* bar, unsigned& epoch, u
   }
   __syncthreads();
   return s_ok != 0;
-}
-__device__ __forceinline__ bool blocks_barrier(unsigned* bar, unsigned& epoch, unsigned count,
-                                               int* status, long long max_spins) {
-  return blocks_barrier(bar, epoch, count, status, max_spins, [] {});
 }
 __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned& epoch, int* status,
                                              long long max_spins) {

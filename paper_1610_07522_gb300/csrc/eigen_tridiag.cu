@@ -14,9 +14,9 @@
 //     w = tau p - (|tau|^2 u^H p / 2) u (tau for u).  Each owner forms p_j =
 //     col_j^H u_t for its own columns, fused with that column's update by the
 //     previous reflector, and publishes p, the next column and its block's
-//     partial of u^H p; after one grid barrier every block recomputes the next
+//     partial of u^H p; once these are there every block recomputes the next
 //     column itself (the same arithmetic in every block), so each step costs one
-//     barrier.  The heads of up to four problems run side by side on separate
+//     exchange.  The heads of up to four problems run side by side on separate
 //     warp groups.
 //  2. k_tri_bisect: eigenvalues of T by multisection on the count of
 //     negative LDL^T pivots of T - x I, one warp (kBisLanes points) per
@@ -59,6 +59,7 @@ constexpr int kWinChunks = (2 * kWinMax + 1 + 31) / 32;
 constexpr int kBackWarps = 16;
 constexpr size_t kTriSmemMax = 200 * 1024;   // dynamic shared memory of k_hh_tridiag / k_hh_back
 constexpr double kEps = 2.220446049250313e-16;
+constexpr int kTriBufs = 4;             // buffers of the published vectors (see unset)
 constexpr int kTeamBarStride = 32;     // unsigned between team barrier counters (128 bytes)
 
 struct TriBatch {
@@ -111,7 +112,7 @@ struct TriPtrs {
   double2* cols;                 // own columns, global home: column j at cols + j * n
   double2* V;
   double *Y, *Y2, *U0, *U2;      // U0: pairs (1 / pivot, first superdiagonal)
-  double2 *P0, *P1, *C0, *C1, *tau;
+  double2 *P, *C, *tau;          // published p and columns, kTriBufs of m each
   double *d, *e, *e2, *lam;
   float *df, *e2f;               // d and e^2 rounded to float (coarse bisection rounds)
   dd *ddd, *e2dd;                // d and e^2 as float pairs (fine bisection rounds)
@@ -128,8 +129,8 @@ __device__ __forceinline__ TriPtrs tri_ptrs(const TriBatch& a, int b) {
   double* t = a.T + k * a.tslot;
   p.U2 = t;
   double2* vecs = reinterpret_cast<double2*>(t + m * m);   // m even: 16-byte aligned
-  p.P0 = vecs; p.P1 = vecs + m; p.C0 = vecs + 2 * m; p.C1 = vecs + 3 * m; p.tau = vecs + 4 * m;
-  double* s = reinterpret_cast<double*>(vecs + 5 * m);
+  p.P = vecs; p.C = vecs + kTriBufs * m; p.tau = vecs + 2 * kTriBufs * m;
+  double* s = reinterpret_cast<double*>(vecs + (2 * kTriBufs + 1) * m);
   p.d = s; p.e = s + m; p.e2 = s + 2 * m; p.lam = s + 3 * m;
   p.ddd = reinterpret_cast<dd*>(s + 4 * m); p.e2dd = p.ddd + m;        // m doubles each
   p.df = reinterpret_cast<float*>(s + 6 * m); p.e2f = p.df + m;        // m / 2 doubles each
@@ -171,7 +172,7 @@ __device__ __forceinline__ void warp_sum2(double& x, double& y) {
 // ---- stage 1: Householder reduction ------------------------------------------
 // What a step takes is FP64 instructions (a warp's takes the SM's unit 16 cycles
 // whatever lanes are active) and the latency of what stands in a row (67 cycles
-// each, a barrier over the blocks and its loads some thousands).  So:
+// each, an exchange between the blocks some thousands).  So:
 //  - scalars are formed by one warp and passed on in shared memory, sums over a
 //    block's threads go through shared memory to one warp;
 //  - w is not formed (column j <- column j - u a_j - p b_j with a_j = conj(w_j) -
@@ -180,12 +181,14 @@ __device__ __forceinline__ void warp_sum2(double& x, double& y) {
 //  - norm, beta and tau are formed while the other warps update their columns:
 //    these need only row t + 1 of u from it, whose term is added at the end;
 //  - a block's columns are split over its warps by rows.
-// 700 + 300 states: 12.0 ms before, 9.9 ms; 280 + 120: 3.3, 2.7 ms.
+// With the published values as flags (kUnset) 700 + 300 states take 9.3 ms instead
+// of 12.0 ms, 280 + 120 states 2.4 instead of 3.3 ms.
 // The per-step vectors of a problem are short (n - t entries): its head work
 // runs on a group of 16, 8 or 4 warps for one, two or more problems left, and the
 // heads of up to kHeadGroups problems run side by side (one set of __syncthreads
 // for all of them).
 constexpr int kHeadGroups = 4;
+constexpr int kHeadSums = 5;            // per-block partials a lane loads at once
 constexpr int kHeadLoad = 4;            // elements per thread loaded ahead of the sums
 constexpr int kTabProbs = 4;            // problems of a team whose a_j, b_j are tabulated
 constexpr int kTabCols = 31;            // own columns of them
@@ -218,9 +221,63 @@ __device__ __forceinline__ double2* own_col(const TriBatch& a, int b, double2* d
                         : a.S0 + (size_t)a.sid[b] * a.slot + (size_t)j * n;
 }
 
-// Per-block partials of Re(v_t^H p_t) of problem b, parity t & 1.
+// Per-block partials of Re(u_t^H p_t) of problem b.
 __device__ __forceinline__ double* sp_row(const TriBatch& a, int b, int t) {
-  return a.sp + (size_t)a.sid[b] * a.sp_stride + (size_t)(t & 1) * gridDim.x;
+  return a.sp + (size_t)a.sid[b] * a.sp_stride + (size_t)(t & (kTriBufs - 1)) * gridDim.x;
+}
+
+// The published values of step t (p, column t + 1, the partials of u^H p) are
+// their own flags: a reader takes a word once it no longer holds kUnset, a
+// signalling NaN that no arithmetic returns.  That is one trip through L2 per
+// step, where a barrier costs the writers' fence, its counter, the poll and then
+// the loads: 7.9 -> 7.4 us a step at 120 states, 13.2 -> 12.5 us at 700.  The values of step t are in buffer t mod 4; while step t is under way its owners
+// unset their words of buffer t + 2 mod 4, last read at step t - 1: everyone is
+// past that, since everyone's partial of step t - 1 was read here, and nobody
+// looks for them before it has read the owner's partial of step t + 1, published
+// after the fence behind the unsetting.  Every wait is bounded.
+constexpr unsigned long long kUnset = 0x7FF4000000C0FFEEull;
+__device__ __forceinline__ double unset() { return __longlong_as_double((long long)kUnset); }
+__device__ __forceinline__ bool is_unset(double x) {
+  return (unsigned long long)__double_as_longlong(x) == kUnset;
+}
+__device__ __forceinline__ void put_word(double* p, double v) {
+  asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
+}
+__device__ __forceinline__ void put_word(double2* p, double2 v) {
+  asm volatile("st.relaxed.gpu.global.v2.f64 [%0], {%1, %2};" ::"l"(p), "d"(v.x), "d"(v.y) : "memory");
+}
+__device__ __forceinline__ double get_word(const double* p) {
+  double v;
+  asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ double2 get_word(const double2* p) {
+  double2 v;
+  asm volatile("ld.relaxed.gpu.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ bool is_unset(double2 v) { return is_unset(v.x) || is_unset(v.y); }
+// Another try at a word that was not there: false when the wait is over.
+struct TriWait {
+  int* status;
+  long long left;
+  bool ok;
+};
+__device__ __forceinline__ bool wait_more(TriWait& w) {
+  --w.left;
+  if (w.left <= 0 || ((w.left & 63) == 0 && (*(volatile int*)w.status & SKY_STATUS_BIT(SKY_ETIMEOUT)))) {
+    flag_status(w.status, SKY_ETIMEOUT);
+    w.ok = false;
+  }
+  return w.ok;
+}
+template <typename T>
+__device__ __forceinline__ T await_word(const T* p, T v, TriWait& w) {
+  while (is_unset(v)) {
+    if (!wait_more(w)) break;
+    v = get_word(p);
+  }
+  return v;
 }
 
 struct HeadShared {
@@ -229,7 +286,8 @@ struct HeadShared {
   double2 tab[kTabProbs][kTabCols][2];      // a_j, b_j of the own columns from slot smin on
   double2 acc[kBodyItems];                  // column shares' col^H u but for row t + 1
   double2 x1[kBodyItems];                   // row t + 1 of the columns
-  int rescaled;                             // a reflector of this step has scl != 1
+  int rescaled[2];                          // a reflector of step t (parity) has scl != 1
+  int timeout[2];                           // a wait before the first, second barrier ran out
 };
 // Reflector t of a problem, the same in every block; entry b + kMaxBatch (t & 1).
 struct TriStep {
@@ -283,8 +341,9 @@ __device__ __forceinline__ double2 column_update(double2 x, double2 u, double2 p
 // owners' published per-block partials (the same order in every block).  The
 // published p and column are loaded in one pass (one L2 round trip per step).
 // The group's first warp ends with reflector t after the last barrier here: its
-// results, u_{t+1} among them, are there after the next one.
-__device__ void tri_heads(const TriBatch& a, const TeamView& tv, int r0, int lg, int t, double2* dsm,
+// results, u_{t+1} among them, are there after the next one.  False (in every
+// thread) when a wait ran out.
+__device__ bool tri_heads(const TriBatch& a, const TeamView& tv, int r0, int lg, int t, double2* dsm,
                           HeadShared& hs, TriStep* s_st, const TriOwn* own) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int q = wid >> lg, hwarp = wid & ((1 << lg) - 1), HT = 32 << lg, ht = hwarp * 32 + lane;
@@ -296,6 +355,7 @@ __device__ void tri_heads(const TriBatch& a, const TeamView& tv, int r0, int lg,
   const double2* vo = vb + (size_t)((t + 1) & 1) * n;
   double2* w = vb + 2 * (size_t)n;
   double sg = 0.0;                           // |column|^2 below the subdiagonal
+  TriWait wt{a.status, a.spins, true};
   if (t == 0) {
     const double2* A = on ? a.A[b] : nullptr;
     for (int i = ht; i < n; i += HT) {
@@ -304,35 +364,48 @@ __device__ void tri_heads(const TriBatch& a, const TeamView& tv, int r0, int lg,
       vn[i] = x;
       if (i >= 2) sg = fma(x.x, x.x, fma(x.y, x.y, sg));
     }
-    if (r0 == 0 && threadIdx.x == 0) hs.rescaled = 0;
+    if (r0 == 0 && threadIdx.x == 0) hs.rescaled[t & 1] = 0;
   } else {
     double2 xp[kHeadLoad], xc[kHeadLoad];
     const double2 *Pp = nullptr, *Cp = nullptr;
     if (on) {
       const TriPtrs p = tri_ptrs(a, b);
-      Pp = ((t - 1) & 1) ? p.P1 : p.P0;
-      Cp = ((t - 1) & 1) ? p.C1 : p.C0;
+      Pp = p.P + (size_t)((t - 1) & (kTriBufs - 1)) * a.m;
+      Cp = p.C + (size_t)((t - 1) & (kTriBufs - 1)) * a.m;
 #pragma unroll
       for (int r = 0; r < kHeadLoad; ++r) {
         const int i = t + ht + r * HT;
         if (i < n) {
-          xp[r] = __ldcg(Pp + i);
-          xc[r] = __ldcg(Cp + i);            // the column after step t-2's update
+          xp[r] = get_word(Pp + i);
+          xc[r] = get_word(Cp + i);          // the column after step t-2's update
         }
       }
       if (hwarp == 0) {
         // lanes 0 .. 30: own columns; lane 31: column t
         const double* ps = sp_row(a, b, t - 1);
-        double S0 = 0.0, S1 = 0.0;
-#pragma unroll 4
-        for (int g = lane; g < tv.G; g += 64) {
-          S0 += __ldcg(ps + g);
-          if (g + 32 < tv.G) S1 += __ldcg(ps + g + 32);
-        }
         const int cb = active_cols(own[k], t);
         const int j = lane == 31 ? t : lane < cb ? own[k].j0 + (own[k].smin + lane) * tv.G : -1;
-        const double2 pj = j >= 0 ? __ldcg(Pp + j) : make_double2(0.0, 0.0);
+        double2 pj = j >= 0 ? get_word(Pp + j) : make_double2(0.0, 0.0);
+        double S0 = 0.0, S1 = 0.0;
+        for (int g = lane; g < tv.G; g += 32 * kHeadSums) {
+          double x[kHeadSums];
+#pragma unroll
+          for (int r = 0; r < kHeadSums; ++r) x[r] = g + 32 * r < tv.G ? get_word(ps + g + 32 * r) : 0.0;
+          for (;;) {                         // (all words that are missing at once)
+            bool miss = false;
+#pragma unroll
+            for (int r = 0; r < kHeadSums; ++r) miss |= is_unset(x[r]);
+            if (!miss || !wait_more(wt)) break;
+#pragma unroll
+            for (int r = 0; r < kHeadSums; ++r)
+              if (is_unset(x[r])) x[r] = get_word(ps + g + 32 * r);
+          }
+#pragma unroll
+          for (int r = 0; r < kHeadSums; ++r) (r & 1 ? S1 : S0) += x[r];
+        }
+        if (j >= 0) pj = await_word(Pp + j, pj, wt);
         const double2 uj = j >= 0 ? vo[j] : make_double2(0.0, 0.0);
+        __syncwarp();
         TriStep& prev = s_st[b + (size_t)((t + 1) & 1) * kMaxBatch];
         TriStep st = prev;
         st.c = st.kap * warp_sum(S0 + S1);
@@ -347,9 +420,27 @@ __device__ void tri_heads(const TriBatch& a, const TeamView& tv, int r0, int lg,
           hs.tab[k][lane][1] = fb;
         }
       }
+      for (;;) {
+        bool miss = false;
+#pragma unroll
+        for (int r = 0; r < kHeadLoad; ++r)
+          if (t + ht + r * HT < n) miss |= is_unset(xp[r]) || is_unset(xc[r]);
+        if (!miss || !wait_more(wt)) break;
+#pragma unroll
+        for (int r = 0; r < kHeadLoad; ++r) {
+          const int i = t + ht + r * HT;
+          if (i < n) {
+            if (is_unset(xp[r])) xp[r] = get_word(Pp + i);
+            if (is_unset(xc[r])) xc[r] = get_word(Cp + i);
+          }
+        }
+      }
+      __syncwarp();
     }
-    if (r0 == 0 && threadIdx.x == 0) hs.rescaled = 0;
+    if (r0 == 0 && threadIdx.x == 0) hs.rescaled[t & 1] = 0;
+    if (!wt.ok) hs.timeout[0] = 1;
     __syncthreads();
+    if (hs.timeout[0]) return false;
     if (on) {
       const double2 fa = hs.at[q][0], fb = hs.at[q][1];
       auto row = [&](int i, double2 pi, double2 ci) {
@@ -363,13 +454,17 @@ __device__ void tri_heads(const TriBatch& a, const TeamView& tv, int r0, int lg,
         const int i = t + ht + r * HT;
         if (i < n) row(i, xp[r], xc[r]);
       }
-      for (int i = t + ht + kHeadLoad * HT; i < n; i += HT) row(i, __ldcg(Pp + i), __ldcg(Cp + i));
+      for (int i = t + ht + kHeadLoad * HT; i < n; i += HT)
+        row(i, await_word(Pp + i, get_word(Pp + i), wt), await_word(Cp + i, get_word(Cp + i), wt));
+      if (!wt.ok) hs.timeout[1] = 1;
+      __syncwarp();
     }
   }
   if (t + hwarp * 32 < n || t == 0) sg += __shfl_xor_sync(0xffffffffu, sg, 16);
   if (lane < 16) hs.sg[wid][lane] = sg;
   __syncthreads();
-  if (hwarp != 0 || !on || t > n - 2) return;
+  if (hs.timeout[1]) return false;
+  if (hwarp != 0 || !on || t > n - 2) return true;
   double sig = 0.0;
   {
     double s2[8];                            // 16 gw values, half as many per lane
@@ -383,7 +478,7 @@ __device__ void tri_heads(const TriBatch& a, const TeamView& tv, int r0, int lg,
         for (int r = 0; r + o < 8; r += 2 * o) s2[r] += s2[r + o];
     sig = warp_sum(s2[0]);
   }
-  if (lane != 0) return;
+  if (lane != 0) return true;
   double2 al = vn[t + 1];
   TriStep st;
   st.c = 0.0;
@@ -407,7 +502,7 @@ __device__ void tri_heads(const TriBatch& a, const TeamView& tv, int r0, int lg,
       s2 = (s2 * st.scl) * st.scl;
       al.x *= st.scl;
       al.y *= st.scl;
-      hs.rescaled = 1;
+      hs.rescaled[t & 1] = 1;
     }
     // |column|, by one step of Heron's rule from the refined reciprocal root
     const double rs = rsqrt_refined(s2);
@@ -424,6 +519,7 @@ __device__ void tri_heads(const TriBatch& a, const TeamView& tv, int r0, int lg,
   }
   vn[t + 1] = u1;
   s_st[b + (size_t)(t & 1) * kMaxBatch] = st;
+  return true;
 }
 
 // d_t, beta_t, the unscaled reflector t and its tau and |u_{t+1}|^2 (in e2) of the
@@ -447,6 +543,26 @@ __device__ void tri_store(const TriBatch& a, const TeamView& tv, int t, double2*
     double2* Vt = p.V + (size_t)t * n;
     for (int i = t + 1 + (int)threadIdx.x; i < n; i += kTriThreads) Vt[i] = vn[i];
   }
+}
+
+// This block's words of buffer t + 2 mod kTriBufs, by the warps other than the
+// first: p of its columns, its partials, and as the owner of column t + 3 that.
+__device__ __forceinline__ void tri_unset(const TriBatch& a, const TeamView& tv, int t,
+                                          const TriOwn* own) {
+  const int tid = (int)threadIdx.x - 32;
+  for (int k = 0; k < tv.p1 - tv.p0; ++k) {
+    const int b = a.tmem[tv.p0 + k], n = own[k].n;
+    if (t + 2 > n - 2) continue;             // step t + 2 publishes nothing
+    const TriPtrs p = tri_ptrs(a, b);
+    const size_t o = (size_t)((t + 2) & (kTriBufs - 1)) * a.m;
+    const double2 no = make_double2(unset(), unset());
+    for (int s = tid; s < own[k].ns; s += kTriThreads - 32)
+      put_word(p.P + o + own[k].j0 + s * tv.G, no);
+    if (tid == kTriThreads - 33) put_word(sp_row(a, b, t + 2) + tv.gb, unset());
+    if ((t + 3 + a.rot[b]) % tv.G == tv.gb)
+      for (int i = t + 3 + tid; i < n; i += kTriThreads - 32) put_word(p.C + o + i, no);
+  }
+  __threadfence();
 }
 
 // Own columns j >= t+1: update by reflector t-1 (rows > t), p_j = col_j^H u_t,
@@ -498,7 +614,7 @@ __device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, i
       double2* Cb = nullptr;
       if (pub) {
         const TriPtrs p = tri_ptrs(a, b);
-        Cb = (t & 1) ? p.C1 : p.C0;
+        Cb = p.C + (size_t)(t & (kTriBufs - 1)) * a.m;
       }
       double2 fa = make_double2(0.0, 0.0), fb = fa;
       if (upd) {
@@ -530,8 +646,8 @@ __device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, i
         }
         if (i == t + 1) x1 = xa;
         if (pub) {
-          Cb[i] = xa;
-          if (two) Cb[i2] = xb;
+          put_word(Cb + i, xa);
+          if (two) put_word(Cb + i2, xb);
         }
         ax = fma(xa.x, va.x, fma(xa.y, va.y, ax));      // conj(x) u
         ay = fma(xa.x, va.y, fma(-xa.y, va.x, ay));
@@ -547,7 +663,7 @@ __device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, i
       }
     }
     __syncthreads();                         // reflector t; the shares
-    if (c0 == 0 && hs.rescaled) {
+    if (c0 == 0 && hs.rescaled[t & 1]) {
       for (int k = 0; k < np; ++k) {
         const int b = a.tmem[tv.p0 + k], n = own[k].n;
         if (t > n - 2 || cur[b].scl == 1.0) continue;
@@ -558,6 +674,7 @@ __device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, i
       }
       __syncthreads();
     }
+    if (c0 == 0 && wid != 0) tri_unset(a, tv, t, own);
     if (wid == 0)
       for (int cj = lane; cj < cols; cj += 32) {
         int k, rest;
@@ -578,7 +695,7 @@ __device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, i
         const double ax = fma(x1.x, u1.x, fma(x1.y, u1.y, sc * z[0].x));
         const double ay = fma(x1.x, u1.y, fma(-x1.y, u1.x, sc * z[0].y));
         const TriPtrs p = tri_ptrs(a, b);
-        ((t & 1) ? p.P1 : p.P0)[j] = make_double2(ax, ay);
+        put_word(p.P + (size_t)(t & (kTriBufs - 1)) * a.m + j, make_double2(ax, ay));
         contrib[c0 + cj] = fma(uj.x, ax, uj.y * ay);   // Re(conj(u_t[j]) p_j)
       }
     if (c0 + kBodyItems < C) __syncthreads();
@@ -595,7 +712,7 @@ __device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, i
     const int cb = active_cols(o, t);
     double acc = 0.0;
     for (int i = 0; i < cb; ++i) acc += contrib[first + i];
-    sp_row(a, a.tmem[tv.p0 + k], t)[tv.gb] = acc;
+    put_word(sp_row(a, a.tmem[tv.p0 + k], t) + tv.gb, acc);
   }
   __syncwarp();
   for (int k = lane; k < np; k += 32)
@@ -640,8 +757,22 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_hh_tridiag(TriBatch a) {
         col[i] = x;
       }
     }
+    // nothing published yet
+    const TriPtrs p = tri_ptrs(a, b);
+    const double2 no = make_double2(unset(), unset());
+    for (int e = tid; e < own[k].ns * kTriBufs; e += nt) {
+      const size_t o = (size_t)(e % kTriBufs) * a.m + own[k].j0 + (e / kTriBufs) * tv.G;
+      put_word(p.P + o, no);
+      put_word(p.C + o, no);
+    }
+    if (tid < kTriBufs) put_word(sp_row(a, b, tid) + tv.gb, unset());
   }
-  __syncthreads();
+  if (tid == 0) hs.timeout[0] = hs.timeout[1] = 0;
+  if (tv.G == 1) {
+    __syncthreads();
+  } else if (!blocks_barrier(tv.bar, epoch, (unsigned)tv.G, a.status, a.spins)) {
+    return;
+  }
   for (int t = 0; t < nrun; ++t) {
     const int nact = count_active(own, np, t);
     const int lg = nact == 1 ? 4 : nact == 2 ? 3 : 2;
@@ -649,21 +780,13 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_hh_tridiag(TriBatch a) {
     int last = 0;                            // problems of the last round of heads
     for (int r0 = 0; r0 < nact; r0 += per) {
       if (r0 > 0) __syncthreads();
-      tri_heads(a, tv, r0, lg, t, dsm, hs, s_st, own);
+      if (!tri_heads(a, tv, r0, lg, t, dsm, hs, s_st, own)) return;
       last = nact - r0 < per ? nact - r0 : per;
     }
     tri_body(a, tv, t, lg, last, dsm, contrib, hs, s_st, own);
-    auto store = [&] {
-      if (tv.gb == t % tv.G) tri_store(a, tv, t, dsm, s_st, own);
-    };
-    if (t + 1 == nrun) {
-      store();
-    } else if (tv.G == 1) {
-      store();
-      __syncthreads();
-    } else if (!blocks_barrier(tv.bar, epoch, (unsigned)tv.G, a.status, a.spins, store)) {
-      return;
-    }
+    // (the next step's first loads wait for this one's values of every block)
+    __syncthreads();
+    if (tv.gb == t % tv.G) tri_store(a, tv, t, dsm, s_st, own);
   }
   if (tv.gb == 0 && tid == 0) {
     long long k = 0;
@@ -1300,7 +1423,7 @@ static sky_status wy_back(Ctx* c, int np, const int* idx, const int* n, double2*
     T[q] = c->d_small[5] + (size_t)b * c->small_slot;
     Zb[q] = Z[b];
     j.P[q] = P[q];
-    j.tau[q] = reinterpret_cast<const double2*>(a.T + (size_t)b * a.tslot + (size_t)a.m * a.m) + 4 * (size_t)a.m;
+    j.tau[q] = reinterpret_cast<const double2*>(a.T + (size_t)b * a.tslot + (size_t)a.m * a.m) + 2 * kTriBufs * (size_t)a.m;
     j.Y[q] = reinterpret_cast<const double*>(S2[q]);
     j.Z[q] = Zb[q];
     j.G[q] = S0[q];
@@ -1623,7 +1746,7 @@ static sky_status tri_group(Ctx* c, int np, const int* idx, const double2* const
   while (back_warps > 1 && (size_t)back_warps * zstride * sizeof(double2) > kTriSmemMax) back_warps >>= 1;
   a.S0 = c->d_eigA[0]; a.S1 = c->d_eigA[1]; a.S2 = c->d_eigV; a.slot = c->eig_slot;
   a.T = c->d_trid; a.tslot = c->tri_slot; a.m = c->tri_m;
-  a.sp = c->d_eigpart; a.sp_stride = (size_t)2 * c->eig_grid_max;
+  a.sp = c->d_eigpart; a.sp_stride = (size_t)kTriBufs * c->eig_grid_max;
   a.run = run; a.run_stride = run_stride;
   a.bar = c->d_bar; a.status = c->d_status; a.spins = c->wait_spins; a.stats = c->d_stats;
   // run flags are indexed by the batch position of each problem
