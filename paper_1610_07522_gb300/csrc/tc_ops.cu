@@ -137,13 +137,20 @@ int tc_nsplit(sky_prec p) { return p == SKY_F32_BF16X6 ? 3 : 2; }
 // in L2 (kSmallPartials), they are half as long: it costs nothing there (small
 // boxes have too few tiles to fill the GPU otherwise) and halves the error (12^3,
 // 43 states: the energy 5e-5 MeV per nucleon from that of 64-value partials
-// with 2048, 2e-5 with 1024).
+// with 2048, 2e-5 with 1024).  The six products of the x6 form, which is there for
+// its accuracy, take half-length partials up to 1 GB of them: the diagonal's
+// truncation is 1.1e-5 with 2048 values in either form (32^3, 700 states), 7e-6 with
+// 1024, which the recombination's own (1.1e-5 before, 3.9e-6 with the states read
+// as stored) no longer hides.
 constexpr long long kMaxAccK = 2048;
-constexpr long long kSmallPartials = 4LL << 20;   // fp32 values of all partials
-int tc_min_splits(long long K, int I) {
-  const long long z = (K + kMaxAccK / 2 - 1) / (kMaxAccK / 2);
+static long long half_partials(int nsplit) {      // fp32 values of all partials
+  return nsplit == 3 ? 256LL << 20 : 4LL << 20;
+}
+static long long half_splits(long long K) { return (K + kMaxAccK / 2 - 1) / (kMaxAccK / 2); }
+int tc_min_splits(long long K, int I, int nsplit) {
+  const long long z = half_splits(K);
   const long long ldd = (2LL * I + 3) / 4 * 4;
-  return (int)(z * I * ldd <= kSmallPartials ? z : (K + kMaxAccK - 1) / kMaxAccK);
+  return (int)(z * I * ldd <= half_partials(nsplit) ? z : (K + kMaxAccK - 1) / kMaxAccK);
 }
 
 // Scratch (bf16 elements per piece / fp32 partials) for I states of V complex.
@@ -160,8 +167,11 @@ void tc_scratch_sizes(int I, long long V, int num_sms, size_t* piece_a, size_t* 
   if (z < zacc) z = zacc;
   if (z < 1) z = 1;
   *partial = (size_t)z * I * ldd;
-  // fewer states may take more splits (kSmallPartials values at most)
-  if (*partial < (size_t)kSmallPartials) *partial = (size_t)kSmallPartials;
+  // half-length partials of these states, or of fewer, as x6 takes them (a context can
+  // change between the forms)
+  const long long half = half_splits(K) * I * ldd, most = half_partials(3);
+  const size_t need = (size_t)(half < most ? half : most);
+  if (*partial < need) *partial = need;
 }
 
 sky_status tc_overlap(Ctx* c, const void* a, const void* b, int I, double2* X) {
@@ -184,7 +194,7 @@ sky_status tc_overlap(Ctx* c, const void* a, const void* b, int I, double2* X) {
   // tc_waves 0: the fewest splits the accumulation bound allows (for boxes
   // that share the GPU with others), else about that many waves of SMs
   int z = c->tc_waves * c->num_sms / tiles;
-  if (z < tc_min_splits(K, I)) z = tc_min_splits(K, I);   // bounded FP32 accumulation length
+  if (z < tc_min_splits(K, I, n)) z = tc_min_splits(K, I, n);   // bounded FP32 accumulation length
   if (z < 1) z = 1;
   const long long sstride = (long long)I * ldd;
   if ((size_t)z * sstride > c->tc_partial_elems) z = (int)(c->tc_partial_elems / sstride);
