@@ -181,7 +181,7 @@ __device__ __forceinline__ void warp_sum2(double& x, double& y) {
 //  - norm, beta and tau are formed while the other warps update their columns:
 //    these need only row t + 1 of u from it, whose term is added at the end;
 //  - a block's columns are split over its warps by rows.
-// With the published values as flags (kUnset) 700 + 300 states take 9.3 ms instead
+// With the published values as flags (kUnset) 700 + 300 states take 8.9 ms instead
 // of 12.0 ms, 280 + 120 states 2.4 instead of 3.3 ms.
 // The per-step vectors of a problem are short (n - t entries): its head work
 // runs on a group of 16, 8 or 4 warps for one, two or more problems left, and the
@@ -194,6 +194,9 @@ constexpr int kTabProbs = 4;            // problems of a team whose a_j, b_j are
 constexpr int kTabCols = 31;            // own columns of them
 constexpr int kBodyItems = 64;          // column shares per pass of tri_body
 constexpr int kMaxParts = 8;            // row shares of a column at most
+constexpr int kPartWarps = 4;           // warps that share the block's columns, if fewer (each
+                                        // costs a sum over its lanes; 700 states: 8.42 ms
+                                        // with 4, 8.45 with 6, 8.56 with 9, 8.75 with 15 shares)
 
 __device__ __forceinline__ TeamView team_view(const TriBatch& a) {
   const int k = find_prob(a.tg0, a.nteam, (int)blockIdx.x);
@@ -230,7 +233,7 @@ __device__ __forceinline__ double* sp_row(const TriBatch& a, int b, int t) {
 // their own flags: a reader takes a word once it no longer holds kUnset, a
 // signalling NaN that no arithmetic returns.  That is one trip through L2 per
 // step, where a barrier costs the writers' fence, its counter, the poll and then
-// the loads: 7.9 -> 7.4 us a step at 120 states, 13.2 -> 12.5 us at 700.  The values of step t are in buffer t mod 4; while step t is under way its owners
+// the loads: 7.9 -> 7.4 us a step at 120 states, 13.2 -> 12.5 us at 700 when it came.  The values of step t are in buffer t mod 4; while step t is under way its owners
 // unset their words of buffer t + 2 mod 4, last read at step t - 1: everyone is
 // past that, since everyone's partial of step t - 1 was read here, and nobody
 // looks for them before it has read the owner's partial of step t + 1, published
@@ -314,6 +317,28 @@ __device__ __forceinline__ int count_active(const TriOwn* own, int np, int t) {
   for (int k = 0; k < np; ++k) c += t < own[k].n;
   return c;
 }
+// A warp group's problem in tri_heads (k < 0: none), found again only when the
+// number of problems at work changes: the walk to it and its pointers took 1000
+// cycles of each step.
+struct TriHead {
+  int k, b, n;
+  double2* vb;                              // work vectors
+  double2 *P, *C;
+  double* sp;
+};
+__device__ __forceinline__ TriHead head_of(const TriBatch& a, const TeamView& tv, const TriOwn* own,
+                                           int t, int r, double2* dsm) {
+  TriHead h;
+  h.k = nth_active(own, tv.p1 - tv.p0, t, r);
+  h.b = h.k >= 0 ? a.tmem[tv.p0 + h.k] : 0;
+  h.n = h.k >= 0 ? own[h.k].n : 0;
+  const TriPtrs p = tri_ptrs(a, h.b);
+  h.vb = h.k >= 0 ? vec_base(a, h.b, dsm) : dsm;
+  h.P = p.P;
+  h.C = p.C;
+  h.sp = sp_row(a, h.b, 0);
+  return h;
+}
 // Active own columns of a problem at step t (none at its last).
 __device__ __forceinline__ int active_cols(const TriOwn& o, int t) {
   return t < o.n - 1 ? o.ns - o.smin : 0;
@@ -334,8 +359,8 @@ __device__ __forceinline__ double2 column_update(double2 x, double2 u, double2 p
       fma(-u.x, fa.y, fma(-u.y, fa.x, fma(-p.x, fb.y, fma(-p.y, fb.x, x.y)))));
 }
 
-// Heads of the problems at active positions r0 .. r0 + 16 / gw - 1, step t, every
-// block of the team alike, gw = 2^lg warps each: column t of the trailing matrix
+// The heads of a round's problems (h: this warp group's; 2^lg warps each), step t,
+// every block of the team alike: column t of the trailing matrix
 // (updated by reflector t-1 from the published copy) into vn, the published p
 // into w, and reflector t.  vo = u_{t-1}.  u_{t-1}^H p_{t-1} is the sum of the
 // owners' published per-block partials (the same order in every block).  The
@@ -343,17 +368,15 @@ __device__ __forceinline__ double2 column_update(double2 x, double2 u, double2 p
 // The group's first warp ends with reflector t after the last barrier here: its
 // results, u_{t+1} among them, are there after the next one.  False (in every
 // thread) when a wait ran out.
-__device__ bool tri_heads(const TriBatch& a, const TeamView& tv, int r0, int lg, int t, double2* dsm,
-                          HeadShared& hs, TriStep* s_st, const TriOwn* own) {
+__device__ bool tri_heads(const TriBatch& a, const TeamView& tv, const TriHead& h, bool first, int lg,
+                          int t, HeadShared& hs, TriStep* s_st, const TriOwn* own) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int q = wid >> lg, hwarp = wid & ((1 << lg) - 1), HT = 32 << lg, ht = hwarp * 32 + lane;
-  const int k = nth_active(own, tv.p1 - tv.p0, t, r0 + q);
+  const int k = h.k, b = h.b, n = h.n;
   const bool on = k >= 0;
-  const int b = on ? a.tmem[tv.p0 + k] : 0, n = on ? own[k].n : 0;
-  double2* vb = on ? vec_base(a, b, dsm) : dsm;
-  double2* vn = vb + (size_t)(t & 1) * n;
-  const double2* vo = vb + (size_t)((t + 1) & 1) * n;
-  double2* w = vb + 2 * (size_t)n;
+  double2* vn = h.vb + (size_t)(t & 1) * n;
+  const double2* vo = h.vb + (size_t)((t + 1) & 1) * n;
+  double2* w = h.vb + 2 * (size_t)n;
   double sg = 0.0;                           // |column|^2 below the subdiagonal
   TriWait wt{a.status, a.spins, true};
   if (t == 0) {
@@ -364,14 +387,12 @@ __device__ bool tri_heads(const TriBatch& a, const TeamView& tv, int r0, int lg,
       vn[i] = x;
       if (i >= 2) sg = fma(x.x, x.x, fma(x.y, x.y, sg));
     }
-    if (r0 == 0 && threadIdx.x == 0) hs.rescaled[t & 1] = 0;
+    if (first && threadIdx.x == 0) hs.rescaled[t & 1] = 0;
   } else {
     double2 xp[kHeadLoad], xc[kHeadLoad];
-    const double2 *Pp = nullptr, *Cp = nullptr;
+    const double2* Pp = h.P + (size_t)((t - 1) & (kTriBufs - 1)) * a.m;
+    const double2* Cp = h.C + (size_t)((t - 1) & (kTriBufs - 1)) * a.m;
     if (on) {
-      const TriPtrs p = tri_ptrs(a, b);
-      Pp = p.P + (size_t)((t - 1) & (kTriBufs - 1)) * a.m;
-      Cp = p.C + (size_t)((t - 1) & (kTriBufs - 1)) * a.m;
 #pragma unroll
       for (int r = 0; r < kHeadLoad; ++r) {
         const int i = t + ht + r * HT;
@@ -382,7 +403,7 @@ __device__ bool tri_heads(const TriBatch& a, const TeamView& tv, int r0, int lg,
       }
       if (hwarp == 0) {
         // lanes 0 .. 30: own columns; lane 31: column t
-        const double* ps = sp_row(a, b, t - 1);
+        const double* ps = h.sp + (size_t)((t - 1) & (kTriBufs - 1)) * gridDim.x;
         const int cb = active_cols(own[k], t);
         const int j = lane == 31 ? t : lane < cb ? own[k].j0 + (own[k].smin + lane) * tv.G : -1;
         double2 pj = j >= 0 ? get_word(Pp + j) : make_double2(0.0, 0.0);
@@ -437,7 +458,7 @@ __device__ bool tri_heads(const TriBatch& a, const TeamView& tv, int r0, int lg,
       }
       __syncwarp();
     }
-    if (r0 == 0 && threadIdx.x == 0) hs.rescaled[t & 1] = 0;
+    if (first && threadIdx.x == 0) hs.rescaled[t & 1] = 0;
     if (!wt.ok) hs.timeout[0] = 1;
     __syncthreads();
     if (hs.timeout[0]) return false;
@@ -582,8 +603,8 @@ __device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, i
     C += active_cols(own[k], t);
     mmax = own[k].n - t > mmax ? own[k].n - t : mmax;
   }
-  // at least two rows per lane and share; no more shares than warps
-  int parts = C > 0 ? (kTriWarps - 1) / C : 1;
+  // at least two rows per lane and share
+  int parts = C > 0 ? (kPartWarps + C - 1) / C : 1;
   const int most = (mmax + 63) >> 6;
   parts = parts > most ? most : parts;
   parts = parts < 1 ? 1 : parts > kMaxParts ? kMaxParts : parts;
@@ -773,6 +794,8 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_hh_tridiag(TriBatch a) {
   } else if (!blocks_barrier(tv.bar, epoch, (unsigned)tv.G, a.status, a.spins)) {
     return;
   }
+  TriHead h{};
+  int seen = -1;
   for (int t = 0; t < nrun; ++t) {
     const int nact = count_active(own, np, t);
     const int lg = nact == 1 ? 4 : nact == 2 ? 3 : 2;
@@ -780,7 +803,9 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_hh_tridiag(TriBatch a) {
     int last = 0;                            // problems of the last round of heads
     for (int r0 = 0; r0 < nact; r0 += per) {
       if (r0 > 0) __syncthreads();
-      if (!tri_heads(a, tv, r0, lg, t, dsm, hs, s_st, own)) return;
+      if (nact != seen || nact > per) h = head_of(a, tv, own, t, r0 + (tid >> (5 + lg)), dsm);
+      seen = nact;
+      if (!tri_heads(a, tv, h, r0 == 0, lg, t, hs, s_st, own)) return;
       last = nact - r0 < per ? nact - r0 : per;
     }
     tri_body(a, tv, t, lg, last, dsm, contrib, hs, s_st, own);
