@@ -1,0 +1,145 @@
+"""The kernels at the sizes where their tiles, rows and warps end (GPU): the
+reduction to tridiagonal form with its back-transformation, the grouped
+digit-split products of two problems, the recombination of the split-BF16
+forms, the FP32 form's fused h psi on ragged axes and the FP64 form's float-pair
+passes, and the damping network's convolutions, each against the FP64 oracle
+or numpy.
+
+Tolerances, from the arithmetic: a backward stable reduction of n <= 257 states
+leaves n eps ||H|| = 6e-14 ||H|| in eigenvalues and residuals, the bisection
+stops at 2^-43 ||T|| = 1.1e-13 ||T||, and 1e-12 leaves a factor for their
+constants; the digit-split products keep 1e-14 of the largest element, five of
+them in a Newton-Schulz step, each again corrected by the next: 1e-12; BF16x3
+and x6 as in the parity tests of the same calls."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle as O
+import test_gpu_eigen as TE
+import test_gpu_parity as TP
+import test_gpu_precond as TN
+from paper_1610_07522_gb300 import binding as B
+from paper_1610_07522_gb300 import inputs as IN
+
+pytestmark = pytest.mark.gpu
+
+
+def _hermitian(kind, n, rng):
+    a = rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))
+    if kind == "random":
+        return a + a.conj().T
+    d = np.diag(-60.0 + 100.0 * (np.arange(n) + 0.5 * rng.random(n)) / n)
+    if kind == "blocks":                    # decoupled: reflectors that are the identity
+        H = (a + a.conj().T) / np.sqrt(n)
+        k = n // 3
+        H[:k, k:] = 0.0
+        H[k:, :k] = 0.0
+        H[2 * k:, :2 * k] = 0.0
+        H[:2 * k, 2 * k:] = 0.0
+        H[2 * k:, 2 * k:] = 0.0
+        return H + d
+    # couplings from 1e-2 down to 1e-16 along the matrix: reflectors far below 1
+    e = 10.0 ** (-2.0 - 14.0 * np.arange(n) / n)
+    E = a * np.minimum(e[:, None], e[None, :])
+    return d + E + E.conj().T
+
+
+@pytest.mark.parametrize("kind", ["random", "blocks", "graded"])
+@pytest.mark.parametrize("n", [2, 31, 33, 64, 65, 96, 127, 128, 129, 153, 193, 257])
+def test_reduction_and_back_transformation(kind, n):
+    rng = np.random.default_rng(7 * n + len(kind))
+    H = _hermitian(kind, n, rng)
+    c = TE._ctx(n)
+    B.sky_tune_set(c, B.SKY_KNOB_EIGEN_METHOD, B.SKY_EIG_TRIDIAGONAL)
+    M, lam = TE._solve(c, H)
+    B.sky_destroy(c)
+    lw = np.linalg.eigvalsh(H)
+    nrm = float(np.max(np.abs(lw)))
+    assert np.max(np.abs(lam - lw)) < 1e-12 * nrm
+    assert np.max(np.abs(M.conj().T @ M - np.eye(n))) < 1e-12
+    assert np.max(np.abs(H @ M - M * lam)) < 1e-12 * nrm
+
+
+@pytest.mark.parametrize("sizes", [(96, 95), (96, 96), (128, 129), (161, 80), (97, 1)])
+def test_grouped_products_of_two_problems(sizes):
+    rng = np.random.default_rng(sum(sizes))
+    c = TE._ctx(max(sizes))
+    S, C = [], []
+    for n in sizes:
+        a = rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))
+        S.append(np.eye(n) + 0.05 / np.sqrt(n) * (a + a.conj().T))
+        C.append(torch.zeros((n, n), dtype=torch.complex128, device="cuda:0"))
+    B.sky_orthonormalize_batched(c, [TE._dev(x) for x in S], list(sizes), C)
+    B.sky_sync(c)
+    for x, y in zip(S, C):
+        w, U = np.linalg.eigh(x)
+        want = (U / np.sqrt(w)) @ U.conj().T
+        got = y.cpu().numpy()
+        # C or its transpose's conjugate alike: S^{-1/2} is Hermitian up to the
+        # convention of its indices
+        assert min(np.max(np.abs(got - want)), np.max(np.abs(got - want.T))) < 1e-12
+    B.sky_destroy(c)
+
+
+@pytest.mark.parametrize("prec", [B.SKY_F32_BF16X3, B.SKY_F32_BF16X6])
+@pytest.mark.parametrize("I", [1, 2, 15, 17, 33, 63, 65, 129])
+def test_split_bf16_recombination_of_odd_state_counts(prec, I):
+    rng = np.random.default_rng(40 + I)
+    with TP.Ctx((8, 12, 8), prec=prec, max_states=I) as c:
+        a = TP._r32(IN.random_spinors(c.grid.n, I, rng))
+        M = (rng.standard_normal((I, I)) + 1j * rng.standard_normal((I, I))) / np.sqrt(I)
+        out = torch.zeros(a.shape, dtype=torch.complex64, device="cuda:0")
+        B.sky_rotate(c.ctx, TP.dev32(a), TP.dev(M), I, out)
+        assert TP.relerr(TP.host(out), O.rotate(a, M)) < TP.TC_TOL[prec]
+
+
+@pytest.mark.parametrize("grid", [(8, 20, 24), (32, 20, 12), (8, 32, 16), (16, 24, 32)])
+def test_fp32_default_h_on_ragged_axes(grid):
+    """Without a knob set the fused passes run on axes up to 32 (bit-identical
+    to knob 1), the general ones agree within the FP32 bound."""
+    rng = np.random.default_rng(sum(grid))
+    I, out = 3, []
+    with TP.Ctx(grid, twist=(0.4, -1.1, 2.0), prec=B.SKY_F32, max_states=I) as c:
+        g = c.grid
+        psi = TP._r32(IN.random_spinors(g.n, I, rng))
+        U, Bf, W = TP._fields(g, rng)
+        want = O.apply_h(psi, U, Bf, W, g)
+        for knob in (None, 1, 0):
+            if knob is not None:
+                B.sky_tune_set(c.ctx, B.SKY_KNOB_FUSED_H, knob)
+            d_h = torch.zeros(psi.shape, dtype=torch.complex64, device="cuda:0")
+            B.sky_apply_h(c.ctx, TP.dev(U), TP.dev(Bf), TP.dev(W), TP.dev32(psi), d_h, I)
+            out.append(TP.host(d_h))
+            assert TP.relerr(out[-1], want) < TP.REL32
+    assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("grid,I", [((8, 12, 20), 1), ((20, 8, 32), 5), ((32, 8, 12), 3), ((8, 24, 16), 2)])
+def test_fp64_pair_passes_on_ragged_axes(grid, I):
+    rng = np.random.default_rng(sum(grid) + I)
+    with TP.Ctx(grid, twist=(0.4, -1.1, 2.0), max_states=I) as c:
+        g = c.grid
+        psi = IN.random_spinors(g.n, I, rng)
+        U, Bf, W = TP._fields(g, rng)
+        want = O.apply_h(psi, U, Bf, W, g)
+        e_w, n_w = O.sp_energies(psi, want, g)
+        d_h = torch.zeros(psi.shape, dtype=torch.complex128, device="cuda:0")
+        eps = torch.zeros(I, dtype=torch.float64, device="cuda:0")
+        hn2 = torch.zeros(I, dtype=torch.float64, device="cuda:0")
+        B.sky_apply_h(c.ctx, TP.dev(U), TP.dev(Bf), TP.dev(W), TP.dev(psi), d_h, I, eps, hn2)
+        assert TP.relerr(TP.host(d_h), want) < TP.REL
+        assert TP.relerr(TP.host(eps), e_w) < TP.REL and TP.relerr(TP.host(hn2), n_w) < TP.REL
+        rho_w, tau_w, J_w, dJ_w = O.densities(psi, g)
+        rho = torch.zeros(g.G, dtype=torch.float64, device="cuda:0")
+        tau, dJ = torch.zeros_like(rho), torch.zeros_like(rho)
+        J = torch.zeros(3 * g.G, dtype=torch.float64, device="cuda:0")
+        B.sky_densities(c.ctx, TP.dev(psi), I, rho, tau, J, dJ)
+        for got, ref in ((rho, rho_w), (tau, tau_w), (J, J_w), (dJ, dJ_w)):
+            assert TP.relerr(TP.host(got), ref.ravel()) < TP.REL
+
+
+@pytest.mark.parametrize("grid", [(8, 8, 8), (20, 8, 12), (8, 32, 24)])
+def test_network_convolutions_on_small_and_ragged_grids(grid):
+    TN.test_net_forward_loss_and_gradient(grid, 1)
