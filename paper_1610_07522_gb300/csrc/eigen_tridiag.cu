@@ -76,7 +76,7 @@ struct TriBatch {
   int off[kMaxBatch + 1];        // prefix sums of n: eigenvalue / column items
   int sid[kMaxBatch];            // workspace slot of each problem
   int np;
-  double2* S0;                   // per problem: own columns (global home), later U0, U1
+  double2* S0;                   // per problem: own columns (global home), later U0
   double2* S1;                   // per problem: reflectors V[t * n + i]
   double2* S2;                   // per problem: Y and its Loewdin ping-pong buffer
   size_t slot;                   // double2 per problem in S0, S1, S2
