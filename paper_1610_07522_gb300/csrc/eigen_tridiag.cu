@@ -233,11 +233,19 @@ __device__ __forceinline__ double* sp_row(const TriBatch& a, int b, int t) {
 // their own flags: a reader takes a word once it no longer holds kUnset, a
 // signalling NaN that no arithmetic returns.  That is one trip through L2 per
 // step, where a barrier costs the writers' fence, its counter, the poll and then
-// the loads: 7.9 -> 7.4 us a step at 120 states, 13.2 -> 12.5 us at 700 when it came.  The values of step t are in buffer t mod 4; while step t is under way its owners
-// unset their words of buffer t + 2 mod 4, last read at step t - 1: everyone is
-// past that, since everyone's partial of step t - 1 was read here, and nobody
-// looks for them before it has read the owner's partial of step t + 1, published
-// after the fence behind the unsetting.  Every wait is bounded.
+// the loads: 7.9 -> 7.4 us a step at 120 states, 13.2 -> 12.5 us at 700 when it came.
+// The values of step t are in buffer t mod 4; while step t is under way its owners
+// unset their words of buffer t + 2 mod 4, last read at step t - 1.  Two things
+// order that, both by one fence of the heads' first warps (the ones that read and
+// publish the partials) between the heads of a step and its partials:
+//  - everyone is past those reads: each block's fence stands between its reads of
+//    step t - 1 and its partial of that step, and the partials were read here, a
+//    fence and a barrier before the unsetting;
+//  - nobody takes an old word of buffer t + 2 for a new one: its reads come at step
+//    t + 3, behind the fence and the barrier of step t + 2, whose head read the
+//    owner's partial of step t + 1, which the owner published after the barrier
+//    behind the unsetting and the fence of step t + 1.
+// Every wait is bounded.
 constexpr unsigned long long kUnset = 0x7FF4000000C0FFEEull;
 __device__ __forceinline__ double unset() { return __longlong_as_double((long long)kUnset); }
 __device__ __forceinline__ bool is_unset(double x) {
@@ -583,7 +591,6 @@ __device__ __forceinline__ void tri_unset(const TriBatch& a, const TeamView& tv,
     if ((t + 3 + a.rot[b]) % tv.G == tv.gb)
       for (int i = t + 3 + tid; i < n; i += kTriThreads - 32) put_word(p.C + o + i, no);
   }
-  __threadfence();
 }
 
 // Own columns j >= t+1: update by reflector t-1 (rows > t), p_j = col_j^H u_t,
@@ -598,6 +605,7 @@ __device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, i
   const int grp = wid >> lg;
   const int rank = grp >= ng ? wid - ng
                              : (wid & ((1 << lg) - 1)) == 0 ? kTriWarps - ng + grp : wid - grp - 1;
+  if ((wid & ((1 << lg) - 1)) == 0) __threadfence();   // see kUnset
   int C = 0, mmax = 0;
   for (int k = 0; k < np; ++k) {
     C += active_cols(own[k], t);
