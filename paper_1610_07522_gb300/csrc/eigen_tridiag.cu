@@ -1061,8 +1061,8 @@ __device__ __forceinline__ void tri_forward(const TriCol& c, int n, double scale
   const size_t sn = (size_t)n;
   double rc = scale * *c.Y;
   const double* __restrict__ L = c.L;
-  const double* __restrict__ R = c.Y + sn;   // row i + 1
-  double* __restrict__ W = c.Y;
+  const double* R = c.Y + sn;   // row i + 1
+  double* W = c.Y;
   auto row = [&](double lv, double r0) {
     const double rn = scale * r0;
     const bool piv = piv_of(lv);
@@ -1103,8 +1103,8 @@ __device__ __forceinline__ double tri_backward(const TriCol& c, const double* __
   const size_t sn = (size_t)n;
   const double2* __restrict__ U = c.U + (size_t)(n - 1) * sn;
   const double* __restrict__ L = c.L + (size_t)(n - 1) * sn;
-  const double* __restrict__ R = c.Y + (size_t)(n - 1) * sn;
-  double* __restrict__ W = c.Y + (size_t)(n - 1) * sn;
+  const double* R = c.Y + (size_t)(n - 1) * sn;
+  double* W = c.Y + (size_t)(n - 1) * sn;
   double y1 = 0.0, y2 = 0.0, s0 = 0.0, s1 = 0.0;   // y[i+1], y[i+2]
   auto row = [&](double y, double r, double u1, double u2) {
     const double yi = fma(-u1, y1, fma(-u2, y2, y)) * r;
