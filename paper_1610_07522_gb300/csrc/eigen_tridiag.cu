@@ -782,7 +782,9 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_hh_tridiag(TriBatch a) {
       double2* col = own_col(a, b, dsm, j, s);
       for (int i = tid; i < n; i += nt) {
         double2 x = A[(size_t)j * n + i];
-        x.y = i == j ? 0.0 : -x.y;
+        // (step 0 publishes column 1 as it came: no input may look unset)
+        if (is_unset(x.x)) x.x = NAN;
+        x.y = i == j ? 0.0 : is_unset(x.y) ? NAN : -x.y;
         col[i] = x;
       }
     }

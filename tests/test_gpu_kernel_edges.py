@@ -143,3 +143,20 @@ def test_fp64_pair_passes_on_ragged_axes(grid, I):
 @pytest.mark.parametrize("grid", [(8, 8, 8), (20, 8, 12), (8, 32, 24)])
 def test_network_convolutions_on_small_and_ragged_grids(grid):
     TN.test_net_forward_loss_and_gradient(grid, 1)
+
+
+def test_input_that_looks_like_an_unset_word_does_not_stall_the_reduction():
+    """The reduction's published values are their own flags (a signalling NaN means
+    not there yet) and its first step publishes a column as it came: the same
+    pattern in the input has to end as any NaN does, not in a wait that runs out."""
+    n = 150
+    S = 4.0 * np.eye(n, dtype=np.complex128)
+    S[0, 1:5] = S[1:5, 0] = 0.5
+    S.view(np.uint64)[[1, 3], [2 * 3, 2 * 1]] = 0x7FF4000000C0FFEE     # S[1, 3], S[3, 1]
+    c = TE._ctx(n)
+    C = torch.zeros((n, n), dtype=torch.complex128, device="cuda:0")
+    B.sky_orthonormalize(c, TE._dev(S), n, C)
+    with pytest.raises(B.SkyError) as ei:
+        B.sky_sync(c)
+    assert ei.value.status in (B.SKY_ENOTPD, B.SKY_ENOCONV)   # (SKY_ETIMEOUT would come first)
+    B.sky_destroy(c)
