@@ -829,7 +829,9 @@ sky_status lowdin_batch(Ctx* c, int np, const double2* const* S, const int* I, d
         rj[b] = run[k];
         Ij[b] = I[k];
       }
-      st = zgemm_batch(c, zjobs(nj, false, false, Aj, Bj, Cj, Ij, rj, none));
+      ZJobs both = zjobs(nj, false, false, Aj, Bj, Cj, Ij, rj, none);
+      both.probs = np;
+      st = zgemm_batch(c, both);
     } else {
       st = zgemm_batch(c, zjobs(np, false, false, Y0, (const double2* const*)j.W, Y1, I, run, none));
       if (st == SKY_OK && it > 0)

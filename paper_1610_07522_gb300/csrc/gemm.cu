@@ -186,7 +186,7 @@ ZJobs zjobs(int np, bool ah, bool bh, const double2* const* A, const double2* co
             double2* const* C, const int* n, const int* const* run, const int* const* stop,
             int slices) {
   ZJobs j;
-  j.np = np; j.ah = ah; j.bh = bh; j.slices = slices;
+  j.np = j.probs = np; j.ah = ah; j.bh = bh; j.slices = slices;
   for (int b = 0; b < kMaxBatch; ++b) {
     const bool in = b < np;
     j.A[b] = in ? A[b] : nullptr;
@@ -280,15 +280,26 @@ static void launch_zgemm(Ctx* c, const ZJobs& j, int nmax) {
 }
 
 sky_status zgemm_batch(Ctx* c, const ZJobs& jin) {
-  // several problems: every product in one grouped tensor-core launch sequence
+  // several products: all in one grouped tensor-core launch sequence
   // (oz_zgemm_group), when its buffers hold them.  Up to kOzGroupMin problems
   // only when one has kOzZgemmMin states or more: four launches for all (280 +
   // 120 states: 25 us) instead of four for each large one and an FP64 launch for
-  // the rest (21 + 75 us); batches of small problems stay with the one FP64 launch
+  // the rest (21 + 75 us); batches of small problems stay with the one FP64
+  // launch.  A problem that alone would take FP64 keeps that accuracy: its group
+  // takes seven digits.  (With six, S^{-1/2} of 120 states, alone or beside 280, is
+  // 7e-13 off where FP64 leaves 1.4e-15: Frobenius norm of C S C^H - I over sqrt(n).)
   int nbig = 0;
-  for (int b = 0; b < jin.np; ++b) nbig = jin.n[b] > nbig ? jin.n[b] : nbig;
-  if (jin.np > 1 && (jin.np > kOzGroupMin || nbig >= kOzZgemmMin) && oz_zgemm_group_fits(c, jin.np, jin.n, jin.slices))
-    return oz_zgemm_group(c, jin);
+  bool small = false;
+  for (int b = 0; b < jin.np; ++b) {
+    nbig = jin.n[b] > nbig ? jin.n[b] : nbig;
+    small |= jin.n[b] < (jin.run[b] || jin.stop[b] ? kOzZgemmGated : kOzZgemmMin);
+  }
+  const bool many = jin.probs > kOzGroupMin;
+  if (jin.np > 1 && (many || nbig >= kOzZgemmMin)) {
+    ZJobs j = jin;
+    if (small && !many) j.slices = 7;
+    if (oz_zgemm_group_fits(c, j.np, j.n, j.slices)) return oz_zgemm_group(c, j);
+  }
   // problems of kOzZgemmMin states or more: tensor-core digit-split products
   // (one launch sequence each, gated like the rest); the others in one
   // batched FP64 launch

@@ -211,6 +211,7 @@ struct ZJobs {
   const int* run[kMaxBatch];
   const int* stop[kMaxBatch];
   int np;
+  int probs;                        // problems they belong to (np, or half as many)
   bool ah, bh;
   int slices;                       // tensor-core products: 6 digits, or 7 (FP64's whole mantissa)
 };

@@ -160,3 +160,28 @@ def test_input_that_looks_like_an_unset_word_does_not_stall_the_reduction():
         B.sky_sync(c)
     assert ei.value.status in (B.SKY_ENOTPD, B.SKY_ENOCONV)   # (SKY_ETIMEOUT would come first)
     B.sky_destroy(c)
+
+
+@pytest.mark.parametrize("sizes", [(120,), (191,), (96, 95), (280, 120), (161, 80), (97, 1), (192, 60, 130)])
+def test_loewdin_factors_of_problems_too_small_for_six_digits(sizes):
+    """S^{-1/2} in the oracle's index convention; problems below 192 states, whose
+    Newton-Schulz products alone are FP64, keep that accuracy beside larger ones:
+    n eps (FP64 sums of n terms, each step corrected by the next) and 16 eps where
+    that is less; the others the six digits' 1e-12."""
+    rng = np.random.default_rng(sum(sizes))
+    c = TE._ctx(max(sizes))
+    B.sky_reserve_batch(c, len(sizes))
+    S, C = [], []
+    for n in sizes:
+        a = rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))
+        S.append(np.eye(n) + 0.05 / np.sqrt(n) * (a + a.conj().T))
+        C.append(torch.zeros((n, n), dtype=torch.complex128, device="cuda:0"))
+    B.sky_orthonormalize_batched(c, [TE._dev(x) for x in S], list(sizes), C)
+    B.sky_sync(c)
+    for n, x, y in zip(sizes, S, C):
+        got = y.cpu().numpy()
+        eps = np.finfo(float).eps
+        tol = max(n, 16) * eps if n < 192 else 1e-12
+        assert np.max(np.abs(got @ x @ got.conj().T - np.eye(n))) < tol
+        assert np.max(np.abs(got - O.loewdin(x))) < (8 * tol if n < 192 else tol)
+    B.sky_destroy(c)
