@@ -239,11 +239,11 @@ sky_status sky_subspace_diag_literal_batched(sky_ctx* ctx, int nb, const double*
 
 /* Raise the batch capacity of the batched calls to nb problems of up to
  * max_states each (1 <= nb <= 128).  Allocates device memory (about
- * 9.5 max_states^2 complex doubles per problem; for nb > 8 also the digit
- * buffers of the grouped tensor-core I x I products, two of them per problem:
- * about 170 max_states bytes per problem and state plus 64 of partials, capped
- * at 2 GiB each) and
- * synchronises the context stream; call it outside stream capture.
+ * 9.5 max_states^2 complex doubles per problem; for nb > 8, or nb > 2 of 96
+ * states or more, also the digit buffers of the grouped tensor-core I x I
+ * products, two of them per problem: about 170 max_states bytes per problem and
+ * state plus 64 of partials, capped at 2 GiB each) and synchronises the context
+ * stream; call it outside stream capture.
  * SKY_ENOMEM leaves the context as it was. */
 sky_status sky_reserve_batch(sky_ctx* ctx, int nb);
 sky_status sky_subspace_diag_batched(sky_ctx* ctx, int nb, const double* const* H,

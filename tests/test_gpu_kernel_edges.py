@@ -185,3 +185,34 @@ def test_loewdin_factors_of_problems_too_small_for_six_digits(sizes):
         assert np.max(np.abs(got @ x @ got.conj().T - np.eye(n))) < tol
         assert np.max(np.abs(got - O.loewdin(x))) < (8 * tol if n < 192 else tol)
     B.sky_destroy(c)
+
+
+@pytest.mark.parametrize("sizes", [(128, 64, 130), (130, 97, 200, 128, 31, 60, 150, 129)])
+def test_diagonalisation_of_three_to_eight_problems(sizes):
+    """Batches of up to eight problems: the launches of one problem serve them all,
+    and the eigenvectors come back as those of single problems do."""
+    rng = np.random.default_rng(len(sizes))
+    H = [_hermitian("random", n, rng) for n in sizes]
+    z = lambda n: torch.zeros((n, n), dtype=torch.complex128, device="cuda:0")
+    launches = []
+    for batch in ([H[0]], H):
+        ns = [h.shape[0] for h in batch]
+        c = TE._ctx(max(sizes))
+        B.sky_reserve_batch(c, len(ns))
+        B.sky_tune_set(c, B.SKY_KNOB_EIGEN_METHOD, B.SKY_EIG_TRIDIAGONAL)
+        M, lam = [z(n) for n in ns], [torch.zeros(n, dtype=torch.float64, device="cuda:0") for n in ns]
+        l0 = B.sky_kernel_launches()
+        B.sky_subspace_diag_batched(c, [TE._dev(h) for h in batch],
+                                    [TE._dev(np.eye(n, dtype=np.complex128)) for n in ns], ns, M, lam)
+        launches.append(B.sky_kernel_launches() - l0)
+        B.sky_sync(c)
+        for h, m, w in zip(batch, M, lam):
+            m, w, lw = m.cpu().numpy(), w.cpu().numpy(), np.linalg.eigvalsh(h)
+            nrm = float(np.max(np.abs(lw)))
+            assert np.max(np.abs(w - lw)) < 1e-12 * nrm
+            assert np.max(np.abs(m.conj().T @ m - np.eye(len(w)))) < 1e-12
+            assert np.max(np.abs(h @ m - m * w)) < 1e-12 * nrm
+        B.sky_destroy(c)
+    # two more levels of block doubling at most (200 against 128 states), four
+    # launches a product and one of its own each
+    assert launches[1] <= launches[0] + 2 * (2 * 4 + 1), launches
