@@ -104,7 +104,7 @@ static sky_status alloc_tc_scratch(Ctx* c, int pieces) {
   const int Imax = c->max_states > 0 ? c->max_states : 1;
   const long long V = 2LL * c->G;
   size_t pa, pb, pra, part;
-  tc_scratch_sizes(Imax, V, c->num_sms, &pa, &pb, &pra, &part);
+  tc_scratch_sizes(Imax, V, c->num_sms, pieces, &pa, &pb, &pra, &part);
   sky_status s = SKY_OK;
   for (int k = 0; k < pieces && s == SKY_OK; ++k) {
     if (c->d_tcA[k]) continue;

@@ -253,7 +253,7 @@ sky_status subspace_impl(Ctx* c, const double2* H, const double2* C, int I, doub
                          double* eps);
 int jacobi_max_grid(Ctx* c);
 int tc_nsplit(sky_prec p);
-void tc_scratch_sizes(int I, long long V, int num_sms, size_t* piece_a, size_t* piece_b,
+void tc_scratch_sizes(int I, long long V, int num_sms, int nsplit, size_t* piece_a, size_t* piece_b,
                       size_t* piece_rot_a, size_t* partial);
 sky_status tc_overlap(Ctx* c, const void* a, const void* b, int I, double2* X);
 void oz_scratch_sizes(sky_prec prec, int Imax, long long V, int nsm, size_t* a_elems,

@@ -13,6 +13,9 @@
 //           own layout, psi = (P_re - Q_im, P_im + Q_re) per entry.
 #include <cuda_bf16.h>
 
+#include <cfloat>
+
+#include "dd.cuh"
 #include "tc_gemm.cuh"
 
 namespace sky {
@@ -108,20 +111,57 @@ __global__ void k_split_rot_a(const double2* __restrict__ M, int I, long long ld
   for (int i = 0; i < n; ++i) d[i][e] = s[i];
 }
 
-// X[a][b] = dV sum_z (D_z[a][b] + i D_z[a][I + b]) for a >= b, mirrored.
-__global__ void k_tc_overlap_reduce(const float* __restrict__ D, int nz, long long sstride,
-                                    long long ldd, int I, double dV, double2* X) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long long)I * I) return;
-  const int a = (int)(e / I), b = (int)(e % I);
-  if (a < b) return;
-  double re = 0.0, im = 0.0;
-  for (int z = 0; z < nz; ++z) {
-    const float* Dz = D + z * sstride + (long long)a * ldd;
-    re += Dz[b];
-    im += Dz[I + b];
+// A sum of floats to 72 bits: TwoSum into hi, its errors by TwoSum into mid, theirs
+// into lo.
+struct SumF3 {
+  float hi = 0.0f, mid = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add(float x) {
+    const dd s = two_sum(hi, x);
+    hi = s.hi;
+    const dd m = two_sum(mid, s.lo);
+    mid = m.hi;
+    lo = __fadd_rn(lo, m.lo);
   }
-  const double2 s = make_double2(dV * re, dV * im);
+  __device__ __forceinline__ double value() const { return (double)hi + ((double)mid + (double)lo); }
+};
+
+// X[a][b] (+)= dV sum_z (D_z[a][b] + i D_z[a][I + b]) for a >= b, mirrored.  In
+// FP64 the conversions and additions bound it (32^3, 700 states: 200 us with 64
+// partials, 395 us with 128); with triples of floats, which lose nothing against
+// FP64, the partials' bytes and latency do (33 and 68 us; 83 and 172 us without the
+// loads ahead of the sums).  A sum beyond the floats' range is formed again in FP64.
+constexpr int kRedLoads = 8;            // partials of a thread in flight
+__global__ void __launch_bounds__(128) k_tc_overlap_reduce(const float* __restrict__ D, int nz,
+                                                           long long sstride, long long ldd, int I,
+                                                           double dV, double2* X, int add) {
+  const int a = blockIdx.x, b = blockIdx.y * 128 + threadIdx.x;
+  if (b > a) return;
+  const float* Da = D + (long long)a * ldd + b;
+  SumF3 r, i;
+  for (int z0 = 0; z0 < nz; z0 += kRedLoads) {
+    float x[kRedLoads], y[kRedLoads];
+#pragma unroll
+    for (int k = 0; k < kRedLoads; ++k) {
+      const bool on = z0 + k < nz;
+      x[k] = on ? Da[(z0 + k) * sstride] : 0.0f;
+      y[k] = on ? Da[(z0 + k) * sstride + I] : 0.0f;
+    }
+#pragma unroll
+    for (int k = 0; k < kRedLoads; ++k) {
+      r.add(x[k]);
+      i.add(y[k]);
+    }
+  }
+  double re = r.value(), im = i.value();
+  if (!(fabsf(r.hi) <= FLT_MAX && fabsf(i.hi) <= FLT_MAX)) {
+    re = im = 0.0;
+    for (int z = 0; z < nz; ++z) {
+      re += (double)Da[z * sstride];
+      im += (double)Da[z * sstride + I];
+    }
+  }
+  double2 s = make_double2(dV * re, dV * im);
+  if (add) s = X[(long long)a * I + b] + s;
   X[(long long)a * I + b] = s;
   if (a != b) X[(long long)b * I + a] = conjx(s);
 }
@@ -132,29 +172,29 @@ int tc_nsplit(sky_prec p) { return p == SKY_F32_BF16X6 ? 3 : 2; }
 
 // FP32 accumulation in TMEM loses accuracy over long K (its rounding error
 // grows with the length of the sum): every split-K partial of the overlap
-// covers at most kMaxAccK values of K, and the partials are summed in FP64 by
+// covers at most kMaxAccK values of K, and the partials are summed to FP64 by
 // the reduce.  Where the partials of half that length are small enough to stay
 // in L2 (kSmallPartials), they are half as long: it costs nothing there (small
 // boxes have too few tiles to fill the GPU otherwise) and halves the error (12^3,
 // 43 states: the energy 5e-5 MeV per nucleon from that of 64-value partials
 // with 2048, 2e-5 with 1024).  The six products of the x6 form, which is there for
-// its accuracy, take half-length partials up to 1 GB of them: the diagonal's
-// truncation is 1.1e-5 with 2048 values in either form (32^3, 700 states), 7e-6 with
-// 1024, which the recombination's own (1.1e-5 before, 3.9e-6 with the states read
-// as stored) no longer hides.
+// its accuracy, always take half-length partials: the diagonal's truncation is
+// 1.1e-5 with 2048 values in either form (32^3, 700 states), 7e-6 with 1024, which
+// the recombination's own (3.9e-6) does not hide.  Where they do not fit the buffer
+// at once (kMostPartials), they are formed and summed in several rounds over K.
 constexpr long long kMaxAccK = 2048;
-static long long half_partials(int nsplit) {      // fp32 values of all partials
-  return nsplit == 3 ? 256LL << 20 : 4LL << 20;
-}
+constexpr long long kSmallPartials = 4LL << 20;    // fp32 values: 16 MB
+constexpr long long kMostPartials = 64LL << 20;    // 256 MB: 32^3, 700 states in two rounds (1284 us of
+                                                   // products with 16 to 64 M values, 1277 in one round)
 static long long half_splits(long long K) { return (K + kMaxAccK / 2 - 1) / (kMaxAccK / 2); }
-int tc_min_splits(long long K, int I, int nsplit) {
+static int tc_min_splits(long long K, int I, int nsplit) {
   const long long z = half_splits(K);
   const long long ldd = (2LL * I + 3) / 4 * 4;
-  return (int)(z * I * ldd <= half_partials(nsplit) ? z : (K + kMaxAccK - 1) / kMaxAccK);
+  return (int)(nsplit == 3 || z * I * ldd <= kSmallPartials ? z : (K + kMaxAccK - 1) / kMaxAccK);
 }
 
 // Scratch (bf16 elements per piece / fp32 partials) for I states of V complex.
-void tc_scratch_sizes(int I, long long V, int num_sms, size_t* piece_a, size_t* piece_b,
+void tc_scratch_sizes(int I, long long V, int num_sms, int nsplit, size_t* piece_a, size_t* piece_b,
                       size_t* piece_rot_a, size_t* partial) {
   const long long K = 2 * V;
   *piece_a = (size_t)I * K;              // also the states' pieces of the recombination
@@ -167,9 +207,8 @@ void tc_scratch_sizes(int I, long long V, int num_sms, size_t* piece_a, size_t* 
   if (z < zacc) z = zacc;
   if (z < 1) z = 1;
   *partial = (size_t)z * I * ldd;
-  // half-length partials of these states, or of fewer, as x6 takes them (a context can
-  // change between the forms)
-  const long long half = half_splits(K) * I * ldd, most = half_partials(3);
+  // half-length partials of these states, or of fewer
+  const long long half = half_splits(K) * I * ldd, most = nsplit == 3 ? kMostPartials : kSmallPartials;
   const size_t need = (size_t)(half < most ? half : most);
   if (*partial < need) *partial = need;
 }
@@ -193,19 +232,30 @@ sky_status tc_overlap(Ctx* c, const void* a, const void* b, int I, double2* X) {
   const int tiles = ((I + tc::BM - 1) / tc::BM) * ((2 * I + tc::BN - 1) / tc::BN);
   // tc_waves 0: the fewest splits the accumulation bound allows (for boxes
   // that share the GPU with others), else about that many waves of SMs
-  int z = c->tc_waves * c->num_sms / tiles;
+  const long long sstride = (long long)I * ldd;
+  const long long fit = (long long)(c->tc_partial_elems / sstride);   // partials at once
+  if (fit < 1) return set_err(c, SKY_EINVAL, "tc overlap: partial buffer too small for I=%d", I);
+  long long z = c->tc_waves * c->num_sms / tiles;
+  if (z > fit) z = fit;
   if (z < tc_min_splits(K, I, n)) z = tc_min_splits(K, I, n);   // bounded FP32 accumulation length
   if (z < 1) z = 1;
-  const long long sstride = (long long)I * ldd;
-  if ((size_t)z * sstride > c->tc_partial_elems) z = (int)(c->tc_partial_elems / sstride);
-  const void* pa[3] = {A[0], A[1], A[2]};
-  const void* pb[3] = {Bp[0], Bp[1], Bp[2]};
-  e = tc::gemm_bf16<false>(pa, K, pb, K, n, I, 2 * I, (int)K, &z, c->d_tcPart, ldd, sstride,
-                    c->d_status, c->stream, c->tc_tile_n);
-  if (e != cudaSuccess) return cuda_check(c, e, "tc overlap gemm");
-  k_tc_overlap_reduce<<<div_up((long long)I * I, 256), 256, 0, c->stream>>>(
-      c->d_tcPart, z, sstride, ldd, I, c->dV, X);
-  note_launch();
+  const long long nkb = (K + tc::BK - 1) / tc::BK, per = (nkb + z - 1) / z;   // K blocks of a partial
+  const long long step = fit * per * tc::BK;
+  for (long long k0 = 0; k0 < K; k0 += step) {
+    const long long k = K - k0 < step ? K - k0 : step;
+    const void *pa[3] = {nullptr}, *pb[3] = {nullptr};
+    for (int i = 0; i < n; ++i) {
+      pa[i] = A[i] + k0;
+      pb[i] = Bp[i] + k0;
+    }
+    int zk = (int)((k + per * tc::BK - 1) / (per * tc::BK));
+    e = tc::gemm_bf16<false>(pa, K, pb, K, n, I, 2 * I, (int)k, &zk, c->d_tcPart, ldd, sstride,
+                             c->d_status, c->stream, c->tc_tile_n);
+    if (e != cudaSuccess) return cuda_check(c, e, "tc overlap gemm");
+    k_tc_overlap_reduce<<<dim3(I, div_up(I, 128)), 128, 0, c->stream>>>(
+        c->d_tcPart, zk, sstride, ldd, I, c->dV, X, k0 > 0);
+    note_launch();
+  }
   return cuda_check(c, cudaGetLastError(), "tc overlap reduce");
 }
 

@@ -216,3 +216,35 @@ def test_diagonalisation_of_three_to_eight_problems(sizes):
     # two more levels of block doubling at most (200 against 128 states), four
     # launches a product and one of its own each
     assert launches[1] <= launches[0] + 2 * (2 * 4 + 1), launches
+
+
+def test_x6_overlap_sums_as_short_for_many_states():
+    """The x6 form's sums are 1024 values long whatever the number of states, also
+    where their partials take several rounds (32^3: from 500 states on): the
+    entries of the first states are those of a call with these alone, the partials
+    the same to the bit, their FP64 sum in another order (128 terms)."""
+    I0, I = 200, 1040
+    g = torch.Generator(device="cuda:0").manual_seed(11)
+    a = torch.randn((I, 2 * 32 ** 3), dtype=torch.complex64, device="cuda:0", generator=g)
+    X = []
+    for n in (I0, I):
+        c = B.sky_init((32, 32, 32), (1.0,) * 3, dict(IN.SLY4), False, (0.0,) * 3, B.SKY_F32_BF16X6, n,
+                       torch.cuda.current_stream().cuda_stream)
+        x = torch.zeros((n, n), dtype=torch.complex128, device="cuda:0")
+        B.sky_overlap(c, a[:n].contiguous(), a[:n].contiguous(), n, x)
+        B.sky_sync(c)
+        B.sky_destroy(c)
+        X.append(x[:I0, :I0].cpu().numpy())
+    assert np.max(np.abs(X[0] - X[1])) < 128 * np.finfo(float).eps * np.max(np.abs(X[0]))
+
+
+@pytest.mark.parametrize("prec", [B.SKY_F32_BF16X3, B.SKY_F32_BF16X6])
+def test_split_bf16_overlap_beyond_the_floats_range(prec):
+    """Partials that are floats, a sum that is not: 2048 products of 2.5e35."""
+    I = 3
+    with TP.Ctx((8, 8, 8), prec=prec, max_states=I) as c:
+        a = torch.full((I, 1024), 5e17 * (1 + 1j), dtype=torch.complex64, device="cuda:0")
+        X = torch.zeros((I, I), dtype=torch.complex128, device="cuda:0")
+        B.sky_overlap(c.ctx, a, a, I, X)
+        v = float(np.float32(5e17)) ** 2 * 2048
+        assert TP.relerr(TP.host(X), np.full((I, I), v, dtype=complex)) < TP.TC_TOL[prec]
