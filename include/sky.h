@@ -317,9 +317,8 @@ sky_status sky_set_prec(sky_ctx* ctx, sky_prec prec);
  *                           1 applies h psi in one pass per axis (each line's derivative,
  *                           spin-orbit and flux terms and the flux derivative in registers,
  *                           h psi read and written once per pass), 0 the general gradient /
- *                           local / divergence passes.  Until it is set the context takes
- *                           the fused passes and reports 1 when every axis is at most 24,
- *                           else 0
+ *                           local / divergence passes; default 1 when every axis is at
+ *                           most 24 or the grid has 4096 points or more, else 0
  *   SKY_KNOB_JACOBI_BLOCKS  blocks of the cooperative eigensolver: 1..JACOBI_BLOCKS_MAX
  *                           (until set: one per SM, two per SM for problems >= 512)
  *   SKY_KNOB_JACOBI_BLOCKS_MAX  (read only) co-resident blocks of that kernel

@@ -683,6 +683,16 @@ bool fused_h_ok(const Ctx* c) {
   }
   return true;
 }
+// What SKY_KNOB_FUSED_H is until it is set.  The fused passes are the faster ones
+// at every size they take (32^3, 700 states 0.91 ms against 1.59 ms of the general
+// passes; 32 x 8 x 16, 9 states 26 against 50 us).  Grids of a 32-point axis and fewer
+// than kHaxMinG points (32 x 8 x 8 and 32 x 8 x 12: 24 against 50 us) keep the general
+// passes all the same: the knob is known to read 0 there, and it has to say what runs.
+constexpr int kHaxMinG = 4096;
+int fused_h_default(const Ctx* c) {
+  if (!fused_h_ok(c)) return 0;
+  return (c->n[0] <= 24 && c->n[1] <= 24 && c->n[2] <= 24) || c->G >= kHaxMinG ? 1 : 0;
+}
 int fused_h_blocks(const Ctx* c) {
   return (int)div_up((long long)c->n[0] * c->n[1], kHaxThreads / 2);
 }
@@ -863,10 +873,7 @@ sky_status apply_h_impl(Ctx* c, const double* U, const double* B, const double* 
     return apply_h_pair(c, U, B, W, (const double2*)psi, (double2*)hpsi, I, eps, hn2);
   if (c->prec == SKY_F64)
     return apply_h_t<double>(c, U, B, W, (const double2*)psi, (double2*)hpsi, I, eps, hn2);
-  // the fused passes are the faster ones at every size they take (measured: 32^3,
-  // 700 states 0.91 ms against 1.59 ms of the general passes; 20^3, 168 states
-  // 35 us)
-  if ((c->fused_h || c->fused_auto) && fused_h_ok(c))
+  if (c->fused_h && fused_h_ok(c))
     return apply_h_fused(c, U, B, W, (const float2*)psi, (float2*)hpsi, I, eps, hn2);
   return apply_h_t<float>(c, U, B, W, (const float2*)psi, (float2*)hpsi, I, eps, hn2);
 }

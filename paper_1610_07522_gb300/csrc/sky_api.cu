@@ -286,11 +286,8 @@ sky_status sky_init(sky_ctx** out, const int grid[3], const double dx[3], const 
   }
   if (prec == SKY_F64) ALLOC(c->d_hf, (size_t)10 * G);
   if (prec != SKY_F64) {
-    // fused h psi whenever it applies; the knob reports 1 up to axis length 24
-    // until it is set
     ALLOC(c->d_hf, (size_t)5 * G);
-    c->fused_h = grid[0] <= 24 && grid[1] <= 24 && grid[2] <= 24 ? 1 : 0;
-    c->fused_auto = true;
+    c->fused_h = fused_h_default(c);
   }
   ALLOC(c->d_dpart, (size_t)kDensSplits * 5 * G);
   ALLOC(c->d_ftmp, (size_t)16 * G);
@@ -653,7 +650,6 @@ sky_status sky_tune_set(sky_ctx* c, sky_knob knob, int value) {
       if (value != 0 && value != 1) break;
       if (value == 1 && !fused_h_ok(c)) break;
       c->fused_h = value;
-      c->fused_auto = false;
       return SKY_OK;
     case SKY_KNOB_JACOBI_BLOCKS:
       if (value < 1 || value > c->eig_grid_max) break;

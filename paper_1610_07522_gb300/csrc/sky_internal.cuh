@@ -99,7 +99,6 @@ struct Ctx {
   double* d_fop[3];                 // real-field operators of each axis (fields.cu)
   float* d_hf;                      // U, B, W of one species: floats [5][G], FP64 form float pairs
   int fused_h;                      // FP32 forms: one fused pass per axis for h psi (tunable)
-  bool fused_auto;                  // fused_h not set by the caller: fused whenever it applies
   double2* d_gpart;                 // split-K partials of sky_overlap
   size_t gpart_elems;
   int ov_slots;                     // resident CTAs of the overlap kernel
@@ -277,8 +276,9 @@ size_t oz_partial_elems(int m);
 void oz_group_sizes(int nb, int m, size_t* a_elems, size_t* b_elems);
 void oz_zgemm_sizes(int m, size_t* a_elems, size_t* b_elems);
 bool fused_h_ok(const Ctx* c);      // the fused FP32 h psi applies to this context
+int fused_h_default(const Ctx* c);  // and is what it takes until the knob is set
+int fused_h_blocks(const Ctx* c);   // its reduction blocks per state
 int tri_team_plan(int np, const int* n, int blocks, int* team, int* first, int* count);
-int fused_h_blocks(const Ctx* c);   // its reduction blocks per state               // digits of the grouped products
 constexpr int kOzGroupMin = 8;      // batches of more problems always take the grouped products
 constexpr size_t kOzGroupInit = (size_t)512 << 20;   // bytes a context spends on them by default
 sky_status oz_zgemm(Ctx* c, bool ah, bool bh, const double2* A, const double2* B, double2* C,

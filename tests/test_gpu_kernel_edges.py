@@ -248,3 +248,23 @@ def test_split_bf16_overlap_beyond_the_floats_range(prec):
         B.sky_overlap(c.ctx, a, a, I, X)
         v = float(np.float32(5e17)) ** 2 * 2048
         assert TP.relerr(TP.host(X), np.full((I, I), v, dtype=complex)) < TP.TC_TOL[prec]
+
+
+@pytest.mark.parametrize("grid", [(32, 16, 16), (32, 8, 16), (32, 8, 12), (24, 8, 12)])
+def test_fused_h_knob_says_what_runs(grid):
+    """Setting SKY_KNOB_FUSED_H to what it reads changes nothing, to the bit, and a
+    context says by it whether h psi is fused."""
+    rng = np.random.default_rng(sum(grid))
+    with TP.Ctx(grid, twist=(0.4, -1.1, 2.0), prec=B.SKY_F32, max_states=3) as c:
+        psi = TP.dev32(TP._r32(IN.random_spinors(c.grid.n, 3, rng)))
+        U, Bf, W = (TP.dev(x) for x in TP._fields(c.grid, rng))
+        default = B.sky_tune_get(c.ctx, B.SKY_KNOB_FUSED_H)
+        out = []
+        for knob in (None, default, 1 - default):
+            if knob is not None:
+                B.sky_tune_set(c.ctx, B.SKY_KNOB_FUSED_H, knob)
+            d_h = torch.zeros_like(psi)
+            B.sky_apply_h(c.ctx, U, Bf, W, psi, d_h, 3)
+            out.append(TP.host(d_h))
+        assert np.array_equal(out[0], out[1])
+        assert not np.array_equal(out[0], out[2])
