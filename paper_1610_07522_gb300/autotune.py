@@ -80,8 +80,14 @@ def tune_box(solver, reps=5, cache=None):
     h = lambda: B.sky_apply_h(ctx, solver.U[q], solver.Bf[q], solver.W[q], solver.psi[q], solver.h[q], I)
     ov = lambda: B.sky_overlap(ctx, solver.psi[q], solver.h[q], I, solver.H[q])
     res = {}
+    # line-pass shapes on the general h psi passes, which use them
+    fused = B.sky_tune_get(ctx, B.SKY_KNOB_FUSED_H)
+    if fused:
+        B.sky_tune_set(ctx, B.SKY_KNOB_FUSED_H, 0)
     for knob in (B.SKY_KNOB_LINE_YZ, B.SKY_KNOB_LINE_X):
         res[NAMES[knob]] = _pick(ctx, knob, CANDIDATES[knob], h, st, reps)
+    if fused:
+        B.sky_tune_set(ctx, B.SKY_KNOB_FUSED_H, fused)
     if solver.prec in TC_FORMS:
         rot = lambda: B.sky_rotate(ctx, solver.phi[q], solver.M[q], I, solver.h[q])
         res[NAMES[B.SKY_KNOB_TC_TILE_N]] = _pick(ctx, B.SKY_KNOB_TC_TILE_N,
