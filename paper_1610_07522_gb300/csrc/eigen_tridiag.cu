@@ -359,6 +359,11 @@ __device__ __forceinline__ void column_factors(const TriStep& st, double2 pj, do
                     fma(c2, uj.y, -fma(st.tau.x, pj.y, st.tau.y * pj.x)));
   fb = make_double2(fma(st.tau.x, uj.x, st.tau.y * uj.y), fma(st.tau.y, uj.x, -st.tau.x * uj.y));
 }
+// w = tau p - c u; with it the update of column j is x - u conj(w_j) - w conj(u_j).
+__device__ __forceinline__ double2 w_entry(const TriStep& st, double2 p, double2 u) {
+  return make_double2(fma(-st.c, u.x, fma(st.tau.x, p.x, -st.tau.y * p.y)),
+                      fma(-st.c, u.y, fma(st.tau.x, p.y, st.tau.y * p.x)));
+}
 // x - u a - p b.
 __device__ __forceinline__ double2 column_update(double2 x, double2 u, double2 p, double2 fa,
                                                  double2 fb) {
@@ -376,6 +381,7 @@ __device__ __forceinline__ double2 column_update(double2 x, double2 u, double2 p
 // The group's first warp ends with reflector t after the last barrier here: its
 // results, u_{t+1} among them, are there after the next one.  False (in every
 // thread) when a wait ran out.
+template <bool ONE>
 __device__ bool tri_heads(const TriBatch& a, const TeamView& tv, const TriHead& h, bool first, int lg,
                           int t, HeadShared& hs, TriStep* s_st, const TriOwn* own) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -439,12 +445,17 @@ __device__ bool tri_heads(const TriBatch& a, const TeamView& tv, const TriHead& 
         TriStep st = prev;
         st.c = st.kap * warp_sum(S0 + S1);
         double2 fa, fb;
-        column_factors(st, pj, uj, fa, fb);
+        if constexpr (!ONE) {
+          column_factors(st, pj, uj, fa, fb);
+        } else {
+          fa = conjx(w_entry(st, pj, uj));
+          fb = conjx(uj);
+        }
         if (lane == 31) {
           hs.at[q][0] = fa;
           hs.at[q][1] = fb;
           prev.c = st.c;
-        } else if (lane < cb && k < kTabProbs) {
+        } else if (!ONE && lane < cb && k < kTabProbs) {
           hs.tab[k][lane][0] = fa;
           hs.tab[k][lane][1] = fb;
         }
@@ -472,7 +483,9 @@ __device__ bool tri_heads(const TriBatch& a, const TeamView& tv, const TriHead& 
     if (hs.timeout[0]) return false;
     if (on) {
       const double2 fa = hs.at[q][0], fb = hs.at[q][1];
+      const TriStep& prev = s_st[b + (size_t)((t + 1) & 1) * kMaxBatch];
       auto row = [&](int i, double2 pi, double2 ci) {
+        if constexpr (ONE) pi = w_entry(prev, pi, vo[i]);
         const double2 y = column_update(ci, vo[i], pi, fa, fb);
         w[i] = pi;
         vn[i] = y;
@@ -599,13 +612,15 @@ __device__ __forceinline__ void tri_unset(const TriBatch& a, const TeamView& tv,
 // A column's rows go to `parts` warps in turn.  The first shares are begun while
 // the first warps of the last ng groups of heads are at reflector t (so those get
 // theirs last), and row t + 1 of u is added after the barrier.
+template <bool ONE>
 __device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, int ng, double2* dsm,
                          double* contrib, HeadShared& hs, const TriStep* s_st, TriOwn* own) {
   const int G = tv.G, np = tv.p1 - tv.p0, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int grp = wid >> lg;
   const int rank = grp >= ng ? wid - ng
                              : (wid & ((1 << lg) - 1)) == 0 ? kTriWarps - ng + grp : wid - grp - 1;
-  if ((wid & ((1 << lg) - 1)) == 0) __threadfence();   // see kUnset
+  // see kUnset (a team of one block reads its words behind its own barrier)
+  if (!ONE && (wid & ((1 << lg) - 1)) == 0) __threadfence();
   int C = 0, mmax = 0;
   for (int k = 0; k < np; ++k) {
     C += active_cols(own[k], t);
@@ -647,7 +662,10 @@ __device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, i
       }
       double2 fa = make_double2(0.0, 0.0), fb = fa;
       if (upd) {
-        if (k < kTabProbs && rest < kTabCols) {
+        if constexpr (ONE) {
+          fa = conjx(w[j]);
+          fb = conjx(vo[j]);
+        } else if (k < kTabProbs && rest < kTabCols) {
           fa = hs.tab[k][rest][0];
           fb = hs.tab[k][rest][1];
         } else {
@@ -703,9 +721,9 @@ __device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, i
       }
       __syncthreads();
     }
-    if (c0 == 0 && wid != 0) tri_unset(a, tv, t, own);
-    if (wid == 0)
-      for (int cj = lane; cj < cols; cj += 32) {
+    if (!ONE && c0 == 0 && wid != 0) tri_unset(a, tv, t, own);
+    if (ONE || wid == 0)
+      for (int cj = ONE ? (int)threadIdx.x : lane; cj < cols; cj += ONE ? kTriThreads : 32) {
         int k, rest;
         find(c0 + cj, k, rest);
         const int b = a.tmem[tv.p0 + k], n = own[k].n, j = own[k].j0 + (own[k].smin + rest) * G;
@@ -729,11 +747,25 @@ __device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, i
       }
     if (c0 + kBodyItems < C) __syncthreads();
   }
-  // per-problem partials, one lane per problem, own columns in order; the next
-  // step's first own columns
+  // per-problem partials, one lane per problem, own columns in order (one block has
+  // all columns: one warp per problem); the next step's first own columns
+  if constexpr (ONE) {
+    __syncthreads();
+    for (int k = wid; k < np; k += kTriWarps) {
+      if (t > own[k].n - 2) continue;
+      int first = 0;
+      for (int kq = 0; kq < k; ++kq) first += active_cols(own[kq], t);
+      const int cb = active_cols(own[k], t);
+      double acc = 0.0;
+      for (int i = lane; i < cb; i += 32) acc += contrib[first + i];
+      acc = warp_sum(acc);
+      if (lane == 0) put_word(sp_row(a, a.tmem[tv.p0 + k], t) + tv.gb, acc);
+    }
+    __syncthreads();                         // smin is read above
+  }
   if (wid != 0) return;
   __syncwarp();
-  for (int k = lane; k < np; k += 32) {
+  for (int k = lane; k < np && !ONE; k += 32) {
     TriOwn& o = own[k];
     if (t > o.n - 2) continue;
     int first = 0;
@@ -746,6 +778,40 @@ __device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, i
   __syncwarp();
   for (int k = lane; k < np; k += 32)
     if (own[k].smin < own[k].ns && own[k].j0 + own[k].smin * G < t + 2) ++own[k].smin;
+}
+
+// All steps of a team.  False when a wait ran out.  ONE: a team of one block, which
+// has every column.  It reads its own words behind its barrier (nothing to unset, no
+// fence), takes w instead of p (one entry per row; factors per column cost 10 FP64
+// instructions for each of up to hundreds of columns), and all its warps finish
+// the columns and sum the partials (one warp did, column after column: 8400 cycles of
+// a step at 125 columns).  One 100-state problem per block: 3.09 ms as the
+// teams of several blocks do it, 2.70 ms; 128 problems of 37 to 290 states: 17.4 and
+// 14.8 ms.
+template <bool ONE>
+__device__ bool tri_steps(const TriBatch& a, const TeamView& tv, int nrun, double2* dsm, double* contrib,
+                          HeadShared& hs, TriStep* s_st, TriOwn* own) {
+  const int tid = threadIdx.x, np = tv.p1 - tv.p0;
+  TriHead h{};
+  int seen = -1;
+  for (int t = 0; t < nrun; ++t) {
+    const int nact = count_active(own, np, t);
+    const int lg = nact == 1 ? 4 : nact == 2 ? 3 : 2;
+    const int per = kTriWarps >> lg;
+    int last = 0;                            // problems of the last round of heads
+    for (int r0 = 0; r0 < nact; r0 += per) {
+      if (r0 > 0) __syncthreads();
+      if (nact != seen || nact > per) h = head_of(a, tv, own, t, r0 + (tid >> (5 + lg)), dsm);
+      seen = nact;
+      if (!tri_heads<ONE>(a, tv, h, r0 == 0, lg, t, hs, s_st, own)) return false;
+      last = nact - r0 < per ? nact - r0 : per;
+    }
+    tri_body<ONE>(a, tv, t, lg, last, dsm, contrib, hs, s_st, own);
+    // (the next step's first loads wait for this one's values of every block)
+    __syncthreads();
+    if (tv.gb == t % tv.G) tri_store(a, tv, t, dsm, s_st, own);
+  }
+  return true;
 }
 
 __global__ void __launch_bounds__(kTriThreads, 1) k_hh_tridiag(TriBatch a) {
@@ -804,25 +870,9 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_hh_tridiag(TriBatch a) {
   } else if (!blocks_barrier(tv.bar, epoch, (unsigned)tv.G, a.status, a.spins)) {
     return;
   }
-  TriHead h{};
-  int seen = -1;
-  for (int t = 0; t < nrun; ++t) {
-    const int nact = count_active(own, np, t);
-    const int lg = nact == 1 ? 4 : nact == 2 ? 3 : 2;
-    const int per = kTriWarps >> lg;
-    int last = 0;                            // problems of the last round of heads
-    for (int r0 = 0; r0 < nact; r0 += per) {
-      if (r0 > 0) __syncthreads();
-      if (nact != seen || nact > per) h = head_of(a, tv, own, t, r0 + (tid >> (5 + lg)), dsm);
-      seen = nact;
-      if (!tri_heads(a, tv, h, r0 == 0, lg, t, hs, s_st, own)) return;
-      last = nact - r0 < per ? nact - r0 : per;
-    }
-    tri_body(a, tv, t, lg, last, dsm, contrib, hs, s_st, own);
-    // (the next step's first loads wait for this one's values of every block)
-    __syncthreads();
-    if (tv.gb == t % tv.G) tri_store(a, tv, t, dsm, s_st, own);
-  }
+  if (!(tv.G == 1 ? tri_steps<true>(a, tv, nrun, dsm, contrib, hs, s_st, own)
+                  : tri_steps<false>(a, tv, nrun, dsm, contrib, hs, s_st, own)))
+    return;
   if (tv.gb == 0 && tid == 0) {
     long long k = 0;
     for (int q = 0; q < np; ++q) k += own[q].n > 0;
