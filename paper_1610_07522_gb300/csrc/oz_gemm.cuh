@@ -440,15 +440,20 @@ __device__ __forceinline__ void oz_gemm_body(const OzArgs& a, const OzGroup* grp
 
   if (warp == 0) {
     // stage layout: A slices 0..S-1, then B slices 0..S-1.  Lane 0 arms the
-    // stage's barrier and copies B; lane i copies run i % 3 (a row tile of A) of
-    // slice i / 3.
+    // stage's barrier and copies B (a partly filled tile of B: lane i slice i of
+    // it); lane i copies run i % 3 (a row tile of A) of slice i / 3.
     static_assert(3 * S <= 32 && 2 * BNT >= BM, "runs of A");
     long long g = 0;
     bool ok = true;
     for (int w = 0, t; (t = item_index(w)) >= 0 && ok; ++w) {
       OzItem it;
       if (!item_at<GROUP>(a, grp, BNT, t, it)) continue;
-      const int end = it.m0 + BM < it.nta * BNT ? it.m0 + BM : it.nta * BNT;   // rows that exist
+      // rows that hold an operand's, in whole groups of 8 (the padding of a tile
+      // is not fetched: 32^3, 5 FP32 states, whose tiles of B are 9/10 padding, one
+      // overlap 160 us with it, 132 us)
+      const int ma = (it.M + 7) & ~7, mb = (it.N - it.n0 + 7) & ~7;
+      const int end = it.m0 + BM < ma ? it.m0 + BM : ma;
+      const int rows_b = mb < BNT ? mb : BNT;
       const int p = lane / 3, ta = it.m0 / BNT + lane % 3;
       const int lo = ta * BNT > it.m0 ? ta * BNT : it.m0;
       const int hi = (ta + 1) * BNT < end ? (ta + 1) * BNT : end;
@@ -468,10 +473,13 @@ __device__ __forceinline__ void oz_gemm_body(const OzArgs& a, const OzGroup* grp
         }
         const uint32_t sa = smem_u32(base + s * STAGE);
         if (lane == 0) {
-          mbar_expect_tx(full(s), (uint32_t)(S * (end - it.m0) * (BK * 2) + S * TILE_B));
-          bulk_load(sa + S * TILE_A, srcB, S * TILE_B, full(s));
+          mbar_expect_tx(full(s), (uint32_t)(S * (end - it.m0 + rows_b) * (BK * 2)));
+          if (rows_b == BNT) bulk_load(sa + S * TILE_A, srcB, S * TILE_B, full(s));
         }
         __syncwarp();
+        if (rows_b < BNT && lane < S)
+          bulk_load(sa + S * TILE_A + lane * TILE_B, srcB + lane * (BNT * BK), (uint32_t)(rows_b * (BK * 2)),
+                    full(s));
         if (mine) bulk_load(sa + dstA, srcA, (uint32_t)((hi - lo) * (BK * 2)), full(s));
       }
     }
