@@ -155,7 +155,7 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool v
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// 2^k as a float, k in [-128, 127] (-127, -128: subnormal).
+// 2^k as a float, k in [-150, 128] (subnormal below -126, 0 at -150, infinity at 128).
 __device__ __forceinline__ float pow2f(int k) {
   return __int_as_float(k >= -126 ? (k + 127) << 23 : 0x00400000 >> (-127 - k));
 }
@@ -208,8 +208,11 @@ __device__ __forceinline__ dd pair_of_groups(float g0, float g1, float g2, float
   const dd t = two_sum(a.hi, u.hi);
   return fast_two_sum(t.hi, __fadd_rn(t.lo, __fadd_rn(u.lo, __fadd_rn(b.lo, g4))));
 }
-// An exponent whose power of two pow2f forms (pairs beyond it have no FP32 value).
-__device__ __forceinline__ int clamp_exp(int k) { return k < -128 ? -128 : k > 127 ? 127 : k; }
+// An exponent whose power of two pow2f forms: what is beyond the floats becomes 0 or
+// infinity.
+__device__ __forceinline__ int clamp_exp(int k) { return k < -150 ? -150 : k > 128 ? 128 : k; }
+// exp_of for the lines of pairs, whose smallest values may be subnormal.
+__device__ __forceinline__ int exp_of_pair(float x) { return x == 0.0f ? INT_MIN : max(exp_of(x), -126); }
 __device__ __forceinline__ unsigned bf16x2(float lo, float hi) {   // lo in the low half
   unsigned r;
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
@@ -472,7 +475,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_deriv(const DerivArgs a) {
       int E = INT_MIN;
 #pragma unroll
       for (int j = 0; j < H0; ++j) {
-        if constexpr (IN == kInPair) E = max(E, max(exp_of(v[j].x), exp_of(v[j].z)));
+        if constexpr (IN == kInPair) E = max(E, max(exp_of_pair(v[j].x), exp_of_pair(v[j].z)));
         else E = max(E, max(exp_of(v[j].x), exp_of(v[j].y)));
       }
       if constexpr (PF) {
@@ -491,7 +494,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_deriv(const DerivArgs a) {
         break;
       }
       if (hh == 0) s_ea[slot * BM + r] = E;
-      const float sc = IN == kInPair ? pow2f(-(E < 128 ? E : 128)) : 1.0f;   // pairs: |E| <= 129
+      const float sc = IN == kInPair ? pow2f(-E) : 1.0f;   // pairs: -126 <= E <= 129
       unsigned char* ta = ring + s * STAGE;
 #pragma unroll
       for (int c = 0; c < H0 / 4; ++c) {

@@ -268,3 +268,24 @@ def test_fused_h_knob_says_what_runs(grid):
             out.append(TP.host(d_h))
         assert np.array_equal(out[0], out[1])
         assert not np.array_equal(out[0], out[2])
+
+
+def _decaying_states(g, I, rng):
+    """States that fall off to 1e-16 of their largest value and below."""
+    r2 = np.meshgrid(*[(np.arange(n) - n / 2.0) ** 2 for n in g.shape], indexing="ij")
+    return IN.random_spinors(g.n, I, rng) * np.exp(-sum(r2) / 8.0)
+
+
+@pytest.mark.parametrize("grid", [(12, 16, 20), (32, 24, 8)])
+@pytest.mark.parametrize("power", [-100, -64, 64, 100])
+def test_fp64_h_psi_scales_with_the_states(grid, power):
+    """States times a power of two: h psi times it at the bound of the unscaled call,
+    though float pairs hold it between the passes (lines below 2^-126 among them)."""
+    rng = np.random.default_rng(power + 200)
+    I, s = 4, 2.0 ** power
+    with TP.Ctx(grid, twist=(0.3, -0.2, 0.7), max_states=I) as c:
+        psi = _decaying_states(c.grid, I, rng)
+        U, Bf, W = TP._fields(c.grid, rng)
+        d_h = torch.zeros(psi.shape, dtype=torch.complex128, device="cuda:0")
+        B.sky_apply_h(c.ctx, TP.dev(U), TP.dev(Bf), TP.dev(W), TP.dev(psi * s), d_h, I)
+        assert TP.relerr(TP.host(d_h) / s, O.apply_h(psi, U, Bf, W, c.grid)) < 1e-12
