@@ -945,6 +945,26 @@ sky_status damped_step_impl(Ctx* c, int q, const void* psi, const void* hpsi,
                          x0, E0, w);
 }
 
+// The terms of one state at one point in FP64.
+__device__ __forceinline__ void dens_terms(double2 a0, double2 a1, const double2 (&d0)[3],
+                                           const double2 (&d1)[3], double& rho, double& tau, double& jx,
+                                           double& jy, double& jz) {
+  rho += a0.x * a0.x + a0.y * a0.y + a1.x * a1.x + a1.y * a1.y;
+  double imx[3], imy[3], imz[3];   // Im M_{x,j}, Im M_{y,j}, Im M_{z,j}
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    tau += d0[j].x * d0[j].x + d0[j].y * d0[j].y + d1[j].x * d1[j].x + d1[j].y * d1[j].y;
+    const double2 c01 = cmulc(a0, d1[j]), c10 = cmulc(a1, d0[j]);   // conj(a0) d1, conj(a1) d0
+    const double2 c00 = cmulc(a0, d0[j]), c11 = cmulc(a1, d1[j]);
+    imx[j] = c01.y + c10.y;
+    imy[j] = c10.x - c01.x;
+    imz[j] = c00.y - c11.y;
+  }
+  jx += imz[1] - imy[2];
+  jy += imx[2] - imz[0];
+  jz += imy[0] - imx[1];
+}
+
 // ------------------------------------------------------------ densities
 // Partial rho, tau, J over the states of one split:
 //   M_kj = psi^+ sigma_k G_j, J_x = Im M_zy - Im M_yz, J_y = Im M_xz - Im M_zx,
@@ -995,22 +1015,9 @@ __global__ void __launch_bounds__(128) k_dens_accum(const cx<T>* __restrict__ ps
   } else {
   for (int s = s_beg; s < s_end; ++s) {
     const long long o0 = (long long)s * 2 * G + p, o1 = o0 + G;
-    const double2 a0 = to_d2(psi[o0]), a1 = to_d2(psi[o1]);
-    rho += a0.x * a0.x + a0.y * a0.y + a1.x * a1.x + a1.y * a1.y;
-    double imx[3], imy[3], imz[3];   // Im M_{x,j}, Im M_{y,j}, Im M_{z,j}
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const double2 d0 = to_d2(gs[j][o0]), d1 = to_d2(gs[j][o1]);
-      tau += d0.x * d0.x + d0.y * d0.y + d1.x * d1.x + d1.y * d1.y;
-      const double2 c01 = cmulc(a0, d1), c10 = cmulc(a1, d0);   // conj(a0) d1, conj(a1) d0
-      const double2 c00 = cmulc(a0, d0), c11 = cmulc(a1, d1);
-      imx[j] = c01.y + c10.y;
-      imy[j] = c10.x - c01.x;
-      imz[j] = c00.y - c11.y;
-    }
-    jx += imz[1] - imy[2];
-    jy += imx[2] - imz[0];
-    jz += imy[0] - imx[1];
+    const double2 d0[3] = {to_d2(gs[0][o0]), to_d2(gs[1][o0]), to_d2(gs[2][o0])};
+    const double2 d1[3] = {to_d2(gs[0][o1]), to_d2(gs[1][o1]), to_d2(gs[2][o1])};
+    dens_terms(to_d2(psi[o0]), to_d2(psi[o1]), d0, d1, rho, tau, jx, jy, jz);
   }
   }
   double* dst = part + (long long)blockIdx.y * 5 * G;
@@ -1052,7 +1059,9 @@ struct AccD {
 // route): rho in FP64 from psi itself (four operations per state and point), tau
 // and J, whose gradients carry 48 bits, as sums of pair products on the FP32 pipe
 // (36 products; some 85 FP64 operations per state and point bound the pass
-// before: densities of 24^3, 280 states 889 us, now 464).
+// before: densities of 24^3, 280 states 889 us, now 464).  Where a point's sums
+// leave the range in which floats hold a product and its error (2^-90 .. 2^100: far
+// below the noise of normalised states) they are formed again in FP64.
 __global__ void __launch_bounds__(128) k_dens_accum_pair(const double2* __restrict__ psi,
                                                          const float4* __restrict__ g0,
                                                          const float4* __restrict__ g1,
@@ -1092,12 +1101,25 @@ __global__ void __launch_bounds__(128) k_dens_accum_pair(const double2* __restri
     az.re_cj<1>(a1, x0); az.re_cj<-1>(a0, x1);
     az.im_cj<-1>(a0, y1); az.im_cj<-1>(a1, y0);
   }
+  double rho = (r[0] + r[1]) + (r[2] + r[3]), tau = ta.value(), jx = ax.value(), jy = ay.value(),
+         jz = az.value();
+  if (!(rho > 0x1p-90 && rho < 0x1p100 && ta.hi > 0x1p-90f && ta.hi < 0x1p100f) &&
+      !(rho == 0.0 && ta.hi == 0.0f)) {
+    rho = tau = jx = jy = jz = 0.0;
+    auto full = [](float4 v) { return make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w); };
+    for (int s = s_beg; s < s_end; ++s) {
+      const long long o0 = (long long)s * 2 * G + p, o1 = o0 + G;
+      const double2 d0[3] = {full(g0[o0]), full(g1[o0]), full(g2[o0])};
+      const double2 d1[3] = {full(g0[o1]), full(g1[o1]), full(g2[o1])};
+      dens_terms(psi[o0], psi[o1], d0, d1, rho, tau, jx, jy, jz);
+    }
+  }
   double* dst = part + (long long)blockIdx.y * 5 * G;
-  dst[p] = (r[0] + r[1]) + (r[2] + r[3]);
-  dst[G + p] = ta.value();
-  dst[2 * G + p] = ax.value();
-  dst[3 * G + p] = ay.value();
-  dst[4 * G + p] = az.value();
+  dst[p] = rho;
+  dst[G + p] = tau;
+  dst[2 * G + p] = jx;
+  dst[3 * G + p] = jy;
+  dst[4 * G + p] = jz;
 }
 
 // Sum the splits in order; accumulate onto the outputs after the first chunk.

@@ -289,3 +289,21 @@ def test_fp64_h_psi_scales_with_the_states(grid, power):
         d_h = torch.zeros(psi.shape, dtype=torch.complex128, device="cuda:0")
         B.sky_apply_h(c.ctx, TP.dev(U), TP.dev(Bf), TP.dev(W), TP.dev(psi * s), d_h, I)
         assert TP.relerr(TP.host(d_h) / s, O.apply_h(psi, U, Bf, W, c.grid)) < 1e-12
+
+
+@pytest.mark.parametrize("grid", [(12, 16, 20), (32, 24, 8)])
+@pytest.mark.parametrize("power", [-100, -64, 64, 100])
+def test_fp64_densities_scale_with_the_states(grid, power):
+    """States times a power of two: the densities times its square at the bounds of
+    the unscaled call (1e-12, and 1e-11 for div J, one more derivative), also where
+    the products of the gradients leave the range of the floats."""
+    rng = np.random.default_rng(power + 200)
+    I, s = 4, 2.0 ** power
+    with TP.Ctx(grid, twist=(0.3, -0.2, 0.7), max_states=I) as c:
+        g = c.grid
+        psi = _decaying_states(g, I, rng)
+        z = lambda n: torch.zeros(n, dtype=torch.float64, device="cuda:0")
+        got = [z(g.G), z(g.G), z(3 * g.G), z(g.G)]
+        B.sky_densities(c.ctx, TP.dev(psi * s), I, *got)
+        for x, w, tol in zip(got, O.densities(psi, g), (1e-12, 1e-12, 1e-12, 1e-11)):
+            assert TP.relerr(TP.host(x) / s / s, w.ravel()) < tol
