@@ -307,3 +307,65 @@ def test_fp64_densities_scale_with_the_states(grid, power):
         B.sky_densities(c.ctx, TP.dev(psi * s), I, *got)
         for x, w, tol in zip(got, O.densities(psi, g), (1e-12, 1e-12, 1e-12, 1e-11)):
             assert TP.relerr(TP.host(x) / s / s, w.ravel()) < tol
+
+
+@pytest.mark.parametrize("grid", [(48, 8, 12), (8, 64, 8), (12, 16, 48), (64, 48, 16)])
+@pytest.mark.parametrize("coulomb", [True, False])
+def test_real_fields_on_long_axes(grid, coulomb):
+    """The direct sums of the real-field derivatives and of the Coulomb transform up
+    to their longest axes, at the bounds of the short ones (the parity test of the
+    same calls)."""
+    rng = np.random.default_rng(sum(grid))
+    with TP.Ctx(grid, dx=(0.9, 1.0, 1.1), coulomb=coulomb, prec=B.SKY_F32, max_states=2) as c:
+        g = c.grid
+        rho = np.stack([0.08 + 0.01 * IN.random_smooth_field(g.n, rng, 0.0, 1.0) for _ in range(2)])
+        tau, dJ = 0.6 * rho, 0.1 * rho - 0.005
+        U_w, B_w, W_w = O.mean_fields(rho, tau, dJ, TP.P, g, coulomb)
+        E_w = O.energy(rho, tau, dJ, TP.P, g, coulomb)
+        z = lambda *n: torch.zeros(n, dtype=torch.float64, device="cuda:0")
+        U, Bf, W, out = z(2, g.G), z(2, g.G), z(2, 3, g.G), z(8)
+        B.sky_mean_fields(c.ctx, TP.dev(rho), TP.dev(tau), TP.dev(dJ), U, Bf, W)
+        B.sky_energy(c.ctx, TP.dev(rho), TP.dev(tau), TP.dev(dJ), out)
+        assert TP.relerr(TP.host(U), U_w.reshape(2, -1)) < 1e-11
+        assert TP.relerr(TP.host(Bf), B_w.reshape(2, -1)) < 1e-12
+        assert TP.relerr(TP.host(W), W_w.reshape(2, 3, -1)) < 1e-11
+        for e, k in zip(TP.host(out), ["total", "kin", "rho", "tau", "drho", "nJ", "coul", "A"]):
+            assert abs(e - E_w[k]) <= 1e-11 * max(1.0, abs(E_w[k])), k
+        psi = TP.dev32(TP._r32(IN.random_spinors(g.n, 2, rng)))
+        r, t, J, d = z(g.G), z(g.G), z(3 * g.G), z(g.G)
+        B.sky_densities(c.ctx, psi, 2, r, t, J, d)
+        Jh = TP.host(J).reshape((3,) + g.shape)
+        assert TP.relerr(TP.host(d), sum(O.deriv_real(Jh[j], j, g) for j in range(3)).ravel()) < 1e-11
+
+
+@pytest.mark.parametrize("grid,I", [((24, 24, 24), 231), ((32, 32, 32), 97)])
+def test_fp32_fused_h_in_uneven_chunks(grid, I):
+    """More states than a chunk of the fused h psi holds (227 at 24^3, 96 at 32^3):
+    two chunks, the last one smaller; states on both sides of the seam against the
+    oracle, every state against the same states alone (the same arithmetic)."""
+    rng = np.random.default_rng(I)
+    with TP.Ctx(grid, twist=(1.3, -0.2, 0.9), prec=B.SKY_F32, max_states=I) as c:
+        g = c.grid
+        B.sky_tune_set(c.ctx, B.SKY_KNOB_FUSED_H, 1)
+        psi = TP._r32(IN.random_spinors(g.n, I, rng))
+        U, Bf, W = TP._fields(g, rng)
+        d_psi, fields = TP.dev32(psi), [TP.dev(x) for x in (U, Bf, W)]
+
+        def run(a, b):
+            d_h = torch.zeros_like(d_psi[a:b])
+            e = torch.zeros(b - a, dtype=torch.float64, device="cuda:0")
+            n2 = torch.zeros_like(e)
+            B.sky_apply_h(c.ctx, *fields, d_psi[a:b].contiguous(), d_h, b - a, e, n2)
+            return TP.host(d_h), TP.host(e), TP.host(n2)
+
+        h, e, n2 = run(0, I)
+        seam = (I + 1) // 2
+        for a, b in ((0, 60), (seam - 30, seam + 30), (I - 60, I)):
+            for got, want in zip(run(a, b), (h, e, n2)):
+                assert np.array_equal(got, want[a:b])
+        for s in (0, seam - 1, seam, I - 1):
+            want = O.apply_h(psi[s:s + 1], U, Bf, W, g)
+            ew, nw = O.sp_energies(psi[s:s + 1], want, g)
+            assert TP.relerr(h[s:s + 1], want) < TP.REL32
+            assert TP.relerr(e[s:s + 1], ew) < TP.REL32
+            assert TP.relerr(n2[s:s + 1], nw) < TP.REL32
