@@ -1383,7 +1383,11 @@ __global__ void __launch_bounds__(kBackWarps * 32) k_hh_back(TriBatch a, int zst
 // and residuals stay what they were (128 to 1000 states, dense and nearly diagonal
 // matrices: 6e-15 to 6e-14 sqrt(n), both ways).
 constexpr int kWyBlock = 64;
-constexpr int kWyMin = 128;            // smallest largest problem of a batch it is used for
+// It is used from kWyMin states on (one diagonalisation, reflectors one by one and
+// compact WY: 160 states 2.13 and 2.17 ms, 192 2.60 and 2.58, 256 3.51 and 3.21), and
+// from kWyManyMin states on in batches of kWyMany states in all (6 of 128: 2.79 and
+// 2.82 ms, 12 of 128: 2.32 and 2.26 ms).
+constexpr int kWyMin = 192, kWyManyMin = 128, kWyMany = 1536;
 
 struct WyJobs {
   double2* P[kMaxBatch];               // in: row t = v_t; out: row t = v_t^H
@@ -1857,7 +1861,7 @@ static sky_status tri_group(Ctx* c, int np, const int* idx, const double2* const
   note_launch(5);
   // the products by tensor cores, unless the batch is gated (skipped products
   // still cost their launches) or its problems are small
-  if (!run && nmax >= kWyMin) {
+  if (!run && (nmax >= kWyMin || (nmax >= kWyManyMin && ntot >= kWyMany))) {
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_check(c, e, "tridiagonal eigensolver");
     return wy_back(c, np, idx, n, Z, a);
   }

@@ -280,7 +280,10 @@ int fused_h_default(const Ctx* c);  // and is what it takes until the knob is se
 int fused_h_blocks(const Ctx* c);   // its reduction blocks per state
 int tri_team_plan(int np, const int* n, int blocks, int* team, int* first, int* count);
 constexpr int kOzGroupMin = 8;      // batches of more problems always take the grouped products
-constexpr size_t kOzGroupInit = (size_t)512 << 20;   // bytes a context spends on them by default
+// bytes a context spends on them by default, for the products of two species: enough
+// for 1064 states (41 MiB at 290, 219 MiB at 700).  Beyond, one by one costs little
+// (1100 + 700 states, one diagonalisation: 36.5 ms grouped, 38.3 ms).
+constexpr size_t kOzGroupInit = (size_t)512 << 20;
 sky_status oz_zgemm(Ctx* c, bool ah, bool bh, const double2* A, const double2* B, double2* C,
                     int n, const int* run, const int* stop, int slices = 6);
 sky_status tc_rotate(Ctx* c, const void* phi, const double2* M, int I, void* out);
