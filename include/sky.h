@@ -81,7 +81,12 @@ typedef struct {
  * SKY_ENOMEM / SKY_ECUDA on failure with *out = NULL.  With the environment
  * variable SKY_FILL_SCRATCH_NAN=1, every device buffer a context allocates
  * (here or later) starts filled with 0xFF bytes, NaN in every floating-point
- * format: a check that no kernel reads scratch it has not written. */
+ * format: a check that no kernel reads scratch it has not written.
+ * Besides what scales with the states, a context of 96 states or more owns the
+ * digit buffers of four I x I products (two species, two products at once: 41 MiB
+ * at 290 states, 219 MiB at 700, none beyond 512 MiB); the split-BF16 forms own
+ * FP32 partials of the overlap (at least those of 2048-value sums, for x6 up to
+ * 256 MiB of 1024-value sums). */
 sky_status sky_init(sky_ctx** out, const int grid[3], const double dx[3],
                     const sky_skyrme* params, const double twist[3],
                     sky_prec prec, int max_states, void* stream);
@@ -144,8 +149,10 @@ int sky_tri_team_plan(int np, const int* n, int blocks, int* team, int* first, i
  * spinors, must not overlap.  eps (nullable, [I]) receives <psi|h|psi>,
  * hnorm2 (nullable, [I]) receives <h psi|h psi> (= <psi|h^2|psi>), both
  * with the volume element dx^3 (FP32 forms: sums of exact float products kept
- * in float pairs, about 2^-48 of the sum per term, totals in FP64).  Stored as
- * the paper's hampsi (Sec. 3.4). */
+ * in float pairs, about 2^-48 of the sum per term, totals in FP64).  The FP64
+ * form's operator products (SKY_KNOB_LINE_ARITH 2) keep what passes between
+ * their kernels in float pairs too: 48 bits, states of 2^-100 to 2^100.  Stored
+ * as the paper's hampsi (Sec. 3.4). */
 sky_status sky_apply_h(sky_ctx* ctx, const double* U, const double* B, const double* W,
                        const void* psi, void* hpsi, int I, double* eps, double* hnorm2);
 

@@ -87,7 +87,6 @@ struct TriBatch {
   int run_stride;
   double* sp;                    // per problem slot: [2][gridDim.x] partials of Re(v^H p)
   size_t sp_stride;
-  unsigned* bar;
   int* status;
   long long spins;
   long long* stats;
@@ -1837,7 +1836,7 @@ static sky_status tri_group(Ctx* c, int np, const int* idx, const double2* const
   a.T = c->d_trid; a.tslot = c->tri_slot; a.m = c->tri_m;
   a.sp = c->d_eigpart; a.sp_stride = (size_t)kTriBufs * c->eig_grid_max;
   a.run = run; a.run_stride = run_stride;
-  a.bar = c->d_bar; a.status = c->d_status; a.spins = c->wait_spins; a.stats = c->d_stats;
+  a.status = c->d_status; a.spins = c->wait_spins; a.stats = c->d_stats;
   // run flags are indexed by the batch position of each problem
   if (run) {
     bool ident = true;

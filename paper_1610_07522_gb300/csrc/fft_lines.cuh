@@ -244,8 +244,8 @@ __global__ void __launch_bounds__(kLineThreads) k_line_yz(Op op, LineGeom g) {
 // Lines along x: a block stages blockDim.x (<= kLinesX) consecutive lines
 // through shared memory.  Consecutive x lines are consecutive in memory, also
 // from one array to the next, so element e of the block is element
-// s_r[0] N + e counted from the start of the first line's array: no division
-// per element, and up to kXChunk bytes of loads in flight per thread (one load
+// i0 + e counted from the start of the first line's array (i0 its first line's
+// first point): no division per element, and up to kXChunk bytes of loads in flight per thread (one load
 // per round trip to memory had bound the pass: 32^3, 700 FP32 states, 316 us
 // with one, 214 us with eight, 194 us with 32; the y pass takes 107 us).
 constexpr int kXChunk = 256;

@@ -515,10 +515,6 @@ sky_status oz_zgemm(Ctx* c, bool ah, bool bh, const double2* A, const double2* B
                            : oz_zgemm_t<oz::kS64, oz::kBN64>(c, ah, bh, A, B, C, n, run, stop);
 }
 
-// The products C_b = opA(A_b) opB(B_b) of every problem of a batch (n_b <=
-// the context's state count) in one grouped launch sequence: two digit
-// splits, one tensor-core launch over all problems' tiles, one reduction
-// (the per-problem form above, stacked; gates per problem).
 // Operand buffer sizes (elements) of one product of m states with the given
 // digits; of the larger of both forms; and of the grouped products of nb problems
 // of up to m.
@@ -558,6 +554,10 @@ bool oz_zgemm_group_fits(const Ctx* c, int np, const int* n, int slices) {
   return rows <= c->ozg_rows && ae <= c->ozg_a_elems && be <= c->ozg_b_elems && p <= (long long)c->ozg_p_elems;
 }
 
+// The products C_b = opA(A_b) opB(B_b) of every problem of a batch (n_b <=
+// the context's state count) in one grouped launch sequence: two digit
+// splits, one tensor-core launch over all problems' tiles, one reduction
+// (the per-problem form above, stacked; gates per problem).
 template <int S, int BN>
 static sky_status oz_zgemm_group_t(Ctx* c, const ZJobs& j) {
   cudaStream_t st = c->stream;

@@ -148,7 +148,8 @@ struct Ctx {
   size_t oz_a_elems, oz_b_elems, oz_p_elems;
   // grouped I x I products of a batched eigensolve (oz_zgemm_group): digits of
   // every problem's operands, partials, row exponents (ozg_rows stacked rows);
-  // allocated by sky_reserve_batch for batches of more than kOzGroupMin problems
+  // allocated at creation for two species of kOzZgemmMin states or more (up to
+  // kOzGroupInit bytes), by sky_reserve_batch for larger batches
   void* d_ozgA;
   void* d_ozgB;
   float2* d_ozgP;
