@@ -461,7 +461,13 @@ __device__ __forceinline__ void oz_gemm_body(const OzArgs& a, const OzGroup* grp
       const long long ka = (long long)it.nta * S * (BNT * BK), kb = (long long)it.ntb * S * (BNT * BK);
       const unsigned short* srcA =
           it.A + it.kb0 * ka + ((long long)ta * S + p) * (BNT * BK) + (long long)(lo - ta * BNT) * BK;
-      const unsigned short* srcB = it.B + it.kb0 * kb + (long long)(it.n0 / BNT) * S * (BNT * BK);
+      const bool whole_b = rows_b == BNT;
+      const unsigned short* srcB = it.B + it.kb0 * kb + (long long)(it.n0 / BNT) * S * (BNT * BK) +
+                                   (whole_b ? 0 : lane * (BNT * BK));
+      const uint32_t dstB = (uint32_t)(S * TILE_A + (whole_b ? 0 : lane * TILE_B));
+      const uint32_t bytes_b = whole_b ? (lane == 0 ? S * TILE_B : 0) : (lane < S ? rows_b * (BK * 2) : 0);
+      const uint32_t bytes_a = mine ? (hi - lo) * (BK * 2) : 0;
+      const uint32_t bytes = S * (end - it.m0 + rows_b) * (BK * 2);
       const uint32_t dstA = (uint32_t)(p * TILE_A + (lo - it.m0) * (BK * 2));
       for (int j = 0; j < it.nkb; ++j, ++g, srcA += ka, srcB += kb) {
         const int s = (int)(g % STAGES);
@@ -472,15 +478,10 @@ __device__ __forceinline__ void oz_gemm_body(const OzArgs& a, const OzGroup* grp
           break;
         }
         const uint32_t sa = smem_u32(base + s * STAGE);
-        if (lane == 0) {
-          mbar_expect_tx(full(s), (uint32_t)(S * (end - it.m0 + rows_b) * (BK * 2)));
-          if (rows_b == BNT) bulk_load(sa + S * TILE_A, srcB, S * TILE_B, full(s));
-        }
+        if (lane == 0) mbar_expect_tx(full(s), bytes);
         __syncwarp();
-        if (rows_b < BNT && lane < S)
-          bulk_load(sa + S * TILE_A + lane * TILE_B, srcB + lane * (BNT * BK), (uint32_t)(rows_b * (BK * 2)),
-                    full(s));
-        if (mine) bulk_load(sa + dstA, srcA, (uint32_t)((hi - lo) * (BK * 2)), full(s));
+        if (bytes_b) bulk_load(sa + dstB, srcB, bytes_b, full(s));
+        if (bytes_a) bulk_load(sa + dstA, srcA, bytes_a, full(s));
       }
     }
   } else if (warp == 1) {
