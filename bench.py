@@ -662,13 +662,13 @@ NPROD = {0: 21, 1: 10, 2: 3, 3: 6}
 # apply_h; profiles/), divided by its I.  Keyed by (workload, form); absent
 # until captured for the current kernels.
 HPSI_TRAFFIC_PER_SPINOR = {
-    # 2.784 GB over the 8 kernels of one I = 280 call (profiles/sky_apply_h_sly4_24cubed_280n_fp64.md)
-    ("sly4_24cubed_280n120p_coulomb_fp64", "fp64"): 2784466176.0 / 280,
+    # 2.456 GB over the 8 kernels of one I = 280 call (profiles/sky_apply_h_sly4_24cubed_280n_fp64.md)
+    ("sly4_24cubed_280n120p_coulomb_fp64", "fp64"): 2455737856.0 / 280,
 }
 # ncu dram__bytes_read.sum + dram__bytes_write.sum of one k_oz_deriv launch
-# along y over the 560 neutron spin components of the 24^3 workload
-# (profiles/k_oz_deriv_sly4_24cubed_280n_fp64.md): 124.2 + 71.5 MB
-DERIV_TRAFFIC = {("sly4_24cubed_280n120p_coulomb_fp64", "fp64"): 195.7e6}
+# along y over the 560 neutron spin components of the 24^3 workload (bench.py
+# --probe-call derivative; profiles/k_oz_deriv_sly4_24cubed_280n_fp64.md): 124.0 + 64.4 MB
+DERIV_TRAFFIC = {("sly4_24cubed_280n120p_coulomb_fp64", "fp64"): 188.4e6}
 
 
 def derivative_roofline(dev, w, prec, peaks, form, reps=20):
@@ -774,7 +774,8 @@ def call_rooflines(events, grid, prec, peaks, csize):
         by = sum(I for I, _, _ in ev) * b1 / len(ev)
         pk = peaks["fp64" if prec == 0 else "fp32"]
         out["apply_h"] = {
-            "kernel": "sky_apply_h (line-pass FFTs, k_h_local, k_h_sum)",
+            "kernel": ("sky_apply_h (k_oz_deriv operator passes, k_h_local_pair, k_h_totals)" if prec == 0
+                       else "sky_apply_h (fused line passes k_h_axis_*, or the general line passes)"),
             "bound": "alu", "unit": "TFLOP/s", "avg_call_ms": ms,
             "mean_I": sum(I for I, _, _ in ev) / len(ev),
             "achieved": fl / (ms / 1e3) / 1e12, "peak": pk,
@@ -871,6 +872,8 @@ def probe_call(args):
     n0 = B.sky_kernel_launches()
     if args.probe_call == "apply_h":
         B.sky_apply_h(ctx, U, Bf, W, psi, out, I)
+    elif args.probe_call == "derivative":     # the launch that derivative_roofline times
+        B.sky_derivative(ctx, 1, psi, out, 2 * I)
     elif args.probe_call == "overlap":
         B.sky_overlap(ctx, psi, psi, I, X)
     elif args.probe_call == "rotate":
@@ -1167,7 +1170,7 @@ def main():
                     help="skip the time-dependent stepping leg")
     ap.add_argument("--no-convergence", action="store_true",
                     help="skip the time-to-convergence comparison of the forms")
-    ap.add_argument("--probe-call", default=None, choices=["apply_h", "overlap", "rotate", "ritz", "batched"],
+    ap.add_argument("--probe-call", default=None, choices=["apply_h", "derivative", "overlap", "rotate", "ritz", "batched"],
                     help="run one library call on the workload's shapes and exit (for ncu)")
     ap.add_argument("--line-arith", type=int, default=None, choices=[0, 1],
                     help="--probe-call only: FP64 form's derivative line passes in FP64 (0) "
