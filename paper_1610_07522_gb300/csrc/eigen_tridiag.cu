@@ -59,7 +59,7 @@ constexpr int kWinChunks = (2 * kWinMax + 1 + 31) / 32;
 constexpr int kBackWarps = 16;
 constexpr size_t kTriSmemMax = 200 * 1024;   // dynamic shared memory of k_hh_tridiag / k_hh_back
 constexpr double kEps = 2.220446049250313e-16;
-constexpr int kTriBufs = 4;             // buffers of the published vectors (see unset)
+constexpr int kTriBufs = 8;             // buffers of the published vectors (see unset)
 constexpr int kTeamBarStride = 32;     // unsigned between team barrier counters (128 bytes)
 
 struct TriBatch {
@@ -233,18 +233,20 @@ __device__ __forceinline__ double* sp_row(const TriBatch& a, int b, int t) {
 // signalling NaN that no arithmetic returns.  That is one trip through L2 per
 // step, where a barrier costs the writers' fence, its counter, the poll and then
 // the loads: 7.9 -> 7.4 us a step at 120 states, 13.2 -> 12.5 us at 700 when it came.
-// The values of step t are in buffer t mod 4; while step t is under way its owners
-// unset their words of buffer t + 2 mod 4, last read at step t - 1.  Two things
-// order that, both by one fence of the heads' first warps (the ones that read and
-// publish the partials) between the heads of a step and its partials:
-//  - everyone is past those reads: each block's fence stands between its reads of
-//    step t - 1 and its partial of that step, and the partials were read here, a
-//    fence and a barrier before the unsetting;
-//  - nobody takes an old word of buffer t + 2 for a new one: its reads come at step
-//    t + 3, behind the fence and the barrier of step t + 2, whose head read the
-//    owner's partial of step t + 1, which the owner published after the barrier
-//    behind the unsetting and the fence of step t + 1.
-// Every wait is bounded.
+// The values of step t are in buffer t mod kTriBufs; while step t is under way its
+// owners unset their words of the buffer of step t + 4, which held those of step t - 4.
+// Two fences a step order that, both where their warps would only wait: (F) the warp
+// that publishes the partials (the last one) before its shares, (A) the warps that
+// read the partials (the heads' first ones) behind the shares.
+//  - Everyone has read step t - 4: each block did in the head of step t - 3, its F and
+//    its partial of that step follow; that partial was read here in the head of step
+//    t - 2; A and a barrier of that step precede the unsetting.
+//  - Nobody takes an old word for one of step t + 4: the unsetting, a barrier, F and
+//    the partial of step t + 1; the others read that in the head of step t + 2, then A
+//    and a barrier, and look for the words of step t + 4 in the head of step t + 5.
+// (One fence between the heads and the shares, in the heads' first warps, with four
+// buffers: it stands behind the reflector's scalars and costs 1 to 5 % of the
+// reduction.)  Every wait is bounded.
 constexpr unsigned long long kUnset = 0x7FF4000000C0FFEEull;
 __device__ __forceinline__ double unset() { return __longlong_as_double((long long)kUnset); }
 __device__ __forceinline__ bool is_unset(double x) {
@@ -586,22 +588,22 @@ __device__ void tri_store(const TriBatch& a, const TeamView& tv, int t, double2*
   }
 }
 
-// This block's words of buffer t + 2 mod kTriBufs, by the warps other than the
-// first: p of its columns, its partials, and as the owner of column t + 3 that.
+// This block's words of the buffer of step t + 4, by the warps other than the last:
+// p of its columns, its partials, and as the owner of column t + 5 that.
 __device__ __forceinline__ void tri_unset(const TriBatch& a, const TeamView& tv, int t,
                                           const TriOwn* own) {
-  const int tid = (int)threadIdx.x - 32;
+  const int tid = (int)threadIdx.x;
   for (int k = 0; k < tv.p1 - tv.p0; ++k) {
     const int b = a.tmem[tv.p0 + k], n = own[k].n;
-    if (t + 2 > n - 2) continue;             // step t + 2 publishes nothing
+    if (t + 4 > n - 2) continue;             // step t + 4 publishes nothing
     const TriPtrs p = tri_ptrs(a, b);
-    const size_t o = (size_t)((t + 2) & (kTriBufs - 1)) * a.m;
+    const size_t o = (size_t)((t + 4) & (kTriBufs - 1)) * a.m;
     const double2 no = make_double2(unset(), unset());
     for (int s = tid; s < own[k].ns; s += kTriThreads - 32)
       put_word(p.P + o + own[k].j0 + s * tv.G, no);
-    if (tid == kTriThreads - 33) put_word(sp_row(a, b, t + 2) + tv.gb, unset());
-    if ((t + 3 + a.rot[b]) % tv.G == tv.gb)
-      for (int i = t + 3 + tid; i < n; i += kTriThreads - 32) put_word(p.C + o + i, no);
+    if (tid == kTriThreads - 33) put_word(sp_row(a, b, t + 4) + tv.gb, unset());
+    if ((t + 5 + a.rot[b]) % tv.G == tv.gb)
+      for (int i = t + 5 + tid; i < n; i += kTriThreads - 32) put_word(p.C + o + i, no);
   }
 }
 
@@ -618,8 +620,9 @@ __device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, i
   const int grp = wid >> lg;
   const int rank = grp >= ng ? wid - ng
                              : (wid & ((1 << lg) - 1)) == 0 ? kTriWarps - ng + grp : wid - grp - 1;
-  // see kUnset (a team of one block reads its words behind its own barrier)
-  if (!ONE && (wid & ((1 << lg) - 1)) == 0) __threadfence();
+  // F of kUnset (a team of one block reads its words behind its own barrier)
+  constexpr int kLast = kTriWarps - 1;
+  if (!ONE && wid == kLast) __threadfence();
   int C = 0, mmax = 0;
   for (int k = 0; k < np; ++k) {
     C += active_cols(own[k], t);
@@ -720,8 +723,11 @@ __device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, i
       }
       __syncthreads();
     }
-    if (!ONE && c0 == 0 && wid != 0) tri_unset(a, tv, t, own);
-    if (ONE || wid == 0)
+    if (!ONE && c0 == 0 && wid != kLast) {
+      if ((wid & ((1 << lg) - 1)) == 0) __threadfence();   // A of kUnset
+      tri_unset(a, tv, t, own);
+    }
+    if (ONE || wid == kLast)
       for (int cj = ONE ? (int)threadIdx.x : lane; cj < cols; cj += ONE ? kTriThreads : 32) {
         int k, rest;
         find(c0 + cj, k, rest);
@@ -762,7 +768,7 @@ __device__ void tri_body(const TriBatch& a, const TeamView& tv, int t, int lg, i
     }
     __syncthreads();                         // smin is read above
   }
-  if (wid != 0) return;
+  if (wid != kLast) return;
   __syncwarp();
   for (int k = lane; k < np && !ONE; k += 32) {
     TriOwn& o = own[k];

@@ -346,7 +346,7 @@ sky_status sky_init(sky_ctx** out, const int grid[3], const double dx[3], const 
     c->eig_grid_max = jacobi_max_grid(c);
     c->eig_grid = c->eig_grid_max < c->num_sms ? c->eig_grid_max : c->num_sms;   // one per SM
     c->eig_grid_auto = true;
-    ALLOC(c->d_eigpart, (size_t)4 * c->eig_grid_max * kMaxBatch);
+    ALLOC(c->d_eigpart, (size_t)8 * c->eig_grid_max * kMaxBatch);
   }
 #undef ALLOC
   if (s == SKY_OK) {

@@ -245,7 +245,7 @@ cudaError_t damp_tc(Ctx* c, int q, const double2* psi, const double2* hpsi, cons
                     double2* phi, int I, double x0, const float* w);
 bool tri_vectors_global(int n);
 size_t tri_vec_elems(int m, int nb, int nsm);
-inline size_t tri_slot_doubles(int m) { return (size_t)m * m + 26 * (size_t)m; }
+inline size_t tri_slot_doubles(int m) { return (size_t)m * m + 42 * (size_t)m; }
 sky_status eigh_impl(Ctx* c, const double2* A, int I, double* w, double2* Z,
                      const int* run = nullptr);
 sky_status lowdin_impl(Ctx* c, const double2* S, int I, double2* C);

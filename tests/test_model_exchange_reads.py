@@ -1,17 +1,17 @@
 """CPU model of the exchange of the tridiagonal reduction (values that are their
-own flags, four buffers in turn, unset two steps ahead) with loads that may be
-served early as well as stores that may be seen late: between two fences of a
-block a load may return what memory held at any time since the first of them.
+own flags, eight buffers in turn, unset four steps ahead) with loads that may be
+served early as well as stores that may be seen late.
 
-A block at step t: wait for everyone's partial of step t-1, take everyone's words
-of that step, fence, unset its word of step t+2's buffer, publish its word and
-its partial of step t.  The fence both orders the unsetting of step t-1 and the
-reads before the partial and keeps later loads behind the partials read."""
+A block at step t: wait for everyone's partial of step t-1, take everyone's words of
+that step; a fence of the warp that publishes the partials, behind which nothing
+stored before stays unseen; publish the step's word and partial, unset the word of
+step t+4's buffer; a fence of the warps that read the partials, behind which (and the
+step's last barrier) no load of the next step is served early."""
 import random
 
 import pytest
 
-BUFS = 4
+BUFS, AHEAD = 8, 4
 
 
 def run(blocks, steps, seed, acquire):
@@ -23,7 +23,7 @@ def run(blocks, steps, seed, acquire):
             for b in range(blocks):
                 hist[k, s, b] = [(0, None)]
     pending = [[] for _ in range(blocks)]     # stores not yet seen, any order between fences
-    since = [0] * blocks                       # time of the block's last fence
+    since = [0] * blocks                       # time of the block's last reading fence
     pc = [("part", 0, 0)] * blocks
     end, now = 0, 0
 
@@ -58,13 +58,15 @@ def run(blocks, steps, seed, acquire):
         elif what == "fence":
             if pending[g]:
                 continue                       # what was stored before is seen first
+            pc[g] = ("store", t, 0)
+        elif what == "store":
+            if t + AHEAD < steps:
+                pending[g] += [((k, (t + AHEAD) % BUFS, g), None) for k in ("word", "part")]
+            pending[g] += [((k, t % BUFS, g), (t, g)) for k in ("word", "part")]
+            pc[g] = ("acquire", t, 0)
+        else:
             if acquire:
                 since[g] = now                 # later loads stay behind
-            pc[g] = ("store", t, 0)
-        else:
-            if t + 2 < steps:
-                pending[g] += [((k, (t + 2) % BUFS, g), None) for k in ("word", "part")]
-            pending[g] += [((k, t % BUFS, g), (t, g)) for k in ("word", "part")]
             if t + 1 == steps:
                 pc[g] = ("end", t, 0)
                 end += 1
@@ -73,12 +75,12 @@ def run(blocks, steps, seed, acquire):
     return True
 
 
-@pytest.mark.parametrize("blocks,steps", [(2, 30), (3, 30), (5, 20)])
-def test_one_fence_per_step_orders_the_exchange(blocks, steps):
-    assert all(run(blocks, steps, seed, True) for seed in range(40))
+@pytest.mark.parametrize("blocks,steps", [(2, 40), (3, 40), (5, 30)])
+def test_the_fences_of_a_step_order_the_exchange(blocks, steps):
+    assert all(run(blocks, steps, seed, True) for seed in range(60))
 
 
 def test_ordered_stores_alone_are_not_enough():
-    """A fence that orders the stores only: a word of four steps ago passes for a
+    """A fence that orders the stores only: a word of eight steps ago passes for a
     new one."""
-    assert not all(run(3, 30, seed, False) for seed in range(40))
+    assert not all(run(3, 40, seed, False) for seed in range(60))
