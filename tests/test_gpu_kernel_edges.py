@@ -367,3 +367,53 @@ def test_fp32_fused_h_in_uneven_chunks(grid, I):
             assert TP.relerr(h[s:s + 1], want) < TP.REL32
             assert TP.relerr(e[s:s + 1], ew) < TP.REL32
             assert TP.relerr(n2[s:s + 1], nw) < TP.REL32
+
+
+def test_x6_overlap_of_a_context_made_for_x3():
+    """A context keeps the partial buffer of the form it was made for: after
+    sky_set_prec the x6 overlap takes it in rounds (24^3, 400 states: two) and gives
+    what an x6 context gives, but for the FP64 sum of 54 terms in another order."""
+    I, X = 400, []
+    g = torch.Generator(device="cuda:0").manual_seed(5)
+    a = torch.randn((I, 2 * 24 ** 3), dtype=torch.complex64, device="cuda:0", generator=g)
+    for first in (B.SKY_F32_BF16X3, B.SKY_F32_BF16X6):
+        c = B.sky_init((24, 24, 24), (1.0,) * 3, dict(IN.SLY4), False, (0.0,) * 3, first, I,
+                       torch.cuda.current_stream().cuda_stream)
+        B.sky_set_prec(c, B.SKY_F32_BF16X6)
+        x = torch.zeros((I, I), dtype=torch.complex128, device="cuda:0")
+        B.sky_overlap(c, a, a, I, x)
+        B.sky_sync(c)
+        B.sky_destroy(c)
+        X.append(x.cpu().numpy())
+    assert np.max(np.abs(X[0] - X[1])) < 54 * np.finfo(float).eps * np.max(np.abs(X[0]))
+
+
+@pytest.mark.parametrize("sizes", [(129, 100), (97, 60), (200, 193)])
+def test_subspace_of_two_problems_with_their_loewdin_factors(sizes):
+    """C from S, then M from C^H H C, both for two problems at once: M^H S M = I and
+    M^H H M = diag(lambda) with the eigenvalues of the pencil (H, S).  Bounds: the
+    grouped products' 1e-12 of the largest entry, five factors in a row, and the
+    reduction's 1e-12 ||H||."""
+    from scipy.linalg import eigh
+
+    rng = np.random.default_rng(sum(sizes))
+    c = TE._ctx(max(sizes))
+    S, H = [], []
+    for n in sizes:
+        a = rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))
+        S.append(np.eye(n) + 0.1 / np.sqrt(n) * (a + a.conj().T))
+        H.append(_hermitian("random", n, rng))
+    z = lambda n: torch.zeros((n, n), dtype=torch.complex128, device="cuda:0")
+    C, M = [z(n) for n in sizes], [z(n) for n in sizes]
+    lam = [torch.zeros(n, dtype=torch.float64, device="cuda:0") for n in sizes]
+    B.sky_orthonormalize_batched(c, [TE._dev(x) for x in S], list(sizes), C)
+    B.sky_subspace_diag_batched(c, [TE._dev(x) for x in H], C, list(sizes), M, lam)
+    B.sky_sync(c)
+    B.sky_destroy(c)
+    for s, h, m, w in zip(S, H, M, lam):
+        m, w = m.cpu().numpy(), w.cpu().numpy()
+        lw = eigh(h, s, eigvals_only=True)
+        nrm = float(np.max(np.abs(lw)))
+        assert np.max(np.abs(w - lw)) < 5e-12 * nrm
+        assert np.max(np.abs(m.conj().T @ s @ m - np.eye(len(w)))) < 5e-12
+        assert np.max(np.abs(m.conj().T @ h @ m - np.diag(w))) < 5e-12 * nrm
