@@ -450,7 +450,7 @@ __device__ __forceinline__ void oz_gemm_body(const OzArgs& a, const OzGroup* grp
       if (!item_at<GROUP>(a, grp, BNT, t, it)) continue;
       // rows that hold an operand's, in whole groups of 8 (the padding of a tile
       // is not fetched: 32^3, 5 FP32 states, whose tiles of B are 9/10 padding, one
-      // overlap 160 us with it, 132 us)
+      // overlap 160 us with it, 127 us)
       const int ma = (it.M + 7) & ~7, mb = (it.N - it.n0 + 7) & ~7;
       const int end = it.m0 + BM < ma ? it.m0 + BM : ma;
       const int rows_b = mb < BNT ? mb : BNT;
